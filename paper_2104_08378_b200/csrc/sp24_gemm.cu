@@ -11,10 +11,11 @@
 //            owns the tensor-memory allocation;
 //   warps 2-9 epilogue, two per tensor-memory lane quarter taking alternate 32-column boxes:
 //            tcgen05.ld accumulator -> registers (the next box's load already under way), alpha /
-//            beta / conversion in registers, then one of two forms.  Row-major 2-byte outputs: the
-//            warps load C and store D themselves, through small per-warp transposing buffers, and
-//            hand the accumulators back as soon as their last box is in registers.  Other outputs:
-//            a staging box per warp, C boxes TMA-loaded a few boxes ahead, TMA store of the D box.
+//            beta / conversion in registers, then one of two forms.  4-byte row-major outputs: a
+//            staging box per warp, C boxes TMA-loaded a few boxes ahead, TMA store of the D box, if
+//            shared memory has room for the boxes.  All others: the warps load C and store D
+//            themselves, through small per-warp transposing buffers, and hand the accumulators back
+//            as soon as their last box is in registers.
 // CTAS == 2 runs a pair of CTAs (cluster of two): each CTA loads its 128 rows of A / metadata per
 // m-block and its half of B, CTA 0 issues cta_group::2 MMAs (M = 256) for both.
 // MBLK == 2 gives every CTA two m-blocks (two accumulators, one B tile): what an SM can pull in
@@ -120,7 +121,7 @@ struct Cfg {
   static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
   static_assert(kMinStagesFit >= 2, "need at least two stages");
   // the epilogue moves 32-column boxes; a last box of 16 columns (240-column tiles) is handled only by
-  // the epilogue for row-major outputs, which bounds every access by the tile's last column
+  // epilogue_direct, which bounds every access by the tile's last column
   static_assert(BLOCK_N % 16 == 0, "tile width");
   static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte alignment of the atoms");
   static_assert(kECol + (SPARSE ? 2 * MBLK * 8 : 0) <= (int)kTmemCols, "tensor memory overflow");
@@ -211,14 +212,26 @@ __device__ __forceinline__ float2 unpack_16bit(uint32_t w, bool bf) {
 }
 
 // One thread's row of a 32-column box: out = alpha * acc + beta * c (or the dequantising form) as
-// the packed words of the output row: 16 words for 2-byte outputs (CS = 2), 32 for 4-byte ones.
+// the packed words of the output row: 8 words for 1-byte outputs (CS = 1: the dequantising form),
+// 16 for 2-byte outputs (CS = 2), 32 for 4-byte ones.
 // `c` holds the row's C values in the same packing and is read only if has_c.  One multiply and
 // one fused multiply-add per element, whichever path stores the row.
 template <int KIND, int CS>
 __device__ __forceinline__ void compute_row(const uint32_t (&r)[32], const uint32_t (&c)[8 * CS], bool has_c,
                                             const GemmParams& p, float scale, float bias, uint32_t (&o)[8 * CS]) {
   const bool bf = p.cd_type == SP24_BF16;
-  if constexpr (CS == 4) {
+  if constexpr (CS == 1) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      uint32_t word = 0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int q = requant_i8(dequant_value(r[4 * e + b], scale, bias, p.relu), p.out_inv_scale);
+        word |= ((uint32_t)q & 0xFFu) << (8 * b);
+      }
+      o[e] = word;
+    }
+  } else if constexpr (CS == 4) {
     if (KIND == 1 && p.dequant) {
 #pragma unroll
       for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(dequant_value(r[e], scale, bias, p.relu));
@@ -280,100 +293,36 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
     *reinterpret_cast<uint4*>(row + ((v ^ (lane & 7)) << 4)) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
 }
 
-// int8 output of the dequantising epilogue: rows of 32 bytes, no swizzle
-__device__ __forceinline__ void convert_row_dequant_i8(const uint32_t (&r)[32], uint8_t* buf, int lane, const GemmParams& p,
-                                                       float scale, float bias) {
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    uint32_t w[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      uint32_t word = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        int q = requant_i8(dequant_value(r[16 * v + 4 * e + b], scale, bias, p.relu), p.out_inv_scale);
-        word |= ((uint32_t)q & 0xFFu) << (8 * b);
-      }
-      w[e] = word;
-    }
-    *reinterpret_cast<uint4*>(buf + lane * 32 + v * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// Column-major output of the dequantising epilogue: box transposed in the staging buffer.
-__device__ __forceinline__ void convert_row_dequant_transposed(const uint32_t (&r)[32], uint8_t* buf, int lane,
-                                                               const GemmParams& p, float scale, float bias) {
-#pragma unroll
-  for (int n = 0; n < 32; ++n) {
-    const float y = dequant_value(r[n], scale, bias, p.relu);
-    if (p.cd_type == SP24_F32) {
-      *reinterpret_cast<float*>(buf + n * 128 + ((((lane >> 2) ^ (n & 7))) << 4) + (lane & 3) * 4) = y;
-    } else if (p.cd_type == SP24_I8) {
-      *reinterpret_cast<int8_t*>(buf + n * 32 + lane) = (int8_t)requant_i8(y, p.out_inv_scale);
-    } else {
-      uint16_t* u = reinterpret_cast<uint16_t*>(buf + n * 64 + ((((lane >> 3) ^ ((n >> 1) & 3))) << 4) + (lane & 7) * 2);
-      if (p.cd_type == SP24_BF16) {
-        __nv_bfloat16 o = __float2bfloat16_rn(y);
-        *u = *reinterpret_cast<uint16_t*>(&o);
-      } else {
-        __half o = __float2half_rn(y);
-        *u = *reinterpret_cast<uint16_t*>(&o);
-      }
-    }
-  }
-}
-
-// Column-major C / D: the staging buffer holds the box transposed (32 rows of n, m contiguous), so
-// this thread's 32 values go to 32 different rows, one element each.
-template <int KIND>
-__device__ __forceinline__ void convert_row_transposed(const uint32_t (&r)[32], uint8_t* buf, int lane,
-                                                       const GemmParams& p) {
-  const bool wide = KIND == 1 || p.cd_type == SP24_F32;
-#pragma unroll
-  for (int n = 0; n < 32; ++n) {
-    if (wide) {
-      uint32_t* u = reinterpret_cast<uint32_t*>(buf + n * 128 + ((((lane >> 2) ^ (n & 7))) << 4) + (lane & 3) * 4);
-      if (KIND == 1) {
-        *u = r[n] + (p.has_c ? *u : 0u);
-      } else {
-        float f = p.alpha * __uint_as_float(r[n]);
-        if (p.has_c) f += p.beta * __uint_as_float(*u);
-        *u = __float_as_uint(f);
-      }
-    } else {
-      uint16_t* u = reinterpret_cast<uint16_t*>(buf + n * 64 + ((((lane >> 3) ^ ((n >> 1) & 3))) << 4) + (lane & 7) * 2);
-      float f = p.alpha * __uint_as_float(r[n]);
-      if (p.cd_type == SP24_BF16) {
-        if (p.has_c) f += p.beta * __bfloat162float(*reinterpret_cast<__nv_bfloat16*>(u));
-        __nv_bfloat16 o = __float2bfloat16_rn(f);
-        *u = *reinterpret_cast<uint16_t*>(&o);
-      } else {
-        if (p.has_c) f += p.beta * __half2float(*reinterpret_cast<__half*>(u));
-        __half o = __float2half_rn(f);
-        *u = *reinterpret_cast<uint16_t*>(&o);
-      }
-    }
-  }
-}
-
-// ---- epilogue for row-major C / D of 2- or 4-byte elements ------------------------------------
-// The epilogue warps move C and D themselves.  C: every thread loads the 32 values of ITS
-// accumulator row straight from global memory into registers, the first boxes of a tile before
-// the tile's accumulators are even complete, the later ones a few boxes ahead, so that no load
-// latency is left on the path that holds the accumulators (tensor memory cannot be handed back to
-// the MMA issuer before it is drained).  D: the row is converted in registers, written to a small
-// per-warp buffer in shared memory and read back transposed, so that the global stores of a warp
-// cover whole 64-byte row segments.  A "pass" is 32 rows x 64 bytes (2 KB): a whole box of a 2-byte
-// type, half a box of a 4-byte type.
-template <int KIND, int CS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
-__device__ __forceinline__ void epilogue_rows(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
+// ---- epilogue in which the warps move C and D themselves -----------------------------------------
+// C is loaded straight from global memory into registers, the first boxes of a tile before the
+// tile's accumulators are even complete, the later ones a few boxes ahead, so that no load latency
+// is left on the path that holds the accumulators (tensor memory cannot be handed back to the MMA
+// issuer before it is drained).
+// Row-major outputs: each thread loads the C values of ITS accumulator row; D: the row is converted
+// in registers, written to a small per-warp buffer in shared memory and read back transposed, so
+// that the global stores of a warp cover whole 64-byte row segments.  A "pass" is 32 rows x 64 bytes
+// (2 KB): a whole box of a 1- or 2-byte type, half a box of a 4-byte type.
+// Column-major outputs (D stored [N][M], M contiguous): the lanes of a warp hold 32 consecutive m of
+// each column, so a 4-byte box is stored straight from registers, one 128-byte line per column; the
+// 1- and 2-byte boxes are transposed on the way out of the same per-warp buffer by ldmatrix.trans.
+// The eight rows of ldmatrix matrix i are m = 8 j + 2 i + b (j = 0..3, b = 0, 1), which leaves each
+// thread with eight consecutive m of one column (2-byte) or of two columns (1-byte): 16- and 8-byte
+// stores.  16-byte unit u of buffer row m sits at u ^ (((m >> 1) ^ (m >> 3)) & 3): no bank conflicts
+// in the row-wise writes, the row-wise reads or the ldmatrix reads.
+// Measured against TMA boxes with scalar shared-memory stores (one 1-2 KB box per warp in flight, each
+// store waited for): int8 3072 x 4096 x 768 -> int8 44.7 -> 17.3 us, fp8 16384 x 8192 x 8192 -> bf16
+// 600 -> 514 us, the 3x3 convolution 50176 pixels x 256 x 2304 46.7 -> 36 us (with 240-column tiles, which
+// this form can store), int8 4096 x 32 x 4096 -> bf16 10.7 -> 9.0 us.
+template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
+__device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
                                               int lane) {
   constexpr int kSub = (BLOCK_N + 31) / 32, kIters = MBLK * kSub;  // the last box of a 240-column tile is half a box
   constexpr int kBoxes = (kIters + 1) / 2;  // boxes per warp and tile (the two warps of a lane quarter alternate)
   constexpr int W = 8 * CS;                 // 32-bit words of one box row
   constexpr int P = CS == 2 ? 4 : 1;        // boxes whose C values are held in registers (16 or 32 registers each)
-  constexpr int kPasses = CS / 2;
+  constexpr int kPasses = CS == 4 ? 2 : 1;
+  constexpr int kUnits = CS == 1 ? 2 : 4;   // 16-byte units of a buffer row that hold data
   constexpr int kUnitElems = 16 / CS;       // elements per 16-byte unit
   const int q = warp & 3, ew = warp - kFirstEpiWarp, half = ew >> 2;
   const int nbuf = p.epi_bytes >= kEpiWarps * 4096 ? 2 : 1;
@@ -382,7 +331,11 @@ __device__ __forceinline__ void epilogue_rows(const GemmParams& p, Shared* sh, u
   uint8_t* Db = static_cast<uint8_t*>(p.D);
   const size_t ldc_b = (size_t)p.ldc * CS, ldd_b = (size_t)p.ldd * CS;
   const int M = (int)p.M, N = (int)p.N;
-  const bool has_c = p.has_c != 0;
+  const bool has_c = CS != 1 && p.has_c != 0;
+  // ldmatrix / stmatrix: this lane's row m of the buffer (its unit 0 under the swizzle: xor the unit into bits 4..5)
+  const int tm_i = lane >> 3, tm_j = (lane & 7) >> 1;
+  const uint32_t tm_row = ptx::smem_u32(stage) + (uint32_t)((8 * tm_j + 2 * tm_i + (lane & 1)) * 64 + ((tm_i ^ tm_j) << 4));
+  const int sw = ((lane >> 1) ^ (lane >> 3)) & 3;  // swizzle of buffer row `lane`
   uint32_t creg[P][W];
   int acc = 0;
   uint32_t acc_phase = 0, pass_no = 0;
@@ -402,6 +355,27 @@ __device__ __forceinline__ void epilogue_rows(const GemmParams& p, Shared* sh, u
     auto load_c = [&](int n, uint32_t (&c)[W]) {
       int row0, col0, tcol;
       if (!geom(n, row0, col0, tcol)) return;
+      if constexpr (COLS) {
+        if constexpr (CS == 2) {
+          const int m = row0 + 8 * (lane & 3);
+          if (m >= M) return;
+#pragma unroll
+          for (int nb = 0; nb < 4; ++nb) {
+            const int n1 = col0 + 8 * nb + (lane >> 2);
+            if (n1 < col_end) {
+              const uint4 x = *reinterpret_cast<const uint4*>(Cb + (size_t)n1 * ldc_b + (size_t)m * CS);
+              c[4 * nb] = x.x; c[4 * nb + 1] = x.y; c[4 * nb + 2] = x.z; c[4 * nb + 3] = x.w;
+            }
+          }
+        } else if constexpr (CS == 4) {
+          if (row0 + lane >= M) return;
+          const uint8_t* src = Cb + (size_t)col0 * ldc_b + (size_t)(row0 + lane) * CS;
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (col0 + e < col_end) c[e] = *reinterpret_cast<const uint32_t*>(src + (size_t)e * ldc_b);
+        }
+        return;
+      }
       const int row = row0 + lane;
       if (row >= M) return;
       const uint4* src = reinterpret_cast<const uint4*>(Cb + (size_t)row * ldc_b + (size_t)col0 * CS);
@@ -447,7 +421,24 @@ __device__ __forceinline__ void epilogue_rows(const GemmParams& p, Shared* sh, u
       int row0, col0, tcol;
       const bool live = geom(n, row0, col0, tcol);  // same answer for the whole warp
       uint32_t o[W];
+      const uint32_t buf_off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
       if (live) {
+        if constexpr (CS == 2 && COLS) {
+          if (has_c) {
+            // C arrived in the order of the column stores: through the buffer to the rows' owners
+            if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
+            uint32_t (&c)[W] = creg[n % P];
+#pragma unroll
+            for (int nb = 0; nb < 4; ++nb)
+              ptx::stmatrix_x4_trans((tm_row + buf_off) ^ (uint32_t)(nb << 4), c[4 * nb], c[4 * nb + 1], c[4 * nb + 2], c[4 * nb + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const uint4 x = *reinterpret_cast<const uint4*>(stage + buf_off + lane * 64 + ((u ^ sw) << 4));
+              c[4 * u] = x.x; c[4 * u + 1] = x.y; c[4 * u + 2] = x.z; c[4 * u + 3] = x.w;
+            }
+          }
+        }
         uint32_t (&r)[32] = racc[n & 1];
         if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
         float scale = 1.f, bias = 0.f;
@@ -460,22 +451,56 @@ __device__ __forceinline__ void epilogue_rows(const GemmParams& p, Shared* sh, u
       }
       // the C registers of box n are free: fetch box n + P into them (also when box n lies outside the matrix)
       if (has_c && n + P < kBoxes) load_c(n + P, creg[n % P]);
-      if (live) {
+      if (!live) continue;
+      if constexpr (CS == 4 && COLS) {
+        if (row0 + lane < M) {
+          uint8_t* dst = Db + (size_t)col0 * ldd_b + (size_t)(row0 + lane) * CS;
+#pragma unroll
+          for (int e = 0; e < 4 * W / CS; ++e)
+            if (col0 + e < col_end) *reinterpret_cast<uint32_t*>(dst + (size_t)e * ldd_b) = o[e];
+        }
+      } else {
 #pragma unroll
         for (int ps = 0; ps < kPasses; ++ps) {
-          uint8_t* buf = stage + (nbuf == 2 ? (pass_no & 1u) * 2048 : 0);
+          const uint32_t off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
+          uint8_t* buf = stage + off;
           if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            *reinterpret_cast<uint4*>(buf + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) =
+          for (int u = 0; u < kUnits; ++u)
+            *reinterpret_cast<uint4*>(buf + lane * 64 + ((u ^ sw) << 4)) =
                 make_uint4(o[16 * ps + 4 * u], o[16 * ps + 4 * u + 1], o[16 * ps + 4 * u + 2], o[16 * ps + 4 * u + 3]);
           __syncwarp();
+          if constexpr (COLS) {
+            const int m = row0 + 8 * (lane & 3);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int i = lane + 32 * k, rr = i >> 2, u = i & 3;
-            const uint4 x = *reinterpret_cast<const uint4*>(buf + rr * 64 + ((u ^ ((rr >> 1) & 3)) << 4));
-            const int grow = row0 + rr, gcol = col0 + ps * (64 / CS) + u * kUnitElems;
-            if (grow < M && gcol < col_end) *reinterpret_cast<uint4*>(Db + (size_t)grow * ldd_b + (size_t)gcol * CS) = x;
+            for (int nb = 0; nb < kUnits; ++nb) {
+              uint32_t w[4];
+              ptx::ldmatrix_x4_trans((tm_row + off) ^ (uint32_t)(nb << 4), w[0], w[1], w[2], w[3]);
+              if (m < M) {
+                if constexpr (CS == 2) {
+                  const int n1 = col0 + 8 * nb + (lane >> 2);
+                  if (n1 < col_end)
+                    *reinterpret_cast<uint4*>(Db + (size_t)n1 * ldd_b + (size_t)m * CS) = make_uint4(w[0], w[1], w[2], w[3]);
+                } else {
+                  // 16-bit units hold two neighbouring columns: split them
+                  const int n1 = col0 + 16 * nb + 2 * (lane >> 2);
+                  if (n1 < col_end) {
+                    uint8_t* dst = Db + (size_t)n1 * ldd_b + m;
+                    *reinterpret_cast<uint2*>(dst) = make_uint2(__byte_perm(w[0], w[1], 0x6420), __byte_perm(w[2], w[3], 0x6420));
+                    *reinterpret_cast<uint2*>(dst + ldd_b) =
+                        make_uint2(__byte_perm(w[0], w[1], 0x7531), __byte_perm(w[2], w[3], 0x7531));
+                  }
+                }
+              }
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < kUnits; ++k) {
+              const int i = lane + 32 * k, rr = i / kUnits, u = i % kUnits;
+              const uint4 x = *reinterpret_cast<const uint4*>(buf + rr * 64 + ((u ^ (((rr >> 1) ^ (rr >> 3)) & 3)) << 4));
+              const int grow = row0 + rr, gcol = col0 + ps * (64 / CS) + u * kUnitElems;
+              if (grow < M && gcol < col_end) *reinterpret_cast<uint4*>(Db + (size_t)grow * ldd_b + (size_t)gcol * CS) = x;
+            }
           }
           ++pass_no;
         }
@@ -518,8 +543,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     ptx::prefetch_tensormap(&map_a);
     ptx::prefetch_tensormap(&map_b);
     if (SPARSE) ptx::prefetch_tensormap(&map_e);
-    if (p.has_c) ptx::prefetch_tensormap(&map_c);
-    ptx::prefetch_tensormap(&map_d);
+    if (!p.epi_lsu) {
+      if (p.has_c) ptx::prefetch_tensormap(&map_c);
+      ptx::prefetch_tensormap(&map_d);
+    }
   }
   if (warp == 1) {
     ptx::tmem_alloc<CTAS>(&sh->tmem_base, kTmemCols);
@@ -703,34 +730,36 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // ------------------------------ epilogue ------------------------------
     const int cs = elem_bytes((sp24_dtype)p.cd_type);
     if (p.epi_lsu) {
-      // row-major C / D: loads and stores by the epilogue warps themselves
-      if (KIND != 2 && cs == 2)
-        epilogue_rows<KIND, 2, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
-                                                                   num_clusters, num_tiles, warp, lane);
-      else
-        epilogue_rows<KIND, 4, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
-                                                                   num_clusters, num_tiles, warp, lane);
+      // loads and stores by the epilogue warps themselves
+#define SP24_EPILOGUE(CS_, COLS_)                                                                                    \
+  epilogue_direct<KIND, CS_, COLS_, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id, \
+                                                                        num_clusters, num_tiles, warp, lane)
+      if (p.cd_col_major) {
+        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, true);
+        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, true);
+        else SP24_EPILOGUE(4, true);
+      } else {
+        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, false);
+        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, false);
+        else SP24_EPILOGUE(4, false);
+      }
+#undef SP24_EPILOGUE
     } else {
-    // Column-major C / D, 1-byte outputs, and 4-byte row-major outputs when every epilogue warp can have
-    // a box buffer of its own.  Each warp owns 32 accumulator rows and walks its tiles in 32 x 32 boxes:
-    // TMA load of the C box (if beta != 0) into a staging buffer a few boxes ahead, tcgen05.ld of the
-    // accumulator columns, convert in place, TMA store of the D box.  Boxes outside the matrix are
-    // clipped by the TMA.
+    // 4-byte row-major outputs when every epilogue warp can have a box buffer of its own.  The two warps
+    // of a lane quarter own its 32 accumulator rows and take its 32 x 32 boxes in turn: TMA load of the C
+    // box (if beta != 0) into a staging buffer a few boxes ahead, tcgen05.ld of the accumulator columns,
+    // convert in place, TMA store of the D box.  Boxes outside the matrix are clipped by the TMA.
     const int q = warp & 3;  // tensor-memory lane quarter this warp may read
     const int ew = warp - kFirstEpiWarp;  // epilogue warp 0..7: warps ew and ew + 4 share a lane quarter
-    const int buf_bytes = 1024 * cs;
-    // Both warps of a quarter work (alternate boxes) when each can have a staging buffer of its own;
-    // otherwise the second one only takes part in handing the accumulators back.
-    const int split = (p.epi_bytes / kEpiWarps >= buf_bytes) ? 2 : 1;
+    constexpr int buf_bytes = 4096, split = 2;
     const int first_it = ew >> 2;
-    const bool active = first_it < split;
-    const int warp_bytes = p.epi_bytes / (4 * split);
-    const int nbuf = min(4, warp_bytes / buf_bytes);  // staging buffers of this warp: 1, 2 or 4
+    const int warp_bytes = p.epi_bytes / kEpiWarps;
+    const int nbuf = min(4, warp_bytes / buf_bytes);  // staging buffers of this warp: 1 or 2
     const int ahead = nbuf > 1 ? nbuf - 1 : 1;      // boxes the C loads run ahead (their latency is what the epilogue waits on)
     // stores that may still be reading their buffer when the next buffer is claimed: with C the
     // buffer of box seq + ahead is claimed at the end of box seq, without C that of box seq + 1
     const int pending_ok = p.has_c ? nbuf - ahead : nbuf - 1;
-    uint8_t* my_bufs = epi + (ew & (4 * split - 1)) * warp_bytes;
+    uint8_t* my_bufs = epi + ew * warp_bytes;
     constexpr int kSub = BLOCK_N / 32;
     constexpr int kIters = MBLK * kSub;
 
@@ -759,14 +788,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (live_box) {
           const int b = pf_seq % nbuf;
           ptx::mbar_expect_tx(&sh->c_full[ew][b], (uint32_t)buf_bytes);
-          ptx::tma_load_2d(my_bufs + b * buf_bytes, &map_c, &sh->c_full[ew][b], p.cd_col_major ? row0 : col0,
-                           p.cd_col_major ? col0 : row0);
+          ptx::tma_load_2d(my_bufs + b * buf_bytes, &map_c, &sh->c_full[ew][b], col0, row0);
           ++pf_seq;
           return;
         }
       }
     };
-    if (p.has_c && active && lane == 0)
+    if (p.has_c && lane == 0)
       for (int i = 0; i < ahead; ++i) issue_c_load();
 
     int acc = 0;
@@ -778,13 +806,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::tc_fence_after();
       uint32_t r_next[32];
       const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-      if (active) {
-        const int j0 = first_it / kSub, sc0 = first_it - j0 * kSub;
-        ptx::tmem_ld_32x32b_x32(t_acc + j0 * BLOCK_N + sc0 * 32, r_next);
-      }
+      ptx::tmem_ld_32x32b_x32(t_acc + first_it * 32, r_next);
       bool ok = true;
 #pragma unroll 1
-      for (int it = active ? first_it : kIters; it < kIters; it += split) {
+      for (int it = first_it; it < kIters; it += split) {
         uint32_t r[32];
         ptx::tmem_ld_wait();
 #pragma unroll
@@ -799,22 +824,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         uint8_t* buf = my_bufs + b * buf_bytes;
         if (p.has_c && !bounded_wait(&sh->c_full[ew][b], (seq / nbuf) & 1u, sh, p.status, 5u, p.wait_limit)) { ok = false; break; }
         if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
+        float scale = 1.f, bias = 0.f;
         if (KIND == 1 && p.dequant) {
           // this thread's output row: its scale and bias
           const int row = min(row0 + lane, (int)p.M - 1);
-          const float scale = __ldg(p.row_scale + row), bias = p.bias ? __ldg(p.bias + row) : 0.f;
-          if (p.cd_col_major) convert_row_dequant_transposed(r, buf, lane, p, scale, bias);
-          else if (cs == 1) convert_row_dequant_i8(r, buf, lane, p, scale, bias);
-          else convert_row_staged<KIND>(r, buf, lane, p, scale, bias);
-        } else if (p.cd_col_major) {
-          convert_row_transposed<KIND>(r, buf, lane, p);
-        } else {
-          convert_row_staged<KIND>(r, buf, lane, p, 1.f, 0.f);
+          scale = __ldg(p.row_scale + row);
+          bias = p.bias ? __ldg(p.bias + row) : 0.f;
         }
+        convert_row_staged<KIND>(r, buf, lane, p, scale, bias);
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          ptx::tma_store_2d(&map_d, buf, p.cd_col_major ? row0 : col0, p.cd_col_major ? col0 : row0);
+          ptx::tma_store_2d(&map_d, buf, col0, row0);
           ptx::bulk_commit_group();
           // the buffer claimed next is free once the store that used it last has read it
           if (pending_ok >= 3) ptx::bulk_wait_group_read<3>();
@@ -1042,42 +1063,31 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   } else {
     map_e = map_a;
   }
-  // C and D move in 32 x 32 boxes whose rows are 64 bytes (2-byte types) or 128 bytes (4-byte types)
-  CUtensorMap map_c, map_d;
   const int cs = elem_bytes(d->cd_type);
-  const uint64_t cd_rows = p.cd_col_major ? d->N : d->M, cd_cols = p.cd_col_major ? d->M : d->N;
-  st = make_map(&map_d, p.D, cs, cd_rows, cd_cols, d->ldd * cs, 32, 32, 32 * cs);
-  if (st != SP24_OK) return st;
-  if (p.has_c) {
-    st = make_map(&map_c, p.C, cs, cd_rows, cd_cols, d->ldc * cs, 32, 32, 32 * cs);
-    if (st != SP24_OK) return st;
-  } else {
-    map_c = map_d;
-  }
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
-  // stage less cost the int8 configuration 9 %); staging gets what is left, up to two boxes per
-  // epilogue warp (16 boxes of 1024 output elements), in powers of two from 16 KB.
-  {
-    p.stages = C::kMinStagesFit > C::kMaxStages ? C::kMaxStages : C::kMinStagesFit;
-    const int room = C::kSmemLimit - p.stages * C::kStageBytes;
-    // Epilogue form.  Row-major 2-byte outputs: the warps' own loads and stores through two 2 KB
-    // transposing buffers per warp (measured against the TMA form: bf16 BERT FFN 26.6 against 28.7 us,
-    // fp8 16384 x 8192 x 8192 440 against 472 us, the 256 x 256 x 512 problem 12 against 17 us, the large
-    // bf16 GEMM within 3 %).  Row-major 4-byte outputs: TMA boxes if every epilogue warp can have a 4 KB
-    // box of its own (int8 4096 x 8192 x 4096: 77 against 80 us), else the warps' own stores (two-m-block
-    // int8 tiles, 16 KB of staging: 465 against 504 us on 16384 x 8192 x 8192).  Column-major and 1-byte
-    // outputs: TMA boxes, staging in powers of two from 16 KB up to two boxes per epilogue warp.
-    int epi = 16384;
-    p.epi_lsu = 0;
-    if (!p.cd_col_major && cs == 2) {
-      p.epi_lsu = 1;
-      if (room >= kEpiWarps * 4096) epi = kEpiWarps * 4096;
-    } else if (!p.cd_col_major && cs == 4 && room < kEpiWarps * 4096) {
-      p.epi_lsu = 1;
-    } else {
-      while (epi < 16 * 1024 * cs && 2 * epi <= room) epi *= 2;
-    }
-    p.epi_bytes = epi;
+  // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
+  p.stages = C::kMinStagesFit > C::kMaxStages ? C::kMaxStages : C::kMinStagesFit;
+  const int room = C::kSmemLimit - p.stages * C::kStageBytes;
+  // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
+  // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
+  // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
+  // (against the TMA form: bf16 BERT FFN 26.6 against 28.7 us, fp8 16384 x 8192 x 8192 440 against 472 us,
+  // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
+  // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
+  // epilogue_direct).
+  p.epi_lsu = (p.cd_col_major || cs != 4 || room < kEpiWarps * 4096) ? 1 : 0;
+  p.epi_bytes = room >= kEpiWarps * 4096 ? kEpiWarps * 4096 : 16384;
+  CUtensorMap map_c, map_d;
+  if (p.epi_lsu) {
+    map_c = map_d = map_a;  // not used
+  } else {
+    while (p.epi_bytes < 16 * 4096 && 2 * p.epi_bytes <= room) p.epi_bytes *= 2;
+    // C and D move in 32 x 32 boxes whose rows are 128 bytes
+    st = make_map(&map_d, p.D, cs, d->M, d->N, d->ldd * cs, 32, 32, 128);
+    if (st != SP24_OK) return st;
+    map_c = map_d;
+    if (p.has_c) st = make_map(&map_c, p.C, cs, d->M, d->N, d->ldc * cs, 32, 32, 128);
+    if (st != SP24_OK) return st;
   }
   auto kernel = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   {
@@ -1126,7 +1136,7 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
 // tile.  The tile times are measured ratios (unit: one 256 x 224 tile per unit of K; interleaved runs on
 // 2048..8192-row problems with K = 4096..16384):
 //   256 x 224, two accumulator buffers (epilogue overlapped)      K                 the reference
-//   256 x 240, the same (16-bit kinds, 16-bit row-major output)    1.04 K            operand bytes per k
+//   256 x 240, the same (16-bit kinds, 16-bit output)              1.04 K            operand bytes per k
 //   256 x 256, one accumulator buffer (epilogue exposed)           1.09 K + 450
 //   512 x 224, two m-blocks per CTA share a B tile (epilogue exposed): twice the work in
 //              1.65 K + 1150 (16-bit kinds), 1.80 K + 820 (8-bit floats), 1.98 K + 200 (int8 -> int32)
@@ -1142,7 +1152,7 @@ static void choose_tile(const sp24_gemm_desc* d, int& ctas, int& block_n, int& m
   const bool k_major_b = d->order_b == SP24_COL_MAJOR;
   const int64_t pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
   const bool bits16 = d->ab_type == SP24_F16 || d->ab_type == SP24_BF16;
-  const bool has_240 = bits16 && k_major_b && d->order_d == SP24_ROW_MAJOR && elem_bytes(d->cd_type) == 2;
+  const bool has_240 = bits16 && k_major_b && elem_bytes(d->cd_type) == 2;
   if (d->a_is_dense) {
     if (d->M >= 512 && (d->M / 512) * n224 >= 444) {
       mblk = 2;
@@ -1344,7 +1354,7 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   if (ctas == 2 && block_n == 256 && mblk == 2 && !sparse && !b_mn && !tf32)  // dense variant only
     return f8 ? launch<3, false, 256, 2, 2, false>(d, p, A, meta, B, s)
               : (i8 ? launch<1, false, 256, 2, 2, false>(d, p, A, meta, B, s) : launch<0, false, 256, 2, 2, false>(d, p, A, meta, B, s));
-  if (ctas == 2 && block_n == 240 && mblk == 1 && !b_mn && !tf32 && !f8 && !i8 && !p.cd_col_major && elem_bytes(d->cd_type) == 2)
+  if (ctas == 2 && block_n == 240 && mblk == 1 && !b_mn && !tf32 && !f8 && !i8 && elem_bytes(d->cd_type) == 2)
     return SP24_LAUNCH(0, 240, 2, 1, false);
   SP24_DISPATCH_TF32(1, 128, 1)
   SP24_DISPATCH_TF32(2, 224, 1)
