@@ -11,7 +11,9 @@ import fails, and every call needs a CUDA device.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+from ctypes import byref
 
 import torch
 
@@ -114,8 +116,12 @@ def _check(status: int, where: str):
         raise Sp24Error(status, where)
 
 
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """The current device's current stream as a handle (no Stream object is made for it)."""
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dtype_of(t: torch.Tensor, dtype: str | None) -> str:
@@ -125,13 +131,14 @@ def _dtype_of(t: torch.Tensor, dtype: str | None) -> str:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def values_bytes(dtype: str, M: int, K: int) -> int:
     return lib.sp24_values_bytes(DTYPE_CODE[dtype], M, K)
 
 
+@functools.lru_cache(maxsize=256)
 def meta_bytes(dtype: str, M: int, K: int, layout: int = META_TCGEN05) -> int:
     return lib.sp24_meta_bytes(DTYPE_CODE[dtype], M, K, layout)
 
@@ -153,8 +160,8 @@ def compress(x: torch.Tensor, layout: int = META_TCGEN05, dtype: str | None = No
     """sp24_compress: returns (vals [M, K/2], meta uint8 [meta_bytes], dropped tensor or None)."""
     dt = _dtype_of(x, dtype)
     M, K = x.shape
-    vals = torch.empty((M, K // 2), dtype=x.dtype, device=x.device)
-    meta = torch.empty(meta_bytes(dt, M, K, layout), dtype=torch.uint8, device=x.device)
+    vals = x.new_empty((M, K // 2))
+    meta = x.new_empty(meta_bytes(dt, M, K, layout), dtype=torch.uint8)
     dropped = torch.zeros(1, dtype=torch.int64, device=x.device) if count_dropped else None
     _check(lib.sp24_compress(DTYPE_CODE[dt], M, K, _ptr(x), x.stride(0) if M > 1 else K, _ptr(vals),
                              K // 2, _ptr(meta), layout, _ptr(dropped), _stream()), "sp24_compress")
@@ -176,8 +183,8 @@ def prune_compress(x: torch.Tensor, layout: int = META_TCGEN05, dtype: str | Non
     dt = _dtype_of(x, dtype)
     M, K = x.shape
     pruned = torch.empty_like(x) if pruned is None else pruned
-    vals = torch.empty((M, K // 2), dtype=x.dtype, device=x.device) if vals is None else vals
-    meta = torch.empty(meta_bytes(dt, M, K, layout), dtype=torch.uint8, device=x.device) if meta is None else meta
+    vals = x.new_empty((M, K // 2)) if vals is None else vals
+    meta = x.new_empty(meta_bytes(dt, M, K, layout), dtype=torch.uint8) if meta is None else meta
     dropped = torch.zeros(1, dtype=torch.int64, device=x.device) if count_dropped else None
     _check(lib.sp24_prune_compress(DTYPE_CODE[dt], M, K, _ptr(x), x.stride(0) if M > 1 else K, _ptr(pruned),
                                    pruned.stride(0) if M > 1 else K, _ptr(vals), vals.stride(0) if M > 1 else K // 2,
@@ -203,18 +210,38 @@ def make_desc(ab: str, cd: str, M: int, N: int, K: int, lda: int, ldb: int, ldc:
                     ROW_MAJOR if b_row_major else COL_MAJOR, cd_order, cd_order, 1 if a_is_dense else 0)
 
 
+@functools.lru_cache(maxsize=512)
+def _desc_ref(*args):
+    """A reference to make_desc(*args) for the calls below, which only read it: a problem is described once."""
+    return byref(make_desc(*args))
+
+
 def _scalar(ab: str, v):
     return ctypes.c_float(float(v)) if ab != "i8" else ctypes.c_int32(int(v))
+
+
+# The scalars of most calls, made once (the library only reads them).
+_FLOAT_ONE, _FLOAT_ZERO = byref(ctypes.c_float(1.0)), byref(ctypes.c_float(0.0))
+
+
+def _scalar_refs(ab: str, alpha, beta):
+    if ab == "i8":
+        return byref(ctypes.c_int32(int(alpha))), byref(ctypes.c_int32(int(beta)))
+    return (_FLOAT_ONE if type(alpha) is float and alpha == 1.0 else byref(ctypes.c_float(float(alpha))),
+            _FLOAT_ZERO if type(beta) is float and beta == 0.0 else byref(ctypes.c_float(float(beta))))
 
 
 _workspaces: dict = {}
 
 
-def workspace(device) -> torch.Tensor:
-    key = (torch.device(device).index, torch.cuda.current_stream().cuda_stream)
-    if key not in _workspaces:
-        _workspaces[key] = torch.zeros(256, dtype=torch.uint8, device=device)
-    return _workspaces[key]
+def workspace(device, stream: int | None = None) -> torch.Tensor:
+    if type(device) is not torch.device:
+        device = torch.device(device)
+    key = (device.index, _stream() if stream is None else stream)
+    ws = _workspaces.get(key)
+    if ws is None:
+        ws = _workspaces.setdefault(key, torch.zeros(256, dtype=torch.uint8, device=device))
+    return ws
 
 
 def gemm(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor, *, alpha=1.0, beta=0.0,
@@ -225,21 +252,22 @@ def gemm(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor, *, alpha=
     (K contiguous), or with b_row_major=True the K x N matrix itself, [K, N] (N contiguous); C/D: [M, N],
     or with cd_col_major=True their transposes [N, M] (M contiguous)."""
     ab = _dtype_of(A, ab)
-    M = A.shape[0]
-    K = A.shape[1] if a_is_dense else 2 * A.shape[1]
-    N = Bt.shape[1] if b_row_major else Bt.shape[0]
-    assert (Bt.shape[0] if b_row_major else Bt.shape[1]) == K
+    a_shape, b_shape = A.shape, Bt.shape
+    M = a_shape[0]
+    K = a_shape[1] if a_is_dense else 2 * a_shape[1]
+    N = b_shape[1 if b_row_major else 0]
+    assert b_shape[0 if b_row_major else 1] == K
     cd = cd or ("i32" if ab == "i8" else ("bf16" if ab in ("e4m3", "e5m2") else ab))
     if out is None:
-        out = torch.empty((N, M) if cd_col_major else (M, N), dtype=TORCH_DTYPE[cd], device=A.device)
-    ws = ws if ws is not None else workspace(A.device)
-    desc = make_desc(ab, cd, M, N, K, A.stride(0), Bt.stride(0),
+        out = A.new_empty((N, M) if cd_col_major else (M, N), dtype=TORCH_DTYPE[cd])
+    stream = _stream()
+    ws = ws if ws is not None else workspace(A.device, stream)
+    desc = _desc_ref(ab, cd, M, N, K, A.stride(0), Bt.stride(0),
                      C.stride(0) if C is not None else (M if cd_col_major else N), out.stride(0), a_is_dense,
                      b_row_major, cd_col_major)
-    a, b = _scalar(ab, alpha), _scalar(ab, beta)
+    a, b = _scalar_refs(ab, alpha, beta)
     fn = lib.sp24_gemm_f16acc if acc_f16 else lib.sp24_gemm
-    _check(fn(ctypes.byref(desc), ctypes.byref(a), _ptr(A), _ptr(meta), _ptr(Bt),
-              ctypes.byref(b), _ptr(C), _ptr(out), _ptr(ws), ws.numel(), _stream()),
+    _check(fn(desc, a, _ptr(A), _ptr(meta), _ptr(Bt), b, _ptr(C), _ptr(out), _ptr(ws), ws.numel(), stream),
            "sp24_gemm_f16acc" if acc_f16 else "sp24_gemm")
     return out
 
@@ -247,7 +275,7 @@ def gemm(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor, *, alpha=
 def gemm_plan(desc: GemmDesc) -> str:
     """sp24_gemm_plan: the tile shape the library picks for this problem, as "<ctas>x<block_n>x<mblk>"."""
     c, n, m = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
-    _check(lib.sp24_gemm_plan(ctypes.byref(desc), ctypes.byref(c), ctypes.byref(n), ctypes.byref(m)), "sp24_gemm_plan")
+    _check(lib.sp24_gemm_plan(byref(desc), byref(c), byref(n), byref(m)), "sp24_gemm_plan")
     return f"{c.value}x{n.value}x{m.value}"
 
 
@@ -295,11 +323,11 @@ def gemm_static_ws(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor,
     K = A.shape[1] if a_is_dense else 2 * A.shape[1]
     N = Bt.shape[0]
     cd = cd or ("i32" if ab == "i8" else ("bf16" if ab in ("e4m3", "e5m2") else ab))
-    desc = make_desc(ab, cd, M, N, K, A.stride(0), Bt.stride(0), C.stride(0) if C is not None else N,
+    desc = _desc_ref(ab, cd, M, N, K, A.stride(0), Bt.stride(0), C.stride(0) if C is not None else N,
                      out.stride(0), a_is_dense)
-    a, b = _scalar(ab, alpha), _scalar(ab, beta)
-    _check(lib.sp24_gemm_static_ws(ctypes.byref(desc), ctypes.byref(a), _ptr(A), _ptr(meta), _ptr(Bt),
-                                   ctypes.byref(b), _ptr(C), _ptr(out), _stream()), "sp24_gemm_static_ws")
+    a, b = _scalar_refs(ab, alpha, beta)
+    _check(lib.sp24_gemm_static_ws(desc, a, _ptr(A), _ptr(meta), _ptr(Bt), b, _ptr(C), _ptr(out), _stream()),
+           "sp24_gemm_static_ws")
     return out
 
 
@@ -308,17 +336,19 @@ def gemm_i8_dequant(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor
                     out: torch.Tensor | None = None, a_is_dense: bool = False, ws: torch.Tensor | None = None,
                     b_row_major: bool = False, cd_col_major: bool = False) -> torch.Tensor:
     """sp24_gemm_i8_dequant: int8 sparse GEMM, D = act(row_scale[i] * acc + bias[i]) as cd (bf16/f16/f32/i8)."""
-    M = A.shape[0]
-    K = A.shape[1] if a_is_dense else 2 * A.shape[1]
-    N = Bt.shape[1] if b_row_major else Bt.shape[0]
+    a_shape = A.shape
+    M = a_shape[0]
+    K = a_shape[1] if a_is_dense else 2 * a_shape[1]
+    N = Bt.shape[1 if b_row_major else 0]
     if out is None:
-        out = torch.empty((N, M) if cd_col_major else (M, N), dtype=TORCH_DTYPE[cd], device=A.device)
-    ws = ws if ws is not None else workspace(A.device)
-    desc = make_desc("i8", cd, M, N, K, A.stride(0), Bt.stride(0), M if cd_col_major else N, out.stride(0),
+        out = A.new_empty((N, M) if cd_col_major else (M, N), dtype=TORCH_DTYPE[cd])
+    stream = _stream()
+    ws = ws if ws is not None else workspace(A.device, stream)
+    desc = _desc_ref("i8", cd, M, N, K, A.stride(0), Bt.stride(0), M if cd_col_major else N, out.stride(0),
                      a_is_dense, b_row_major, cd_col_major)
-    _check(lib.sp24_gemm_i8_dequant(ctypes.byref(desc), _ptr(A), _ptr(meta), _ptr(Bt), _ptr(row_scale), _ptr(bias),
-                                    1 if relu else 0, ctypes.c_float(out_scale), _ptr(out), _ptr(ws), ws.numel(),
-                                    _stream()), "sp24_gemm_i8_dequant")
+    _check(lib.sp24_gemm_i8_dequant(desc, _ptr(A), _ptr(meta), _ptr(Bt), _ptr(row_scale), _ptr(bias),
+                                    1 if relu else 0, out_scale, _ptr(out), _ptr(ws), ws.numel(), stream),
+           "sp24_gemm_i8_dequant")
     return out
 
 
@@ -333,13 +363,14 @@ def conv3x3_nhwc(A: torch.Tensor, meta: torch.Tensor | None, x: torch.Tensor, *,
     K, N = 9 * Cin, Nb * H * W
     cd = cd or ("i32" if ab == "i8" else ("bf16" if ab in ("e4m3", "e5m2") else ab))
     if out is None:
-        out = torch.empty((N, M) if nhwc_out else (M, N), dtype=TORCH_DTYPE[cd], device=A.device)
-    ws = ws if ws is not None else workspace(A.device)
-    desc = make_desc(ab, cd, M, N, K, A.stride(0), K, C.stride(0) if C is not None else (M if nhwc_out else N),
+        out = A.new_empty((N, M) if nhwc_out else (M, N), dtype=TORCH_DTYPE[cd])
+    stream = _stream()
+    ws = ws if ws is not None else workspace(A.device, stream)
+    desc = _desc_ref(ab, cd, M, N, K, A.stride(0), K, C.stride(0) if C is not None else (M if nhwc_out else N),
                      out.stride(0), a_is_dense, False, nhwc_out)
-    a, b = _scalar(ab, alpha), _scalar(ab, beta)
-    _check(lib.sp24_conv3x3_nhwc(ctypes.byref(desc), Nb, H, W, Cin, ctypes.byref(a), _ptr(A), _ptr(meta), _ptr(x),
-                                 ctypes.byref(b), _ptr(C), _ptr(out), _ptr(ws), ws.numel(), _stream()),
+    a, b = _scalar_refs(ab, alpha, beta)
+    _check(lib.sp24_conv3x3_nhwc(desc, Nb, H, W, Cin, a, _ptr(A), _ptr(meta), _ptr(x), b, _ptr(C), _ptr(out), _ptr(ws),
+                                 ws.numel(), stream),
            "sp24_conv3x3_nhwc")
     return out
 
