@@ -444,8 +444,8 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
         float scale = 1.f, bias = 0.f;
         if (KIND == 1 && p.dequant) {
           const int row = min(row0 + lane, M - 1);
-          scale = __ldg(p.row_scale + row);
-          bias = p.bias ? __ldg(p.bias + row) : 0.f;
+          scale = p.row_scale[row];
+          bias = p.bias ? p.bias[row] : 0.f;
         }
         compute_row<KIND, CS>(r, creg[n % P], has_c, p, scale, bias, o);
       }
@@ -557,6 +557,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   if (CTAS == 2) ptx::cluster_sync();
   ptx::tc_fence_after();
   const uint32_t tmem_base = sh->tmem_base;
+  let_next_start();
+  wait_for_stream();
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
@@ -828,8 +830,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (KIND == 1 && p.dequant) {
           // this thread's output row: its scale and bias
           const int row = min(row0 + lane, (int)p.M - 1);
-          scale = __ldg(p.row_scale + row);
-          bias = p.bias ? __ldg(p.bias + row) : 0.f;
+          scale = p.row_scale[row];
+          bias = p.bias ? p.bias[row] : 0.f;
         }
         convert_row_staged<KIND>(r, buf, lane, p, scale, bias);
         ptx::fence_proxy_async_smem();
@@ -1105,20 +1107,8 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   const int tiles = p.m_tiles * p.n_tiles;
   int clusters = sm_count() / CTAS;
   if (clusters > tiles) clusters = tiles;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(clusters * CTAS), 1, 1);
-  cfg.blockDim = dim3(kNumThreads, 1, 1);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CTAS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  SP24_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, map_e, map_c, map_d, p));
-  return SP24_OK;
+  return launch_overlapped(kernel, dim3((unsigned)(clusters * CTAS)), dim3(kNumThreads), C::kSmemBytes, stream, CTAS, map_a,
+                           map_b, map_e, map_c, map_d, p);
 }
 
 }  // namespace

@@ -148,9 +148,11 @@ __global__ void __launch_bounds__(kThreads) kept_magnitude_perm_kernel(const uin
 // Vector path: one thread per 16 columns (four groups = 16 metadata bits), threads along a row.
 template <int ES>
 __global__ void __launch_bounds__(kThreads) apply_mask_vec_kernel(const uint8_t* w, int64_t row_bytes_w,
-                                                                  const uint8_t* __restrict__ meta, int layout,
+                                                                  const uint8_t* meta, int layout,
                                                                   uint8_t* y, int64_t row_bytes_y, int64_t M, int64_t K,
                                                                   int64_t KB) {
+  let_next_start();
+  wait_for_stream();
   const int64_t chunk = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (chunk >= (K >> 4)) return;
   const int cl = (int)(chunk & 7);
@@ -394,12 +396,10 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
   if (K % 16 == 0 && aligned16(w) && aligned16(y) && aligned16(meta) && (ldw * es) % 16 == 0 && (ldy * es) % 16 == 0) {
     dim3 grid((unsigned)((K / 16 + kThreads - 1) / kThreads), (unsigned)(M < 8192 ? M : 8192), 1);
     if (es == 2)
-      apply_mask_vec_kernel<2><<<grid, kThreads, 0, s>>>((const uint8_t*)w, ldw * es, (const uint8_t*)meta, (int)l,
-                                                         (uint8_t*)y, ldy * es, M, K, KB);
-    else
-      apply_mask_vec_kernel<1><<<grid, kThreads, 0, s>>>((const uint8_t*)w, ldw * es, (const uint8_t*)meta, (int)l,
-                                                         (uint8_t*)y, ldy * es, M, K, KB);
-    return cuda_status(cudaGetLastError());
+      return launch_overlapped(apply_mask_vec_kernel<2>, grid, dim3(kThreads), 0, s, 1, (const uint8_t*)w, ldw * es,
+                               (const uint8_t*)meta, (int)l, (uint8_t*)y, ldy * es, M, K, KB);
+    return launch_overlapped(apply_mask_vec_kernel<1>, grid, dim3(kThreads), 0, s, 1, (const uint8_t*)w, ldw * es,
+                             (const uint8_t*)meta, (int)l, (uint8_t*)y, ldy * es, M, K, KB);
   }
   const unsigned blocks = (unsigned)((total + kThreads - 1) / kThreads);
   if (elem_bytes(t) == 2)

@@ -214,7 +214,7 @@ __device__ __forceinline__ uint4 prune_vec(uint4 v, const uint32_t* table, int f
 
 // One 16-byte vector per thread and unroll step; `vpr` vectors per row.
 template <int ES, int UNROLL>
-__global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* __restrict__ x, int64_t row_bytes_x,
+__global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* x, int64_t row_bytes_x,
                                                              uint8_t* y, int64_t row_bytes_y, int64_t vpr,
                                                              int64_t rows, int f8) {
   __shared__ uint32_t table[64];
@@ -223,6 +223,8 @@ __global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* __re
     if (t < 64) table[t] = prune_selectors<ES>((uint32_t)t);
     __syncthreads();
   }
+  let_next_start();
+  wait_for_stream();
   const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows;
        row += (int64_t)gridDim.y * blockDim.y) {
@@ -279,6 +281,8 @@ __global__ void __launch_bounds__(kThreads, 4) compress16_kernel(const uint8_t* 
     if (t < 64) ptable[t] = prune_selectors<2>((uint32_t)t);
   }
   build_selection_table(table);
+  let_next_start();
+  wait_for_stream();
   const uint32_t halves = (uint32_t)(K >> 3), halves_pad = (uint32_t)chunks_pad * 2, KB = (uint32_t)(chunks_pad >> 3);
   const uint32_t h0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   // metadata offset of this thread's chunks inside a row: fixed for the whole kernel
@@ -349,6 +353,8 @@ __global__ void __launch_bounds__(kThreads, 4) compress8_kernel(const uint8_t* x
     if (t < 64) ptable[t] = prune_selectors<1>((uint32_t)t);
   }
   build_selection_table(table);
+  let_next_start();
+  wait_for_stream();
   const uint32_t chunks = (uint32_t)(K >> 4), cpad = (uint32_t)chunks_pad, KB = (uint32_t)(chunks_pad >> 3);
   const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   uint32_t moff[UNROLL];
@@ -693,9 +699,11 @@ extern "C" sp24_status sp24_prune(sp24_dtype t, int64_t M, int64_t K, const void
     RowLaunch L(vpr, rows, UNROLL);
     int64_t rbx = ldx == K && ldy == K ? vpr * 16 : ldx * es, rby = ldx == K && ldy == K ? vpr * 16 : ldy * es;
     if (es == 2)
-      prune_vec_kernel<2, UNROLL><<<L.grid, L.block, 0, s>>>((const uint8_t*)x, rbx, (uint8_t*)y, rby, vpr, rows, f8);
+      return launch_overlapped(prune_vec_kernel<2, UNROLL>, L.grid, L.block, 0, s, 1, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
+                               vpr, rows, f8);
     else
-      prune_vec_kernel<1, UNROLL><<<L.grid, L.block, 0, s>>>((const uint8_t*)x, rbx, (uint8_t*)y, rby, vpr, rows, f8);
+      return launch_overlapped(prune_vec_kernel<1, UNROLL>, L.grid, L.block, 0, s, 1, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
+                               vpr, rows, f8);
   } else {
     int64_t gpr = K / 4, total = M * gpr;
     unsigned blocks = blocks_for(total, kThreads);
@@ -711,16 +719,16 @@ namespace sp24 {
 namespace {
 
 template <int ES, bool COUNT, bool HW, bool FULL, bool PRUNE>
-void launch_compress_vec(const RowLaunch& L, cudaStream_t s, const uint8_t* xs, int64_t rbx, uint8_t* vs, int64_t rbv,
-                         uint8_t* ms, int64_t M, int64_t K, int64_t rows_pad, int64_t chunks_pad,
-                         unsigned long long* dropped, int f8, uint8_t* ys, int64_t rby) {
+sp24_status launch_compress_vec(const RowLaunch& L, cudaStream_t s, const uint8_t* xs, int64_t rbx, uint8_t* vs, int64_t rbv,
+                                uint8_t* ms, int64_t M, int64_t K, int64_t rows_pad, int64_t chunks_pad,
+                                unsigned long long* dropped, int f8, uint8_t* ys, int64_t rby) {
   constexpr int UNROLL = 4;
-  if (ES == 2)
-    compress16_kernel<UNROLL, COUNT, HW, FULL, PRUNE><<<L.grid, L.block, 0, s>>>(xs, rbx, vs, rbv, ms, M, K, rows_pad,
-                                                                                chunks_pad, dropped, ys, rby);
+  if constexpr (ES == 2)
+    return launch_overlapped(compress16_kernel<UNROLL, COUNT, HW, FULL, PRUNE>, L.grid, L.block, 0, s, 1, xs, rbx, vs, rbv, ms,
+                             M, K, rows_pad, chunks_pad, dropped, ys, rby);
   else
-    compress8_kernel<UNROLL, COUNT, HW, FULL, PRUNE><<<L.grid, L.block, 0, s>>>(xs, rbx, vs, rbv, ms, M, K, rows_pad,
-                                                                               chunks_pad, dropped, f8, ys, rby);
+    return launch_overlapped(compress8_kernel<UNROLL, COUNT, HW, FULL, PRUNE>, L.grid, L.block, 0, s, 1, xs, rbx, vs, rbv, ms,
+                             M, K, rows_pad, chunks_pad, dropped, f8, ys, rby);
 }
 
 // compress (y == nullptr) or fused prune + compress (y = pruned matrix, vector kernels only: returns
@@ -754,10 +762,10 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
 #define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                            \
   case V:                                                                                                             \
     if (es == 2)                                                                                                      \
-      launch_compress_vec<2, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
+      st = launch_compress_vec<2, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
                                                      dropped, f8, ys, ldy * es);                                      \
     else                                                                                                              \
-      launch_compress_vec<1, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
+      st = launch_compress_vec<1, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
                                                      dropped, f8, ys, ldy * es);                                      \
     break;
     switch (variant) {
@@ -780,6 +788,7 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
         SP24_CV(15, true, true, true, true)
     }
 #undef SP24_CV
+    return st;
   } else {
     if (y != nullptr) return SP24_ERR_UNSUPPORTED;
     int64_t bytes_pad = k_pad / 8, total = rows_pad * bytes_pad;
