@@ -69,6 +69,7 @@ struct GemmParams {
   long long wait_limit;       // SM cycles after which a device-side wait gives up
   int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
   int32_t band;       // m-tiles per band of the tile sweep
+  int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout)
   // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
   int32_t conv, conv_h, conv_w, conv_c;
@@ -92,6 +93,7 @@ struct Cfg {
   static constexpr int kABoxes = SPARSE ? 1 : kBBoxes;
   static constexpr int kBRows = BLOCK_N / CTAS;                    // B rows (N) this CTA loads
   static constexpr int kABlockBytes = kABoxes * kBlockM * kAtomBytes;  // one m-block
+  static_assert(MBLK == 1 || kABoxes == 1, "the m-blocks of a stage are one box of rows");
   static constexpr int kABytes = MBLK * kABlockBytes;
   static constexpr int kAtomElems = KIND == 0 ? 64 : (one_byte_operands(KIND) ? 128 : 32);  // elements per 128-byte row
   static constexpr int kKPerStage = kAtomElems * kBBoxes;  // logical K per stage
@@ -183,6 +185,19 @@ __device__ __forceinline__ uint32_t make_idesc(bool sparse, bool b_mn_major, int
   d |= (uint32_t)(n >> 3) << 17;
   d |= (uint32_t)(m >> 4) << 24;
   return d;                                        // no negate, no saturate
+}
+
+// Rows of A of a tile.  One m-block: rank 0 has the first 128 rows, rank 1 the next.  Two m-blocks: a CTA's
+// blocks are neighbours (rank 0 rows 0-255 of the tile, rank 1 rows 256-511), so that one load brings
+// both; in a last tile of at most 256 rows each CTA has one block instead of rank 0 having two.
+template <int CTAS, int MBLK>
+__device__ __forceinline__ int live_blocks(int mt, int M) {
+  return MBLK == 1 ? 1 : (M - mt * (MBLK * CTAS * kBlockM) > CTAS * kBlockM ? 2 : 1);
+}
+template <int CTAS, int MBLK>
+__device__ __forceinline__ int first_row(int mt, int cta_rank, int M) {
+  static_assert(MBLK == 1 || (CTAS == 2 && MBLK == 2), "tile shape");
+  return mt * (MBLK * CTAS * kBlockM) + cta_rank * kBlockM * live_blocks<CTAS, MBLK>(mt, M);
 }
 
 // ---- epilogue helpers ----------------------------------------------------------------------------
@@ -343,14 +358,15 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
     int mt, nt;
     tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
     const int col_end = min(N, (nt + 1) * BLOCK_N);  // columns of this tile stop here
+    const int tile_row = first_row<CTAS, MBLK>(mt, cta_rank, M), live_j = live_blocks<CTAS, MBLK>(mt, M);
     // box n of this warp in this tile: first row / column, accumulator column, inside the matrix?
     auto geom = [&](int n, int& row0, int& col0, int& tcol) -> bool {
       const int it = half + 2 * n;
       const int j = it / kSub, sc = it - j * kSub;
-      row0 = ((mt * MBLK + j) * CTAS + cta_rank) * kBlockM + q * 32;
+      row0 = tile_row + j * kBlockM + q * 32;
       col0 = nt * BLOCK_N + sc * 32;
       tcol = j * BLOCK_N + sc * 32;
-      return it < kIters && row0 < M && col0 < col_end;
+      return it < kIters && j < live_j && row0 < M && col0 < col_end;
     };
     auto load_c = [&](int n, uint32_t (&c)[W]) {
       int row0, col0, tcol;
@@ -563,19 +579,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (ptx::elect_one()) {
+      // (Shared-memory and barrier addresses as plain integers, as few loads per stage as the boxes allow: the
+      // thread that issues them is busy for about 100 cycles per load, which delays the refill of a stage.
+      // Three loads instead of six (two m-blocks) or four: 49152 x 32 x 12288 bf16 123.1 -> 119.6 us, int8
+      // 4096 x 8192 x 4096 79.3 -> 77.2, 256 x 256 x 512 4.55 -> 4.47.)
       int stage = 0;
       uint32_t phase = 0;
-      const int box_elems = C::kAtomElems;  // elements per 128-byte atom row
+      constexpr int box_elems = C::kAtomElems;  // elements per 128-byte atom row
+      const uint32_t ring = ptx::smem_u32(smem);
+      const uint32_t full0 = CTAS == 2 ? ptx::map_to_cta(ptx::smem_u32(&sh->full[0]), 0) : ptx::smem_u32(&sh->full[0]);
       for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
         int mt, nt;
         tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
         // the last n-tile may be narrower: the pair then splits only the columns that exist
         const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
         const int col0 = nt * BLOCK_N + (int)cta_rank * (n_eff / CTAS);  // first B row (N index)
-        // m-blocks of this tile that have rows at all (the rest are neither loaded nor multiplied)
-        const int live = min(MBLK, (int)((p.M - (int64_t)mt * MBLK * CTAS * kBlockM + CTAS * kBlockM - 1) /
-                                         (CTAS * kBlockM)));
-        const uint32_t tx_bytes = (uint32_t)((live * (C::kABlockBytes + C::kEBlockBytes) + C::kBBytes) * CTAS);
+        const int row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M);
+        constexpr uint32_t tx_bytes = (uint32_t)((C::kABytes + C::kEBytes + C::kBBytes) * CTAS);
         // implicit convolution: (image, row, column) of this CTA's first output pixel
         int conv_n = 0, conv_p = 0, conv_q = 0;
         if (p.conv) {
@@ -596,59 +616,34 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             continue;
           }
-          uint8_t* sa = smem + stage * C::kStageBytes;
-          uint8_t* sb = sa + C::kABytes;
-          uint8_t* se = sb + C::kBBytes;
-          uint64_t* full = &sh->full[stage];
-          if (cta_rank == 0) ptx::mbar_expect_tx(full, tx_bytes);
+          const uint32_t sa = ring + stage * C::kStageBytes, sb = sa + C::kABytes, se = sb + C::kBBytes;
+          const uint32_t full = full0 + 8 * stage;
+          if (cta_rank == 0) ptx::mbar_expect_tx(&sh->full[stage], tx_bytes);
+          // both m-blocks' rows and metadata blocks are neighbours: one box each
+          if (SPARSE) ptx::tma_load_3d<CTAS>(se, &map_e, full, 0, 16 * kb * C::kEBlocks, row0 / kBlockM);
 #pragma unroll
-          for (int j = 0; j < MBLK; ++j) {
-            if (j >= live) break;
-            const int mb = (mt * MBLK + j) * CTAS + (int)cta_rank;  // 128-row block of A
-#pragma unroll
-            for (int i = 0; i < C::kABoxes; ++i) {
-              uint8_t* dst = sa + j * C::kABlockBytes + i * kBlockM * kAtomBytes;
-              int x = (kb * C::kABoxes + i) * box_elems;
-              if (CTAS == 1) ptx::tma_load_2d(dst, &map_a, full, x, mb * kBlockM);
-              else ptx::tma_load_2d_pair(dst, &map_a, full, 0, x, mb * kBlockM);
-            }
-            if (SPARSE) {
-              // metadata viewed as rows of 128 bytes: block (mb, kb128) starts at row 16 * (mb * KB + kb128)
-              int y = 16 * (mb * p.meta_kb + kb * C::kEBlocks);
-              if (CTAS == 1) ptx::tma_load_2d(se + j * C::kEBlockBytes, &map_e, full, 0, y);
-              else ptx::tma_load_2d_pair(se + j * C::kEBlockBytes, &map_e, full, 0, 0, y);
-            }
-          }
+          for (int i = 0; i < C::kABoxes; ++i)
+            ptx::tma_load_2d<CTAS>(sa + i * MBLK * kBlockM * kAtomBytes, &map_a, full, (kb * C::kABoxes + i) * box_elems, row0);
           if (B_MN) {
             // B stored N-contiguous: boxes of 128 bytes along N x all k-rows of the stage
 #pragma unroll
-            for (int c = 0; c < C::kBChunks; ++c) {
-              int x = col0 + c * C::kBChunkElems, y = kb * C::kKPerStage;
-              if (CTAS == 1) ptx::tma_load_2d(sb + c * C::kBChunkBytes, &map_b, full, x, y);
-              else ptx::tma_load_2d_pair(sb + c * C::kBChunkBytes, &map_b, full, 0, x, y);
-            }
+            for (int c = 0; c < C::kBChunks; ++c)
+              ptx::tma_load_2d<CTAS>(sb + c * C::kBChunkBytes, &map_b, full, col0 + c * C::kBChunkElems, kb * C::kKPerStage);
           } else if (p.conv) {
             // k = (r * 3 + s) * C + c: a stage holds channels of one filter tap; rows = output pixels
             const int k0 = kb * C::kKPerStage;
             const int tap = k0 / p.conv_c, c0 = k0 - tap * p.conv_c;
             const int r = tap / 3, sx = tap - 3 * r;
 #pragma unroll
-            for (int i = 0; i < C::kBBoxes; ++i) {
-              uint8_t* dst = sb + i * C::kBRows * kAtomBytes;
-              if (CTAS == 1)
-                ptx::tma_load_im2col_4d(dst, &map_b, full, c0 + i * box_elems, conv_q - 1, conv_p - 1, conv_n,
-                                        (uint16_t)sx, (uint16_t)r);
-              else
-                ptx::tma_load_im2col_4d_pair(dst, &map_b, full, 0, c0 + i * box_elems, conv_q - 1, conv_p - 1, conv_n,
-                                             (uint16_t)sx, (uint16_t)r);
-            }
+            for (int i = 0; i < C::kBBoxes; ++i)
+              ptx::tma_load_im2col_4d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, c0 + i * box_elems, conv_q - 1,
+                                            conv_p - 1, conv_n, (uint16_t)sx, (uint16_t)r);
+          } else if (p.b_3d) {
+            ptx::tma_load_3d<CTAS>(sb, &map_b, full, 0, col0, kb * C::kBBoxes);
           } else {
 #pragma unroll
-            for (int i = 0; i < C::kBBoxes; ++i) {
-              int x = (kb * C::kBBoxes + i) * box_elems;
-              if (CTAS == 1) ptx::tma_load_2d(sb + i * C::kBRows * kAtomBytes, &map_b, full, x, col0);
-              else ptx::tma_load_2d_pair(sb + i * C::kBRows * kAtomBytes, &map_b, full, 0, x, col0);
-            }
+            for (int i = 0; i < C::kBBoxes; ++i)
+              ptx::tma_load_2d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * box_elems, col0);
           }
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
@@ -664,8 +659,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
         // instruction N = the columns this tile really has (a multiple of 16, of 32 for int8)
         const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
-        const int live = min(MBLK, (int)((p.M - (int64_t)mt * MBLK * CTAS * kBlockM + CTAS * kBlockM - 1) /
-                                         (CTAS * kBlockM)));
+        const int live = live_blocks<CTAS, MBLK>(mt, (int)p.M);  // m-blocks with rows (others are not multiplied)
         const uint32_t idesc = make_idesc<KIND>(SPARSE, B_MN, p.a_fmt, kBlockM * CTAS, n_eff, KIND == 0 && p.acc_f16);
         if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
         ptx::tc_fence_after();
@@ -768,9 +762,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // box `it` of the tile (mt, nt): first row / column and whether any of it lies inside the matrix
     auto box_of = [&](int mt, int nt, int it, int& row0, int& col0) -> bool {
       const int j = it / kSub, sc = it - j * kSub;
-      row0 = ((mt * MBLK + j) * CTAS + (int)cta_rank) * kBlockM + q * 32;
+      row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M) + j * kBlockM + q * 32;
       col0 = nt * BLOCK_N + sc * 32;
-      return row0 < p.M && col0 < p.N;
+      return j < live_blocks<CTAS, MBLK>(mt, (int)p.M) && row0 < p.M && col0 < p.N;
     };
     // cursor of the C loads over the same stream of boxes, `ahead` live boxes in front of the consumer
     // (the tile coordinates cost two divisions: once per tile, not per box)
@@ -790,7 +784,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (live_box) {
           const int b = pf_seq % nbuf;
           ptx::mbar_expect_tx(&sh->c_full[ew][b], (uint32_t)buf_bytes);
-          ptx::tma_load_2d(my_bufs + b * buf_bytes, &map_c, &sh->c_full[ew][b], col0, row0);
+          ptx::tma_load_2d<1>(ptx::smem_u32(my_bufs + b * buf_bytes), &map_c, ptx::smem_u32(&sh->c_full[ew][b]), col0, row0);
           ++pf_seq;
           return;
         }
@@ -934,27 +928,34 @@ sp24_status make_im2col_map(CUtensorMap* map, const void* x, int es, uint64_t nb
   return r == CUDA_SUCCESS ? SP24_OK : SP24_ERR_CUDA;
 }
 
-// 2-D tensor map over a row-major (rows x cols) array of `es`-byte elements with `ld_bytes`
-// between rows; box = box_cols x box_rows elements.
 constexpr int kSwizzle128Atom32 = 1280;
 
-sp24_status encode_map(CUtensorMap* map, const void* base, int es, uint64_t rows, uint64_t cols, uint64_t ld_bytes,
-                       uint32_t box_cols, uint32_t box_rows, int swizzle_bytes) {
+// Up to three dimensions, innermost first: sizes in elements, strides of the outer ones in bytes.
+struct MapShape {
+  const void* base;
+  uint64_t dims[3], strides[2];  // dims[2] == 0: two dimensions
+  uint32_t box[3];
+  int32_t es, swizzle;  // swizzle: 0, 64, 128, or kSwizzle128Atom32 = the 128-byte pattern in 32-byte units
+  bool operator==(const MapShape& o) const {
+    return base == o.base && dims[0] == o.dims[0] && dims[1] == o.dims[1] && dims[2] == o.dims[2] &&
+           strides[0] == o.strides[0] && strides[1] == o.strides[1] && box[0] == o.box[0] && box[1] == o.box[1] &&
+           box[2] == o.box[2] && es == o.es && swizzle == o.swizzle;
+  }
+};
+
+sp24_status encode_map(CUtensorMap* map, const MapShape& m) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return SP24_ERR_CUDA;
-  cuuint64_t dims[2] = {cols, rows};
-  cuuint64_t strides[1] = {ld_bytes};
-  cuuint32_t box[2] = {box_cols, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUtensorMapDataType dt = es == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32
-                                   : (es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8);
-  // swizzle_bytes: 0, 64, 128, or kSwizzle128Atom32 = the 128-byte pattern in 32-byte units
-  CUtensorMapSwizzle sw = swizzle_bytes == kSwizzle128Atom32
+  const cuuint64_t dims[3] = {m.dims[0], m.dims[1], m.dims[2]}, strides[2] = {m.strides[0], m.strides[1]};
+  const cuuint32_t box[3] = {m.box[0], m.box[1], m.box[2]}, estr[3] = {1, 1, 1};
+  CUtensorMapDataType dt = m.es == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32
+                                     : (m.es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8);
+  CUtensorMapSwizzle sw = m.swizzle == kSwizzle128Atom32
                               ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B
-                              : (swizzle_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                                      : (swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE));
-  CUresult r = fn(map, dt, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                              : (m.swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                                  : (m.swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE));
+  CUresult r = fn(map, dt, m.dims[2] ? 3 : 2, const_cast<void*>(m.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? SP24_OK : SP24_ERR_CUDA;
 }
 
@@ -962,38 +963,32 @@ sp24_status encode_map(CUtensorMap* map, const void* base, int es, uint64_t rows
 // dimension, element size, box, swizzle): a layer that is multiplied again with the same buffers
 // finds its five maps here instead of encoding them again.  One small table per host thread (no
 // lock), replaced round-robin.
-struct MapKey {
-  const void* base;
-  uint64_t rows, cols, ld_bytes;
-  uint32_t box_cols, box_rows;
-  int32_t es, swizzle;
-  bool operator==(const MapKey& o) const {
-    return base == o.base && rows == o.rows && cols == o.cols && ld_bytes == o.ld_bytes && box_cols == o.box_cols &&
-           box_rows == o.box_rows && es == o.es && swizzle == o.swizzle;
-  }
-};
 struct MapCache {
   static constexpr int kEntries = 32;
-  MapKey keys[kEntries];
+  MapShape keys[kEntries];
   CUtensorMap maps[kEntries];
   int used = 0, next = 0;
 };
 
-sp24_status make_map(CUtensorMap* map, const void* base, int es, uint64_t rows, uint64_t cols, uint64_t ld_bytes,
-                     uint32_t box_cols, uint32_t box_rows, int swizzle_bytes) {
+sp24_status make_map(CUtensorMap* map, const MapShape& key) {
   static thread_local MapCache cache;
-  const MapKey key = {base, rows, cols, ld_bytes, box_cols, box_rows, es, swizzle_bytes};
   for (int i = 0; i < cache.used; ++i)
     if (cache.keys[i] == key) {
       *map = cache.maps[i];
       return SP24_OK;
     }
-  sp24_status st = encode_map(map, base, es, rows, cols, ld_bytes, box_cols, box_rows, swizzle_bytes);
+  sp24_status st = encode_map(map, key);
   if (st != SP24_OK) return st;
   const int slot = cache.used < MapCache::kEntries ? cache.used++ : (cache.next++ % MapCache::kEntries);
   cache.keys[slot] = key;
   cache.maps[slot] = *map;
   return SP24_OK;
+}
+// 2-D map over a row-major (rows x cols) array of `es`-byte elements with `ld_bytes` between rows; box = box_cols x
+// box_rows elements.
+sp24_status make_map(CUtensorMap* map, const void* base, int es, uint64_t rows, uint64_t cols, uint64_t ld_bytes,
+                     uint32_t box_cols, uint32_t box_rows, int swizzle) {
+  return make_map(map, MapShape{base, {cols, rows, 0}, {ld_bytes, 0}, {box_cols, box_rows, 1}, es, swizzle});
 }
 
 int sm_count() {
@@ -1043,7 +1038,7 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   CUtensorMap map_a, map_b, map_e;
   const uint32_t atom_elems = kAtomBytes / es;
   const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, kBlockM, 128);
+  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, MBLK * kBlockM, 128);
   if (st != SP24_OK) return st;
   if (p.conv) {
     // B = im2col view of the NHWC activation: boxes of kBRows output pixels x one 128-byte run of channels
@@ -1054,13 +1049,20 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   } else if (B_MN) {
     st = make_map(&map_b, B, es, d->K, d->N, d->ldb * es, C::kBChunkElems, C::kKPerStage,
                   KIND == 2 ? kSwizzle128Atom32 : 128);
+  } else if (C::kBBoxes > 1 && d->K % atom_elems == 0) {
+    // K in whole 128-byte atoms: the atoms of a stage are a third dimension, one load brings them all (a K tail
+    // needs the zeros that only the two-dimensional map gives it)
+    p.b_3d = 1;
+    st = make_map(&map_b, MapShape{B, {atom_elems, (uint64_t)d->N, (uint64_t)d->K / atom_elems},
+                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, (uint32_t)C::kBRows, (uint32_t)C::kBBoxes}, es, 128});
   } else {
     st = make_map(&map_b, B, es, d->N, d->K, d->ldb * es, atom_elems, C::kBRows, 128);
   }
   if (st != SP24_OK) return st;
   if (SPARSE) {
-    uint64_t meta_rows = (uint64_t)((d->M + 127) / 128) * p.meta_kb * 16;  // rows of 128 bytes
-    st = make_map(&map_e, meta, 1, meta_rows, 128, 128, 128, 16 * C::kEBlocks, 0);
+    // metadata as rows of 128 bytes: 16 * meta_kb of them per 128 rows of A
+    st = make_map(&map_e, MapShape{meta, {128, (uint64_t)p.meta_kb * 16, (uint64_t)((d->M + 127) / 128)},
+                                   {128, (uint64_t)p.meta_kb * 2048}, {128, 16 * C::kEBlocks, MBLK}, 1, 0});
     if (st != SP24_OK) return st;
   } else {
     map_e = map_a;
