@@ -286,7 +286,7 @@ sp24_status sp24_gemm_static_ws_status(void* stream);
 
 /* Benchmarking and test support (no counterpart in the paper): forces the tile shape of every
  * following sp24_gemm / sp24_gemm_i8_dequant / sp24_conv3x3_nhwc call in this process.
- *   ctas: 1 or 2 CTAs per tile; block_n: columns per tile; mblk: 128-row blocks per CTA (1 or 2);
+ *   ctas: 1 or 2 CTAs per tile; block_n: columns per tile; mblk: 128-row blocks per CTA (1 to 3);
  *   the shape must be one of the built ones, else those calls return SP24_ERR_UNSUPPORTED.
  *   ctas == 0 restores the automatic choice.  band: m-tiles per band of the tile sweep, 0 = default.
  * The environment variables SP24_TILE=<ctas>x<block_n>x<mblk>, SP24_BAND=<band> and SP24_LOG=1

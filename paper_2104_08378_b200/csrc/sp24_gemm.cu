@@ -69,6 +69,7 @@ struct GemmParams {
   long long wait_limit;       // SM cycles after which a device-side wait gives up
   int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
   int32_t band;       // m-tiles per band of the tile sweep
+  int32_t mblk, b_rows, b_stages;  // tall tiles only: m-blocks of a tile, rows of a B box, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout)
   // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
@@ -84,6 +85,13 @@ struct GemmParams {
 
 // MMA kinds: 0 = f16 / bf16, 1 = int8, 2 = tf32, 3 = 8-bit floating point (e4m3 / e5m2)
 __host__ __device__ constexpr bool one_byte_operands(int kind) { return kind == 1 || kind == 3; }
+
+// Tall tiles (CTAS == 1, MBLK == kTallBlocks; sparse A, K-major B): up to 128 columns, two or three m-blocks (set
+// per launch) that share each B box.  Their ring is finer: one slot per m-block and k-block (A and metadata) and
+// a second ring for the B boxes, so that a slot is refilled as soon as its four MMAs are done.
+constexpr int kTallBlocks = 3;
+template <int CTAS, int MBLK>
+constexpr bool is_tall = CTAS == 1 && MBLK == kTallBlocks;
 
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
 struct Cfg {
@@ -115,9 +123,9 @@ struct Cfg {
   // The split between ring stages and epilogue staging is made per launch (the output type
   // decides how much staging is useful).
   static constexpr int kSmemLimit = 232448 - 1024 - 512;
-  static constexpr int kMaxStages = 8;
+  static constexpr int kMaxStages = is_tall<CTAS, MBLK> ? 12 : 8;
   static constexpr int kMinStagesFit = (kSmemLimit - 16384) / kStageBytes;  // with the smallest staging
-  static constexpr int kAccStages = MBLK == 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
+  static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
   static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
   static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block
   static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
@@ -126,12 +134,13 @@ struct Cfg {
   // epilogue_direct, which bounds every access by the tile's last column
   static_assert(BLOCK_N % 16 == 0, "tile width");
   static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte alignment of the atoms");
-  static_assert(kECol + (SPARSE ? 2 * MBLK * 8 : 0) <= (int)kTmemCols, "tensor memory overflow");
+  static_assert(kECol + (SPARSE ? (is_tall<CTAS, MBLK> ? kMaxStages * 8 : 2 * MBLK * 8) : 0) <= (int)kTmemCols,
+                "tensor memory overflow");
 };
 
 struct Shared {
-  uint64_t full[8], empty[8], tmem_full[2], tmem_empty[2];
-  uint64_t c_full[kEpiWarps][4];   // per epilogue warp and staging buffer: C box has landed
+  uint64_t full[12], empty[12], tmem_full[2], tmem_empty[2];
+  uint64_t c_full[kEpiWarps][2];   // per epilogue warp and staging buffer: C box has landed
   uint32_t tmem_base;
   volatile uint32_t abort;
 };
@@ -192,11 +201,11 @@ __device__ __forceinline__ uint32_t make_idesc(bool sparse, bool b_mn_major, int
 // both; in a last tile of at most 256 rows each CTA has one block instead of rank 0 having two.
 template <int CTAS, int MBLK>
 __device__ __forceinline__ int live_blocks(int mt, int M) {
-  return MBLK == 1 ? 1 : (M - mt * (MBLK * CTAS * kBlockM) > CTAS * kBlockM ? 2 : 1);
+  return MBLK != 2 ? 1 : (M - mt * (MBLK * CTAS * kBlockM) > CTAS * kBlockM ? 2 : 1);
 }
 template <int CTAS, int MBLK>
 __device__ __forceinline__ int first_row(int mt, int cta_rank, int M) {
-  static_assert(MBLK == 1 || (CTAS == 2 && MBLK == 2), "tile shape");
+  static_assert(MBLK == 1 || (CTAS == 2 && MBLK == 2) || is_tall<CTAS, MBLK>, "tile shape");  // (tall: not used)
   return mt * (MBLK * CTAS * kBlockM) + cta_rank * kBlockM * live_blocks<CTAS, MBLK>(mt, M);
 }
 
@@ -358,19 +367,9 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
     int mt, nt;
     tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
     const int col_end = min(N, (nt + 1) * BLOCK_N);  // columns of this tile stop here
-    const int tile_row = first_row<CTAS, MBLK>(mt, cta_rank, M), live_j = live_blocks<CTAS, MBLK>(mt, M);
-    // box n of this warp in this tile: first row / column, accumulator column, inside the matrix?
-    auto geom = [&](int n, int& row0, int& col0, int& tcol) -> bool {
-      const int it = half + 2 * n;
-      const int j = it / kSub, sc = it - j * kSub;
-      row0 = tile_row + j * kBlockM + q * 32;
-      col0 = nt * BLOCK_N + sc * 32;
-      tcol = j * BLOCK_N + sc * 32;
-      return it < kIters && j < live_j && row0 < M && col0 < col_end;
-    };
-    auto load_c = [&](int n, uint32_t (&c)[W]) {
-      int row0, col0, tcol;
-      if (!geom(n, row0, col0, tcol)) return;
+    // C values of the box at (row0, col0): row-major in the accumulators' order (this thread's row), column-major
+    // in the order of the stores
+    auto load_c = [&](int row0, int col0, uint32_t (&c)[W]) {
       if constexpr (COLS) {
         if constexpr (CS == 2) {
           const int m = row0 + 8 * (lane & 3);
@@ -403,71 +402,35 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
         }
       }
     };
-    if (has_c) {
-#pragma unroll
-      for (int n = 0; n < P; ++n)
-        if (n < kBoxes) load_c(n, creg[n]);
-    }
-    if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-    ptx::tc_fence_after();
-    const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-    uint32_t racc[2][32];
-    {
-      int row0, col0, tcol;
-      geom(0, row0, col0, tcol);
-      ptx::tmem_ld_32x32b_x32(t_acc + tcol, racc[0]);
-    }
-#pragma unroll
-    for (int n = 0; n < kBoxes; ++n) {
-      if (half + 2 * n >= kIters) break;  // same answer for the whole warp
-      ptx::tmem_ld_wait();
-      if (half + 2 * (n + 1) < kIters) {
-        int row1, col1, tcol1;
-        geom(n + 1, row1, col1, tcol1);
-        ptx::tmem_ld_32x32b_x32(t_acc + tcol1, racc[(n + 1) & 1]);
-      } else {
-        // this warp's part of the accumulators is in registers: hand it back to the MMA issuer (CTA 0 of the pair)
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (CTAS == 1) ptx::mbar_arrive(&sh->tmem_empty[acc]);
-          else ptx::mbar_arrive_cluster(&sh->tmem_empty[acc], 0);
-        }
-      }
-      int row0, col0, tcol;
-      const bool live = geom(n, row0, col0, tcol);  // same answer for the whole warp
-      uint32_t o[W];
+    // accumulators (and C) of a box -> packed output rows
+    auto convert = [&](uint32_t (&r)[32], uint32_t (&c)[W], int row0, uint32_t (&o)[W]) {
       const uint32_t buf_off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
-      if (live) {
-        if constexpr (CS == 2 && COLS) {
-          if (has_c) {
-            // C arrived in the order of the column stores: through the buffer to the rows' owners
-            if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
-            uint32_t (&c)[W] = creg[n % P];
+      if constexpr (CS == 2 && COLS) {
+        if (has_c) {
+          // C arrived in the order of the column stores: through the buffer to the rows' owners
+          if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
 #pragma unroll
-            for (int nb = 0; nb < 4; ++nb)
-              ptx::stmatrix_x4_trans((tm_row + buf_off) ^ (uint32_t)(nb << 4), c[4 * nb], c[4 * nb + 1], c[4 * nb + 2], c[4 * nb + 3]);
-            __syncwarp();
+          for (int nb = 0; nb < 4; ++nb)
+            ptx::stmatrix_x4_trans((tm_row + buf_off) ^ (uint32_t)(nb << 4), c[4 * nb], c[4 * nb + 1], c[4 * nb + 2], c[4 * nb + 3]);
+          __syncwarp();
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const uint4 x = *reinterpret_cast<const uint4*>(stage + buf_off + lane * 64 + ((u ^ sw) << 4));
-              c[4 * u] = x.x; c[4 * u + 1] = x.y; c[4 * u + 2] = x.z; c[4 * u + 3] = x.w;
-            }
+          for (int u = 0; u < 4; ++u) {
+            const uint4 x = *reinterpret_cast<const uint4*>(stage + buf_off + lane * 64 + ((u ^ sw) << 4));
+            c[4 * u] = x.x; c[4 * u + 1] = x.y; c[4 * u + 2] = x.z; c[4 * u + 3] = x.w;
           }
         }
-        uint32_t (&r)[32] = racc[n & 1];
-        if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
-        float scale = 1.f, bias = 0.f;
-        if (KIND == 1 && p.dequant) {
-          const int row = min(row0 + lane, M - 1);
-          scale = p.row_scale[row];
-          bias = p.bias ? p.bias[row] : 0.f;
-        }
-        compute_row<KIND, CS>(r, creg[n % P], has_c, p, scale, bias, o);
       }
-      // the C registers of box n are free: fetch box n + P into them (also when box n lies outside the matrix)
-      if (has_c && n + P < kBoxes) load_c(n + P, creg[n % P]);
-      if (!live) continue;
+      if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
+      float scale = 1.f, bias = 0.f;
+      if (KIND == 1 && p.dequant) {
+        const int row = min(row0 + lane, M - 1);
+        scale = p.row_scale[row];
+        bias = p.bias ? p.bias[row] : 0.f;
+      }
+      compute_row<KIND, CS>(r, c, has_c, p, scale, bias, o);
+    };
+    // packed output rows -> D
+    auto store = [&](const uint32_t (&o)[W], int row0, int col0) {
       if constexpr (CS == 4 && COLS) {
         if (row0 + lane < M) {
           uint8_t* dst = Db + (size_t)col0 * ldd_b + (size_t)(row0 + lane) * CS;
@@ -521,6 +484,95 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
           ++pass_no;
         }
       }
+    };
+    auto hand_back = [&] {  // this warp's part of the accumulators is in registers: the MMA issuer (CTA 0 of the pair) may go on
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (CTAS == 1) ptx::mbar_arrive(&sh->tmem_empty[acc]);
+        else ptx::mbar_arrive_cluster(&sh->tmem_empty[acc], 0);
+      }
+    };
+    const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
+    if constexpr (is_tall<CTAS, MBLK>) {
+      // few boxes: a short loop over the ones that exist (unrolled code would be fetched for boxes that do not)
+      const int nsub = (col_end - nt * BLOCK_N + 31) / 32, row_q = mt * p.mblk * kBlockM + q * 32;
+      const int boxes = nsub * max(0, min(p.mblk, (M - row_q + kBlockM - 1) / kBlockM));  // of this lane quarter
+      auto place = [&](int b, int& row0, int& col0, int& tcol) {
+        const int j = b / nsub, sc = b - j * nsub;
+        row0 = row_q + j * kBlockM;
+        col0 = nt * BLOCK_N + sc * 32;
+        tcol = j * BLOCK_N + sc * 32;
+      };
+      int row0 = 0, col0 = 0, tcol = 0;
+      if (half < boxes) {
+        place(half, row0, col0, tcol);
+        if (has_c) load_c(row0, col0, creg[0]);
+      }
+      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
+      ptx::tc_fence_after();
+      if (half >= boxes) hand_back();
+#pragma unroll 1
+      for (int b = half; b < boxes; b += 2) {
+        uint32_t r[32], o[W];
+        ptx::tmem_ld_32x32b_x32(t_acc + tcol, r);
+        ptx::tmem_ld_wait();
+        if (b + 2 >= boxes) hand_back();
+        convert(r, creg[0], row0, o);
+        const int row1 = row0, col1 = col0;
+        if (b + 2 < boxes) {
+          place(b + 2, row0, col0, tcol);
+          if (has_c) load_c(row0, col0, creg[0]);
+        }
+        store(o, row1, col1);
+      }
+    } else {
+      const int tile_row = first_row<CTAS, MBLK>(mt, cta_rank, M), live_j = live_blocks<CTAS, MBLK>(mt, M);
+      // box n of this warp in this tile: first row / column, accumulator column, inside the matrix?
+      auto geom = [&](int n, int& row0, int& col0, int& tcol) -> bool {
+        const int it = half + 2 * n;
+        const int j = it / kSub, sc = it - j * kSub;
+        row0 = tile_row + j * kBlockM + q * 32;
+        col0 = nt * BLOCK_N + sc * 32;
+        tcol = j * BLOCK_N + sc * 32;
+        return it < kIters && j < live_j && row0 < M && col0 < col_end;
+      };
+      auto load_c_of = [&](int n, uint32_t (&c)[W]) {
+        int row0, col0, tcol;
+        if (geom(n, row0, col0, tcol)) load_c(row0, col0, c);
+      };
+      if (has_c) {
+#pragma unroll
+        for (int n = 0; n < P; ++n)
+          if (n < kBoxes) load_c_of(n, creg[n]);
+      }
+      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
+      ptx::tc_fence_after();
+      uint32_t racc[2][32];
+      {
+        int row0, col0, tcol;
+        geom(0, row0, col0, tcol);
+        ptx::tmem_ld_32x32b_x32(t_acc + tcol, racc[0]);
+      }
+#pragma unroll
+      for (int n = 0; n < kBoxes; ++n) {
+        if (half + 2 * n >= kIters) break;  // same answer for the whole warp
+        ptx::tmem_ld_wait();
+        if (half + 2 * (n + 1) < kIters) {
+          int row1, col1, tcol1;
+          geom(n + 1, row1, col1, tcol1);
+          ptx::tmem_ld_32x32b_x32(t_acc + tcol1, racc[(n + 1) & 1]);
+        } else {
+          hand_back();
+        }
+        int row0, col0, tcol;
+        const bool live = geom(n, row0, col0, tcol);  // same answer for the whole warp
+        uint32_t o[W];
+        if (live) convert(racc[n & 1], creg[n % P], row0, o);
+        // the C registers of box n are free: fetch box n + P into them (also when box n lies outside the matrix)
+        if (has_c && n + P < kBoxes) load_c_of(n + P, creg[n % P]);
+        if (live) store(o, row0, col0);
+      }
     }
     if (++acc == ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
   }
@@ -535,7 +587,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   extern __shared__ uint8_t smem_raw[];
   // Operand atoms need 1024-byte alignment for the 128-byte swizzle.
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* epi = smem + p.stages * C::kStageBytes;
+  constexpr bool kTall = is_tall<CTAS, MBLK>;
+  static_assert(!kTall || (SPARSE && !B_MN && C::kABoxes == 1 && C::kBBoxes == 2), "tall tiles: sparse A, K-major B");
+  // tall tiles: [slots of A and metadata | slots of B | epilogue staging]
+  constexpr int kSlotBytes = kTall ? C::kABlockBytes + C::kEBlockBytes : C::kStageBytes;
+  const int b_slot_bytes = kTall ? C::kBBoxes * p.b_rows * kAtomBytes : 0;
+  uint8_t* b_ring = smem + p.stages * kSlotBytes;
+  uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : 0);
   Shared* sh = reinterpret_cast<Shared*>(epi + p.epi_bytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -553,7 +611,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::mbar_init(&sh->tmem_empty[a], kEpiWarps * CTAS);  // one arrival per epilogue warp of the pair
     }
     for (int w = 0; w < kEpiWarps; ++w)
-      for (int b = 0; b < 4; ++b) ptx::mbar_init(&sh->c_full[w][b], 1);
+      for (int b = 0; b < 2; ++b) ptx::mbar_init(&sh->c_full[w][b], 1);
     sh->abort = 0;
     ptx::fence_barrier_init();
     ptx::prefetch_tensormap(&map_a);
@@ -576,7 +634,107 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   let_next_start();
   wait_for_stream();
 
-  if (warp == 0) {
+  // tall tiles: m-blocks of tile row mt that have rows (the rest are neither loaded nor multiplied) ...
+  auto tall_live = [&](int mt) -> int { return min(p.mblk, ((int)p.M - mt * p.mblk * kBlockM + kBlockM - 1) / kBlockM); };
+  // ... and the slots of a CTA's ring.  B's slots have no barriers of their own: the box of k-block kb lands with
+  // the k-block's first m-block, and with at most (b_stages - 1) * (m-blocks of a tile) + 1 slots that m-block's
+  // slot is free only when all of k-block kb - b_stages has been multiplied.
+  auto tall_slots = [&]() -> int {
+    const bool has_last = cluster_id == (p.m_tiles - 1) % num_clusters || p.n_tiles > 1;  // the last tile row may have fewer
+    return min(p.stages, (p.b_stages - 1) * (has_last ? tall_live(p.m_tiles - 1) : p.mblk) + 1);
+  };
+
+  if (kTall && warp == 0) {
+    // ------------------------------ TMA producer, tall tiles ------------------------------
+    if (ptx::elect_one()) {
+      int slot = 0, b_slot = 0;
+      uint32_t phase = 0;
+      const int slots = tall_slots();
+      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), full0 = ptx::smem_u32(&sh->full[0]);
+      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
+        int mt, nt;
+        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
+        const int live = tall_live(mt), blk0 = mt * p.mblk;
+        bool ok = true;
+        for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
+#pragma unroll
+          for (int j = 0; j < MBLK; ++j) {
+            if (j >= live) break;
+            if (!(ok = bounded_wait(&sh->empty[slot], phase ^ 1u, sh, p.status, 1u, p.wait_limit))) break;
+            const uint32_t full = full0 + 8 * slot, sa = ring + slot * kSlotBytes;
+            // (test hook: the slot is neither armed nor loaded, so that the issuer's wait for it expires)
+            if (!(j == 0 && p.test_skip_stage && t == cluster_id && kb == 1)) {
+              ptx::mbar_expect_tx(&sh->full[slot], (uint32_t)(kSlotBytes + (j == 0 ? b_slot_bytes : 0)));
+              if (j == 0) {
+                const uint32_t sb = b_ring_addr + b_slot * b_slot_bytes;
+                if (p.b_3d) {
+                  ptx::tma_load_3d<1>(sb, &map_b, full, 0, nt * BLOCK_N, kb * C::kBBoxes);
+                } else {
+#pragma unroll
+                  for (int i = 0; i < C::kBBoxes; ++i)
+                    ptx::tma_load_2d<1>(sb + i * p.b_rows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * C::kAtomElems,
+                                        nt * BLOCK_N);
+                }
+              }
+              ptx::tma_load_2d<1>(sa, &map_a, full, kb * C::kAtomElems, (blk0 + j) * kBlockM);
+              ptx::tma_load_3d<1>(sa + C::kABlockBytes, &map_e, full, 0, 16 * kb * C::kEBlocks, blk0 + j);
+            }
+            if (++slot == slots) { slot = 0; phase ^= 1u; }
+          }
+          if (++b_slot == p.b_stages) b_slot = 0;
+        }
+      }
+    }
+  } else if (kTall && warp == 1) {
+    // ------------------------------ MMA issuer, tall tiles ------------------------------
+    if (ptx::elect_one()) {
+      int slot = 0, b_slot = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      const int slots = tall_slots();
+      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), b_atom = p.b_rows * kAtomBytes;
+      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
+        int mt, nt;
+        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
+        const int live = tall_live(mt);
+        const uint32_t idesc = make_idesc<KIND>(SPARSE, false, p.a_fmt, kBlockM, min(BLOCK_N, (int)p.N - nt * BLOCK_N),
+                                                KIND == 0 && p.acc_f16);
+        if (!bounded_wait(&sh->tmem_empty[0], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
+        ptx::tc_fence_after();
+        bool ok = true;
+        for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
+          const uint64_t db0 = ptx::smem_desc(b_ring_addr + b_slot * b_slot_bytes, ptx::kLayoutSw128, 1024);
+#pragma unroll
+          for (int j = 0; j < MBLK; ++j) {
+            if (j >= live) break;
+            if (!(ok = bounded_wait(&sh->full[slot], phase, sh, p.status, 3u, p.wait_limit))) break;
+            ptx::tc_fence_after();
+            // (metadata columns per slot: a full slot also says that nothing reads its columns any more)
+            const uint32_t sa = ring + slot * kSlotBytes, e_tmem = tmem_base + C::kECol + slot * 8, d_tmem = tmem_base + j * BLOCK_N;
+#pragma unroll
+            for (int i = 0; i < C::kEBlocks; ++i)
+              ptx::tmem_cp_128x128b<CTAS>(e_tmem + 4 * i, ptx::smem_desc(sa + C::kABlockBytes + i * 2048, ptx::kLayoutNone, 128));
+            const uint64_t da0 = ptx::smem_desc(sa, ptx::kLayoutSw128, 1024);
+#pragma unroll
+            for (int k = 0; k < C::kMmasPerStage; ++k) {
+              // the address fields of the descriptors count 16-byte units
+              const uint64_t da = da0 + (k * 32 >> 4), db = db0 + (((k >> 1) * b_atom + (k & 1) * 64) >> 4);
+              const uint32_t accumulate = (kb > 0 || k > 0) ? 1u : 0u;
+              if (!one_byte_operands(KIND))
+                ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + (k & ~1), idesc | (uint32_t)(k & 1), accumulate);
+              else
+                ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + 2 * k, idesc, accumulate);
+            }
+            ptx::tc_commit(&sh->empty[slot]);
+            if (++slot == slots) { slot = 0; phase ^= 1u; }
+          }
+          if (++b_slot == p.b_stages) b_slot = 0;
+        }
+        if (!ok) break;
+        ptx::tc_commit(&sh->tmem_full[0]);
+        acc_phase ^= 1u;
+      }
+    }
+  } else if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (ptx::elect_one()) {
       // (Shared-memory and barrier addresses as plain integers, as few loads per stage as the boxes allow: the
@@ -725,7 +883,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   } else if (warp >= kFirstEpiWarp) {
     // ------------------------------ epilogue ------------------------------
     const int cs = elem_bytes((sp24_dtype)p.cd_type);
-    if (p.epi_lsu) {
+    if (kTall || p.epi_lsu) {
       // loads and stores by the epilogue warps themselves
 #define SP24_EPILOGUE(CS_, COLS_)                                                                                    \
   epilogue_direct<KIND, CS_, COLS_, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id, \
@@ -750,7 +908,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     constexpr int buf_bytes = 4096, split = 2;
     const int first_it = ew >> 2;
     const int warp_bytes = p.epi_bytes / kEpiWarps;
-    const int nbuf = min(4, warp_bytes / buf_bytes);  // staging buffers of this warp: 1 or 2
+    const int nbuf = min(2, warp_bytes / buf_bytes);  // staging buffers of this warp: 1 or 2
     const int ahead = nbuf > 1 ? nbuf - 1 : 1;      // boxes the C loads run ahead (their latency is what the epilogue waits on)
     // stores that may still be reading their buffer when the next buffer is claimed: with C the
     // buffer of box seq + ahead is claimed at the end of box seq, without C that of box seq + 1
@@ -834,9 +992,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           ptx::tma_store_2d(&map_d, buf, col0, row0);
           ptx::bulk_commit_group();
           // the buffer claimed next is free once the store that used it last has read it
-          if (pending_ok >= 3) ptx::bulk_wait_group_read<3>();
-          else if (pending_ok == 2) ptx::bulk_wait_group_read<2>();
-          else if (pending_ok == 1) ptx::bulk_wait_group_read<1>();
+          if (pending_ok == 1) ptx::bulk_wait_group_read<1>();
           else ptx::bulk_wait_group_read<0>();
           if (p.has_c) issue_c_load();
         }
@@ -1029,7 +1185,24 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   GemmParams p = base;
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
-  const int tile_m = kBlockM * CTAS * MBLK;
+  int tile_m = kBlockM * CTAS * MBLK, ring_stages = C::kMinStagesFit, ring_bytes = C::kStageBytes, b_ring_bytes = 0;
+  uint32_t b_box_rows = C::kBRows;
+  if constexpr (is_tall<CTAS, MBLK>) {
+    p.b_rows = (int32_t)(d->N < BLOCK_N ? d->N : BLOCK_N);
+    tile_m = p.mblk * kBlockM;
+    b_box_rows = p.b_rows;
+    // slots of A (each k-block needs mblk) and of B: the split with the most of A in flight
+    const int b_slot = C::kBBoxes * p.b_rows * kAtomBytes, budget = C::kSmemLimit - 16384;
+    ring_bytes = C::kABlockBytes + C::kEBlockBytes;
+    ring_stages = 0;
+    for (int bs = 2; bs <= 8 && bs * b_slot < budget; ++bs) {
+      int slots = (budget - bs * b_slot) / ring_bytes;
+      if (slots > (bs - 1) * p.mblk + 1) slots = (bs - 1) * p.mblk + 1;
+      if (slots > C::kMaxStages) slots = C::kMaxStages;
+      if (slots > ring_stages) { ring_stages = slots; p.b_stages = bs; }
+    }
+    b_ring_bytes = p.b_stages * b_slot;
+  }
   p.m_tiles = (int)((d->M + tile_m - 1) / tile_m);
   p.n_tiles = (int)((d->N + BLOCK_N - 1) / BLOCK_N);
   p.k_blocks = (int)((d->K + C::kKPerStage - 1) / C::kKPerStage);
@@ -1038,7 +1211,7 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   CUtensorMap map_a, map_b, map_e;
   const uint32_t atom_elems = kAtomBytes / es;
   const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, MBLK * kBlockM, 128);
+  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, (is_tall<CTAS, MBLK> ? 1 : MBLK) * kBlockM, 128);
   if (st != SP24_OK) return st;
   if (p.conv) {
     // B = im2col view of the NHWC activation: boxes of kBRows output pixels x one 128-byte run of channels
@@ -1054,15 +1227,15 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
     // needs the zeros that only the two-dimensional map gives it)
     p.b_3d = 1;
     st = make_map(&map_b, MapShape{B, {atom_elems, (uint64_t)d->N, (uint64_t)d->K / atom_elems},
-                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, (uint32_t)C::kBRows, (uint32_t)C::kBBoxes}, es, 128});
+                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, b_box_rows, (uint32_t)C::kBBoxes}, es, 128});
   } else {
-    st = make_map(&map_b, B, es, d->N, d->K, d->ldb * es, atom_elems, C::kBRows, 128);
+    st = make_map(&map_b, B, es, d->N, d->K, d->ldb * es, atom_elems, b_box_rows, 128);
   }
   if (st != SP24_OK) return st;
   if (SPARSE) {
     // metadata as rows of 128 bytes: 16 * meta_kb of them per 128 rows of A
     st = make_map(&map_e, MapShape{meta, {128, (uint64_t)p.meta_kb * 16, (uint64_t)((d->M + 127) / 128)},
-                                   {128, (uint64_t)p.meta_kb * 2048}, {128, 16 * C::kEBlocks, MBLK}, 1, 0});
+                                   {128, (uint64_t)p.meta_kb * 2048}, {128, 16 * C::kEBlocks, is_tall<CTAS, MBLK> ? 1 : MBLK}, 1, 0});
     if (st != SP24_OK) return st;
   } else {
     map_e = map_a;
@@ -1070,8 +1243,8 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   const int cs = elem_bytes(d->cd_type);
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
-  p.stages = C::kMinStagesFit > C::kMaxStages ? C::kMaxStages : C::kMinStagesFit;
-  const int room = C::kSmemLimit - p.stages * C::kStageBytes;
+  p.stages = ring_stages > C::kMaxStages ? C::kMaxStages : ring_stages;
+  const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
   // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
   // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
   // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
@@ -1079,7 +1252,7 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
   // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
   // epilogue_direct).
-  p.epi_lsu = (p.cd_col_major || cs != 4 || room < kEpiWarps * 4096) ? 1 : 0;
+  p.epi_lsu = (is_tall<CTAS, MBLK> || p.cd_col_major || cs != 4 || room < kEpiWarps * 4096) ? 1 : 0;
   p.epi_bytes = room >= kEpiWarps * 4096 ? kEpiWarps * 4096 : 16384;
   CUtensorMap map_c, map_d;
   if (p.epi_lsu) {
@@ -1123,7 +1296,7 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
   return 256;
 }
 
-// Tile choice.  Small problems: single CTAs, 128 x 128 tiles.  Otherwise a pair of CTAs, and among the
+// Tile choice.  At most 128 columns: see below.  Small problems: single CTAs, 128 x 128 tiles.  Otherwise a pair of CTAs, and among the
 // pair shapes the one with the smallest estimated time = rounds of tiles over the pairs x time of one
 // tile.  The tile times are measured ratios (unit: one 256 x 224 tile per unit of K; interleaved runs on
 // 2048..8192-row problems with K = 4096..16384):
@@ -1138,10 +1311,25 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
 // the fewest rounds.
 static void choose_tile(const sp24_gemm_desc* d, int& ctas, int& block_n, int& mblk) {
   const int64_t n224 = (d->N + 223) / 224;
+  const bool k_major_b = d->order_b == SP24_COL_MAJOR;
   ctas = 1; block_n = 128; mblk = 1;
+  if (!d->a_is_dense && k_major_b && d->N <= 128) {
+    // One column of tiles: all of A is streamed once, and what counts is how evenly its 128-row blocks are spread
+    // over the SMs.  Up to one block per SM: single blocks (us: 12288 x 32 x 4096 bf16 14.9 against 16.0 with
+    // pairs of CTAs, 12288 x 128 x 12288 40.6 against 43.1).  Beyond: tall tiles of the two or three blocks that
+    // give the fewest blocks in a row on one SM, three if equal (B is loaded once per tile): 49152 rows x 12288,
+    // bf16, 32 / 64 / 128 columns 103 / 107 / 118 us against 120 / 128 / 131 with single blocks or pairs; 24576
+    // rows 55 against 77; int8 30560 x 32 x 576 4.7 against 8.6, 24576 x 96 x 4096 18.2 against 19.1.  (The floor
+    // of the 49152-row weight is 104 us at the copy rate.)
+    const int64_t sms = sm_count(), blocks = (d->M + kBlockM - 1) / kBlockM;
+    if (blocks > sms) {
+      const int64_t chain2 = 2 * ((blocks + 2 * sms - 1) / (2 * sms)), chain3 = 3 * ((blocks + 3 * sms - 1) / (3 * sms));
+      mblk = chain2 < chain3 ? 2 : 3;
+    }
+    return;
+  }
   if (d->M < 256 || (d->M / 256) * n224 < 32) return;
   ctas = 2; block_n = 224;
-  const bool k_major_b = d->order_b == SP24_COL_MAJOR;
   const int64_t pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
   const bool bits16 = d->ab_type == SP24_F16 || d->ab_type == SP24_BF16;
   const bool has_240 = bits16 && k_major_b && elem_bytes(d->cd_type) == 2;
@@ -1319,6 +1507,8 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
     block_n = cfg.block_n.load(std::memory_order_relaxed);
     mblk = cfg.mblk.load(std::memory_order_relaxed);
   }
+  if (cv && ctas == 1) mblk = 1;  // tall tiles load no im2col view
+  p.mblk = mblk;
   if (const int b = cfg.band.load(std::memory_order_relaxed)) p.band = b;
   const bool b_mn = d->order_b == SP24_ROW_MAJOR;  // B stored N-contiguous
   if (cfg.log.load(std::memory_order_relaxed))
@@ -1359,6 +1549,11 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   SP24_DISPATCH_MN(1, 128, 1)
   SP24_DISPATCH_MN(2, 224, 1)
   SP24_DISPATCH_MN(2, 224, 2)
+  if (ctas == 1 && block_n == 128 && (mblk == 2 || mblk == kTallBlocks) && sparse && !b_mn)
+    return tf32 ? launch<2, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
+                : (f8 ? launch<3, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
+                      : (i8 ? launch<1, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
+                            : launch<0, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)));
 #undef SP24_DISPATCH
 #undef SP24_DISPATCH_MN
 #undef SP24_DISPATCH_TF32
