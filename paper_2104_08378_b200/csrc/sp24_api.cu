@@ -10,14 +10,14 @@ sp24_status check_arch() {
   // per-device answer: 0 = not asked yet, 1 = sm_100, 2 = something else (callers may be on several threads)
   static std::atomic<int> known[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return SP24_ERR_CUDA;
+  SP24_CUDA_CHECK(cudaGetDevice(&dev));
   const bool cacheable = dev >= 0 && dev < 64;
   if (cacheable) {
     const int k = known[dev].load(std::memory_order_relaxed);
     if (k != 0) return k == 1 ? SP24_OK : SP24_ERR_ARCH;
   }
   int major = 0;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return SP24_ERR_CUDA;
+  SP24_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
   if (cacheable) known[dev].store(major == 10 ? 1 : 2, std::memory_order_relaxed);
   return major == 10 ? SP24_OK : SP24_ERR_ARCH;
 }

@@ -30,7 +30,13 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // The current device must be a compute-capability 10.x part; the answer is cached per device.
 sp24_status check_arch();
 
-inline sp24_status cuda_status(cudaError_t e) { return e == cudaSuccess ? SP24_OK : SP24_ERR_CUDA; }
+// The status of a runtime call.  A call that fails also leaves its code behind as the thread's last error, which the
+// plain launches read back with cudaGetLastError(): cleared here, so that only the call that failed reports it.
+inline sp24_status cuda_status(cudaError_t e) {
+  if (e == cudaSuccess) return SP24_OK;
+  (void)cudaGetLastError();
+  return SP24_ERR_CUDA;
+}
 
 // ---- launches that may start before the kernel ahead of them in the stream has ended -----------------
 // A kernel launched through launch_overlapped() is set up (blocks scheduled as the ones of the kernel
@@ -70,10 +76,9 @@ inline sp24_status launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
     if (cond) return (code);       \
   } while (0)
 
-#define SP24_CUDA_CHECK(expr)                    \
-  do {                                           \
-    cudaError_t e__ = (expr);                    \
-    if (e__ != cudaSuccess) return SP24_ERR_CUDA; \
+#define SP24_CUDA_CHECK(expr)                                    \
+  do {                                                           \
+    if (cuda_status(expr) != SP24_OK) return SP24_ERR_CUDA;      \
   } while (0)
 
 }  // namespace sp24

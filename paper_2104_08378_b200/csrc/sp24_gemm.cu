@@ -1674,7 +1674,8 @@ sp24_status static_workspace(void** out) {
   std::lock_guard<std::mutex> lock(g_static_ws_mutex);
   if (g_static_ws_ptr[dev] == nullptr) {
     void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_workspace) != cudaSuccess || ptr == nullptr) return SP24_ERR_CUDA;
+    SP24_CUDA_CHECK(cudaGetSymbolAddress(&ptr, g_static_workspace));
+    if (ptr == nullptr) return SP24_ERR_CUDA;
     g_static_ws_ptr[dev] = ptr;
   }
   *out = g_static_ws_ptr[dev];
