@@ -116,12 +116,10 @@ def _check(status: int, where: str):
         raise Sp24Error(status, where)
 
 
-_raw_stream = torch._C._cuda_getCurrentRawStream
-
-
 def _stream() -> int:
     """The current device's current stream as a handle (no Stream object is made for it)."""
-    return _raw_stream(torch.cuda.current_device())
+    device = torch.cuda.current_device()     # (first: it says what is missing on a CPU-only build of torch)
+    return torch._C._cuda_getCurrentRawStream(device)
 
 
 def _dtype_of(t: torch.Tensor, dtype: str | None) -> str:

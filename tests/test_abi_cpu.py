@@ -3,6 +3,8 @@ argument validation answers before any device work."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 from paper_2104_08378_b200 import build
 
@@ -94,3 +96,16 @@ def test_tile_plan_and_support_calls_answer_without_a_device():
     assert lib.sp24_gemm_f16acc(ctypes.byref(desc), ctypes.byref(a), one, one, one, ctypes.byref(b), None, one, one,
                                 256, None) == 2                                # FP16 operands only
     assert lib.sp24_gemm_status(None, None) == 1
+
+
+def test_the_binding_imports_without_the_cuda_parts_of_torch():
+    """The size helpers and the host-side rejections work on a CPU-only build of torch, which lacks the private CUDA
+    functions of torch._C."""
+    code = (
+        "import torch\n"
+        "for name in [n for n in dir(torch._C) if n.startswith('_cuda_')]: delattr(torch._C, name)\n"
+        "from paper_2104_08378_b200 import binding as sp\n"
+        "assert sp.values_bytes('bf16', 64, 128) == 64 * 64 * 2\n"
+        "assert sp.gemm_plan(sp.make_desc('bf16', 'bf16', 0, 32, 64, 32, 64, 32, 32)) is None\n")
+    done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert "Sp24Error" in done.stderr and "status 3" in done.stderr, done.stderr
