@@ -7,9 +7,10 @@ from paper_2104_08378_b200 import build
 
 HARNESS = r"""
 #include "sp24_common.cuh"
+using namespace sp24;
 __global__ void nothing() {}
 // A launch without blocks: refused on the host, with or without a device.
-extern "C" int failed_launch() { return sp24::launch_overlapped(nothing, dim3(0), dim3(32), 0, nullptr, 1); }
+extern "C" int failed_launch() { return launch_overlapped(nothing, dim3(0), dim3(32), 0, nullptr, 1); }
 static sp24_status checked() { SP24_CUDA_CHECK(cudaSetDevice(-1)); return SP24_OK; }
 extern "C" int failed_call() { return checked(); }
 extern "C" int last_error() { return (int)cudaPeekAtLastError(); }
