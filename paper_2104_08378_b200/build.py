@@ -1,9 +1,11 @@
-"""Compile the CUDA library in-tree: csrc/*.cu -> libsp24.so (sm_100a SASS only)."""
+"""Compile the CUDA library in-tree: csrc/*.cu -> libsp24.so (sm_100a SASS only), the sources side by side."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
@@ -13,7 +15,7 @@ HEADERS = sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cuh"))) + [os.path.joi
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "--shared", "-Xcompiler", "-fPIC", "-cudart", "static",
+    "-Xcompiler", "-fPIC", "-cudart", "static",
     "-I", os.path.join(_ROOT, "include"),
 ]
 
@@ -36,8 +38,11 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     """Run nvcc if the library is missing or older than its sources; returns the .so path."""
     if force or needs_build():
         tmp = f"{LIB_PATH}.{os.getpid()}.tmp"
-        cmd = [_nvcc()] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + SOURCES
-        subprocess.check_call(cmd)
+        compile_ = [_nvcc()] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else [])
+        with tempfile.TemporaryDirectory() as objects, ThreadPoolExecutor(os.cpu_count()) as pool:
+            names = [os.path.join(objects, os.path.basename(src) + ".o") for src in SOURCES]
+            list(pool.map(lambda pair: subprocess.check_call(compile_ + ["-c", "-o", *pair]), zip(names, SOURCES)))
+            subprocess.check_call([_nvcc()] + NVCC_FLAGS + ["--shared", "-o", tmp] + names)
         os.replace(tmp, LIB_PATH)
     return LIB_PATH
 

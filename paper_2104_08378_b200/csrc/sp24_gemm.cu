@@ -1,1036 +1,14 @@
-// D = alpha * A * B + beta * C on the sm_100a tensor cores (Section 3.2, Figure 2 of arXiv
-// 2104.08378): A is either 2:4-compressed (values + metadata, tcgen05.mma.sp) or dense
-// (tcgen05.mma, the "dense variant" that supplies the sparse-vs-dense speedup).
-//
-// One persistent, warp-specialised kernel:
-//   warp 0   TMA producer: compressed-A tiles, metadata blocks and B tiles of one k-block into a
-//            ring of shared-memory stages (mbarrier expect_tx / complete_tx);
-//   warp 1   MMA issuer (one elected thread): copies the stage's metadata shared -> tensor
-//            memory (tcgen05.cp), issues the tcgen05.mma[.sp] of the stage, commits the stage
-//            back to the producer and, after the last k-block, the accumulators to the epilogue;
-//            owns the tensor-memory allocation;
-//   warps 2-9 epilogue, two per tensor-memory lane quarter taking alternate 32-column boxes:
-//            tcgen05.ld accumulator -> registers (the next box's load already under way), alpha /
-//            beta / conversion in registers, then one of two forms.  4-byte row-major outputs: a
-//            staging box per warp, C boxes TMA-loaded a few boxes ahead, TMA store of the D box, if
-//            shared memory has room for the boxes.  All others: the warps load C and store D
-//            themselves, through small per-warp transposing buffers, and hand the accumulators back
-//            as soon as their last box is in registers.
-// CTAS == 2 runs a pair of CTAs (cluster of two): each CTA loads its 128 rows of A / metadata per
-// m-block and its half of B, CTA 0 issues cta_group::2 MMAs (M = 256) for both.
-// MBLK == 2 gives every CTA two m-blocks (two accumulators, one B tile): what an SM can pull in
-// from the L2 per clock, not the tensor pipe, bounds this kernel, and sharing the B tile between
-// two m-blocks cuts the bytes per flop by about a third.  The two accumulators then fill tensor
-// memory, so the epilogue is not overlapped with the next tile's main loop; MBLK == 1 keeps two
-// accumulator buffers and overlaps it.
-// Every wait is bounded: on expiry the role records a code in the status record and all roles
-// leave through the normal teardown (no trap, no endless spin).  The kernel never clears the
-// record: it stays at the first expired wait, across launches, until the host reads it.
-#include <cuda.h>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
+// Host side of the GEMM (kernel: sp24_gemm_kernel.cuh): tensor maps, tile choice, argument checks, entry points.
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
 
-#include "sp24_common.cuh"
-#include "sp24_ptx.cuh"
+#include "sp24_gemm_kernel.cuh"
 
 namespace sp24 {
 namespace {
 
-constexpr int kBlockM = 128;              // rows of A per CTA and m-block (tensor-memory lanes)
-constexpr int kAtomBytes = 128;           // bytes per row of one swizzle-128B operand atom
-constexpr int kEpiWarps = 8;              // two per tensor-memory lane quarter, taking alternate boxes
-constexpr int kFirstEpiWarp = 2;          // warp 0: TMA producer, warp 1: MMA issuer
-constexpr int kNumThreads = 32 * (kFirstEpiWarp + kEpiWarps);
-// (Ten warps leave three on two of the SM's four sub-partitions, which caps the kernel at 168
-// registers per thread; trading registers between the roles with setmaxnreg was tried and made the
-// compiler spill far more than it saved.)
-constexpr long long kWaitTimeoutCycles = 2000ll * 1000ll * 1000ll;  // per wait: 1-2 s of SM clock
-constexpr uint32_t kTmemCols = 512;
-
-struct GemmParams {
-  int64_t M, N, K;
-  int64_t ldc, ldd;   // elements
-  const void* C;
-  void* D;
-  uint32_t* status;   // [0] = 0 ok, else code of the first wait that expired; [1] = number of expired waits
-  float alpha, beta;
-  int32_t m_tiles, n_tiles, k_blocks;
-  int32_t meta_kb;    // 128-column metadata blocks per 128-row block (K padded to 256)
-  int32_t a_fmt;      // 0 f16, 1 bf16 (kind::f16); ignored for int8
-  int32_t cd_type;    // sp24_dtype of C / D
-  int32_t has_c;
-  int32_t stages, epi_bytes;  // shared memory: ring stages and bytes of epilogue staging
-  int32_t epi_lsu;            // epilogue form: 1 = the warps' own loads and stores, 0 = TMA through staging boxes
-  long long wait_limit;       // SM cycles after which a device-side wait gives up
-  int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
-  int32_t band;       // m-tiles per band of the tile sweep
-  int32_t mblk, b_rows, b_stages;  // tall tiles only: m-blocks of a tile, rows of a B box, slots of the B ring
-  int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
-  int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout)
-  // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
-  int32_t conv, conv_h, conv_w, conv_c;
-  // int8 dequantising epilogue (sp24_gemm_i8_dequant): out = act(row_scale[i] * acc + bias[i]),
-  // requantised with out_inv_scale when the output type is int8
-  int32_t dequant, relu;
-  int32_t acc_f16;    // FP16 accumulation (kind::f16 with a binary16 accumulator; FP16 operands only)
-  const float* row_scale;
-  const float* bias;
-  float out_inv_scale;
-};
-
-// MMA kinds: 0 = f16 / bf16, 1 = int8, 2 = tf32, 3 = 8-bit floating point (e4m3 / e5m2)
-__host__ __device__ constexpr bool one_byte_operands(int kind) { return kind == 1 || kind == 3; }
-
-// Tall tiles (CTAS == 1, MBLK == kTallBlocks; sparse A, K-major B): up to 128 columns, two or three m-blocks (set
-// per launch) that share each B box.  Their ring is finer: one slot per m-block and k-block (A and metadata) and
-// a second ring for the B boxes, so that a slot is refilled as soon as its four MMAs are done.
-constexpr int kTallBlocks = 3;
-template <int CTAS, int MBLK>
-constexpr bool is_tall = CTAS == 1 && MBLK == kTallBlocks;
-
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
-struct Cfg {
-  // 128-byte atoms per stage: sparse A is half as wide as B; the dense variant with two
-  // m-blocks takes one atom per operand so that four stages still fit
-  static constexpr int kBBoxes = SPARSE ? 2 : (MBLK == 2 ? 1 : 2);
-  static constexpr int kABoxes = SPARSE ? 1 : kBBoxes;
-  static constexpr int kBRows = BLOCK_N / CTAS;                    // B rows (N) this CTA loads
-  static constexpr int kABlockBytes = kABoxes * kBlockM * kAtomBytes;  // one m-block
-  static_assert(MBLK == 1 || kABoxes == 1, "the m-blocks of a stage are one box of rows");
-  static constexpr int kABytes = MBLK * kABlockBytes;
-  static constexpr int kAtomElems = KIND == 0 ? 64 : (one_byte_operands(KIND) ? 128 : 32);  // elements per 128-byte row
-  static constexpr int kKPerStage = kAtomElems * kBBoxes;  // logical K per stage
-  // B with N contiguous (MN-major operand): 128-byte chunks along N, each kKPerStage k-rows of 128 bytes
-  static constexpr int kBChunkElems = kAtomElems;
-  static constexpr int kBChunks = (kBRows + kBChunkElems - 1) / kBChunkElems;
-  static constexpr int kBChunkBytes = kKPerStage * kAtomBytes;
-  static constexpr int kBKStepBytes = (SPARSE ? 2 : 1) * (kAtomElems / 4) * kAtomBytes;  // k-rows of one MMA
-  // an MN-major tf32 operand exists only in the 128-byte swizzle with 32-byte units (groups of 4 k-rows)
-  static constexpr uint32_t kBMnLayout = KIND == 2 ? ptx::kLayoutSw128Base32 : ptx::kLayoutSw128;
-  static constexpr uint32_t kBMnSbo = KIND == 2 ? 512 : 1024;
-  static constexpr int kBBytes = B_MN ? kBChunks * kBChunkBytes : kBBoxes * kBRows * kAtomBytes;
-  static constexpr int kEBlocks = SPARSE ? (one_byte_operands(KIND) ? 2 : 1) : 0;  // 2048-byte metadata blocks per m-block and stage
-  static constexpr int kEBlockBytes = kEBlocks * 2048;
-  static constexpr int kEBytes = MBLK * kEBlockBytes;
-  static constexpr int kEAlloc = (kEBytes + 1023) / 1024 * 1024;
-  static constexpr int kStageBytes = kABytes + kBBytes + kEAlloc;
-  // shared memory: [stage ring | epilogue staging | barriers]; 1 KB of slack for the 1024-byte alignment
-  // The split between ring stages and epilogue staging is made per launch (the output type
-  // decides how much staging is useful).
-  static constexpr int kSmemLimit = 232448 - 1024 - 512;
-  static constexpr int kMaxStages = is_tall<CTAS, MBLK> ? 12 : 8;
-  static constexpr int kMinStagesFit = (kSmemLimit - 16384) / kStageBytes;  // with the smallest staging
-  static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
-  static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
-  static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block
-  static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
-  static_assert(kMinStagesFit >= 2, "need at least two stages");
-  // the epilogue moves 32-column boxes; a last box of 16 columns (240-column tiles) is handled only by
-  // epilogue_direct, which bounds every access by the tile's last column
-  static_assert(BLOCK_N % 16 == 0, "tile width");
-  static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte alignment of the atoms");
-  static_assert(kECol + (SPARSE ? (is_tall<CTAS, MBLK> ? kMaxStages * 8 : 2 * MBLK * 8) : 0) <= (int)kTmemCols,
-                "tensor memory overflow");
-};
-
-struct Shared {
-  uint64_t full[12], empty[12], tmem_full[2], tmem_empty[2];
-  uint64_t c_full[kEpiWarps][2];   // per epilogue warp and staging buffer: C box has landed
-  uint32_t tmem_base;
-  volatile uint32_t abort;
-};
-static_assert(sizeof(Shared) <= 512, "barrier block");
-
-__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, Shared* sh, uint32_t* status,
-                                             uint32_t code, long long limit) {
-  // fast path: poll a while before any bookkeeping; try_wait itself suspends the thread briefly
-#pragma unroll 1
-  for (int i = 0; i < 64; ++i)
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  uint32_t spins = 0;
-  while (true) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    if ((++spins & 255u) == 0) {
-      if (sh->abort) return false;
-      if (clock64() - t0 > limit) {
-        sh->abort = 1;
-        atomicCAS(status, 0u, code);   // sticky: the first code stays until the host reads and clears it
-        atomicAdd(status + 1, 1u);
-        return false;
-      }
-    }
-  }
-}
-
-// tile index -> (m_tile, n_tile): bands of `band_rows` m-tiles are swept n-tile by n-tile so that
-// the tiles in flight at one time share a few A row-panels and B column-panels in the L2; every
-// other band is swept from the last n-tile back, so that the first wave of a band uses the B
-// columns the last wave of the band before has just read.
-__device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int band_rows, int& mt, int& nt) {
-  int per_band = band_rows * n_tiles;
-  int band = t / per_band, in_band = t - band * per_band;
-  int rows = min(band_rows, m_tiles - band * band_rows);
-  nt = in_band / rows;
-  mt = band * band_rows + (in_band - nt * rows);
-  if (band & 1) nt = n_tiles - 1 - nt;
-}
-
-template <int KIND>
-__device__ __forceinline__ uint32_t make_idesc(bool sparse, bool b_mn_major, int a_fmt, int m, int n, bool acc_f16) {
-  uint32_t d = 0;
-  d |= (sparse ? 1u : 0u) << 2;
-  d |= (KIND == 1 ? 2u : (acc_f16 ? 0u : 1u)) << 4;  // accumulator: int32 / fp32 / fp16
-  // kind f16: f16 = 0, bf16 = 1; tf32: 2; int8: 1 = signed; 8-bit floats: e4m3 = 0, e5m2 = 1
-  uint32_t fmt = (KIND == 0 || KIND == 3) ? (uint32_t)a_fmt : (KIND == 1 ? 1u : 2u);
-  d |= fmt << 7;
-  d |= fmt << 10;
-  d |= (b_mn_major ? 1u : 0u) << 16;               // A is always K-major
-  d |= (uint32_t)(n >> 3) << 17;
-  d |= (uint32_t)(m >> 4) << 24;
-  return d;                                        // no negate, no saturate
-}
-
-// Rows of A of a tile.  One m-block: rank 0 has the first 128 rows, rank 1 the next.  Two m-blocks: a CTA's
-// blocks are neighbours (rank 0 rows 0-255 of the tile, rank 1 rows 256-511), so that one load brings
-// both; in a last tile of at most 256 rows each CTA has one block instead of rank 0 having two.
-template <int CTAS, int MBLK>
-__device__ __forceinline__ int live_blocks(int mt, int M) {
-  return MBLK != 2 ? 1 : (M - mt * (MBLK * CTAS * kBlockM) > CTAS * kBlockM ? 2 : 1);
-}
-template <int CTAS, int MBLK>
-__device__ __forceinline__ int first_row(int mt, int cta_rank, int M) {
-  static_assert(MBLK == 1 || (CTAS == 2 && MBLK == 2) || is_tall<CTAS, MBLK>, "tile shape");  // (tall: not used)
-  return mt * (MBLK * CTAS * kBlockM) + cta_rank * kBlockM * live_blocks<CTAS, MBLK>(mt, M);
-}
-
-// ---- epilogue helpers ----------------------------------------------------------------------------
-// Dequantising epilogue of the int8 path, all in fp32 and in exactly this order (the int8 output
-// is compared bit for bit): t = float(acc) (round to nearest), y = fma(scale, t, bias), optional
-// max(y, 0); int8 output: round-to-nearest-even of y * out_inv_scale, clamped to [-127, 127].
-__device__ __forceinline__ float dequant_value(uint32_t acc, float scale, float bias, int relu) {
-  float y = __fmaf_rn(scale, __int2float_rn((int)acc), bias);
-  return relu ? fmaxf(y, 0.f) : y;
-}
-__device__ __forceinline__ int requant_i8(float y, float inv) {
-  int q = __float2int_rn(__fmul_rn(y, inv));
-  return max(-127, min(127, q));
-}
-
-__device__ __forceinline__ uint32_t pack_16bit(float lo, float hi, bool bf) {
-  if (bf) {
-    __nv_bfloat162 o = __float22bfloat162_rn(make_float2(lo, hi));
-    return *reinterpret_cast<uint32_t*>(&o);
-  }
-  __half2 o = __float22half2_rn(make_float2(lo, hi));
-  return *reinterpret_cast<uint32_t*>(&o);
-}
-__device__ __forceinline__ float2 unpack_16bit(uint32_t w, bool bf) {
-  return bf ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w))
-            : __half22float2(*reinterpret_cast<const __half2*>(&w));
-}
-
-// One thread's row of a 32-column box: out = alpha * acc + beta * c (or the dequantising form) as
-// the packed words of the output row: 8 words for 1-byte outputs (CS = 1: the dequantising form),
-// 16 for 2-byte outputs (CS = 2), 32 for 4-byte ones.
-// `c` holds the row's C values in the same packing and is read only if has_c.  One multiply and
-// one fused multiply-add per element, whichever path stores the row.
-template <int KIND, int CS>
-__device__ __forceinline__ void compute_row(const uint32_t (&r)[32], const uint32_t (&c)[8 * CS], bool has_c,
-                                            const GemmParams& p, float scale, float bias, uint32_t (&o)[8 * CS]) {
-  const bool bf = p.cd_type == SP24_BF16;
-  if constexpr (CS == 1) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      uint32_t word = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int q = requant_i8(dequant_value(r[4 * e + b], scale, bias, p.relu), p.out_inv_scale);
-        word |= ((uint32_t)q & 0xFFu) << (8 * b);
-      }
-      o[e] = word;
-    }
-  } else if constexpr (CS == 4) {
-    if (KIND == 1 && p.dequant) {
-#pragma unroll
-      for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(dequant_value(r[e], scale, bias, p.relu));
-    } else if (KIND == 1) {
-#pragma unroll
-      for (int e = 0; e < 32; ++e) o[e] = r[e] + (has_c ? c[e] : 0u);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        float f = __fmul_rn(p.alpha, __uint_as_float(r[e]));
-        if (has_c) f = __fmaf_rn(p.beta, __uint_as_float(c[e]), f);
-        o[e] = __float_as_uint(f);
-      }
-    }
-  } else {
-    if (KIND == 1) {  // dequantised to a 16-bit type (the plain int8 GEMM writes 4-byte results)
-#pragma unroll
-      for (int e = 0; e < 16; ++e)
-        o[e] = pack_16bit(dequant_value(r[2 * e], scale, bias, p.relu), dequant_value(r[2 * e + 1], scale, bias, p.relu), bf);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        float f0 = __fmul_rn(p.alpha, __uint_as_float(r[2 * e])), f1 = __fmul_rn(p.alpha, __uint_as_float(r[2 * e + 1]));
-        if (has_c) {
-          const float2 g = unpack_16bit(c[e], bf);
-          f0 = __fmaf_rn(p.beta, g.x, f0);
-          f1 = __fmaf_rn(p.beta, g.y, f1);
-        }
-        o[e] = pack_16bit(f0, f1, bf);
-      }
-    }
-  }
-}
-
-// FP16 accumulation: every accumulator cell of tensor memory holds a binary16 value in its low half
-__device__ __forceinline__ void widen_f16_accumulators(uint32_t (&r)[32]) {
-#pragma unroll
-  for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__half2float(__ushort_as_half((unsigned short)(r[e] & 0xFFFFu))));
-}
-
-// TMA-staged form of a 4-byte row-major box (rows of 128 bytes in the TMA's 128-byte swizzle: 16-byte
-// unit v of row r sits at unit v ^ (r & 7), which also keeps the row-per-thread accesses free of bank
-// conflicts): C, if any, is in the staging buffer; the result replaces it there.
-template <int KIND>
-__device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint8_t* buf, int lane, const GemmParams& p,
-                                                   float scale, float bias) {
-  uint32_t c[32], o[32];
-  uint8_t* row = buf + lane * 128;
-  if (p.has_c) {
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-      const uint4 x = *reinterpret_cast<const uint4*>(row + ((v ^ (lane & 7)) << 4));
-      c[4 * v] = x.x; c[4 * v + 1] = x.y; c[4 * v + 2] = x.z; c[4 * v + 3] = x.w;
-    }
-  }
-  compute_row<KIND, 4>(r, c, p.has_c != 0, p, scale, bias, o);
-#pragma unroll
-  for (int v = 0; v < 8; ++v)
-    *reinterpret_cast<uint4*>(row + ((v ^ (lane & 7)) << 4)) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
-}
-
-// ---- epilogue in which the warps move C and D themselves -----------------------------------------
-// C is loaded straight from global memory into registers, the first boxes of a tile before the
-// tile's accumulators are even complete, the later ones a few boxes ahead, so that no load latency
-// is left on the path that holds the accumulators (tensor memory cannot be handed back to the MMA
-// issuer before it is drained).
-// Row-major outputs: each thread loads the C values of ITS accumulator row; D: the row is converted
-// in registers, written to a small per-warp buffer in shared memory and read back transposed, so
-// that the global stores of a warp cover whole 64-byte row segments.  A "pass" is 32 rows x 64 bytes
-// (2 KB): a whole box of a 1- or 2-byte type, half a box of a 4-byte type.
-// Column-major outputs (D stored [N][M], M contiguous): the lanes of a warp hold 32 consecutive m of
-// each column, so a 4-byte box is stored straight from registers, one 128-byte line per column; the
-// 1- and 2-byte boxes are transposed on the way out of the same per-warp buffer by ldmatrix.trans.
-// The eight rows of ldmatrix matrix i are m = 8 j + 2 i + b (j = 0..3, b = 0, 1), which leaves each
-// thread with eight consecutive m of one column (2-byte) or of two columns (1-byte): 16- and 8-byte
-// stores.  16-byte unit u of buffer row m sits at u ^ (((m >> 1) ^ (m >> 3)) & 3): no bank conflicts
-// in the row-wise writes, the row-wise reads or the ldmatrix reads.
-// Measured against TMA boxes with scalar shared-memory stores (one 1-2 KB box per warp in flight, each
-// store waited for): int8 3072 x 4096 x 768 -> int8 44.7 -> 17.3 us, fp8 16384 x 8192 x 8192 -> bf16
-// 600 -> 514 us, the 3x3 convolution 50176 pixels x 256 x 2304 46.7 -> 36 us (with 240-column tiles, which
-// this form can store), int8 4096 x 32 x 4096 -> bf16 10.7 -> 9.0 us.
-template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
-__device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
-                                              int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
-                                              int lane) {
-  constexpr int kSub = (BLOCK_N + 31) / 32, kIters = MBLK * kSub;  // the last box of a 240-column tile is half a box
-  constexpr int kBoxes = (kIters + 1) / 2;  // boxes per warp and tile (the two warps of a lane quarter alternate)
-  constexpr int W = 8 * CS;                 // 32-bit words of one box row
-  constexpr int P = CS == 2 ? 4 : 1;        // boxes whose C values are held in registers (16 or 32 registers each)
-  constexpr int kPasses = CS == 4 ? 2 : 1;
-  constexpr int kUnits = CS == 1 ? 2 : 4;   // 16-byte units of a buffer row that hold data
-  constexpr int kUnitElems = 16 / CS;       // elements per 16-byte unit
-  const int q = warp & 3, ew = warp - kFirstEpiWarp, half = ew >> 2;
-  const int nbuf = p.epi_bytes >= kEpiWarps * 4096 ? 2 : 1;
-  uint8_t* stage = epi + ew * (nbuf * 2048);
-  const uint8_t* Cb = static_cast<const uint8_t*>(p.C);
-  uint8_t* Db = static_cast<uint8_t*>(p.D);
-  const size_t ldc_b = (size_t)p.ldc * CS, ldd_b = (size_t)p.ldd * CS;
-  const int M = (int)p.M, N = (int)p.N;
-  const bool has_c = CS != 1 && p.has_c != 0;
-  // ldmatrix / stmatrix: this lane's row m of the buffer (its unit 0 under the swizzle: xor the unit into bits 4..5)
-  const int tm_i = lane >> 3, tm_j = (lane & 7) >> 1;
-  const uint32_t tm_row = ptx::smem_u32(stage) + (uint32_t)((8 * tm_j + 2 * tm_i + (lane & 1)) * 64 + ((tm_i ^ tm_j) << 4));
-  const int sw = ((lane >> 1) ^ (lane >> 3)) & 3;  // swizzle of buffer row `lane`
-  uint32_t creg[P][W];
-  int acc = 0;
-  uint32_t acc_phase = 0, pass_no = 0;
-  for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-    int mt, nt;
-    tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-    const int col_end = min(N, (nt + 1) * BLOCK_N);  // columns of this tile stop here
-    // C values of the box at (row0, col0): row-major in the accumulators' order (this thread's row), column-major
-    // in the order of the stores
-    auto load_c = [&](int row0, int col0, uint32_t (&c)[W]) {
-      if constexpr (COLS) {
-        if constexpr (CS == 2) {
-          const int m = row0 + 8 * (lane & 3);
-          if (m >= M) return;
-#pragma unroll
-          for (int nb = 0; nb < 4; ++nb) {
-            const int n1 = col0 + 8 * nb + (lane >> 2);
-            if (n1 < col_end) {
-              const uint4 x = *reinterpret_cast<const uint4*>(Cb + (size_t)n1 * ldc_b + (size_t)m * CS);
-              c[4 * nb] = x.x; c[4 * nb + 1] = x.y; c[4 * nb + 2] = x.z; c[4 * nb + 3] = x.w;
-            }
-          }
-        } else if constexpr (CS == 4) {
-          if (row0 + lane >= M) return;
-          const uint8_t* src = Cb + (size_t)col0 * ldc_b + (size_t)(row0 + lane) * CS;
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (col0 + e < col_end) c[e] = *reinterpret_cast<const uint32_t*>(src + (size_t)e * ldc_b);
-        }
-        return;
-      }
-      const int row = row0 + lane;
-      if (row >= M) return;
-      const uint4* src = reinterpret_cast<const uint4*>(Cb + (size_t)row * ldc_b + (size_t)col0 * CS);
-#pragma unroll
-      for (int v = 0; v < W / 4; ++v) {
-        if (col0 + v * kUnitElems < col_end) {
-          const uint4 x = src[v];
-          c[4 * v] = x.x; c[4 * v + 1] = x.y; c[4 * v + 2] = x.z; c[4 * v + 3] = x.w;
-        }
-      }
-    };
-    // accumulators (and C) of a box -> packed output rows
-    auto convert = [&](uint32_t (&r)[32], uint32_t (&c)[W], int row0, uint32_t (&o)[W]) {
-      const uint32_t buf_off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
-      if constexpr (CS == 2 && COLS) {
-        if (has_c) {
-          // C arrived in the order of the column stores: through the buffer to the rows' owners
-          if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
-#pragma unroll
-          for (int nb = 0; nb < 4; ++nb)
-            ptx::stmatrix_x4_trans((tm_row + buf_off) ^ (uint32_t)(nb << 4), c[4 * nb], c[4 * nb + 1], c[4 * nb + 2], c[4 * nb + 3]);
-          __syncwarp();
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint4 x = *reinterpret_cast<const uint4*>(stage + buf_off + lane * 64 + ((u ^ sw) << 4));
-            c[4 * u] = x.x; c[4 * u + 1] = x.y; c[4 * u + 2] = x.z; c[4 * u + 3] = x.w;
-          }
-        }
-      }
-      if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
-      float scale = 1.f, bias = 0.f;
-      if (KIND == 1 && p.dequant) {
-        const int row = min(row0 + lane, M - 1);
-        scale = p.row_scale[row];
-        bias = p.bias ? p.bias[row] : 0.f;
-      }
-      compute_row<KIND, CS>(r, c, has_c, p, scale, bias, o);
-    };
-    // packed output rows -> D
-    auto store = [&](const uint32_t (&o)[W], int row0, int col0) {
-      if constexpr (CS == 4 && COLS) {
-        if (row0 + lane < M) {
-          uint8_t* dst = Db + (size_t)col0 * ldd_b + (size_t)(row0 + lane) * CS;
-#pragma unroll
-          for (int e = 0; e < 4 * W / CS; ++e)
-            if (col0 + e < col_end) *reinterpret_cast<uint32_t*>(dst + (size_t)e * ldd_b) = o[e];
-        }
-      } else {
-#pragma unroll
-        for (int ps = 0; ps < kPasses; ++ps) {
-          const uint32_t off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
-          uint8_t* buf = stage + off;
-          if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
-#pragma unroll
-          for (int u = 0; u < kUnits; ++u)
-            *reinterpret_cast<uint4*>(buf + lane * 64 + ((u ^ sw) << 4)) =
-                make_uint4(o[16 * ps + 4 * u], o[16 * ps + 4 * u + 1], o[16 * ps + 4 * u + 2], o[16 * ps + 4 * u + 3]);
-          __syncwarp();
-          if constexpr (COLS) {
-            const int m = row0 + 8 * (lane & 3);
-#pragma unroll
-            for (int nb = 0; nb < kUnits; ++nb) {
-              uint32_t w[4];
-              ptx::ldmatrix_x4_trans((tm_row + off) ^ (uint32_t)(nb << 4), w[0], w[1], w[2], w[3]);
-              if (m < M) {
-                if constexpr (CS == 2) {
-                  const int n1 = col0 + 8 * nb + (lane >> 2);
-                  if (n1 < col_end)
-                    *reinterpret_cast<uint4*>(Db + (size_t)n1 * ldd_b + (size_t)m * CS) = make_uint4(w[0], w[1], w[2], w[3]);
-                } else {
-                  // 16-bit units hold two neighbouring columns: split them
-                  const int n1 = col0 + 16 * nb + 2 * (lane >> 2);
-                  if (n1 < col_end) {
-                    uint8_t* dst = Db + (size_t)n1 * ldd_b + m;
-                    *reinterpret_cast<uint2*>(dst) = make_uint2(__byte_perm(w[0], w[1], 0x6420), __byte_perm(w[2], w[3], 0x6420));
-                    *reinterpret_cast<uint2*>(dst + ldd_b) =
-                        make_uint2(__byte_perm(w[0], w[1], 0x7531), __byte_perm(w[2], w[3], 0x7531));
-                  }
-                }
-              }
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < kUnits; ++k) {
-              const int i = lane + 32 * k, rr = i / kUnits, u = i % kUnits;
-              const uint4 x = *reinterpret_cast<const uint4*>(buf + rr * 64 + ((u ^ (((rr >> 1) ^ (rr >> 3)) & 3)) << 4));
-              const int grow = row0 + rr, gcol = col0 + ps * (64 / CS) + u * kUnitElems;
-              if (grow < M && gcol < col_end) *reinterpret_cast<uint4*>(Db + (size_t)grow * ldd_b + (size_t)gcol * CS) = x;
-            }
-          }
-          ++pass_no;
-        }
-      }
-    };
-    auto hand_back = [&] {  // this warp's part of the accumulators is in registers: the MMA issuer (CTA 0 of the pair) may go on
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (CTAS == 1) ptx::mbar_arrive(&sh->tmem_empty[acc]);
-        else ptx::mbar_arrive_cluster(&sh->tmem_empty[acc], 0);
-      }
-    };
-    const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-    if constexpr (is_tall<CTAS, MBLK>) {
-      // few boxes: a short loop over the ones that exist (unrolled code would be fetched for boxes that do not)
-      const int nsub = (col_end - nt * BLOCK_N + 31) / 32, row_q = mt * p.mblk * kBlockM + q * 32;
-      const int boxes = nsub * max(0, min(p.mblk, (M - row_q + kBlockM - 1) / kBlockM));  // of this lane quarter
-      auto place = [&](int b, int& row0, int& col0, int& tcol) {
-        const int j = b / nsub, sc = b - j * nsub;
-        row0 = row_q + j * kBlockM;
-        col0 = nt * BLOCK_N + sc * 32;
-        tcol = j * BLOCK_N + sc * 32;
-      };
-      int row0 = 0, col0 = 0, tcol = 0;
-      if (half < boxes) {
-        place(half, row0, col0, tcol);
-        if (has_c) load_c(row0, col0, creg[0]);
-      }
-      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-      ptx::tc_fence_after();
-      if (half >= boxes) hand_back();
-#pragma unroll 1
-      for (int b = half; b < boxes; b += 2) {
-        uint32_t r[32], o[W];
-        ptx::tmem_ld_32x32b_x32(t_acc + tcol, r);
-        ptx::tmem_ld_wait();
-        if (b + 2 >= boxes) hand_back();
-        convert(r, creg[0], row0, o);
-        const int row1 = row0, col1 = col0;
-        if (b + 2 < boxes) {
-          place(b + 2, row0, col0, tcol);
-          if (has_c) load_c(row0, col0, creg[0]);
-        }
-        store(o, row1, col1);
-      }
-    } else {
-      const int tile_row = first_row<CTAS, MBLK>(mt, cta_rank, M), live_j = live_blocks<CTAS, MBLK>(mt, M);
-      // box n of this warp in this tile: first row / column, accumulator column, inside the matrix?
-      auto geom = [&](int n, int& row0, int& col0, int& tcol) -> bool {
-        const int it = half + 2 * n;
-        const int j = it / kSub, sc = it - j * kSub;
-        row0 = tile_row + j * kBlockM + q * 32;
-        col0 = nt * BLOCK_N + sc * 32;
-        tcol = j * BLOCK_N + sc * 32;
-        return it < kIters && j < live_j && row0 < M && col0 < col_end;
-      };
-      auto load_c_of = [&](int n, uint32_t (&c)[W]) {
-        int row0, col0, tcol;
-        if (geom(n, row0, col0, tcol)) load_c(row0, col0, c);
-      };
-      if (has_c) {
-#pragma unroll
-        for (int n = 0; n < P; ++n)
-          if (n < kBoxes) load_c_of(n, creg[n]);
-      }
-      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-      ptx::tc_fence_after();
-      uint32_t racc[2][32];
-      {
-        int row0, col0, tcol;
-        geom(0, row0, col0, tcol);
-        ptx::tmem_ld_32x32b_x32(t_acc + tcol, racc[0]);
-      }
-#pragma unroll
-      for (int n = 0; n < kBoxes; ++n) {
-        if (half + 2 * n >= kIters) break;  // same answer for the whole warp
-        ptx::tmem_ld_wait();
-        if (half + 2 * (n + 1) < kIters) {
-          int row1, col1, tcol1;
-          geom(n + 1, row1, col1, tcol1);
-          ptx::tmem_ld_32x32b_x32(t_acc + tcol1, racc[(n + 1) & 1]);
-        } else {
-          hand_back();
-        }
-        int row0, col0, tcol;
-        const bool live = geom(n, row0, col0, tcol);  // same answer for the whole warp
-        uint32_t o[W];
-        if (live) convert(racc[n & 1], creg[n % P], row0, o);
-        // the C registers of box n are free: fetch box n + P into them (also when box n lies outside the matrix)
-        if (has_c && n + P < kBoxes) load_c_of(n + P, creg[n % P]);
-        if (live) store(o, row0, col0);
-      }
-    }
-    if (++acc == ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
-  }
-}
-
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
-__global__ void __launch_bounds__(kNumThreads, 1)
-gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_c,
-            const __grid_constant__ CUtensorMap map_d, const GemmParams p) {
-  using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
-  extern __shared__ uint8_t smem_raw[];
-  // Operand atoms need 1024-byte alignment for the 128-byte swizzle.
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr bool kTall = is_tall<CTAS, MBLK>;
-  static_assert(!kTall || (SPARSE && !B_MN && C::kABoxes == 1 && C::kBBoxes == 2), "tall tiles: sparse A, K-major B");
-  // tall tiles: [slots of A and metadata | slots of B | epilogue staging]
-  constexpr int kSlotBytes = kTall ? C::kABlockBytes + C::kEBlockBytes : C::kStageBytes;
-  const int b_slot_bytes = kTall ? C::kBBoxes * p.b_rows * kAtomBytes : 0;
-  uint8_t* b_ring = smem + p.stages * kSlotBytes;
-  uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : 0);
-  Shared* sh = reinterpret_cast<Shared*>(epi + p.epi_bytes);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t cta_rank = CTAS == 2 ? ptx::cluster_ctarank() : 0;
-  const int cluster_id = blockIdx.x / CTAS, num_clusters = gridDim.x / CTAS;
-  const int num_tiles = p.m_tiles * p.n_tiles;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) {
-      ptx::mbar_init(&sh->full[s], 1);
-      ptx::mbar_init(&sh->empty[s], 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      ptx::mbar_init(&sh->tmem_full[a], 1);
-      ptx::mbar_init(&sh->tmem_empty[a], kEpiWarps * CTAS);  // one arrival per epilogue warp of the pair
-    }
-    for (int w = 0; w < kEpiWarps; ++w)
-      for (int b = 0; b < 2; ++b) ptx::mbar_init(&sh->c_full[w][b], 1);
-    sh->abort = 0;
-    ptx::fence_barrier_init();
-    ptx::prefetch_tensormap(&map_a);
-    ptx::prefetch_tensormap(&map_b);
-    if (SPARSE) ptx::prefetch_tensormap(&map_e);
-    if (!p.epi_lsu) {
-      if (p.has_c) ptx::prefetch_tensormap(&map_c);
-      ptx::prefetch_tensormap(&map_d);
-    }
-  }
-  if (warp == 1) {
-    ptx::tmem_alloc<CTAS>(&sh->tmem_base, kTmemCols);
-    ptx::tmem_relinquish<CTAS>();
-  }
-  ptx::tc_fence_before();
-  __syncthreads();
-  if (CTAS == 2) ptx::cluster_sync();
-  ptx::tc_fence_after();
-  const uint32_t tmem_base = sh->tmem_base;
-  let_next_start();
-  wait_for_stream();
-
-  // tall tiles: m-blocks of tile row mt that have rows (the rest are neither loaded nor multiplied) ...
-  auto tall_live = [&](int mt) -> int { return min(p.mblk, ((int)p.M - mt * p.mblk * kBlockM + kBlockM - 1) / kBlockM); };
-  // ... and the slots of a CTA's ring.  B's slots have no barriers of their own: the box of k-block kb lands with
-  // the k-block's first m-block, and with at most (b_stages - 1) * (m-blocks of a tile) + 1 slots that m-block's
-  // slot is free only when all of k-block kb - b_stages has been multiplied.
-  auto tall_slots = [&]() -> int {
-    const bool has_last = cluster_id == (p.m_tiles - 1) % num_clusters || p.n_tiles > 1;  // the last tile row may have fewer
-    return min(p.stages, (p.b_stages - 1) * (has_last ? tall_live(p.m_tiles - 1) : p.mblk) + 1);
-  };
-
-  if (kTall && warp == 0) {
-    // ------------------------------ TMA producer, tall tiles ------------------------------
-    if (ptx::elect_one()) {
-      int slot = 0, b_slot = 0;
-      uint32_t phase = 0;
-      const int slots = tall_slots();
-      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), full0 = ptx::smem_u32(&sh->full[0]);
-      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-        int mt, nt;
-        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-        const int live = tall_live(mt), blk0 = mt * p.mblk;
-        bool ok = true;
-        for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
-#pragma unroll
-          for (int j = 0; j < MBLK; ++j) {
-            if (j >= live) break;
-            if (!(ok = bounded_wait(&sh->empty[slot], phase ^ 1u, sh, p.status, 1u, p.wait_limit))) break;
-            const uint32_t full = full0 + 8 * slot, sa = ring + slot * kSlotBytes;
-            // (test hook: the slot is neither armed nor loaded, so that the issuer's wait for it expires)
-            if (!(j == 0 && p.test_skip_stage && t == cluster_id && kb == 1)) {
-              ptx::mbar_expect_tx(&sh->full[slot], (uint32_t)(kSlotBytes + (j == 0 ? b_slot_bytes : 0)));
-              if (j == 0) {
-                const uint32_t sb = b_ring_addr + b_slot * b_slot_bytes;
-                if (p.b_3d) {
-                  ptx::tma_load_3d<1>(sb, &map_b, full, 0, nt * BLOCK_N, kb * C::kBBoxes);
-                } else {
-#pragma unroll
-                  for (int i = 0; i < C::kBBoxes; ++i)
-                    ptx::tma_load_2d<1>(sb + i * p.b_rows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * C::kAtomElems,
-                                        nt * BLOCK_N);
-                }
-              }
-              ptx::tma_load_2d<1>(sa, &map_a, full, kb * C::kAtomElems, (blk0 + j) * kBlockM);
-              ptx::tma_load_3d<1>(sa + C::kABlockBytes, &map_e, full, 0, 16 * kb * C::kEBlocks, blk0 + j);
-            }
-            if (++slot == slots) { slot = 0; phase ^= 1u; }
-          }
-          if (++b_slot == p.b_stages) b_slot = 0;
-        }
-      }
-    }
-  } else if (kTall && warp == 1) {
-    // ------------------------------ MMA issuer, tall tiles ------------------------------
-    if (ptx::elect_one()) {
-      int slot = 0, b_slot = 0;
-      uint32_t phase = 0, acc_phase = 0;
-      const int slots = tall_slots();
-      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), b_atom = p.b_rows * kAtomBytes;
-      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-        int mt, nt;
-        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-        const int live = tall_live(mt);
-        const uint32_t idesc = make_idesc<KIND>(SPARSE, false, p.a_fmt, kBlockM, min(BLOCK_N, (int)p.N - nt * BLOCK_N),
-                                                KIND == 0 && p.acc_f16);
-        if (!bounded_wait(&sh->tmem_empty[0], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
-        ptx::tc_fence_after();
-        bool ok = true;
-        for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
-          const uint64_t db0 = ptx::smem_desc(b_ring_addr + b_slot * b_slot_bytes, ptx::kLayoutSw128, 1024);
-#pragma unroll
-          for (int j = 0; j < MBLK; ++j) {
-            if (j >= live) break;
-            if (!(ok = bounded_wait(&sh->full[slot], phase, sh, p.status, 3u, p.wait_limit))) break;
-            ptx::tc_fence_after();
-            // (metadata columns per slot: a full slot also says that nothing reads its columns any more)
-            const uint32_t sa = ring + slot * kSlotBytes, e_tmem = tmem_base + C::kECol + slot * 8, d_tmem = tmem_base + j * BLOCK_N;
-#pragma unroll
-            for (int i = 0; i < C::kEBlocks; ++i)
-              ptx::tmem_cp_128x128b<CTAS>(e_tmem + 4 * i, ptx::smem_desc(sa + C::kABlockBytes + i * 2048, ptx::kLayoutNone, 128));
-            const uint64_t da0 = ptx::smem_desc(sa, ptx::kLayoutSw128, 1024);
-#pragma unroll
-            for (int k = 0; k < C::kMmasPerStage; ++k) {
-              // the address fields of the descriptors count 16-byte units
-              const uint64_t da = da0 + (k * 32 >> 4), db = db0 + (((k >> 1) * b_atom + (k & 1) * 64) >> 4);
-              const uint32_t accumulate = (kb > 0 || k > 0) ? 1u : 0u;
-              if (!one_byte_operands(KIND))
-                ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + (k & ~1), idesc | (uint32_t)(k & 1), accumulate);
-              else
-                ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + 2 * k, idesc, accumulate);
-            }
-            ptx::tc_commit(&sh->empty[slot]);
-            if (++slot == slots) { slot = 0; phase ^= 1u; }
-          }
-          if (++b_slot == p.b_stages) b_slot = 0;
-        }
-        if (!ok) break;
-        ptx::tc_commit(&sh->tmem_full[0]);
-        acc_phase ^= 1u;
-      }
-    }
-  } else if (warp == 0) {
-    // ------------------------------ TMA producer ------------------------------
-    if (ptx::elect_one()) {
-      // (Shared-memory and barrier addresses as plain integers, as few loads per stage as the boxes allow: the
-      // thread that issues them is busy for about 100 cycles per load, which delays the refill of a stage.
-      // Three loads instead of six (two m-blocks) or four: 49152 x 32 x 12288 bf16 123.1 -> 119.6 us, int8
-      // 4096 x 8192 x 4096 79.3 -> 77.2, 256 x 256 x 512 4.55 -> 4.47.)
-      int stage = 0;
-      uint32_t phase = 0;
-      constexpr int box_elems = C::kAtomElems;  // elements per 128-byte atom row
-      const uint32_t ring = ptx::smem_u32(smem);
-      const uint32_t full0 = CTAS == 2 ? ptx::map_to_cta(ptx::smem_u32(&sh->full[0]), 0) : ptx::smem_u32(&sh->full[0]);
-      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-        int mt, nt;
-        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-        // the last n-tile may be narrower: the pair then splits only the columns that exist
-        const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
-        const int col0 = nt * BLOCK_N + (int)cta_rank * (n_eff / CTAS);  // first B row (N index)
-        const int row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M);
-        constexpr uint32_t tx_bytes = (uint32_t)((C::kABytes + C::kEBytes + C::kBBytes) * CTAS);
-        // implicit convolution: (image, row, column) of this CTA's first output pixel
-        int conv_n = 0, conv_p = 0, conv_q = 0;
-        if (p.conv) {
-          conv_n = col0 / (p.conv_h * p.conv_w);
-          const int rem = col0 - conv_n * p.conv_h * p.conv_w;
-          conv_p = rem / p.conv_w;
-          conv_q = rem - conv_p * p.conv_w;
-        }
-        // (Walking K backwards in every other tile of a CTA, so that a wave first meets the END of the A
-        // panel the wave before it has just finished with, saves 12 % of the DRAM reads and 1.5 % of the
-        // time, but makes the rounding of a result depend on which CTA computed its tile: the same rows
-        // and columns would no longer give the same bits when M or N is split differently.  Not done.)
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
-          if (p.test_skip_stage && t == cluster_id && kb == 1) {
-            // test hook: this k-block of the first tile is neither armed nor loaded by either CTA, so
-            // the MMA issuer's wait for it expires and every role leaves through the abort path
-            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
-            continue;
-          }
-          const uint32_t sa = ring + stage * C::kStageBytes, sb = sa + C::kABytes, se = sb + C::kBBytes;
-          const uint32_t full = full0 + 8 * stage;
-          if (cta_rank == 0) ptx::mbar_expect_tx(&sh->full[stage], tx_bytes);
-          // both m-blocks' rows and metadata blocks are neighbours: one box each
-          if (SPARSE) ptx::tma_load_3d<CTAS>(se, &map_e, full, 0, 16 * kb * C::kEBlocks, row0 / kBlockM);
-#pragma unroll
-          for (int i = 0; i < C::kABoxes; ++i)
-            ptx::tma_load_2d<CTAS>(sa + i * MBLK * kBlockM * kAtomBytes, &map_a, full, (kb * C::kABoxes + i) * box_elems, row0);
-          if (B_MN) {
-            // B stored N-contiguous: boxes of 128 bytes along N x all k-rows of the stage
-#pragma unroll
-            for (int c = 0; c < C::kBChunks; ++c)
-              ptx::tma_load_2d<CTAS>(sb + c * C::kBChunkBytes, &map_b, full, col0 + c * C::kBChunkElems, kb * C::kKPerStage);
-          } else if (p.conv) {
-            // k = (r * 3 + s) * C + c: a stage holds channels of one filter tap; rows = output pixels
-            const int k0 = kb * C::kKPerStage;
-            const int tap = k0 / p.conv_c, c0 = k0 - tap * p.conv_c;
-            const int r = tap / 3, sx = tap - 3 * r;
-#pragma unroll
-            for (int i = 0; i < C::kBBoxes; ++i)
-              ptx::tma_load_im2col_4d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, c0 + i * box_elems, conv_q - 1,
-                                            conv_p - 1, conv_n, (uint16_t)sx, (uint16_t)r);
-          } else if (p.b_3d) {
-            ptx::tma_load_3d<CTAS>(sb, &map_b, full, 0, col0, kb * C::kBBoxes);
-          } else {
-#pragma unroll
-            for (int i = 0; i < C::kBBoxes; ++i)
-              ptx::tma_load_2d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * box_elems, col0);
-          }
-          if (++stage == p.stages) { stage = 0; phase ^= 1u; }
-        }
-      }
-    }
-  } else if (warp == 1) {
-    // ------------------------------ MMA issuer ------------------------------
-    if (cta_rank == 0 && ptx::elect_one()) {
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0, e_buf = 0;
-      for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-        int mt, nt;
-        tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-        // instruction N = the columns this tile really has (a multiple of 16, of 32 for int8)
-        const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
-        const int live = live_blocks<CTAS, MBLK>(mt, (int)p.M);  // m-blocks with rows (others are not multiplied)
-        const uint32_t idesc = make_idesc<KIND>(SPARSE, B_MN, p.a_fmt, kBlockM * CTAS, n_eff, KIND == 0 && p.acc_f16);
-        if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
-        ptx::tc_fence_after();
-        bool ok = true;
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
-          ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem + stage * C::kStageBytes);
-          const uint32_t sb = sa + C::kABytes;
-          const uint32_t se = sb + C::kBBytes;
-          // metadata columns alternate between two small tensor-memory buffers from k-block to k-block
-          const uint32_t e_base = tmem_base + C::kECol + e_buf * (MBLK * 8);
-          e_buf ^= 1u;
-          if (SPARSE) {
-#pragma unroll
-            for (int j = 0; j < MBLK; ++j) {
-              if (j >= live) break;
-#pragma unroll
-              for (int i = 0; i < C::kEBlocks; ++i)
-                ptx::tmem_cp_128x128b<CTAS>(e_base + j * 8 + 4 * i,
-                                            ptx::smem_desc(se + j * C::kEBlockBytes + i * 2048, ptx::kLayoutNone, 128));
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < MBLK; ++j) {
-            if (j >= live) break;
-            const uint32_t d_tmem = tmem_base + (acc * MBLK + j) * BLOCK_N;
-            const uint32_t e_tmem = e_base + j * 8;
-            const uint32_t saj = sa + j * C::kABlockBytes;
-#pragma unroll
-            for (int k = 0; k < C::kMmasPerStage; ++k) {
-              const uint32_t accumulate = (kb > 0 || k > 0) ? 1u : 0u;
-              if (SPARSE) {
-                // 32 bytes of compressed A and 64 bytes of B per instruction
-                uint64_t da = ptx::smem_desc(saj + k * 32, ptx::kLayoutSw128, 1024);
-                uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 1) * C::kBRows * kAtomBytes + (k & 1) * 64, ptx::kLayoutSw128, 1024);
-                if (!one_byte_operands(KIND)) {
-                  // one 32-bit metadata column per instruction: even-aligned address + selector
-                  ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + (k & ~1), idesc | (uint32_t)(k & 1), accumulate);
-                } else {
-                  ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + 2 * k, idesc, accumulate);
-                }
-              } else {
-                uint64_t da = ptx::smem_desc(saj + (k >> 2) * kBlockM * kAtomBytes + (k & 3) * 32, ptx::kLayoutSw128, 1024);
-                uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 2) * C::kBRows * kAtomBytes + (k & 3) * 32, ptx::kLayoutSw128, 1024);
-                ptx::mma_dense<KIND, CTAS>(d_tmem, da, db, idesc, accumulate);
-              }
-            }
-          }
-          // the stage may be refilled once these MMAs have read it
-          if (CTAS == 1) ptx::tc_commit(&sh->empty[stage]);
-          else ptx::tc_commit_pair(&sh->empty[stage], 3);
-          if (++stage == p.stages) { stage = 0; phase ^= 1u; }
-        }
-        if (!ok) break;
-        if (CTAS == 1) ptx::tc_commit(&sh->tmem_full[acc]);
-        else ptx::tc_commit_pair(&sh->tmem_full[acc], 3);
-        if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
-      }
-    }
-  } else if (warp >= kFirstEpiWarp) {
-    // ------------------------------ epilogue ------------------------------
-    const int cs = elem_bytes((sp24_dtype)p.cd_type);
-    if (kTall || p.epi_lsu) {
-      // loads and stores by the epilogue warps themselves
-#define SP24_EPILOGUE(CS_, COLS_)                                                                                    \
-  epilogue_direct<KIND, CS_, COLS_, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id, \
-                                                                        num_clusters, num_tiles, warp, lane)
-      if (p.cd_col_major) {
-        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, true);
-        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, true);
-        else SP24_EPILOGUE(4, true);
-      } else {
-        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, false);
-        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, false);
-        else SP24_EPILOGUE(4, false);
-      }
-#undef SP24_EPILOGUE
-    } else {
-    // 4-byte row-major outputs when every epilogue warp can have a box buffer of its own.  The two warps
-    // of a lane quarter own its 32 accumulator rows and take its 32 x 32 boxes in turn: TMA load of the C
-    // box (if beta != 0) into a staging buffer a few boxes ahead, tcgen05.ld of the accumulator columns,
-    // convert in place, TMA store of the D box.  Boxes outside the matrix are clipped by the TMA.
-    const int q = warp & 3;  // tensor-memory lane quarter this warp may read
-    const int ew = warp - kFirstEpiWarp;  // epilogue warp 0..7: warps ew and ew + 4 share a lane quarter
-    constexpr int buf_bytes = 4096, split = 2;
-    const int first_it = ew >> 2;
-    const int warp_bytes = p.epi_bytes / kEpiWarps;
-    const int nbuf = min(2, warp_bytes / buf_bytes);  // staging buffers of this warp: 1 or 2
-    const int ahead = nbuf > 1 ? nbuf - 1 : 1;      // boxes the C loads run ahead (their latency is what the epilogue waits on)
-    // stores that may still be reading their buffer when the next buffer is claimed: with C the
-    // buffer of box seq + ahead is claimed at the end of box seq, without C that of box seq + 1
-    const int pending_ok = p.has_c ? nbuf - ahead : nbuf - 1;
-    uint8_t* my_bufs = epi + ew * warp_bytes;
-    constexpr int kSub = BLOCK_N / 32;
-    constexpr int kIters = MBLK * kSub;
-
-    // box `it` of the tile (mt, nt): first row / column and whether any of it lies inside the matrix
-    auto box_of = [&](int mt, int nt, int it, int& row0, int& col0) -> bool {
-      const int j = it / kSub, sc = it - j * kSub;
-      row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M) + j * kBlockM + q * 32;
-      col0 = nt * BLOCK_N + sc * 32;
-      return j < live_blocks<CTAS, MBLK>(mt, (int)p.M) && row0 < p.M && col0 < p.N;
-    };
-    // cursor of the C loads over the same stream of boxes, `ahead` live boxes in front of the consumer
-    // (the tile coordinates cost two divisions: once per tile, not per box)
-    int pf_t = cluster_id, pf_it = first_it, pf_mt = 0, pf_nt = 0;
-    if (pf_t < num_tiles) tile_coords(pf_t, p.m_tiles, p.n_tiles, p.band, pf_mt, pf_nt);
-    uint32_t pf_seq = 0;
-    auto issue_c_load = [&]() {  // lane 0 only: load the next live box of the stream, if any
-      while (pf_t < num_tiles) {
-        int row0, col0;
-        const bool live_box = box_of(pf_mt, pf_nt, pf_it, row0, col0);
-        pf_it += split;
-        if (pf_it >= kIters) {
-          pf_it = first_it;
-          pf_t += num_clusters;
-          if (pf_t < num_tiles) tile_coords(pf_t, p.m_tiles, p.n_tiles, p.band, pf_mt, pf_nt);
-        }
-        if (live_box) {
-          const int b = pf_seq % nbuf;
-          ptx::mbar_expect_tx(&sh->c_full[ew][b], (uint32_t)buf_bytes);
-          ptx::tma_load_2d<1>(ptx::smem_u32(my_bufs + b * buf_bytes), &map_c, ptx::smem_u32(&sh->c_full[ew][b]), col0, row0);
-          ++pf_seq;
-          return;
-        }
-      }
-    };
-    if (p.has_c && lane == 0)
-      for (int i = 0; i < ahead; ++i) issue_c_load();
-
-    int acc = 0;
-    uint32_t acc_phase = 0, seq = 0;
-    for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
-      int mt, nt;
-      tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-      ptx::tc_fence_after();
-      uint32_t r_next[32];
-      const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-      ptx::tmem_ld_32x32b_x32(t_acc + first_it * 32, r_next);
-      bool ok = true;
-#pragma unroll 1
-      for (int it = first_it; it < kIters; it += split) {
-        uint32_t r[32];
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) r[e] = r_next[e];
-        if (it + split < kIters) {
-          const int jn = (it + split) / kSub, scn = (it + split) - jn * kSub;
-          ptx::tmem_ld_32x32b_x32(t_acc + jn * BLOCK_N + scn * 32, r_next);
-        }
-        int row0, col0;
-        if (!box_of(mt, nt, it, row0, col0)) continue;  // same answer for the whole warp
-        const int b = seq % nbuf;
-        uint8_t* buf = my_bufs + b * buf_bytes;
-        if (p.has_c && !bounded_wait(&sh->c_full[ew][b], (seq / nbuf) & 1u, sh, p.status, 5u, p.wait_limit)) { ok = false; break; }
-        if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
-        float scale = 1.f, bias = 0.f;
-        if (KIND == 1 && p.dequant) {
-          // this thread's output row: its scale and bias
-          const int row = min(row0 + lane, (int)p.M - 1);
-          scale = p.row_scale[row];
-          bias = p.bias ? p.bias[row] : 0.f;
-        }
-        convert_row_staged<KIND>(r, buf, lane, p, scale, bias);
-        ptx::fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          ptx::tma_store_2d(&map_d, buf, col0, row0);
-          ptx::bulk_commit_group();
-          // the buffer claimed next is free once the store that used it last has read it
-          if (pending_ok == 1) ptx::bulk_wait_group_read<1>();
-          else ptx::bulk_wait_group_read<0>();
-          if (p.has_c) issue_c_load();
-        }
-        __syncwarp();
-        ++seq;
-      }
-      if (!ok) break;
-      // accumulators drained: hand them back to the MMA issuer (CTA 0 of the pair)
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (CTAS == 1) ptx::mbar_arrive(&sh->tmem_empty[acc]);
-        else ptx::mbar_arrive_cluster(&sh->tmem_empty[acc], 0);
-      }
-      if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
-    }
-    if (lane == 0) ptx::bulk_wait_group_read<0>();  // staging buffers must outlive the stores that read them
-    }
-  }
-
-  // ------------------------------ teardown ------------------------------
-  ptx::tc_fence_before();
-  __syncthreads();
-  if (sh->abort) {
-    // copies issued before the abort may still be landing in this CTA's shared memory
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
-  }
-  if (CTAS == 2) ptx::cluster_sync();
-  if (warp == 1) {
-    __syncwarp();
-    ptx::tc_fence_after();
-    ptx::tmem_dealloc<CTAS>(tmem_base, kTmemCols);
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// host side
-// ---------------------------------------------------------------------------------------------
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1066,6 +44,8 @@ EncodeIm2colFn encode_im2col_fn() {
   return fn;
 }
 
+}  // namespace
+
 // im2col tensor map over an NHWC activation for a 3x3, stride-1, pad-1 convolution: the bounding box
 // of the filter's anchor starts one pixel before the image and ends one pixel before its far edge, so
 // that anchor + tap (0..2) covers rows/columns -1 .. H, W with zeros outside.
@@ -1084,20 +64,7 @@ sp24_status make_im2col_map(CUtensorMap* map, const void* x, int es, uint64_t nb
   return r == CUDA_SUCCESS ? SP24_OK : SP24_ERR_CUDA;
 }
 
-constexpr int kSwizzle128Atom32 = 1280;
-
-// Up to three dimensions, innermost first: sizes in elements, strides of the outer ones in bytes.
-struct MapShape {
-  const void* base;
-  uint64_t dims[3], strides[2];  // dims[2] == 0: two dimensions
-  uint32_t box[3];
-  int32_t es, swizzle;  // swizzle: 0, 64, 128, or kSwizzle128Atom32 = the 128-byte pattern in 32-byte units
-  bool operator==(const MapShape& o) const {
-    return base == o.base && dims[0] == o.dims[0] && dims[1] == o.dims[1] && dims[2] == o.dims[2] &&
-           strides[0] == o.strides[0] && strides[1] == o.strides[1] && box[0] == o.box[0] && box[1] == o.box[1] &&
-           box[2] == o.box[2] && es == o.es && swizzle == o.swizzle;
-  }
-};
+namespace {
 
 sp24_status encode_map(CUtensorMap* map, const MapShape& m) {
   EncodeTiledFn fn = encode_fn();
@@ -1126,6 +93,8 @@ struct MapCache {
   int used = 0, next = 0;
 };
 
+}  // namespace
+
 sp24_status make_map(CUtensorMap* map, const MapShape& key) {
   static thread_local MapCache cache;
   for (int i = 0; i < cache.used; ++i)
@@ -1140,12 +109,6 @@ sp24_status make_map(CUtensorMap* map, const MapShape& key) {
   cache.maps[slot] = *map;
   return SP24_OK;
 }
-// 2-D map over a row-major (rows x cols) array of `es`-byte elements with `ld_bytes` between rows; box = box_cols x
-// box_rows elements.
-sp24_status make_map(CUtensorMap* map, const void* base, int es, uint64_t rows, uint64_t cols, uint64_t ld_bytes,
-                     uint32_t box_cols, uint32_t box_rows, int swizzle) {
-  return make_map(map, MapShape{base, {cols, rows, 0}, {ld_bytes, 0}, {box_cols, box_rows, 1}, es, swizzle});
-}
 
 int sm_count() {
   static std::atomic<int> known[64];
@@ -1157,6 +120,8 @@ int sm_count() {
   if (cacheable) known[dev].store(n, std::memory_order_relaxed);
   return n;
 }
+
+namespace {
 
 // Process-wide settings: the benchmarking overrides (environment, read once, or sp24_set_tile_override)
 // and the fault-path test hooks (sp24_test_set_fault_hooks only; never read from the environment).
@@ -1177,113 +142,6 @@ Settings& settings() {
     if (const char* env = getenv("SP24_LOG")) st.log = atoi(env) != 0 || env[0] == '\0' ? 1 : 0;
   });
   return st;
-}
-
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
-sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* A, const void* meta, const void* B,
-                   cudaStream_t stream) {
-  using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
-  GemmParams p = base;
-  const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
-  int tile_m = kBlockM * CTAS * MBLK, ring_stages = C::kMinStagesFit, ring_bytes = C::kStageBytes, b_ring_bytes = 0;
-  uint32_t b_box_rows = C::kBRows;
-  if constexpr (is_tall<CTAS, MBLK>) {
-    p.b_rows = (int32_t)(d->N < BLOCK_N ? d->N : BLOCK_N);
-    tile_m = p.mblk * kBlockM;
-    b_box_rows = p.b_rows;
-    // slots of A (each k-block needs mblk) and of B: the split with the most of A in flight
-    const int b_slot = C::kBBoxes * p.b_rows * kAtomBytes, budget = C::kSmemLimit - 16384;
-    ring_bytes = C::kABlockBytes + C::kEBlockBytes;
-    ring_stages = 0;
-    for (int bs = 2; bs <= 8 && bs * b_slot < budget; ++bs) {
-      int slots = (budget - bs * b_slot) / ring_bytes;
-      if (slots > (bs - 1) * p.mblk + 1) slots = (bs - 1) * p.mblk + 1;
-      if (slots > C::kMaxStages) slots = C::kMaxStages;
-      if (slots > ring_stages) { ring_stages = slots; p.b_stages = bs; }
-    }
-    b_ring_bytes = p.b_stages * b_slot;
-  }
-  p.m_tiles = (int)((d->M + tile_m - 1) / tile_m);
-  p.n_tiles = (int)((d->N + BLOCK_N - 1) / BLOCK_N);
-  p.k_blocks = (int)((d->K + C::kKPerStage - 1) / C::kKPerStage);
-  // metadata blocks per 128-row block: 128 columns each (64 for the 1:2 pattern), an even number of them
-  p.meta_kb = KIND == 2 ? (int)(2 * ((d->K + 127) / 128)) : (int)(2 * ((d->K + 255) / 256));
-  CUtensorMap map_a, map_b, map_e;
-  const uint32_t atom_elems = kAtomBytes / es;
-  const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, (is_tall<CTAS, MBLK> ? 1 : MBLK) * kBlockM, 128);
-  if (st != SP24_OK) return st;
-  if (p.conv) {
-    // B = im2col view of the NHWC activation: boxes of kBRows output pixels x one 128-byte run of channels
-    if (B_MN) return SP24_ERR_UNSUPPORTED;
-    if (KIND == 2) return SP24_ERR_UNSUPPORTED;
-    const uint64_t nb = (uint64_t)d->N / ((uint64_t)p.conv_h * p.conv_w);
-    st = make_im2col_map(&map_b, B, es, nb, p.conv_h, p.conv_w, p.conv_c, atom_elems, C::kBRows);
-  } else if (B_MN) {
-    st = make_map(&map_b, B, es, d->K, d->N, d->ldb * es, C::kBChunkElems, C::kKPerStage,
-                  KIND == 2 ? kSwizzle128Atom32 : 128);
-  } else if (C::kBBoxes > 1 && d->K % atom_elems == 0) {
-    // K in whole 128-byte atoms: the atoms of a stage are a third dimension, one load brings them all (a K tail
-    // needs the zeros that only the two-dimensional map gives it)
-    p.b_3d = 1;
-    st = make_map(&map_b, MapShape{B, {atom_elems, (uint64_t)d->N, (uint64_t)d->K / atom_elems},
-                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, b_box_rows, (uint32_t)C::kBBoxes}, es, 128});
-  } else {
-    st = make_map(&map_b, B, es, d->N, d->K, d->ldb * es, atom_elems, b_box_rows, 128);
-  }
-  if (st != SP24_OK) return st;
-  if (SPARSE) {
-    // metadata as rows of 128 bytes: 16 * meta_kb of them per 128 rows of A
-    st = make_map(&map_e, MapShape{meta, {128, (uint64_t)p.meta_kb * 16, (uint64_t)((d->M + 127) / 128)},
-                                   {128, (uint64_t)p.meta_kb * 2048}, {128, 16 * C::kEBlocks, is_tall<CTAS, MBLK> ? 1 : MBLK}, 1, 0});
-    if (st != SP24_OK) return st;
-  } else {
-    map_e = map_a;
-  }
-  const int cs = elem_bytes(d->cd_type);
-  // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
-  // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
-  p.stages = ring_stages > C::kMaxStages ? C::kMaxStages : ring_stages;
-  const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
-  // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
-  // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
-  // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
-  // (against the TMA form: bf16 BERT FFN 26.6 against 28.7 us, fp8 16384 x 8192 x 8192 440 against 472 us,
-  // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
-  // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
-  // epilogue_direct).
-  p.epi_lsu = (is_tall<CTAS, MBLK> || p.cd_col_major || cs != 4 || room < kEpiWarps * 4096) ? 1 : 0;
-  p.epi_bytes = room >= kEpiWarps * 4096 ? kEpiWarps * 4096 : 16384;
-  CUtensorMap map_c, map_d;
-  if (p.epi_lsu) {
-    map_c = map_d = map_a;  // not used
-  } else {
-    while (p.epi_bytes < 16 * 4096 && 2 * p.epi_bytes <= room) p.epi_bytes *= 2;
-    // C and D move in 32 x 32 boxes whose rows are 128 bytes
-    st = make_map(&map_d, p.D, cs, d->M, d->N, d->ldd * cs, 32, 32, 128);
-    if (st != SP24_OK) return st;
-    map_c = map_d;
-    if (p.has_c) st = make_map(&map_c, p.C, cs, d->M, d->N, d->ldc * cs, 32, 32, 128);
-    if (st != SP24_OK) return st;
-  }
-  auto kernel = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
-  {
-    // the shared-memory opt-in is per kernel and device: once is enough
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    SP24_CUDA_CHECK(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !done[dev]) {
-      SP24_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-      if (dev >= 0 && dev < 64) done[dev] = true;
-    }
-  }
-  const int tiles = p.m_tiles * p.n_tiles;
-  int clusters = sm_count() / CTAS;
-  if (clusters > tiles) clusters = tiles;
-  return launch_overlapped(kernel, dim3((unsigned)(clusters * CTAS)), dim3(kNumThreads), C::kSmemBytes, stream, CTAS, map_a,
-                           map_b, map_e, map_c, map_d, p);
 }
 
 }  // namespace
@@ -1516,50 +374,11 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
             (long long)d->N, (long long)d->K, (int)d->ab_type, (int)d->cd_type, sparse ? "sparse" : "dense",
             b_mn ? " B:N-contiguous" : "", ctas, block_n, mblk, p.band, (double)fbeta, dq ? " dequant" : "",
             cv ? " conv3x3" : (acc_f16 ? " fp16-accumulate" : ""));
-#define SP24_LAUNCH(K_, BN, CT, MB, MN)                                                               \
-  (sparse ? launch<K_, true, BN, CT, MB, MN>(d, p, A, meta, B, s) : launch<K_, false, BN, CT, MB, MN>(d, p, A, meta, B, s))
-#define SP24_DISPATCH(CT, BN, MB)                                                                     \
-  if (ctas == CT && block_n == BN && mblk == MB && !b_mn && !tf32 && !f8) return i8 ? SP24_LAUNCH(1, BN, CT, MB, false) : SP24_LAUNCH(0, BN, CT, MB, false);
-#define SP24_DISPATCH_TF32(CT, BN, MB)                                                                \
-  if (ctas == CT && block_n == BN && mblk == MB && !b_mn && tf32) return SP24_LAUNCH(2, BN, CT, MB, false);
-#define SP24_DISPATCH_F8(CT, BN, MB)                                                                  \
-  if (ctas == CT && block_n == BN && mblk == MB && !b_mn && f8) return SP24_LAUNCH(3, BN, CT, MB, false);
-#define SP24_DISPATCH_MN(CT, BN, MB)                                                                  \
-  if (ctas == CT && block_n == BN && mblk == MB && b_mn)                                              \
-    return tf32 ? SP24_LAUNCH(2, BN, CT, MB, true)                                                    \
-                : (f8 ? SP24_LAUNCH(3, BN, CT, MB, true) : (i8 ? SP24_LAUNCH(1, BN, CT, MB, true) : SP24_LAUNCH(0, BN, CT, MB, true)));
-  SP24_DISPATCH(1, 128, 1)
-  SP24_DISPATCH(2, 224, 1)
-  SP24_DISPATCH(2, 224, 2)
-  SP24_DISPATCH(2, 192, 2)
-  SP24_DISPATCH(2, 256, 1)
-  if (ctas == 2 && block_n == 256 && mblk == 2 && !sparse && !b_mn && !tf32)  // dense variant only
-    return f8 ? launch<3, false, 256, 2, 2, false>(d, p, A, meta, B, s)
-              : (i8 ? launch<1, false, 256, 2, 2, false>(d, p, A, meta, B, s) : launch<0, false, 256, 2, 2, false>(d, p, A, meta, B, s));
-  if (ctas == 2 && block_n == 240 && mblk == 1 && !b_mn && !tf32 && !f8 && !i8 && elem_bytes(d->cd_type) == 2)
-    return SP24_LAUNCH(0, 240, 2, 1, false);
-  SP24_DISPATCH_TF32(1, 128, 1)
-  SP24_DISPATCH_TF32(2, 224, 1)
-  SP24_DISPATCH_TF32(2, 224, 2)
-  SP24_DISPATCH_TF32(2, 256, 1)
-  SP24_DISPATCH_F8(1, 128, 1)
-  SP24_DISPATCH_F8(2, 224, 1)
-  SP24_DISPATCH_F8(2, 224, 2)
-  SP24_DISPATCH_F8(2, 256, 1)
-  SP24_DISPATCH_MN(1, 128, 1)
-  SP24_DISPATCH_MN(2, 224, 1)
-  SP24_DISPATCH_MN(2, 224, 2)
-  if (ctas == 1 && block_n == 128 && (mblk == 2 || mblk == kTallBlocks) && sparse && !b_mn)
-    return tf32 ? launch<2, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
-                : (f8 ? launch<3, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
-                      : (i8 ? launch<1, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)
-                            : launch<0, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s)));
-#undef SP24_DISPATCH
-#undef SP24_DISPATCH_MN
-#undef SP24_DISPATCH_TF32
-#undef SP24_DISPATCH_F8
-#undef SP24_LAUNCH
-  return SP24_ERR_UNSUPPORTED;
+  const TileShape tile = {ctas, block_n, mblk};
+  if (i8) return launch_gemm<1>(tile, sparse, b_mn, d, p, A, meta, B, s);
+  if (tf32) return launch_gemm<2>(tile, sparse, b_mn, d, p, A, meta, B, s);
+  if (f8) return launch_gemm<3>(tile, sparse, b_mn, d, p, A, meta, B, s);
+  return launch_gemm<0>(tile, sparse, b_mn, d, p, A, meta, B, s);
 }
 
 extern "C" sp24_status sp24_gemm(const sp24_gemm_desc* d, const void* alpha, const void* A, const void* meta,

@@ -1,0 +1,7 @@
+// The GEMM kernels for INT8 operands.
+#include "sp24_gemm_kernel.cuh"
+
+namespace sp24 {
+template sp24_status launch_gemm<1>(TileShape, bool, bool, const sp24_gemm_desc*, const GemmParams&, const void*, const void*,
+                                    const void*, cudaStream_t);
+}  // namespace sp24

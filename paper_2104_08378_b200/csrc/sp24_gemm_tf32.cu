@@ -1,0 +1,7 @@
+// The GEMM kernels for FP32 operands in TF32 precision.
+#include "sp24_gemm_kernel.cuh"
+
+namespace sp24 {
+template sp24_status launch_gemm<2>(TileShape, bool, bool, const sp24_gemm_desc*, const GemmParams&, const void*, const void*,
+                                    const void*, cudaStream_t);
+}  // namespace sp24
