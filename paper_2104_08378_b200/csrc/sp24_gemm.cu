@@ -1,10 +1,10 @@
-// Host side of the GEMM (kernel: sp24_gemm_kernel.cuh): tensor maps, tile choice, argument checks, entry points.
+// Host side of the GEMM (kernels: sp24_gemm_kernel.cuh): tensor maps, tile choice, argument checks, entry points.
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
 
-#include "sp24_gemm_kernel.cuh"
+#include "sp24_gemm.cuh"
 
 namespace sp24 {
 namespace {
