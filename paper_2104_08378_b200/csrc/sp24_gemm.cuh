@@ -31,13 +31,12 @@ struct GemmParams {
   int32_t cd_type;    // sp24_dtype of C / D
   int32_t has_c;
   int32_t stages, epi_bytes;  // shared memory: ring stages and bytes of epilogue staging
-  int32_t epi_lsu;            // epilogue form: 1 = the warps' own loads and stores, 0 = TMA through staging boxes
   long long wait_limit;       // SM cycles after which a device-side wait gives up
   int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
   int32_t band;       // m-tiles per band of the tile sweep
   int32_t mblk, b_rows, b_stages;  // tall tiles only: m-blocks of a tile, rows of a B box, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
-  int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout)
+  int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout): selects the kernel
   // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
   int32_t conv, conv_h, conv_w, conv_c;
   // int8 dequantising epilogue (sp24_gemm_i8_dequant): out = act(row_scale[i] * acc + bias[i]),

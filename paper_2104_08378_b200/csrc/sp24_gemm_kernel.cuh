@@ -81,6 +81,17 @@ struct Cfg {
   static constexpr int kSmemLimit = 232448 - 1024 - 512;
   static constexpr int kMaxStages = is_tall<CTAS, MBLK> ? 12 : 8;
   static constexpr int kMinStagesFit = (kSmemLimit - 16384) / kStageBytes;  // with the smallest staging
+  static constexpr int kRingStages = kMinStagesFit > kMaxStages ? kMaxStages : kMinStagesFit;
+  // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
+  // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
+  // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
+  // (against the TMA form: bf16 BERT FFN 26.6 against 28.7 us, fp8 16384 x 8192 x 8192 440 against 472 us,
+  // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
+  // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
+  // epilogue_direct).
+  __host__ __device__ static constexpr bool staged_epilogue(int cs, bool cols) {
+    return !is_tall<CTAS, MBLK> && !cols && cs == 4 && kSmemLimit - kRingStages * kStageBytes >= kEpiWarps * 4096;
+  }
   static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
   static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
   static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block
@@ -534,7 +545,10 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   }
 }
 
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
+// CS, COLS: bytes of an output element, column-major output.  A kernel for each form of the output, so that it holds
+// one epilogue: with all of them behind branches of one kernel, a tile's epilogue took up to twice as long whatever
+// the form (us, branches -> own kernels: bf16 24576 x 224 x 4096 with 512 x 224 tiles 39.8 -> 34.3, with C 43.6 -> 37.8).
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS>
 __global__ void __launch_bounds__(kNumThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_c,
@@ -573,7 +587,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     ptx::prefetch_tensormap(&map_a);
     ptx::prefetch_tensormap(&map_b);
     if (SPARSE) ptx::prefetch_tensormap(&map_e);
-    if (!p.epi_lsu) {
+    if (C::staged_epilogue(CS, COLS)) {
       if (p.has_c) ptx::prefetch_tensormap(&map_c);
       ptx::prefetch_tensormap(&map_d);
     }
@@ -838,22 +852,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
   } else if (warp >= kFirstEpiWarp) {
     // ------------------------------ epilogue ------------------------------
-    const int cs = elem_bytes((sp24_dtype)p.cd_type);
-    if (kTall || p.epi_lsu) {
+    if constexpr (!C::staged_epilogue(CS, COLS)) {
       // loads and stores by the epilogue warps themselves
-#define SP24_EPILOGUE(CS_, COLS_)                                                                                    \
-  epilogue_direct<KIND, CS_, COLS_, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id, \
-                                                                        num_clusters, num_tiles, warp, lane)
-      if (p.cd_col_major) {
-        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, true);
-        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, true);
-        else SP24_EPILOGUE(4, true);
-      } else {
-        if (KIND == 1 && cs == 1) SP24_EPILOGUE(1, false);
-        else if (KIND != 2 && cs == 2) SP24_EPILOGUE(2, false);
-        else SP24_EPILOGUE(4, false);
-      }
-#undef SP24_EPILOGUE
+      epilogue_direct<KIND, CS, COLS, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
+                                                                          num_clusters, num_tiles, warp, lane);
     } else {
     // 4-byte row-major outputs when every epilogue warp can have a box buffer of its own.  The two warps
     // of a lane quarter own its 32 accumulator rows and take its 32 x 32 boxes in turn: TMA load of the C
@@ -990,7 +992,7 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   GemmParams p = base;
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
-  int tile_m = kBlockM * CTAS * MBLK, ring_stages = C::kMinStagesFit, ring_bytes = C::kStageBytes, b_ring_bytes = 0;
+  int tile_m = kBlockM * CTAS * MBLK, ring_stages = C::kRingStages, ring_bytes = C::kStageBytes, b_ring_bytes = 0;
   uint32_t b_box_rows = C::kBRows;
   if constexpr (is_tall<CTAS, MBLK>) {
     p.b_rows = (int32_t)(d->N < BLOCK_N ? d->N : BLOCK_N);
@@ -1048,19 +1050,11 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   const int cs = elem_bytes(d->cd_type);
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
-  p.stages = ring_stages > C::kMaxStages ? C::kMaxStages : ring_stages;
+  p.stages = ring_stages;
   const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
-  // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
-  // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
-  // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
-  // (against the TMA form: bf16 BERT FFN 26.6 against 28.7 us, fp8 16384 x 8192 x 8192 440 against 472 us,
-  // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
-  // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
-  // epilogue_direct).
-  p.epi_lsu = (is_tall<CTAS, MBLK> || p.cd_col_major || cs != 4 || room < kEpiWarps * 4096) ? 1 : 0;
   p.epi_bytes = room >= kEpiWarps * 4096 ? kEpiWarps * 4096 : 16384;
   CUtensorMap map_c, map_d;
-  if (p.epi_lsu) {
+  if (!C::staged_epilogue(cs, p.cd_col_major)) {
     map_c = map_d = map_a;  // not used
   } else {
     while (p.epi_bytes < 16 * 4096 && 2 * p.epi_bytes <= room) p.epi_bytes *= 2;
@@ -1071,17 +1065,26 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
     if (p.has_c) st = make_map(&map_c, p.C, cs, d->M, d->N, d->ldc * cs, 32, 32, 128);
     if (st != SP24_OK) return st;
   }
-  auto kernel = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
+  // the kernel of this output form
+  void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams) = nullptr;
+  const int form = 2 * (cs >> 1) + p.cd_col_major;
+#define SP24_FORM(CS_, COLS_) \
+  if (form == 2 * (CS_ >> 1) + COLS_) kernel = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;
+  if constexpr (KIND == 1) { SP24_FORM(1, false) SP24_FORM(1, true) }
+  if constexpr (KIND != 2) { SP24_FORM(2, false) SP24_FORM(2, true) }
+  if constexpr (BLOCK_N % 32 == 0) { SP24_FORM(4, false) SP24_FORM(4, true) }  // 240-column tiles: 2-byte outputs only
+#undef SP24_FORM
+  if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
     // the shared-memory opt-in is per kernel and device: once is enough
     static std::mutex mu;
-    static bool done[64] = {};
+    static bool done[64][6] = {};
     int dev = 0;
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !done[dev]) {
+    if (dev < 0 || dev >= 64 || !done[dev][form]) {
       SP24_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-      if (dev >= 0 && dev < 64) done[dev] = true;
+      if (dev >= 0 && dev < 64) done[dev][form] = true;
     }
   }
   const int tiles = p.m_tiles * p.n_tiles;
@@ -1111,8 +1114,8 @@ sp24_status launch_gemm(TileShape t, bool sparse, bool b_mn, const sp24_gemm_des
   if constexpr (KIND == 0 || KIND == 1) {
     SP24_SHAPE(2, 192, 2, false)
   }
-  if constexpr (KIND == 0) {  // 16-bit outputs only
-    if (elem_bytes(d->cd_type) == 2) SP24_SHAPE(2, 240, 1, false)
+  if constexpr (KIND == 0) {
+    SP24_SHAPE(2, 240, 1, false)  // 2-byte outputs only
   }
   if constexpr (!tf32)  // dense variant only
     if (is(2, 256, 2) && !sparse && !b_mn) return launch<KIND, false, 256, 2, 2, false>(d, p, A, meta, B, s);
