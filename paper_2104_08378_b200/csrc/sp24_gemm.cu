@@ -154,10 +154,28 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
   return 256;
 }
 
-// Tile choice.  At most 128 columns: see below.  Small problems: single CTAs, 128 x 128 tiles.  Otherwise a pair of CTAs, and among the
-// pair shapes the one with the smallest estimated time = rounds of tiles over the pairs x time of one
-// tile.  The tile times are measured ratios (unit: one 256 x 224 tile per unit of K; interleaved runs on
-// 2048..8192-row problems with K = 4096..16384):
+// Whether tall tiles beat pairs of CTAs on `blocks` 128-row blocks and at most 128 columns.  They stream A better but
+// nothing hides their epilogue, so they lose where the output is wide next to A.  `out`: bytes of an output row; with
+// C or column-major, where a byte of it costs more, the limits are lower.  In one round of tiles the limits hardly
+// depend on K (short: all of it is launch and epilogue either way; long: the stream decides); with more rounds each
+// round's epilogue counts, and on a long K a last round that leaves SMs idle does.
+// Measured over 19200..98304 rows x 16..128 columns x 512..12288, every kind, order and C (3960 calls, tall tiles and
+// pairs on each; us, pairs against tall): bf16 -> bf16 49152 x 32 x 12288 123.8 / 104.1, 37888 x 64 x 512 11.4 / 7.5;
+// bf16 -> f32 49152 x 128 x 512 row-major 13.7 / 14.2, with C 17.3 / 20.8; int8 -> int32 98304 x 128 x 1024 23.5 / 29.1;
+// bf16 -> bf16 60000 x 128 x 12288 154.3 / 174.4.  The rule is 0.7 % off the better of the two in the mean.
+static bool tall_tiles_pay(const sp24_gemm_desc* d, bool has_c, int64_t blocks, int64_t sms, int mblk, int64_t chain) {
+  const int64_t out = d->N * elem_bytes(d->cd_type), k_bytes = d->K * elem_bytes(d->ab_type);
+  const bool plain = d->order_d == SP24_ROW_MAJOR && !has_c, short_k = k_bytes <= 2048;
+  if (blocks <= sms * mblk) return out <= (k_bytes >= 24576 || (plain && short_k) ? 512 : (plain ? 384 : 256));
+  if (k_bytes >= 12288 && 5 * sms * chain > 6 * blocks) return false;  // the last round leaves SMs idle
+  if (plain && short_k && chain <= 4) return out <= 512;
+  return d->N <= 96 && out <= (has_c ? 170 : 256);
+}
+
+// Tile choice.  At most 128 columns: see below.  Small problems: single CTAs, 128 x 128 tiles.  Otherwise a
+// pair of CTAs, and among the pair shapes the one with the smallest estimated time = rounds of tiles over
+// the pairs x time of one tile.  The tile times are measured ratios (unit: one 256 x 224 tile per unit of K;
+// interleaved runs on 2048..8192-row problems with K = 4096..16384):
 //   256 x 224, two accumulator buffers (epilogue overlapped)      K                 the reference
 //   256 x 240, the same (16-bit kinds, 16-bit output)              1.04 K            operand bytes per k
 //   256 x 256, one accumulator buffer (epilogue exposed)           1.09 K + 450
@@ -167,24 +185,23 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
 // multiple of 32; 240 is the widest multiple of 16 that fits.)  The dense variant: two m-blocks from six
 // waves of tiles on, 512 x 256 there (no metadata columns needed); below that the one-m-block width with
 // the fewest rounds.
-static void choose_tile(const sp24_gemm_desc* d, int& ctas, int& block_n, int& mblk) {
+static void choose_tile(const sp24_gemm_desc* d, bool has_c, int& ctas, int& block_n, int& mblk) {
   const int64_t n224 = (d->N + 223) / 224;
   const bool k_major_b = d->order_b == SP24_COL_MAJOR;
   ctas = 1; block_n = 128; mblk = 1;
   if (!d->a_is_dense && k_major_b && d->N <= 128) {
     // One column of tiles: all of A is streamed once, and what counts is how evenly its 128-row blocks are spread
     // over the SMs.  Up to one block per SM: single blocks (us: 12288 x 32 x 4096 bf16 14.9 against 16.0 with
-    // pairs of CTAs, 12288 x 128 x 12288 40.6 against 43.1).  Beyond: tall tiles of the two or three blocks that
-    // give the fewest blocks in a row on one SM, three if equal (B is loaded once per tile): 49152 rows x 12288,
-    // bf16, 32 / 64 / 128 columns 103 / 107 / 118 us against 120 / 128 / 131 with single blocks or pairs; 24576
-    // rows 55 against 77; int8 30560 x 32 x 576 4.7 against 8.6, 24576 x 96 x 4096 18.2 against 19.1.  (The floor
-    // of the 49152-row weight is 104 us at the copy rate.)
+    // pairs of CTAs, 12288 x 128 x 12288 40.6 against 43.1).  Beyond, if they pay: tall tiles of the two or three
+    // blocks that give the fewest blocks in a row on one SM, three if equal (B is loaded once per tile).
     const int64_t sms = sm_count(), blocks = (d->M + kBlockM - 1) / kBlockM;
-    if (blocks > sms) {
-      const int64_t chain2 = 2 * ((blocks + 2 * sms - 1) / (2 * sms)), chain3 = 3 * ((blocks + 3 * sms - 1) / (3 * sms));
-      mblk = chain2 < chain3 ? 2 : 3;
+    if (blocks <= sms) return;
+    const int64_t chain2 = 2 * ((blocks + 2 * sms - 1) / (2 * sms)), chain3 = 3 * ((blocks + 3 * sms - 1) / (3 * sms));
+    const int tall = chain2 < chain3 ? 2 : 3;
+    if (tall_tiles_pay(d, has_c, blocks, sms, tall, chain2 < chain3 ? chain2 : chain3)) {
+      mblk = tall;
+      return;
     }
-    return;
   }
   if (d->M < 256 || (d->M / 256) * n224 < 32) return;
   ctas = 2; block_n = 224;
@@ -233,7 +250,7 @@ static void choose_tile(const sp24_gemm_desc* d, int& ctas, int& block_n, int& m
 extern "C" sp24_status sp24_gemm_plan(const sp24_gemm_desc* d, int* ctas, int* block_n, int* mblk) {
   SP24_RETURN_IF(d == nullptr || ctas == nullptr || block_n == nullptr || mblk == nullptr, SP24_ERR_NULL);
   SP24_RETURN_IF(d->M <= 0 || d->N <= 0 || d->K <= 0, SP24_ERR_SHAPE);
-  choose_tile(d, *ctas, *block_n, *mblk);
+  choose_tile(d, false, *ctas, *block_n, *mblk);
   Settings& cfg = settings();
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     *ctas = c;
@@ -358,7 +375,7 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   const bool sparse = !d->a_is_dense;
   const bool i8 = d->ab_type == SP24_I8, tf32 = d->ab_type == SP24_F32, f8 = is_fp8(d->ab_type);
   int ctas, block_n, mblk;
-  choose_tile(d, ctas, block_n, mblk);
+  choose_tile(d, has_c, ctas, block_n, mblk);
   p.band = 16 / mblk;
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     ctas = c;

@@ -89,3 +89,18 @@ def test_expired_wait_is_reported(sp, force_tile):
     again = sp.gemm(vals, meta, x, ws=ws)
     assert torch.equal(again, good)
     assert sp.gemm_status(ws) == 9 and sp.gemm_status(ws) == 0
+
+
+@pytest.mark.parametrize("kind,cd,order,M,N,K,plan", [
+    # wide outputs: pairs of CTAs, whose epilogue overlaps (on the 148 SMs of the device)
+    ("bf16", "f32", True, 49152, 128, 512, "2x224x1"), ("bf16", "f32", False, 98304, 128, 1024, "2x224x1"),
+    ("i8", "i32", False, 98304, 128, 1024, "2x224x1"), ("f32", "f32", True, 60000, 96, 512, "2x224x1"),
+    # a long K and a last round that leaves SMs idle
+    ("bf16", "bf16", False, 60000, 128, 12288, "2x224x2"), ("e4m3", "bf16", True, 60000, 96, 12288, "2x224x2"),
+    # narrow outputs: tall tiles
+    ("bf16", "bf16", True, 49152, 32, 12288, "1x128x3"), ("bf16", "bf16", True, 49152, 128, 12288, "1x128x3"),
+    ("e4m3", "bf16", True, 37888, 128, 4096, "1x128x2"), ("bf16", "f32", True, 49152, 64, 512, "1x128x3"),
+    ("i8", "i32", False, 37888, 96, 1024, "1x128x2"), ("bf16", "bf16", True, 98304, 96, 4096, "1x128x3")])
+def test_tall_tiles_only_where_the_output_is_narrow(sp, kind, cd, order, M, N, K, plan):
+    out = M if order else N
+    assert sp.gemm_plan(sp.make_desc(kind, cd, M, N, K, K // 2, K, out, out, False, False, order)) == plan
