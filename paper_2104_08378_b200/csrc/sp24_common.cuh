@@ -42,11 +42,16 @@ inline sp24_status cuda_status(cudaError_t e) {
 // A kernel launched through launch_overlapped() is set up (blocks scheduled as the ones of the kernel
 // ahead leave their SMs, barriers and tables initialised) while that kernel drains; stream order is kept
 // by wait_for_stream(), which every thread calls before its first access to global memory: it returns when
-// all the work ahead has completed and its writes are visible.  let_next_start() allows the same to the
-// kernel behind; it is a hint and orders nothing.  Such a kernel takes no read-only (non-coherent) loads: its
-// pointers carry no __restrict__ const, so that no load can be moved ahead of the wait.
-// Back-to-back calls (us a call, without and with it): BERT FFN 17.7, 15.9; ragged 1184 x 736 x 1008
-// 10.2, 8.3; int8 3072 x 4096 x 768 -> int8 19.9, 15.6; apply_mask + compress of 12288 x 3072 49.2, 45.6;
+// all the work ahead has completed and its writes are visible.  Such a kernel takes no read-only
+// (non-coherent) loads: its pointers carry no __restrict__ const, so that no load can be moved ahead of the wait.
+// Blocks of the kernel behind may come in once every block of this one has ended or has called
+// let_next_start(); it is a hint and orders nothing.  The GEMM calls it at its start, because its CTAs fill
+// their SMs: the next one can only come to an SM that is idle.  The streaming kernels do not: with a call at
+// the start, waiting blocks take the places of working ones (us a call in a CUDA graph, plain launches / called
+// at the start / not called: prune_compress bf16 1184 x 1008 2.5, 3.3, 2.1; apply_mask i8 4096 x 768 3.9, 4.7, 3.7;
+// apply_mask + compress bf16 1184 x 1008 4.4, 5.3, 4.0, of 12288 x 3072 44.8, 44.3, 44.1).
+// Back-to-back calls (us a call, without and with the overlap): BERT FFN 17.7, 15.9; ragged 1184 x 736 x 1008
+// 10.2, 8.3; int8 3072 x 4096 x 768 -> int8 19.9, 15.6; apply_mask + compress of 12288 x 3072 49.5, 44.7;
 // in a CUDA graph 256 x 256 x 512 5.5, 4.6.
 __device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

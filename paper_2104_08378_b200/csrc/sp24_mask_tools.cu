@@ -151,7 +151,6 @@ __global__ void __launch_bounds__(kThreads) apply_mask_vec_kernel(const uint8_t*
                                                                   const uint8_t* meta, int layout,
                                                                   uint8_t* y, int64_t row_bytes_y, int64_t M, int64_t K,
                                                                   int64_t KB) {
-  let_next_start();
   wait_for_stream();
   const int64_t chunk = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (chunk >= (K >> 4)) return;

@@ -223,7 +223,6 @@ __global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* x, i
     if (t < 64) table[t] = prune_selectors<ES>((uint32_t)t);
     __syncthreads();
   }
-  let_next_start();
   wait_for_stream();
   const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows;
@@ -281,7 +280,6 @@ __global__ void __launch_bounds__(kThreads, 4) compress16_kernel(const uint8_t* 
     if (t < 64) ptable[t] = prune_selectors<2>((uint32_t)t);
   }
   build_selection_table(table);
-  let_next_start();
   wait_for_stream();
   const uint32_t halves = (uint32_t)(K >> 3), halves_pad = (uint32_t)chunks_pad * 2, KB = (uint32_t)(chunks_pad >> 3);
   const uint32_t h0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
@@ -353,7 +351,6 @@ __global__ void __launch_bounds__(kThreads, 4) compress8_kernel(const uint8_t* x
     if (t < 64) ptable[t] = prune_selectors<1>((uint32_t)t);
   }
   build_selection_table(table);
-  let_next_start();
   wait_for_stream();
   const uint32_t chunks = (uint32_t)(K >> 4), cpad = (uint32_t)chunks_pad, KB = (uint32_t)(chunks_pad >> 3);
   const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
