@@ -168,7 +168,7 @@ static bool tall_tiles_pay(const sp24_gemm_desc* d, bool has_c, int64_t blocks, 
   const bool plain = d->order_d == SP24_ROW_MAJOR && !has_c, short_k = k_bytes <= 2048;
   if (blocks <= sms * mblk) return out <= (k_bytes >= 24576 || (plain && short_k) ? 512 : (plain ? 384 : 256));
   if (k_bytes >= 12288 && 5 * sms * chain > 6 * blocks) return false;  // the last round leaves SMs idle
-  if (plain && short_k && chain <= 4) return out <= 512;
+  if (plain && k_bytes <= 8192 && chain <= 4) return out <= (short_k ? 512 : 384);
   return d->N <= 96 && out <= (has_c ? 170 : 256);
 }
 
