@@ -186,7 +186,7 @@ static bool tall_tiles_pay(const sp24_gemm_desc* d, bool has_c, int64_t blocks, 
 // multiple of 32; 240 is the widest multiple of 16 that fits.)  The dense variant: two m-blocks from six
 // waves of tiles on, 512 x 256 there (no metadata columns needed); below that the one-m-block width with
 // the fewest rounds.
-static void choose_tile(const sp24_gemm_desc* d, bool has_c, int& ctas, int& block_n, int& mblk) {
+static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& ctas, int& block_n, int& mblk) {
   const int64_t n224 = (d->N + 223) / 224;
   const bool k_major_b = d->order_b == SP24_COL_MAJOR;
   ctas = 1; block_n = 128; mblk = 1;
@@ -196,7 +196,7 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, int& ctas, int& blo
     // pairs of CTAs, 12288 x 128 x 12288 40.6 against 43.1).  Beyond, if they pay: tall tiles of the two or three
     // blocks that give the fewest blocks in a row on one SM, three if equal (B is loaded once per tile).
     const int64_t sms = sm_count(), blocks = (d->M + kBlockM - 1) / kBlockM;
-    if (blocks <= sms) return;
+    if (blocks <= sms || conv) return;  // (tall tiles load no im2col view)
     const int64_t chain2 = 2 * ((blocks + 2 * sms - 1) / (2 * sms)), chain3 = 3 * ((blocks + 3 * sms - 1) / (3 * sms));
     const int tall = chain2 < chain3 ? 2 : 3;
     if (tall_tiles_pay(d, has_c, blocks, sms, tall, chain2 < chain3 ? chain2 : chain3)) {
@@ -251,7 +251,7 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, int& ctas, int& blo
 extern "C" sp24_status sp24_gemm_plan(const sp24_gemm_desc* d, int* ctas, int* block_n, int* mblk) {
   SP24_RETURN_IF(d == nullptr || ctas == nullptr || block_n == nullptr || mblk == nullptr, SP24_ERR_NULL);
   SP24_RETURN_IF(d->M <= 0 || d->N <= 0 || d->K <= 0, SP24_ERR_SHAPE);
-  choose_tile(d, false, *ctas, *block_n, *mblk);
+  choose_tile(d, false, false, *ctas, *block_n, *mblk);
   Settings& cfg = settings();
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     *ctas = c;
@@ -376,14 +376,14 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   const bool sparse = !d->a_is_dense;
   const bool i8 = d->ab_type == SP24_I8, tf32 = d->ab_type == SP24_F32, f8 = is_fp8(d->ab_type);
   int ctas, block_n, mblk;
-  choose_tile(d, has_c, ctas, block_n, mblk);
+  choose_tile(d, has_c, cv != nullptr, ctas, block_n, mblk);
   p.band = 16 / mblk;
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     ctas = c;
     block_n = cfg.block_n.load(std::memory_order_relaxed);
     mblk = cfg.mblk.load(std::memory_order_relaxed);
   }
-  if (cv && ctas == 1) mblk = 1;  // tall tiles load no im2col view
+  SP24_RETURN_IF(cv && ctas == 1 && mblk != 1, SP24_ERR_UNSUPPORTED);  // a forced tall tile
   p.mblk = mblk;
   if (const int b = cfg.band.load(std::memory_order_relaxed)) p.band = b;
   const bool b_mn = d->order_b == SP24_ROW_MAJOR;  // B stored N-contiguous

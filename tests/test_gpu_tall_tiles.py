@@ -104,3 +104,22 @@ def test_expired_wait_is_reported(sp, force_tile):
 def test_tall_tiles_only_where_the_output_is_narrow(sp, kind, cd, order, M, N, K, plan):
     out = M if order else N
     assert sp.gemm_plan(sp.make_desc(kind, cd, M, N, K, K // 2, K, out, out, False, False, order)) == plan
+
+
+def test_convolutions_take_no_tall_tiles(sp, force_tile):
+    """They have no im2col view of B: a forced one is refused, and the automatic choice, with more 128-row blocks than
+    SMs and 128 output pixels, is the product with the unfolded activation."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(8)
+    M, Cin = 19200, 512
+    vals, meta, _ = sp.compress(_matrix("f16", M, 9 * Cin, g))
+    x = _matrix("f16", 128, Cin, g).view(1, 8, 16, Cin)
+    for tile in ("1x128x2", "1x128x3"):
+        force_tile(tile)
+        with pytest.raises(sp.Sp24Error) as refused:
+            sp.conv3x3_nhwc(vals, meta, x)
+        assert refused.value.status == 6           # not built
+    force_tile(None)
+    got = sp.conv3x3_nhwc(vals, meta, x)
+    want = sp.gemm(vals, meta, sp.im2col_nhwc_3x3(x))
+    assert torch.equal(got, want) and sp.gemm_status(device=x.device) == 0
