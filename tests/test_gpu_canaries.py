@@ -94,11 +94,51 @@ def test_gemm_stays_inside_d(sp, force_tile, kind, tile):
         torch.cuda.synchronize()
         assert sp.gemm_status(ws) == 0
         D.check(f"gemm {kind} {tile}")
-    if kind in ("bf16", "i8") and tile != "2x240x1":   # (240 columns: row-major outputs only)
+    if kind in ("bf16", "i8"):
         Dt = Guarded(N, M, cdt, M + 32)              # column-major D (M contiguous)
         sp.gemm(vals, meta, Bt, out=Dt.t, cd=cd, cd_col_major=True, ws=ws)
         torch.cuda.synchronize()
         Dt.check(f"gemm {kind} {tile} column-major")
+
+
+# Row counts and columns that end half-way through a 32 x 32 box (16-bit and FP32 operands), tall tiles (at most 128
+# columns) among the shapes; the results are, bit for bit, those of 128 x 128 tiles.
+@pytest.mark.parametrize("kind,cd", [("bf16", "bf16"), ("f16", "f32"), ("tf32", "f32"), ("i8", "i32"), ("dq", "i8"),
+                                     ("dq", "bf16"), ("e5m2", "bf16")])
+@pytest.mark.parametrize("tile", ["1x128x1", "1x128x2", "1x128x3", "2x224x1", "2x224x2", "2x240x1", "2x256x1"])
+def test_half_boxes_stay_inside_d(sp, force_tile, kind, cd, tile):
+    if tile == "2x240x1" and (kind not in ("bf16", "f16") or cd == "f32"):
+        pytest.skip("240-column tiles are built for the 16-bit kinds with 16-bit results")
+    one_byte = kind in ("i8", "dq", "e5m2")
+    tall = tile in ("1x128x2", "1x128x3")
+    ab = {"dq": "i8", "tf32": "f32"}.get(kind, kind)
+    cdt = sp.TORCH_DTYPE[cd]
+    K = 288
+    for M, N in ((32, 32), (672, 96), (1184, 64)) if one_byte else ((16, 16), (656, 112), (1200, 48)):
+        if not tall:
+            N += 256
+        if ab == "i8":
+            A, Bt = (torch.randint(-127, 128, (r, K), dtype=torch.int8, device="cuda") for r in (M, N))
+        else:
+            A, Bt = (torch.randn(r, K, device="cuda").to(sp.TORCH_DTYPE[ab]) for r in (M, N))
+        vals, meta, _ = sp.compress(A)
+        scale = torch.rand(M, device="cuda") * 0.01
+        C = torch.randint(-100, 100, (M, N), device="cuda").to(cdt)
+        for cols in (False, True):
+            for beta in (0,) if kind == "dq" else (0, 1):
+                got = []
+                for shape in ("1x128x1", tile):
+                    force_tile(shape)
+                    D = Guarded(N, M, cdt, M + 32) if cols else Guarded(M, N, cdt, N + 32)
+                    if kind == "dq":
+                        sp.gemm_i8_dequant(vals, meta, Bt, scale, relu=True, out_scale=0.1, cd=cd, out=D.t, cd_col_major=cols)
+                    else:
+                        sp.gemm(vals, meta, Bt, beta=beta if ab == "i8" else float(beta), C=(C.t().contiguous() if cols else C)
+                                if beta else None, cd=cd, out=D.t, cd_col_major=cols)
+                    assert sp.gemm_status(device=Bt.device) == 0
+                    D.check(f"{kind} -> {cd} {shape} {M} x {N} beta={beta} column-major={cols}")
+                    got.append(D.t.clone())
+                assert torch.equal(got[0].view(torch.uint8), got[1].view(torch.uint8))
 
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.int8])

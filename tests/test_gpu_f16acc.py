@@ -59,6 +59,21 @@ def test_f16_accumulate_within_its_error_model(sp, force_tile, dense, tile, shap
         assert np.linalg.norm(err) / np.linalg.norm(ref) <= 2.0 ** -10 * np.sqrt(K / 16 + 2) * 2
 
 
+@pytest.mark.parametrize("tile", [None, "1x128x2", "2x224x2"])
+@pytest.mark.parametrize("shape", [(416, 96, 1024, "f16"), (528, 112, 512, "f32")])
+def test_f16_accumulate_few_columns_and_column_major(sp, force_tile, tile, shape):
+    M, N, K, cd = shape
+    cfg = inputs.scaled(inputs.CONFIGS["tiny_f16"], M=M, N=N, K=K)
+    A, Bt = inputs.gen_A(cfg), inputs.gen_Bt(cfg)
+    v_ref, m_ref, _ = oracle.compress(A, "f16")
+    vals, meta, _ = sp.compress(to_device(A, "f16"))
+    force_tile(tile)
+    row, col = (sp.gemm(vals, meta, to_device(Bt, "f16"), cd=cd, acc_f16=True, cd_col_major=cols) for cols in (False, True))
+    assert torch.equal(row.t(), col) and sp.gemm_status(device=row.device) == 0
+    err = np.abs(to_host_f64(row) - oracle.gemm_sparse(v_ref, m_ref, Bt, "f16"))
+    assert (err <= _bound(K, False, oracle.gemm_abs(v_ref, m_ref, Bt, "f16"))).all()
+
+
 def test_f16_accumulate_is_exact_on_small_integers_and_differs_from_fp32_accumulation(sp):
     rng = np.random.default_rng(9)
     M, N, K = 256, 256, 256

@@ -68,3 +68,65 @@ def test_chained_calls_keep_stream_order(sp, size, graph):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
     assert sp.gemm_status(device=w.device) == 0
 
+
+def _mixed(sp, w, x, side, steps, wait):
+    """Copies, fills and work of a second stream (joined by events) between calls that start early."""
+    meta = torch.empty(sp.meta_bytes("bf16", *w.shape), dtype=torch.uint8, device="cuda")
+    vals, masked = torch.empty_like(w[:, : w.shape[1] // 2]).contiguous(), torch.empty_like(w)
+    w, x, out = w.clone(), x.clone(), torch.empty((x.shape[0], w.shape[0]), dtype=x.dtype, device="cuda")
+    main = torch.cuda.current_stream()
+    sync = torch.cuda.synchronize if wait else (lambda: None)
+    for i in range(steps):
+        sp.compress_into(w, vals, meta)
+        sync()
+        sp.apply_mask(w, meta, out=masked)
+        sync()
+        w.copy_(masked)                            # device-to-device copy behind a call, and a call behind it
+        sync()
+        sp.gemm(vals, meta, x, out=out, cd_col_major=True)
+        sync()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):              # the other stream rewrites what the last call read
+            x.copy_(out)
+            x.mul_(0.5)
+            out.zero_()
+        main.wait_stream(side)
+        sync()
+        sp.gemm(vals, meta, x, beta=1.0, C=out, out=out, cd_col_major=True)
+        sync()
+        vals.zero_()                               # a fill of what it read
+        sync()
+        sp.prune(w, out=w)
+        sync()
+        x.copy_(out)
+        x.clamp_(-2, 2)
+        w.add_(w.roll(1, 1), alpha=0.25)
+        sync()
+    return [w, vals, meta, x, out, masked]
+
+
+@pytest.mark.parametrize("size", [256, 1024])
+@pytest.mark.parametrize("graph", [False, True])
+def test_copies_fills_and_other_streams_keep_order(sp, size, graph):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(size)
+    w = (torch.randn((size, size), device="cuda", generator=g) / (0.85 * size) ** 0.5).bfloat16()
+    x = torch.randn((size, size), device="cuda", generator=g).bfloat16()
+    s, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        want = _mixed(sp, w, x, side, 5, True)
+        if graph:
+            gr = torch.cuda.CUDAGraph()
+            torch.cuda.synchronize()
+            with torch.cuda.graph(gr, stream=s, capture_error_mode="thread_local"):
+                got = _mixed(sp, w, x, side, 5, False)
+            gr.replay()
+            gr.replay()
+        else:
+            for _ in range(3):
+                got = _mixed(sp, w, x, side, 5, False)
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+    assert sp.gemm_status(device=w.device) == 0

@@ -5,7 +5,7 @@ import torch
 
 pytestmark = pytest.mark.gpu
 
-OUT = {"bf16": "bf16", "f16": "f16", "i8": "i32", "tf32": "f32", "e4m3": "bf16"}
+OUT = {"bf16": "bf16", "f16": "f16", "i8": "i32", "tf32": "f32", "e4m3": "bf16", "e5m2": "f32"}
 TORCH = {"bf16": torch.bfloat16, "f16": torch.float16, "f32": torch.float32, "i32": torch.int32}
 
 
@@ -18,7 +18,8 @@ def sp():
 def _matrix(kind, rows, cols, g, pad=0):
     if kind == "i8":
         return torch.randint(-128, 128, (rows, cols + pad), dtype=torch.int8, device="cuda", generator=g)[:, :cols]
-    dt = {"bf16": torch.bfloat16, "f16": torch.float16, "tf32": torch.float32, "e4m3": torch.float8_e4m3fn}[kind]
+    dt = {"bf16": torch.bfloat16, "f16": torch.float16, "tf32": torch.float32, "f32": torch.float32,
+          "e4m3": torch.float8_e4m3fn, "e5m2": torch.float8_e5m2}[kind]
     return torch.randn((rows, cols + pad), device="cuda", generator=g).to(dt)[:, :cols]
 
 
@@ -104,6 +105,30 @@ def test_expired_wait_is_reported(sp, force_tile):
 def test_tall_tiles_only_where_the_output_is_narrow(sp, kind, cd, order, M, N, K, plan):
     out = M if order else N
     assert sp.gemm_plan(sp.make_desc(kind, cd, M, N, K, K // 2, K, out, out, False, False, order)) == plan
+
+
+@pytest.mark.parametrize("kind,cd,acc_f16", [("f16", "f16", True), ("f16", "f32", True), ("e5m2", "f32", False),
+                                             ("e5m2", "bf16", False), ("e4m3", "f16", False)])
+def test_other_kinds_and_paddings(sp, force_tile, kind, cd, acc_f16):
+    """FP16 accumulation and both 8-bit floats; the columns between the result and its leading dimension keep their fill."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7)
+    for M, N, K in ((32, 32, 288), (416, 96, 1088), (37920, 128, 320)):
+        vals, meta, _ = sp.compress(_matrix(kind, M, K, g))
+        x, C = _matrix(kind, N, K, g), _matrix(cd, M, N, g)
+        for order in (False, True):
+            for beta in (0.0, -1.5):
+                got = []
+                for tile in ("1x128x1", "1x128x2", "1x128x3"):
+                    force_tile(tile)
+                    out = torch.full((N, M + 32) if order else (M, N + 32), 7, device="cuda").to(TORCH[cd])
+                    width = M if order else N
+                    sp.gemm(vals, meta, x, beta=beta, C=(C.t().contiguous() if order else C) if beta else None, cd=cd,
+                            out=out[:, :width], cd_col_major=order, acc_f16=acc_f16)
+                    assert (out[:, width:] == 7).all() and (out[:, :width] != 7).any()
+                    got.append(out)
+                assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+    assert sp.gemm_status(device=x.device) == 0
 
 
 def test_convolutions_take_no_tall_tiles(sp, force_tile):
