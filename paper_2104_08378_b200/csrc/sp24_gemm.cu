@@ -75,8 +75,7 @@ sp24_status encode_map(CUtensorMap* map, const MapShape& m) {
                                      : (m.es == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8);
   CUtensorMapSwizzle sw = m.swizzle == kSwizzle128Atom32
                               ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B
-                              : (m.swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                                  : (m.swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE));
+                              : (m.swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
   CUresult r = fn(map, dt, m.dims[2] ? 3 : 2, const_cast<void*>(m.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? SP24_OK : SP24_ERR_CUDA;
@@ -84,7 +83,7 @@ sp24_status encode_map(CUtensorMap* map, const MapShape& m) {
 
 // Host-side cache of encoded tensor maps.  A map is a pure function of (address, shape, leading
 // dimension, element size, box, swizzle): a layer that is multiplied again with the same buffers
-// finds its five maps here instead of encoding them again.  One small table per host thread (no
+// finds its maps (three, five with a staged epilogue) here instead of encoding them again.  One small table per host thread (no
 // lock), replaced round-robin.
 struct MapCache {
   static constexpr int kEntries = 32;

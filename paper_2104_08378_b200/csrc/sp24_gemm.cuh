@@ -55,7 +55,7 @@ struct MapShape {
   const void* base;
   uint64_t dims[3], strides[2];  // dims[2] == 0: two dimensions
   uint32_t box[3];
-  int32_t es, swizzle;  // swizzle: 0, 64, 128, or kSwizzle128Atom32 = the 128-byte pattern in 32-byte units
+  int32_t es, swizzle;  // swizzle: 0, 128, or kSwizzle128Atom32 = the 128-byte pattern in 32-byte units
   bool operator==(const MapShape& o) const {
     return base == o.base && dims[0] == o.dims[0] && dims[1] == o.dims[1] && dims[2] == o.dims[2] &&
            strides[0] == o.strides[0] && strides[1] == o.strides[1] && box[0] == o.box[0] && box[1] == o.box[1] &&

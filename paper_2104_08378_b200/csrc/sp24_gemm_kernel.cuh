@@ -12,7 +12,7 @@
 //   warps 2-9 epilogue, two per tensor-memory lane quarter taking alternate 32-column boxes:
 //            tcgen05.ld accumulator -> registers (the next box's load already under way), alpha /
 //            beta / conversion in registers, then one of two forms.  4-byte row-major outputs: a
-//            staging box per warp, C boxes TMA-loaded a few boxes ahead, TMA store of the D box, if
+//            staging box per warp, C boxes TMA-loaded one box ahead, TMA store of the D box, if
 //            shared memory has room for the boxes.  All others: the warps load C and store D
 //            themselves, through small per-warp transposing buffers, and hand the accumulators back
 //            as soon as their last box is in registers.
@@ -286,9 +286,9 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 
 // ---- epilogue in which the warps move C and D themselves -----------------------------------------
 // C is loaded straight from global memory into registers, the first boxes of a tile before the
-// tile's accumulators are even complete, the later ones a few boxes ahead, so that no load latency
-// is left on the path that holds the accumulators (tensor memory cannot be handed back to the MMA
-// issuer before it is drained).
+// tile's accumulators are even complete, the later ones four boxes ahead (2-byte types) or one (4-byte
+// types and tall tiles), so that little load latency is left on the path that holds the accumulators
+// (tensor memory cannot be handed back to the MMA issuer before it is drained).
 // Row-major outputs: each thread loads the C values of ITS accumulator row; D: the row is converted
 // in registers, written to a small per-warp buffer in shared memory and read back transposed, so
 // that the global stores of a warp cover whole 64-byte row segments.  A "pass" is 32 rows x 64 bytes
@@ -299,11 +299,13 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // The eight rows of ldmatrix matrix i are m = 8 j + 2 i + b (j = 0..3, b = 0, 1), which leaves each
 // thread with eight consecutive m of one column (2-byte) or of two columns (1-byte): 16- and 8-byte
 // stores.  16-byte unit u of buffer row m sits at u ^ (((m >> 1) ^ (m >> 3)) & 3): no bank conflicts
-// in the row-wise writes, the row-wise reads or the ldmatrix reads.
+// in the row-wise writes, the ldmatrix reads and the row-wise reads of 64-byte rows (those of 1-byte boxes,
+// half as wide, meet in pairs).
 // Measured against TMA boxes with scalar shared-memory stores (one 1-2 KB box per warp in flight, each
-// store waited for): int8 3072 x 4096 x 768 -> int8 44.7 -> 17.3 us, fp8 16384 x 8192 x 8192 -> bf16
-// 600 -> 514 us, the 3x3 convolution 50176 pixels x 256 x 2304 46.7 -> 36 us (with 240-column tiles, which
-// this form can store), int8 4096 x 32 x 4096 -> bf16 10.7 -> 9.0 us.
+// store waited for), us back to back on the device, early starts and fewer loads per stage in the second
+// figures: int8 3072 x 4096 x 768 -> int8 44.5 -> 14.3, fp8 16384 x 8192 x 8192 -> bf16 692 -> 497, the 3x3
+// convolution 50176 pixels x 256 x 2304 45.2 -> 27.0 (with 240-column tiles, which this form can store), int8
+// 4096 x 32 x 4096 -> bf16 10.6 -> 7.0.
 template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
 __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
@@ -859,7 +861,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     } else {
     // 4-byte row-major outputs when every epilogue warp can have a box buffer of its own.  The two warps
     // of a lane quarter own its 32 accumulator rows and take its 32 x 32 boxes in turn: TMA load of the C
-    // box (if beta != 0) into a staging buffer a few boxes ahead, tcgen05.ld of the accumulator columns,
+    // box (if beta != 0) into a staging buffer one box ahead, tcgen05.ld of the accumulator columns,
     // convert in place, TMA store of the D box.  Boxes outside the matrix are clipped by the TMA.
     const int q = warp & 3;  // tensor-memory lane quarter this warp may read
     const int ew = warp - kFirstEpiWarp;  // epilogue warp 0..7: warps ew and ew + 4 share a lane quarter
@@ -867,10 +869,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int first_it = ew >> 2;
     const int warp_bytes = p.epi_bytes / kEpiWarps;
     const int nbuf = min(2, warp_bytes / buf_bytes);  // staging buffers of this warp: 1 or 2
-    const int ahead = nbuf > 1 ? nbuf - 1 : 1;      // boxes the C loads run ahead (their latency is what the epilogue waits on)
-    // stores that may still be reading their buffer when the next buffer is claimed: with C the
-    // buffer of box seq + ahead is claimed at the end of box seq, without C that of box seq + 1
-    const int pending_ok = p.has_c ? nbuf - ahead : nbuf - 1;
+    // (the buffer of box seq + 1 is claimed, for its C or its result, at the end of box seq: with two buffers one
+    // store may still be reading its own then)
     uint8_t* my_bufs = epi + ew * warp_bytes;
     constexpr int kSub = BLOCK_N / 32;
     constexpr int kIters = MBLK * kSub;
@@ -882,7 +882,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       col0 = nt * BLOCK_N + sc * 32;
       return j < live_blocks<CTAS, MBLK>(mt, (int)p.M) && row0 < p.M && col0 < p.N;
     };
-    // cursor of the C loads over the same stream of boxes, `ahead` live boxes in front of the consumer
+    // cursor of the C loads over the same stream of boxes, one live box in front of the consumer
     // (the tile coordinates cost two divisions: once per tile, not per box)
     int pf_t = cluster_id, pf_it = first_it, pf_mt = 0, pf_nt = 0;
     if (pf_t < num_tiles) tile_coords(pf_t, p.m_tiles, p.n_tiles, p.band, pf_mt, pf_nt);
@@ -906,8 +906,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
       }
     };
-    if (p.has_c && lane == 0)
-      for (int i = 0; i < ahead; ++i) issue_c_load();
+    if (p.has_c && lane == 0) issue_c_load();
 
     int acc = 0;
     uint32_t acc_phase = 0, seq = 0;
@@ -950,7 +949,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           ptx::tma_store_2d(&map_d, buf, col0, row0);
           ptx::bulk_commit_group();
           // the buffer claimed next is free once the store that used it last has read it
-          if (pending_ok == 1) ptx::bulk_wait_group_read<1>();
+          if (nbuf == 2) ptx::bulk_wait_group_read<1>();
           else ptx::bulk_wait_group_read<0>();
           if (p.has_c) issue_c_load();
         }
