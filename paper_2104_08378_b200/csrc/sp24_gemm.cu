@@ -157,18 +157,23 @@ extern "C" size_t sp24_gemm_workspace_bytes(const sp24_gemm_desc* d) {
 // nothing hides their epilogue, so they lose where the output is wide next to A.  `out`: bytes of an output row; with
 // C or column-major, where a byte of it costs more, the limits are lower.  In one round of tiles the limits hardly
 // depend on K (short: all of it is launch and epilogue either way; long: the stream decides); with more rounds each
-// round's epilogue counts, and on a long K a last round that leaves SMs idle does.
+// round's epilogue counts, least on a short K in two rounds of two blocks, and on a long K a last round that leaves
+// SMs idle does.
 // Measured over 19200..98304 rows x 16..128 columns x 512..12288, every kind, order and C (3960 calls, tall tiles and
 // pairs on each; us, pairs against tall): bf16 -> bf16 49152 x 32 x 12288 123.8 / 104.1, 37888 x 64 x 512 11.4 / 7.5;
 // bf16 -> f32 49152 x 128 x 512 row-major 13.7 / 14.2, with C 17.3 / 20.8; int8 -> int32 98304 x 128 x 1024 23.5 / 29.1;
-// bf16 -> bf16 60000 x 128 x 12288 154.3 / 174.4, TF32 60000 x 96 x 1024 38.5 / 38.3.  The
-// rule is 0.7 % off the better of the two in the mean.
+// bf16 -> bf16 60000 x 128 x 12288 154.3 / 174.4, TF32 60000 x 96 x 1024 38.5 / 38.3,
+// 49152 x 128 x 4096 94.3 / 86.9.  The rule is 0.5 % off the better of the two in the mean.
 static bool tall_tiles_pay(const sp24_gemm_desc* d, bool has_c, int64_t blocks, int64_t sms, int mblk, int64_t chain) {
   const int64_t out = d->N * elem_bytes(d->cd_type), k_bytes = d->K * elem_bytes(d->ab_type);
   const bool plain = d->order_d == SP24_ROW_MAJOR && !has_c, short_k = k_bytes <= 2048;
-  if (blocks <= sms * mblk) return out <= (k_bytes >= 24576 || (plain && short_k) ? 512 : (plain ? 384 : 256));
+  if (blocks <= sms * mblk) {  // one round
+    if (k_bytes >= (plain ? 12288 : 24576) || (plain && short_k)) return out <= 512;
+    return out <= (plain ? 384 : 256);
+  }
   if (k_bytes >= 12288 && 5 * sms * chain > 6 * blocks) return false;  // the last round leaves SMs idle
   if (plain && k_bytes <= 8192 && chain <= 4) return out <= (short_k ? 512 : 384);
+  if (elem_bytes(d->ab_type) == 1 && short_k && chain <= 4) return out <= 256;
   return d->N <= 96 && out <= (has_c ? 170 : 256);
 }
 
