@@ -1064,26 +1064,28 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
     if (p.has_c) st = make_map(&map_c, p.C, cs, d->M, d->N, d->ldc * cs, 32, 32, 128);
     if (st != SP24_OK) return st;
   }
-  // the kernel of this output form
-  void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams) = nullptr;
-  const int form = 2 * (cs >> 1) + p.cd_col_major;
-#define SP24_FORM(CS_, COLS_) \
-  if (form == 2 * (CS_ >> 1) + COLS_) kernel = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;
+  // the kernels of the output forms
+  using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams);
+  Kernel forms[6] = {};
+#define SP24_FORM(CS_, COLS_) forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;
   if constexpr (KIND == 1) { SP24_FORM(1, false) SP24_FORM(1, true) }
   if constexpr (KIND != 2) { SP24_FORM(2, false) SP24_FORM(2, true) }
   if constexpr (BLOCK_N % 32 == 0) { SP24_FORM(4, false) SP24_FORM(4, true) }  // 240-column tiles: 2-byte outputs only
 #undef SP24_FORM
+  const Kernel kernel = forms[2 * (cs >> 1) + p.cd_col_major];
   if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
-    // the shared-memory opt-in is per kernel and device: once is enough
+    // the shared-memory opt-in is per kernel and device: once is enough.  All forms at once, so that a call with one
+    // form also loads the others' code: none is loaded for the first time inside a stream capture after that.
     static std::mutex mu;
-    static bool done[64][6] = {};
+    static bool done[64] = {};
     int dev = 0;
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !done[dev][form]) {
-      SP24_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-      if (dev >= 0 && dev < 64) done[dev][form] = true;
+    if (dev < 0 || dev >= 64 || !done[dev]) {
+      for (const Kernel k : forms)
+        if (k != nullptr) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+      if (dev >= 0 && dev < 64) done[dev] = true;
     }
   }
   const int tiles = p.m_tiles * p.n_tiles;
