@@ -116,10 +116,13 @@ def _check(status: int, where: str):
         raise Sp24Error(status, where)
 
 
+# (None on a CPU-only build of torch; the call below then fails in current_device(), which says so)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
     """The current device's current stream as a handle (no Stream object is made for it)."""
-    device = torch.cuda.current_device()     # (first: it says what is missing on a CPU-only build of torch)
-    return torch._C._cuda_getCurrentRawStream(device)
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dtype_of(t: torch.Tensor, dtype: str | None) -> str:
