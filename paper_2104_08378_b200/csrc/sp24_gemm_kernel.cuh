@@ -10,11 +10,11 @@
 //            back to the producer and, after the last k-block, the accumulators to the epilogue;
 //            owns the tensor-memory allocation;
 //   warps 2-9 epilogue, two per tensor-memory lane quarter taking alternate 32-column boxes:
-//            tcgen05.ld accumulator -> registers (the next box's load already under way), alpha /
-//            beta / conversion in registers, then one of two forms.  4-byte row-major outputs: a
+//            tcgen05.ld accumulator -> registers, alpha / beta / conversion in registers, then one of two
+//            forms.  4-byte row-major outputs: a
 //            staging box per warp, C boxes TMA-loaded one box ahead, TMA store of the D box, if
 //            shared memory has room for the boxes.  All others: the warps load C and store D
-//            themselves, through small per-warp transposing buffers, and hand the accumulators back
+//            themselves, through a small transposing buffer per warp, and hand the accumulators back
 //            as soon as their last box is in registers.
 // CTAS == 2 runs a pair of CTAs (cluster of two): each CTA loads its 128 rows of A / metadata per
 // m-block and its half of B, CTA 0 issues cta_group::2 MMAs (M = 256) for both.
@@ -83,12 +83,8 @@ struct Cfg {
   static constexpr int kMinStagesFit = (kSmemLimit - 16384) / kStageBytes;  // with the smallest staging
   static constexpr int kRingStages = kMinStagesFit > kMaxStages ? kMaxStages : kMinStagesFit;
   // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
-  // 4 KB box of its own (int8 4096 x 8192 x 4096: 77 against 80 us).  Everything else takes the warps' own
-  // loads and stores through one or two 2 KB transposing buffers per warp: row-major 2-byte outputs
-  // (against the TMA form: bf16 BERT FFN 26.6 against 28.7 us, fp8 16384 x 8192 x 8192 440 against 472 us,
-  // the 256 x 256 x 512 problem 12 against 17 us, the large bf16 GEMM within 3 %), two-m-block int8 tiles
-  // with 16 KB of staging (465 against 504 us on 16384 x 8192 x 8192), column-major and 1-byte outputs (see
-  // epilogue_direct).
+  // 4 KB box of its own.  Everything else takes the warps' own loads and stores through a 2 KB transposing
+  // buffer per warp (see epilogue_direct).
   __host__ __device__ static constexpr bool staged_epilogue(int cs, bool cols) {
     return !is_tall<CTAS, MBLK> && !cols && cs == 4 && kSmemLimit - kRingStages * kStageBytes >= kEpiWarps * 4096;
   }
@@ -202,18 +198,16 @@ __device__ __forceinline__ float2 unpack_16bit(uint32_t w, bool bf) {
             : __half22float2(*reinterpret_cast<const __half2*>(&w));
 }
 
-// One thread's row of a 32-column box: out = alpha * acc + beta * c (or the dequantising form) as
-// the packed words of the output row: 8 words for 1-byte outputs (CS = 1: the dequantising form),
-// 16 for 2-byte outputs (CS = 2), 32 for 4-byte ones.
+// One thread's row of a box of `cols` columns: out = alpha * acc + beta * c (or the dequantising form) as
+// the packed words of the output row (CS bytes an element; CS = 1 is always the dequantising form).
 // `c` holds the row's C values in the same packing and is read only if has_c.  One multiply and
 // one fused multiply-add per element, whichever path stores the row.
-template <int KIND, int CS>
-__device__ __forceinline__ void compute_row(const uint32_t (&r)[32], const uint32_t (&c)[8 * CS], bool has_c,
-                                            const GemmParams& p, float scale, float bias, uint32_t (&o)[8 * CS]) {
-  const bool bf = p.cd_type == SP24_BF16;
+template <int KIND, int CS, int COLUMNS>
+__device__ __forceinline__ void compute_row(const uint32_t (&r)[COLUMNS], const uint32_t (&c)[COLUMNS * CS / 4], bool has_c,
+                                            const GemmParams& p, float scale, float bias, uint32_t (&o)[COLUMNS * CS / 4]) {
   if constexpr (CS == 1) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int e = 0; e < COLUMNS / 4; ++e) {
       uint32_t word = 0;
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
@@ -225,42 +219,43 @@ __device__ __forceinline__ void compute_row(const uint32_t (&r)[32], const uint3
   } else if constexpr (CS == 4) {
     if (KIND == 1 && p.dequant) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(dequant_value(r[e], scale, bias, p.relu));
+      for (int e = 0; e < COLUMNS; ++e) o[e] = __float_as_uint(dequant_value(r[e], scale, bias, p.relu));
     } else if (KIND == 1) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) o[e] = r[e] + (has_c ? c[e] : 0u);
+      for (int e = 0; e < COLUMNS; ++e) o[e] = r[e] + (has_c ? c[e] : 0u);
     } else {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        float f = __fmul_rn(p.alpha, __uint_as_float(r[e]));
-        if (has_c) f = __fmaf_rn(p.beta, __uint_as_float(c[e]), f);
-        o[e] = __float_as_uint(f);
+      for (int e = 0; e < COLUMNS; e += 2) {
+        float2 f = ptx::mul2(make_float2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), p.alpha);
+        if (has_c) f = ptx::fma2(make_float2(__uint_as_float(c[e]), __uint_as_float(c[e + 1])), p.beta, f);
+        o[e] = __float_as_uint(f.x);
+        o[e + 1] = __float_as_uint(f.y);
       }
     }
   } else {
-    if (KIND == 1) {  // dequantised to a 16-bit type (the plain int8 GEMM writes 4-byte results)
+    auto pack = [&](bool bf) {
 #pragma unroll
-      for (int e = 0; e < 16; ++e)
-        o[e] = pack_16bit(dequant_value(r[2 * e], scale, bias, p.relu), dequant_value(r[2 * e + 1], scale, bias, p.relu), bf);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        float f0 = __fmul_rn(p.alpha, __uint_as_float(r[2 * e])), f1 = __fmul_rn(p.alpha, __uint_as_float(r[2 * e + 1]));
-        if (has_c) {
-          const float2 g = unpack_16bit(c[e], bf);
-          f0 = __fmaf_rn(p.beta, g.x, f0);
-          f1 = __fmaf_rn(p.beta, g.y, f1);
+      for (int e = 0; e < COLUMNS / 2; ++e) {
+        float2 f;
+        if (KIND == 1) {  // dequantised to a 16-bit type (the plain int8 GEMM writes 4-byte results)
+          f = make_float2(dequant_value(r[2 * e], scale, bias, p.relu), dequant_value(r[2 * e + 1], scale, bias, p.relu));
+        } else {
+          f = ptx::mul2(make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), p.alpha);
+          if (has_c) f = ptx::fma2(unpack_16bit(c[e], bf), p.beta, f);
         }
-        o[e] = pack_16bit(f0, f1, bf);
+        o[e] = pack_16bit(f.x, f.y, bf);
       }
-    }
+    };
+    if (p.cd_type == SP24_BF16) pack(true);
+    else pack(false);
   }
 }
 
 // FP16 accumulation: every accumulator cell of tensor memory holds a binary16 value in its low half
-__device__ __forceinline__ void widen_f16_accumulators(uint32_t (&r)[32]) {
+template <int COLUMNS>
+__device__ __forceinline__ void widen_f16_accumulators(uint32_t (&r)[COLUMNS]) {
 #pragma unroll
-  for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__half2float(__ushort_as_half((unsigned short)(r[e] & 0xFFFFu))));
+  for (int e = 0; e < COLUMNS; ++e) r[e] = __float_as_uint(__half2float(__ushort_as_half((unsigned short)(r[e] & 0xFFFFu))));
 }
 
 // TMA-staged form of a 4-byte row-major box (rows of 128 bytes in the TMA's 128-byte swizzle: 16-byte
@@ -278,21 +273,26 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
       c[4 * v] = x.x; c[4 * v + 1] = x.y; c[4 * v + 2] = x.z; c[4 * v + 3] = x.w;
     }
   }
-  compute_row<KIND, 4>(r, c, p.has_c != 0, p, scale, bias, o);
+  compute_row<KIND, 4, 32>(r, c, p.has_c != 0, p, scale, bias, o);
 #pragma unroll
   for (int v = 0; v < 8; ++v)
     *reinterpret_cast<uint4*>(row + ((v ^ (lane & 7)) << 4)) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
 }
 
 // ---- epilogue in which the warps move C and D themselves -----------------------------------------
-// C is loaded straight from global memory into registers, the first boxes of a tile before the
-// tile's accumulators are even complete, the later ones four boxes ahead (2-byte types) or one (4-byte
-// types and tall tiles), so that little load latency is left on the path that holds the accumulators
-// (tensor memory cannot be handed back to the MMA issuer before it is drained).
-// Row-major outputs: each thread loads the C values of ITS accumulator row; D: the row is converted
-// in registers, written to a small per-warp buffer in shared memory and read back transposed, so
-// that the global stores of a warp cover whole 64-byte row segments.  A "pass" is 32 rows x 64 bytes
-// (2 KB): a whole box of a 1- or 2-byte type, half a box of a 4-byte type.
+// What bounds it is how fast eight warps get through their instructions, not the stores: with the boxes of a tile
+// unrolled into straight code a box took a warp 1700 cycles (one pair of CTAs alone on the chip or all of them, the
+// same), a third of them waiting for instructions that were fetched for this one box, and two warps on a scheduler
+// cannot hide that.  So: one short loop over the boxes that exist, with C a loop of four, shared-memory accesses in
+// groups so that they overlap, packed FP32 arithmetic.  Cycles from the accumulators of a 512 x 224 tile being complete
+// to their hand-back, unrolled and now (timestamps included): 16-bit results 12,700 and 5,800, with C 18,400 and 9,600,
+// column-major 14,800 and 6,300, with C 20,800 and 9,500.  More warps make it slower (12 or 16 instead of 8, BERT FFN
+// 12.9 -> 14.7, 17.7 us, 256 x 256 x 512 4.2 -> 4.7, 5.3): registers for fewer boxes of C, and set-up.
+// A box is 32 rows x 64 bytes of output (32 columns, 16 of a 4-byte type; 32 bytes of a 1-byte type).  Per box: the
+// accumulators of this thread's row come out of tensor memory (loaded while the box before is stored), are converted
+// in registers and stored by way of a 2 KB buffer of the warp.
+// Row-major outputs: the rows are written to the buffer and read back transposed, so that the global stores of a warp
+// cover whole 64-byte row segments.
 // Column-major outputs (D stored [N][M], M contiguous): the lanes of a warp hold 32 consecutive m of
 // each column, so a 4-byte box is stored straight from registers, one 128-byte line per column; the
 // 1- and 2-byte boxes are transposed on the way out of the same per-warp buffer by ldmatrix.trans.
@@ -301,102 +301,94 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // stores.  16-byte unit u of buffer row m sits at u ^ (((m >> 1) ^ (m >> 3)) & 3): no bank conflicts
 // in the row-wise writes, the ldmatrix reads and the row-wise reads of 64-byte rows (those of 1-byte boxes,
 // half as wide, meet in pairs).
-// Measured against TMA boxes with scalar shared-memory stores (one 1-2 KB box per warp in flight, each
-// store waited for), us back to back on the device, early starts and fewer loads per stage in the second
-// figures: int8 3072 x 4096 x 768 -> int8 44.5 -> 14.3, fp8 16384 x 8192 x 8192 -> bf16 692 -> 497, the 3x3
-// convolution 50176 pixels x 256 x 2304 45.2 -> 27.0 (with 240-column tiles, which this form can store), int8
-// 4096 x 32 x 4096 -> bf16 10.6 -> 7.0.
+// C is loaded in the order of the stores (whole 64-byte row segments as well) into registers, four boxes ahead, the
+// first four of a tile before its accumulators are complete, and goes to the rows' owners through the buffer.
 template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
 __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
                                               int lane) {
-  constexpr int kSub = (BLOCK_N + 31) / 32, kIters = MBLK * kSub;  // the last box of a 240-column tile is half a box
-  constexpr int kBoxes = (kIters + 1) / 2;  // boxes per warp and tile (the two warps of a lane quarter alternate)
-  constexpr int W = 8 * CS;                 // 32-bit words of one box row
-  constexpr int P = CS == 2 ? 4 : 1;        // boxes whose C values are held in registers (16 or 32 registers each)
-  constexpr int kPasses = CS == 4 ? 2 : 1;
-  constexpr int kUnits = CS == 1 ? 2 : 4;   // 16-byte units of a buffer row that hold data
+  constexpr int kCols = CS == 4 ? 16 : 32;  // columns of a box
+  constexpr int W = kCols * CS / 4;         // 32-bit words of one box row
+  constexpr int P = 4;                      // boxes whose C values are held in registers
+  constexpr int kUnits = W / 4;             // 16-byte units of a buffer row that hold data
   constexpr int kUnitElems = 16 / CS;       // elements per 16-byte unit
-  const int q = warp & 3, ew = warp - kFirstEpiWarp, half = ew >> 2;
-  const int nbuf = p.epi_bytes >= kEpiWarps * 4096 ? 2 : 1;
-  uint8_t* stage = epi + ew * (nbuf * 2048);
+  constexpr int kRowsPerStore = 32 / kUnits;
+  const int q = warp & 3, half = (warp - kFirstEpiWarp) >> 2;
+  uint8_t* stage = epi + (warp - kFirstEpiWarp) * 2048;
   const uint8_t* Cb = static_cast<const uint8_t*>(p.C);
   uint8_t* Db = static_cast<uint8_t*>(p.D);
   const size_t ldc_b = (size_t)p.ldc * CS, ldd_b = (size_t)p.ldd * CS;
   const int M = (int)p.M, N = (int)p.N;
   const bool has_c = CS != 1 && p.has_c != 0;
-  // ldmatrix / stmatrix: this lane's row m of the buffer (its unit 0 under the swizzle: xor the unit into bits 4..5)
+  // this lane's row of the buffer, its unit 0 under the swizzle (xor the unit into bits 4..5) ...
+  const uint32_t own_row = ptx::smem_u32(stage) + (uint32_t)(lane * 64 + ((((lane >> 1) ^ (lane >> 3)) & 3) << 4));
+  // ... for ldmatrix / stmatrix ...
   const int tm_i = lane >> 3, tm_j = (lane & 7) >> 1;
   const uint32_t tm_row = ptx::smem_u32(stage) + (uint32_t)((8 * tm_j + 2 * tm_i + (lane & 1)) * 64 + ((tm_i ^ tm_j) << 4));
-  const int sw = ((lane >> 1) ^ (lane >> 3)) & 3;  // swizzle of buffer row `lane`
-  uint32_t creg[P][W];
+  // ... and in the order of row-major stores: this lane's row and unit of the first store (of the next ones: kRowsPerStore
+  // rows on)
+  const int st_r = lane / kUnits, st_u = lane % kUnits;
+  const uint32_t st_row = ptx::smem_u32(stage) + (uint32_t)(st_r * 64 + ((st_u ^ (((st_r >> 1) ^ (st_r >> 3)) & 3)) << 4));
+  auto st_addr = [&](int k) { return (st_row ^ (uint32_t)(((k * kRowsPerStore) >> 3) << 4)) + k * kRowsPerStore * 64; };
   int acc = 0;
-  uint32_t acc_phase = 0, pass_no = 0;
+  uint32_t acc_phase = 0;
   for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
     int mt, nt;
     tile_coords(t, p.m_tiles, p.n_tiles, p.band, mt, nt);
-    const int col_end = min(N, (nt + 1) * BLOCK_N);  // columns of this tile stop here
-    // C values of the box at (row0, col0): row-major in the accumulators' order (this thread's row), column-major
-    // in the order of the stores
+    const int tile_col = nt * BLOCK_N, col_end = min(N, tile_col + BLOCK_N);  // columns of this tile stop here
+    // the boxes of this lane quarter: `nsub` in a row, `blocks` rows of them (m-blocks); this warp takes every other one
+    const int row_q = (is_tall<CTAS, MBLK> ? mt * p.mblk * kBlockM : first_row<CTAS, MBLK>(mt, cta_rank, M)) + q * 32;
+    const int nsub = (col_end - tile_col + kCols - 1) / kCols;
+    const int blocks = min(is_tall<CTAS, MBLK> ? p.mblk : live_blocks<CTAS, MBLK>(mt, M), (M - row_q + kBlockM - 1) / kBlockM);
+    auto step = [&](int& j, int& sc, int by) {
+      sc += by;
+      while (sc >= nsub) { sc -= nsub; ++j; }
+    };
+    int j = 0, sc = 0;  // the box at hand
+    step(j, sc, half);
+    // C values of a box, in the order of the stores
     auto load_c = [&](int row0, int col0, uint32_t (&c)[W]) {
-      if constexpr (COLS) {
-        if constexpr (CS == 2) {
-          const int m = row0 + 8 * (lane & 3);
-          if (m >= M) return;
+      if constexpr (CS == 1) {
+      } else if constexpr (!COLS) {
+        const int col = col0 + st_u * kUnitElems;
+        const uint8_t* src = Cb + (size_t)(row0 + st_r) * ldc_b + (size_t)col * CS;
 #pragma unroll
-          for (int nb = 0; nb < 4; ++nb) {
-            const int n1 = col0 + 8 * nb + (lane >> 2);
-            if (n1 < col_end) {
-              const uint4 x = *reinterpret_cast<const uint4*>(Cb + (size_t)n1 * ldc_b + (size_t)m * CS);
-              c[4 * nb] = x.x; c[4 * nb + 1] = x.y; c[4 * nb + 2] = x.z; c[4 * nb + 3] = x.w;
-            }
+        for (int k = 0; k < kUnits; ++k) {
+          if (col < col_end && row0 + st_r + k * kRowsPerStore < M) {
+            const uint4 x = *reinterpret_cast<const uint4*>(src + k * kRowsPerStore * ldc_b);
+            c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = x.z; c[4 * k + 3] = x.w;
           }
-        } else if constexpr (CS == 4) {
-          if (row0 + lane >= M) return;
-          const uint8_t* src = Cb + (size_t)col0 * ldc_b + (size_t)(row0 + lane) * CS;
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            if (col0 + e < col_end) c[e] = *reinterpret_cast<const uint32_t*>(src + (size_t)e * ldc_b);
         }
-        return;
-      }
-      const int row = row0 + lane;
-      if (row >= M) return;
-      const uint4* src = reinterpret_cast<const uint4*>(Cb + (size_t)row * ldc_b + (size_t)col0 * CS);
+      } else if constexpr (CS == 2) {
+        const int m = row0 + 8 * (lane & 3);
+        const uint8_t* src = Cb + (size_t)(col0 + (lane >> 2)) * ldc_b + (size_t)m * CS;
 #pragma unroll
-      for (int v = 0; v < W / 4; ++v) {
-        if (col0 + v * kUnitElems < col_end) {
-          const uint4 x = src[v];
-          c[4 * v] = x.x; c[4 * v + 1] = x.y; c[4 * v + 2] = x.z; c[4 * v + 3] = x.w;
+        for (int nb = 0; nb < 4; ++nb) {
+          if (m < M && col0 + 8 * nb + (lane >> 2) < col_end) {
+            const uint4 x = *reinterpret_cast<const uint4*>(src + 8 * nb * ldc_b);
+            c[4 * nb] = x.x; c[4 * nb + 1] = x.y; c[4 * nb + 2] = x.z; c[4 * nb + 3] = x.w;
+          }
         }
+      } else if (row0 + lane < M) {
+        const uint8_t* src = Cb + (size_t)col0 * ldc_b + (size_t)(row0 + lane) * CS;
+#pragma unroll
+        for (int e = 0; e < kCols; ++e)
+          if (col0 + e < col_end) c[e] = *reinterpret_cast<const uint32_t*>(src + e * ldc_b);
       }
     };
-    // accumulators (and C) of a box -> packed output rows
-    auto convert = [&](uint32_t (&r)[32], uint32_t (&c)[W], int row0, uint32_t (&o)[W]) {
-      const uint32_t buf_off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
-      if constexpr (CS == 2 && COLS) {
-        if (has_c) {
-          // C arrived in the order of the column stores: through the buffer to the rows' owners
-          if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
+    // C from the order of the stores to the rows' owners (4-byte column-major boxes are with them already)
+    auto share_c = [&](uint32_t (&c)[W]) {
+      if constexpr (CS == 1 || (CS == 4 && COLS)) return;
+      __syncwarp();  // the reads of the box before are done
 #pragma unroll
-          for (int nb = 0; nb < 4; ++nb)
-            ptx::stmatrix_x4_trans((tm_row + buf_off) ^ (uint32_t)(nb << 4), c[4 * nb], c[4 * nb + 1], c[4 * nb + 2], c[4 * nb + 3]);
-          __syncwarp();
+      for (int k = 0; k < kUnits; ++k) {
+        if constexpr (COLS) ptx::stmatrix_x4_trans(tm_row ^ (uint32_t)(k << 4), c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3]);
+        else ptx::st_shared_v4(st_addr(k), c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3]);
+      }
+      __syncwarp();
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint4 x = *reinterpret_cast<const uint4*>(stage + buf_off + lane * 64 + ((u ^ sw) << 4));
-            c[4 * u] = x.x; c[4 * u + 1] = x.y; c[4 * u + 2] = x.z; c[4 * u + 3] = x.w;
-          }
-        }
-      }
-      if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
-      float scale = 1.f, bias = 0.f;
-      if (KIND == 1 && p.dequant) {
-        const int row = min(row0 + lane, M - 1);
-        scale = p.row_scale[row];
-        bias = p.bias ? p.bias[row] : 0.f;
-      }
-      compute_row<KIND, CS>(r, c, has_c, p, scale, bias, o);
+      for (int u = 0; u < kUnits; ++u)
+        ptx::ld_shared_v4(own_row ^ (uint32_t)(u << 4), c[4 * u], c[4 * u + 1], c[4 * u + 2], c[4 * u + 3]);
     };
     // packed output rows -> D
     auto store = [&](const uint32_t (&o)[W], int row0, int col0) {
@@ -404,53 +396,47 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
         if (row0 + lane < M) {
           uint8_t* dst = Db + (size_t)col0 * ldd_b + (size_t)(row0 + lane) * CS;
 #pragma unroll
-          for (int e = 0; e < 4 * W / CS; ++e)
-            if (col0 + e < col_end) *reinterpret_cast<uint32_t*>(dst + (size_t)e * ldd_b) = o[e];
+          for (int e = 0; e < kCols; ++e)
+            if (col0 + e < col_end) *reinterpret_cast<uint32_t*>(dst + e * ldd_b) = o[e];
         }
       } else {
+        if (!has_c) __syncwarp();  // the reads of the box before are done (with C each lane writes what it alone has read)
 #pragma unroll
-        for (int ps = 0; ps < kPasses; ++ps) {
-          const uint32_t off = nbuf == 2 ? (pass_no & 1u) * 2048u : 0u;
-          uint8_t* buf = stage + off;
-          if (nbuf == 1) __syncwarp();  // the reads of the previous pass are done
+        for (int u = 0; u < kUnits; ++u)
+          ptx::st_shared_v4(own_row ^ (uint32_t)(u << 4), o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
+        __syncwarp();
+        if constexpr (COLS) {
+          const int m = row0 + 8 * (lane & 3);
+          const int n1 = col0 + (CS == 2 ? 1 : 2) * (lane >> 2);
+          uint8_t* dst = Db + (size_t)n1 * ldd_b + (size_t)m * CS;
+          uint32_t x[kUnits][4];
 #pragma unroll
-          for (int u = 0; u < kUnits; ++u)
-            *reinterpret_cast<uint4*>(buf + lane * 64 + ((u ^ sw) << 4)) =
-                make_uint4(o[16 * ps + 4 * u], o[16 * ps + 4 * u + 1], o[16 * ps + 4 * u + 2], o[16 * ps + 4 * u + 3]);
-          __syncwarp();
-          if constexpr (COLS) {
-            const int m = row0 + 8 * (lane & 3);
+          for (int nb = 0; nb < kUnits; ++nb) ptx::ldmatrix_x4_trans(tm_row ^ (uint32_t)(nb << 4), x[nb][0], x[nb][1], x[nb][2], x[nb][3]);
 #pragma unroll
-            for (int nb = 0; nb < kUnits; ++nb) {
-              uint32_t w[4];
-              ptx::ldmatrix_x4_trans((tm_row + off) ^ (uint32_t)(nb << 4), w[0], w[1], w[2], w[3]);
-              if (m < M) {
-                if constexpr (CS == 2) {
-                  const int n1 = col0 + 8 * nb + (lane >> 2);
-                  if (n1 < col_end)
-                    *reinterpret_cast<uint4*>(Db + (size_t)n1 * ldd_b + (size_t)m * CS) = make_uint4(w[0], w[1], w[2], w[3]);
-                } else {
-                  // 16-bit units hold two neighbouring columns: split them
-                  const int n1 = col0 + 16 * nb + 2 * (lane >> 2);
-                  if (n1 < col_end) {
-                    uint8_t* dst = Db + (size_t)n1 * ldd_b + m;
-                    *reinterpret_cast<uint2*>(dst) = make_uint2(__byte_perm(w[0], w[1], 0x6420), __byte_perm(w[2], w[3], 0x6420));
-                    *reinterpret_cast<uint2*>(dst + ldd_b) =
-                        make_uint2(__byte_perm(w[0], w[1], 0x7531), __byte_perm(w[2], w[3], 0x7531));
-                  }
-                }
+          for (int nb = 0; nb < kUnits; ++nb) {
+            const uint32_t(&w)[4] = x[nb];
+            if (m < M && n1 + nb * (16 / CS) < col_end) {
+              uint8_t* at = dst + nb * (16 / CS) * ldd_b;
+              if constexpr (CS == 2) {
+                *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
+              } else {
+                // 16-bit units hold two neighbouring columns: split them
+                *reinterpret_cast<uint2*>(at) = make_uint2(__byte_perm(w[0], w[1], 0x6420), __byte_perm(w[2], w[3], 0x6420));
+                *reinterpret_cast<uint2*>(at + ldd_b) =
+                    make_uint2(__byte_perm(w[0], w[1], 0x7531), __byte_perm(w[2], w[3], 0x7531));
               }
             }
-          } else {
-#pragma unroll
-            for (int k = 0; k < kUnits; ++k) {
-              const int i = lane + 32 * k, rr = i / kUnits, u = i % kUnits;
-              const uint4 x = *reinterpret_cast<const uint4*>(buf + rr * 64 + ((u ^ (((rr >> 1) ^ (rr >> 3)) & 3)) << 4));
-              const int grow = row0 + rr, gcol = col0 + ps * (64 / CS) + u * kUnitElems;
-              if (grow < M && gcol < col_end) *reinterpret_cast<uint4*>(Db + (size_t)grow * ldd_b + (size_t)gcol * CS) = x;
-            }
           }
-          ++pass_no;
+        } else {
+          const int col = col0 + st_u * kUnitElems;
+          uint8_t* dst = Db + (size_t)(row0 + st_r) * ldd_b + (size_t)col * CS;
+          uint4 x[kUnits];
+#pragma unroll
+          for (int k = 0; k < kUnits; ++k) ptx::ld_shared_v4(st_addr(k), x[k].x, x[k].y, x[k].z, x[k].w);
+#pragma unroll
+          for (int k = 0; k < kUnits; ++k)
+            if (col < col_end && row0 + st_r + k * kRowsPerStore < M)
+              *reinterpret_cast<uint4*>(dst + k * kRowsPerStore * ldd_b) = x[k];
         }
       }
     };
@@ -463,84 +449,63 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
       }
     };
     const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-    if constexpr (is_tall<CTAS, MBLK>) {
-      // few boxes: a short loop over the ones that exist (unrolled code would be fetched for boxes that do not)
-      const int nsub = (col_end - nt * BLOCK_N + 31) / 32, row_q = mt * p.mblk * kBlockM + q * 32;
-      const int boxes = nsub * max(0, min(p.mblk, (M - row_q + kBlockM - 1) / kBlockM));  // of this lane quarter
-      auto place = [&](int b, int& row0, int& col0, int& tcol) {
-        const int j = b / nsub, sc = b - j * nsub;
-        row0 = row_q + j * kBlockM;
-        col0 = nt * BLOCK_N + sc * 32;
-        tcol = j * BLOCK_N + sc * 32;
-      };
-      int row0 = 0, col0 = 0, tcol = 0;
-      if (half < boxes) {
-        place(half, row0, col0, tcol);
-        if (has_c) load_c(row0, col0, creg[0]);
+    uint32_t r[kCols], creg[P][W];
+    float scale = 1.f, bias = 0.f;
+    auto load_scale = [&](int row0) {
+      if (KIND == 1 && p.dequant) {
+        const int row = min(row0 + lane, M - 1);
+        scale = p.row_scale[row];
+        bias = p.bias ? p.bias[row] : 0.f;
       }
-      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-      ptx::tc_fence_after();
-      if (half >= boxes) hand_back();
-#pragma unroll 1
-      for (int b = half; b < boxes; b += 2) {
-        uint32_t r[32], o[W];
-        ptx::tmem_ld_32x32b_x32(t_acc + tcol, r);
-        ptx::tmem_ld_wait();
-        if (b + 2 >= boxes) hand_back();
-        convert(r, creg[0], row0, o);
-        const int row1 = row0, col1 = col0;
-        if (b + 2 < boxes) {
-          place(b + 2, row0, col0, tcol);
-          if (has_c) load_c(row0, col0, creg[0]);
-        }
-        store(o, row1, col1);
+    };
+    // One box, with the C values in c; true if there is another one.
+    int cj = j, csc = sc;  // has_c: the next box whose C values are fetched
+    auto fetch_c = [&](uint32_t (&c)[W]) {
+      if (cj < blocks) load_c(row_q + cj * kBlockM, tile_col + csc * kCols, c);
+      step(cj, csc, kEpiWarps / 4);
+    };
+    auto box = [&](uint32_t (&c)[W]) -> bool {
+      const int row0 = row_q + j * kBlockM, col0 = tile_col + sc * kCols, j0 = j;
+      step(j, sc, kEpiWarps / 4);
+      const bool more = j < blocks;
+      uint32_t o[W];
+      if (has_c) share_c(c);
+      ptx::tmem_ld_wait(r);
+      if (!more) hand_back();
+      if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
+      compute_row<KIND, CS, kCols>(r, c, has_c, p, scale, bias, o);
+      if (more) {
+        ptx::tmem_ld_32x32b(t_acc + j * BLOCK_N + sc * kCols, r);
+        if (j != j0) load_scale(row_q + j * kBlockM);
       }
+      if (has_c) fetch_c(c);
+      store(o, row0, col0);
+      return more;
+    };
+    const bool any = j < blocks;
+    if (any) load_scale(row_q + j * kBlockM);
+    if (has_c) {
+#pragma unroll
+      for (int n = 0; n < P; ++n) fetch_c(creg[n]);
+    }
+    if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
+    ptx::tc_fence_after();
+    if (!any) {
+      hand_back();
     } else {
-      const int tile_row = first_row<CTAS, MBLK>(mt, cta_rank, M), live_j = live_blocks<CTAS, MBLK>(mt, M);
-      // box n of this warp in this tile: first row / column, accumulator column, inside the matrix?
-      auto geom = [&](int n, int& row0, int& col0, int& tcol) -> bool {
-        const int it = half + 2 * n;
-        const int j = it / kSub, sc = it - j * kSub;
-        row0 = tile_row + j * kBlockM + q * 32;
-        col0 = nt * BLOCK_N + sc * 32;
-        tcol = j * BLOCK_N + sc * 32;
-        return it < kIters && j < live_j && row0 < M && col0 < col_end;
-      };
-      auto load_c_of = [&](int n, uint32_t (&c)[W]) {
-        int row0, col0, tcol;
-        if (geom(n, row0, col0, tcol)) load_c(row0, col0, c);
-      };
-      if (has_c) {
-#pragma unroll
-        for (int n = 0; n < P; ++n)
-          if (n < kBoxes) load_c_of(n, creg[n]);
-      }
-      if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
-      ptx::tc_fence_after();
-      uint32_t racc[2][32];
-      {
-        int row0, col0, tcol;
-        geom(0, row0, col0, tcol);
-        ptx::tmem_ld_32x32b_x32(t_acc + tcol, racc[0]);
-      }
-#pragma unroll
-      for (int n = 0; n < kBoxes; ++n) {
-        if (half + 2 * n >= kIters) break;  // same answer for the whole warp
-        ptx::tmem_ld_wait();
-        if (half + 2 * (n + 1) < kIters) {
-          int row1, col1, tcol1;
-          geom(n + 1, row1, col1, tcol1);
-          ptx::tmem_ld_32x32b_x32(t_acc + tcol1, racc[(n + 1) & 1]);
-        } else {
-          hand_back();
+      ptx::tmem_ld_32x32b(t_acc + j * BLOCK_N + sc * kCols, r);
+      if (!has_c) {
+#pragma unroll 1
+        while (box(creg[0])) {
         }
-        int row0, col0, tcol;
-        const bool live = geom(n, row0, col0, tcol);  // same answer for the whole warp
-        uint32_t o[W];
-        if (live) convert(racc[n & 1], creg[n % P], row0, o);
-        // the C registers of box n are free: fetch box n + P into them (also when box n lies outside the matrix)
-        if (has_c && n + P < kBoxes) load_c_of(n + P, creg[n % P]);
-        if (live) store(o, row0, col0);
+      } else {
+        bool more = true;
+#pragma unroll 1
+        while (more) {
+#pragma unroll
+          for (int n = 0; n < P; ++n)
+            if (more) more = box(creg[n]);
+        }
       }
     }
     if (++acc == ACC_STAGES) { acc = 0; acc_phase ^= 1u; }
@@ -917,17 +882,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::tc_fence_after();
       uint32_t r_next[32];
       const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-      ptx::tmem_ld_32x32b_x32(t_acc + first_it * 32, r_next);
+      ptx::tmem_ld_32x32b(t_acc + first_it * 32, r_next);
       bool ok = true;
 #pragma unroll 1
       for (int it = first_it; it < kIters; it += split) {
         uint32_t r[32];
-        ptx::tmem_ld_wait();
+        ptx::tmem_ld_wait(r_next);
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = r_next[e];
         if (it + split < kIters) {
           const int jn = (it + split) / kSub, scn = (it + split) - jn * kSub;
-          ptx::tmem_ld_32x32b_x32(t_acc + jn * BLOCK_N + scn * 32, r_next);
+          ptx::tmem_ld_32x32b(t_acc + jn * BLOCK_N + scn * 32, r_next);
         }
         int row0, col0;
         if (!box_of(mt, nt, it, row0, col0)) continue;  // same answer for the whole warp
@@ -1050,13 +1015,14 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
   p.stages = ring_stages;
-  const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
-  p.epi_bytes = room >= kEpiWarps * 4096 ? kEpiWarps * 4096 : 16384;
+  p.epi_bytes = kEpiWarps * 2048;
   CUtensorMap map_c, map_d;
   if (!C::staged_epilogue(cs, p.cd_col_major)) {
     map_c = map_d = map_a;  // not used
   } else {
-    while (p.epi_bytes < 16 * 4096 && 2 * p.epi_bytes <= room) p.epi_bytes *= 2;
+    const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
+    p.epi_bytes = kEpiWarps * 4096;
+    if (2 * p.epi_bytes <= room) p.epi_bytes *= 2;
     // C and D move in 32 x 32 boxes whose rows are 128 bytes
     st = make_map(&map_d, p.D, cs, d->M, d->N, d->ldd * cs, 32, 32, 128);
     if (st != SP24_OK) return st;
