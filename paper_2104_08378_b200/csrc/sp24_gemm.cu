@@ -348,6 +348,8 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
     p.conv_h = (int)cv->h;
     p.conv_w = (int)cv->w;
     p.conv_c = (int)cv->c;
+    p.by_image = FastDiv::by((uint32_t)(cv->h * cv->w));
+    p.by_conv_w = FastDiv::by((uint32_t)cv->w);
   }
   p.acc_f16 = acc_f16 ? 1 : 0;
   if (dq) {

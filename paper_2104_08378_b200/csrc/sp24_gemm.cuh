@@ -18,6 +18,19 @@ constexpr int kNumThreads = 32 * (kFirstEpiWarp + kEpiWarps);
 constexpr long long kWaitTimeoutCycles = 2000ll * 1000ll * 1000ll;  // per wait: 1-2 s of SM clock
 constexpr uint32_t kTmemCols = 512;
 
+// n / d for n < 2^31 by a multiplication: mul / 2^(31 + log) is 1 / d rounded up, by less than 2^-31 / d, with 2^log the
+// first power of two >= d.  (A division by a divisor known only at run time takes the device about 150 cycles, and the
+// first load of a call waits for two.)
+struct FastDiv {
+  uint32_t mul, shift;
+  static FastDiv by(uint32_t d) {
+    uint32_t log = 0;
+    while ((uint64_t(1) << log) < d) ++log;
+    return {(uint32_t)((uint64_t(1) << (31 + log)) / d + 1), 31 + log};
+  }
+  __host__ __device__ __forceinline__ int operator()(int n) const { return (int)(((uint64_t)(uint32_t)n * mul) >> shift); }
+};
+
 struct GemmParams {
   int64_t M, N, K;
   int64_t ldc, ldd;   // elements
@@ -34,11 +47,13 @@ struct GemmParams {
   long long wait_limit;       // SM cycles after which a device-side wait gives up
   int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
   int32_t band;       // m-tiles per band of the tile sweep
+  FastDiv by_band_tiles, by_band, by_last_band;  // tiles of a band; m-tiles of a band and of the last one
   int32_t mblk, b_rows, b_stages;  // tall tiles only: m-blocks of a tile, rows of a B box, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout): selects the kernel
   // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
   int32_t conv, conv_h, conv_w, conv_c;
+  FastDiv by_image, by_conv_w;  // pixels of an image, of an image row
   // int8 dequantising epilogue (sp24_gemm_i8_dequant): out = act(row_scale[i] * acc + bias[i]),
   // requantised with out_inv_scale when the output type is int8
   int32_t dequant, relu;
