@@ -175,9 +175,9 @@ typedef struct {
 
 /* Reports the tile shape sp24_gemm (and its variants) would use for this problem with beta = 0 on the
  * current device: CTAs per tile (1, or 2 = a pair working on one tile), columns per tile, 128-row
- * blocks per CTA.  The output tile is (128 * ctas * mblk) x block_n.  With at most 128 columns the
- * choice may differ with C, and for sp24_conv3x3_nhwc, which has no tiles of one CTA and two or three
- * blocks.  Launches nothing. */
+ * blocks per CTA.  The output tile is (128 * ctas * mblk) x block_n, or narrower where that spreads a
+ * small problem over more SMs.  The choice may differ with C, and for sp24_conv3x3_nhwc, which has no
+ * tiles of one CTA and two or three blocks.  Launches nothing. */
 sp24_status sp24_gemm_plan(const sp24_gemm_desc* d, int* ctas, int* block_n, int* mblk);
 
 /* Bytes of device workspace sp24_gemm needs for this problem (currently a fixed 256 bytes:

@@ -252,10 +252,66 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& cta
   }
 }
 
+// Time of a product with tiles of (128 * ctas * mblk) x tile_n, us on an idle chip: start, and per round of tiles the
+// k-blocks (a fixed part and one per column, the same for all kinds: a k-block is 256 bytes of K), then the epilogue of a
+// tile by its columns (4-byte results and C cost more; 256-column tiles and two m-blocks cannot overlap it).  Fitted to
+// 170 random problems (256..16384 rows, 160..16384 columns, K 256..12288, every kind, with and without C), 11 to 17
+// shapes of each; mean error 5 to 10 % per shape.
+static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n) {
+  const int es = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
+  const double k_blocks = (double)((d->K * es + 255) / 256);
+  const int64_t rows = 128 * ctas * mblk, slots = sm_count() / ctas > 0 ? sm_count() / ctas : 1;
+  const int64_t tiles = ((d->M + rows - 1) / rows) * ((d->N + tile_n - 1) / tile_n);
+  const double rounds = (double)((tiles + slots - 1) / slots), w = tile_n / 100.0;
+  double loaded = w;  // with N contiguous, B comes in chunks of 128 bytes along N
+  if (d->order_b == SP24_ROW_MAJOR) loaded = (double)((tile_n / ctas * es + 127) / 128 * (128 / es) * ctas) / 100.0;
+  const double store = cs == 4 ? (has_c ? 2.0 : 1.0) : (has_c ? 1.4 : 0.6);
+  if (ctas == 1) return 2.4 + rounds * (k_blocks * (0.18 + 0.11 * loaded) + 0.12 + store * w);
+  if (mblk == 2) return 1.6 + 1.08 * rounds * (k_blocks * (es == 4 ? 0.68 : 0.59) + 0.6 + 2.6 * store * w);
+  if (block_n == 256) return 1.5 + rounds * (k_blocks * 0.156 * w + (0.5 + store) * w);
+  if (block_n == 240) return 2.2 + rounds * (k_blocks * 0.151 * w + 1.1 * store * w);
+  return 2.6 + rounds * (k_blocks * (0.165 + 0.085 * loaded) + 0.1 + store * w);
+}
+
+// Columns of a tile.  choose_tile() knows the widest form of each shape; a problem that leaves SMs idle in a round of
+// tiles is faster with narrower ones on more of them (us, device: f16 256 x 256 x 512 4.10 -> 3.23, f16 1184 x 736 x 1008
+// with C 7.6 -> 5.8, int8 992 x 480 x 6176 14.9 -> 9.5, bf16 512 x 192 x 10464 31.2 -> 19.8).  Over 150 other random
+// problems the choice below is 17 % faster in the mean than the widest tiles, one is slower by more than 2 % (int8 128 x
+// 3808 x 352 4.5 -> 4.7 us); over the 170 above it is 1.5 % behind the best of the shapes.  A pair keeps its shape, or its
+// two m-blocks, unless the estimate says 3 %, or 15 %: what it is wrong by.
+static void choose_width(const sp24_gemm_desc* d, bool has_c, int& ctas, int& block_n, int& mblk, int& tile_n) {
+  const int64_t n32 = (d->N + 31) / 32 * 32;
+  auto widest = [&](int bn) { return n32 < bn ? (int)n32 : bn; };
+  tile_n = widest(block_n);
+  if (ctas == 1 && mblk > 1) {  // tall tiles: all the columns there are
+    if (d->N < tile_n) tile_n = (int)d->N;
+    return;
+  }
+  if (ctas == 2 && (d->a_is_dense || d->N <= 128)) return;
+  const double now = tile_time(d, has_c, ctas, block_n, mblk, ctas == 2 ? block_n : tile_n);
+  double best = now * (ctas == 1 ? 1.0 : mblk == 2 ? 0.85 : 0.97);
+  auto try_shape = [&](int c, int bn, int tn) {
+    const double t = tile_time(d, has_c, c, bn, 1, tn);
+    if (t < best) { best = t; ctas = c; block_n = bn; mblk = 1; tile_n = tn; }
+  };
+  const bool pairs = !d->a_is_dense && d->N > 128 && d->M >= 256 && (d->M / 256) * ((d->N + 223) / 224) >= 4;
+  const bool k_major_b = d->order_b == SP24_COL_MAJOR, one = ctas == 1;
+  const bool has_240 = k_major_b && elem_bytes(d->ab_type) == 2 && elem_bytes(d->cd_type) == 2;
+  if (!one) try_shape(1, 128, widest(128));
+  for (int w = 96; w >= 32; w -= 32)
+    if (w < n32) try_shape(1, 128, w);
+  if (!pairs) return;
+  for (int w = 224; w >= 64; w -= 32) try_shape(2, 224, widest(w));
+  if (has_240) try_shape(2, 240, 240);
+  if (k_major_b) try_shape(2, 256, widest(256));
+}
+
 extern "C" sp24_status sp24_gemm_plan(const sp24_gemm_desc* d, int* ctas, int* block_n, int* mblk) {
   SP24_RETURN_IF(d == nullptr || ctas == nullptr || block_n == nullptr || mblk == nullptr, SP24_ERR_NULL);
   SP24_RETURN_IF(d->M <= 0 || d->N <= 0 || d->K <= 0, SP24_ERR_SHAPE);
+  int tile_n;
   choose_tile(d, false, false, *ctas, *block_n, *mblk);
+  choose_width(d, false, *ctas, *block_n, *mblk, tile_n);
   Settings& cfg = settings();
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     *ctas = c;
@@ -382,23 +438,26 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   const bool sparse = !d->a_is_dense;
   const bool i8 = d->ab_type == SP24_I8, tf32 = d->ab_type == SP24_F32, f8 = is_fp8(d->ab_type);
   int ctas, block_n, mblk;
+  int tile_n;
   choose_tile(d, has_c, cv != nullptr, ctas, block_n, mblk);
+  choose_width(d, has_c, ctas, block_n, mblk, tile_n);
   p.band = 16 / mblk;
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     ctas = c;
     block_n = cfg.block_n.load(std::memory_order_relaxed);
     mblk = cfg.mblk.load(std::memory_order_relaxed);
+    tile_n = ctas == 1 && mblk > 1 && d->N < block_n ? (int)d->N : block_n;
   }
   SP24_RETURN_IF(cv && ctas == 1 && mblk != 1, SP24_ERR_UNSUPPORTED);  // a forced tall tile
   p.mblk = mblk;
   if (const int b = cfg.band.load(std::memory_order_relaxed)) p.band = b;
   const bool b_mn = d->order_b == SP24_ROW_MAJOR;  // B stored N-contiguous
   if (cfg.log.load(std::memory_order_relaxed))
-    fprintf(stderr, "sp24_gemm: M=%lld N=%lld K=%lld ab=%d cd=%d %s%s tile=%dx%dx%d band=%d beta=%g%s%s\n", (long long)d->M,
+    fprintf(stderr, "sp24_gemm: M=%lld N=%lld K=%lld ab=%d cd=%d %s%s tile=%dx%dx%d columns=%d band=%d beta=%g%s%s\n", (long long)d->M,
             (long long)d->N, (long long)d->K, (int)d->ab_type, (int)d->cd_type, sparse ? "sparse" : "dense",
-            b_mn ? " B:N-contiguous" : "", ctas, block_n, mblk, p.band, (double)fbeta, dq ? " dequant" : "",
+            b_mn ? " B:N-contiguous" : "", ctas, block_n, mblk, tile_n, p.band, (double)fbeta, dq ? " dequant" : "",
             cv ? " conv3x3" : (acc_f16 ? " fp16-accumulate" : ""));
-  const TileShape tile = {ctas, block_n, mblk};
+  const TileShape tile = {ctas, block_n, mblk, tile_n};
   if (i8) return launch_gemm<1>(tile, sparse, b_mn, d, p, A, meta, B, s);
   if (tf32) return launch_gemm<2>(tile, sparse, b_mn, d, p, A, meta, B, s);
   if (f8) return launch_gemm<3>(tile, sparse, b_mn, d, p, A, meta, B, s);

@@ -48,7 +48,8 @@ struct GemmParams {
   int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
   int32_t band;       // m-tiles per band of the tile sweep
   FastDiv by_band_tiles, by_band, by_last_band;  // tiles of a band; m-tiles of a band and of the last one
-  int32_t mblk, b_rows, b_stages;  // tall tiles only: m-blocks of a tile, rows of a B box, slots of the B ring
+  int32_t tile_n;     // columns of a tile: the kernel's BLOCK_N or fewer
+  int32_t mblk, b_stages;  // tall tiles only: m-blocks of a tile, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout): selects the kernel
   // implicit 3x3 convolution: B is the im2col view of an NHWC activation (never materialised)
@@ -92,10 +93,10 @@ int sm_count();
 
 // ---- in sp24_gemm_{f16,i8,tf32,f8}.cu --------------------------------------------------------------
 // One launch of the kernel for MMA kind KIND (0 = f16 / bf16, 1 = int8, 2 = tf32, 3 = 8-bit floating point (e4m3 /
-// e5m2)) with tiles of ctas x block_n x mblk; SP24_ERR_UNSUPPORTED if that shape is not built.  Each kind is
-// instantiated in a source file of its own, so that they compile side by side.
+// e5m2)) with tiles of ctas x block_n x mblk of which tile_n columns are used; SP24_ERR_UNSUPPORTED if that shape is not
+// built.  Each kind is instantiated in a source file of its own, so that they compile side by side.
 struct TileShape {
-  int ctas, block_n, mblk;
+  int ctas, block_n, mblk, tile_n;
 };
 template <int KIND>
 sp24_status launch_gemm(TileShape tile, bool sparse, bool b_mn, const sp24_gemm_desc* d, const GemmParams& p, const void* A,

@@ -55,7 +55,6 @@ struct Cfg {
   // m-blocks takes one atom per operand so that four stages still fit
   static constexpr int kBBoxes = SPARSE ? 2 : (MBLK == 2 ? 1 : 2);
   static constexpr int kABoxes = SPARSE ? 1 : kBBoxes;
-  static constexpr int kBRows = BLOCK_N / CTAS;                    // B rows (N) this CTA loads
   static constexpr int kABlockBytes = kABoxes * kBlockM * kAtomBytes;  // one m-block
   static_assert(MBLK == 1 || kABoxes == 1, "the m-blocks of a stage are one box of rows");
   static constexpr int kABytes = MBLK * kABlockBytes;
@@ -63,40 +62,48 @@ struct Cfg {
   static constexpr int kKPerStage = kAtomElems * kBBoxes;  // logical K per stage
   // B with N contiguous (MN-major operand): 128-byte chunks along N, each kKPerStage k-rows of 128 bytes
   static constexpr int kBChunkElems = kAtomElems;
-  static constexpr int kBChunks = (kBRows + kBChunkElems - 1) / kBChunkElems;
   static constexpr int kBChunkBytes = kKPerStage * kAtomBytes;
   static constexpr int kBKStepBytes = (SPARSE ? 2 : 1) * (kAtomElems / 4) * kAtomBytes;  // k-rows of one MMA
   // an MN-major tf32 operand exists only in the 128-byte swizzle with 32-byte units (groups of 4 k-rows)
   static constexpr uint32_t kBMnLayout = KIND == 2 ? ptx::kLayoutSw128Base32 : ptx::kLayoutSw128;
   static constexpr uint32_t kBMnSbo = KIND == 2 ? 512 : 1024;
-  static constexpr int kBBytes = B_MN ? kBChunks * kBChunkBytes : kBBoxes * kBRows * kAtomBytes;
+  // A launch may use fewer columns than BLOCK_N (p.tile_n): rows of B (columns of D) a CTA loads per k-block, 128-byte
+  // chunks of them (N contiguous), bytes
+  __host__ __device__ static constexpr int b_rows(int tile_n) { return tile_n / CTAS; }
+  __host__ __device__ static constexpr int b_chunks(int tile_n) { return (b_rows(tile_n) + kBChunkElems - 1) / kBChunkElems; }
+  __host__ __device__ static constexpr int b_bytes(int tile_n) {
+    return B_MN ? b_chunks(tile_n) * kBChunkBytes : kBBoxes * b_rows(tile_n) * kAtomBytes;
+  }
   static constexpr int kEBlocks = SPARSE ? (one_byte_operands(KIND) ? 2 : 1) : 0;  // 2048-byte metadata blocks per m-block and stage
   static constexpr int kEBlockBytes = kEBlocks * 2048;
   static constexpr int kEBytes = MBLK * kEBlockBytes;
   static constexpr int kEAlloc = (kEBytes + 1023) / 1024 * 1024;
-  static constexpr int kStageBytes = kABytes + kBBytes + kEAlloc;
+  __host__ __device__ static constexpr int stage_bytes(int tile_n) { return kABytes + b_bytes(tile_n) + kEAlloc; }
   // shared memory: [stage ring | epilogue staging | barriers]; 1 KB of slack for the 1024-byte alignment
   // The split between ring stages and epilogue staging is made per launch (the output type
   // decides how much staging is useful).
   static constexpr int kSmemLimit = 232448 - 1024 - 512;
-  static constexpr int kMaxStages = is_tall<CTAS, MBLK> ? 12 : 8;
-  static constexpr int kMinStagesFit = (kSmemLimit - 16384) / kStageBytes;  // with the smallest staging
-  static constexpr int kRingStages = kMinStagesFit > kMaxStages ? kMaxStages : kMinStagesFit;
+  static constexpr int kMaxStages = 12;
+  // stages of a ring of slots of `bytes`, the epilogue's staging beside them
+  __host__ __device__ static constexpr int ring_stages(int bytes, int staging) {
+    return (kSmemLimit - staging) / bytes > kMaxStages ? kMaxStages : (kSmemLimit - staging) / bytes;
+  }
   // Epilogue form.  4-byte row-major outputs go through TMA boxes if every epilogue warp can have a
-  // 4 KB box of its own.  Everything else takes the warps' own loads and stores through a 2 KB transposing
+  // 4 KB box of its own without costing the ring of pairs a stage.  Everything else takes the warps' own loads and stores through a 2 KB transposing
   // buffer per warp (see epilogue_direct).
   __host__ __device__ static constexpr bool staged_epilogue(int cs, bool cols) {
-    return !is_tall<CTAS, MBLK> && !cols && cs == 4 && kSmemLimit - kRingStages * kStageBytes >= kEpiWarps * 4096;
+    return CTAS == 2 && !cols && cs == 4 &&
+           ring_stages(stage_bytes(BLOCK_N), kEpiWarps * 4096) == ring_stages(stage_bytes(BLOCK_N), kEpiWarps * 2048);
   }
   static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
   static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
   static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block
   static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
-  static_assert(kMinStagesFit >= 2, "need at least two stages");
+  static_assert(ring_stages(stage_bytes(BLOCK_N), kEpiWarps * 2048) >= 2, "need at least two stages");
   // the epilogue moves 32-column boxes; a last box of 16 columns (240-column tiles) is handled only by
   // epilogue_direct, which bounds every access by the tile's last column
   static_assert(BLOCK_N % 16 == 0, "tile width");
-  static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte alignment of the atoms");
+  static_assert(stage_bytes(32) % 1024 == 0 && stage_bytes(BLOCK_N) % 1024 == 0, "stages must keep the 1024-byte alignment of the atoms");
   static_assert(kECol + (SPARSE ? (is_tall<CTAS, MBLK> ? kMaxStages * 8 : 2 * MBLK * 8) : 0) <= (int)kTmemCols,
                 "tensor memory overflow");
 };
@@ -334,7 +341,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
     int mt, nt;
     tile_coords(t, p, mt, nt);
-    const int tile_col = nt * BLOCK_N, col_end = min(N, tile_col + BLOCK_N);  // columns of this tile stop here
+    const int tile_col = nt * p.tile_n, col_end = min(N, tile_col + p.tile_n);  // columns of this tile stop here
     // the boxes of this lane quarter: `nsub` in a row, `blocks` rows of them (m-blocks); this warp takes every other one
     const int row_q = (is_tall<CTAS, MBLK> ? mt * p.mblk * kBlockM : first_row<CTAS, MBLK>(mt, cta_rank, M)) + q * 32;
     const int nsub = (col_end - tile_col + kCols - 1) / kCols;
@@ -526,9 +533,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   constexpr bool kTall = is_tall<CTAS, MBLK>;
   static_assert(!kTall || (SPARSE && !B_MN && C::kABoxes == 1 && C::kBBoxes == 2), "tall tiles: sparse A, K-major B");
   // tall tiles: [slots of A and metadata | slots of B | epilogue staging]
-  constexpr int kSlotBytes = kTall ? C::kABlockBytes + C::kEBlockBytes : C::kStageBytes;
-  const int b_slot_bytes = kTall ? C::kBBoxes * p.b_rows * kAtomBytes : 0;
-  uint8_t* b_ring = smem + p.stages * kSlotBytes;
+  const int tile_n = p.tile_n, b_bytes = C::b_bytes(tile_n), b_slot_bytes = kTall ? b_bytes : 0;
+  const int slot_bytes = kTall ? C::kABlockBytes + C::kEBlockBytes : C::kABytes + b_bytes + C::kEAlloc;
+  uint8_t* b_ring = smem + p.stages * slot_bytes;
   uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : 0);
   Shared* sh = reinterpret_cast<Shared*>(epi + p.epi_bytes);
 
@@ -604,19 +611,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           for (int j = 0; j < MBLK; ++j) {
             if (j >= live) break;
             if (!(ok = bounded_wait(&sh->empty[slot], phase ^ 1u, sh, p.status, 1u, p.wait_limit))) break;
-            const uint32_t full = full0 + 8 * slot, sa = ring + slot * kSlotBytes;
+            const uint32_t full = full0 + 8 * slot, sa = ring + slot * slot_bytes;
             // (test hook: the slot is neither armed nor loaded, so that the issuer's wait for it expires)
             if (!(j == 0 && p.test_skip_stage && t == cluster_id && kb == 1)) {
-              ptx::mbar_expect_tx(&sh->full[slot], (uint32_t)(kSlotBytes + (j == 0 ? b_slot_bytes : 0)));
+              ptx::mbar_expect_tx(&sh->full[slot], (uint32_t)(slot_bytes + (j == 0 ? b_slot_bytes : 0)));
               if (j == 0) {
                 const uint32_t sb = b_ring_addr + b_slot * b_slot_bytes;
                 if (p.b_3d) {
-                  ptx::tma_load_3d<1>(sb, &map_b, full, 0, nt * BLOCK_N, kb * C::kBBoxes);
+                  ptx::tma_load_3d<1>(sb, &map_b, full, 0, nt * tile_n, kb * C::kBBoxes);
                 } else {
 #pragma unroll
                   for (int i = 0; i < C::kBBoxes; ++i)
-                    ptx::tma_load_2d<1>(sb + i * p.b_rows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * C::kAtomElems,
-                                        nt * BLOCK_N);
+                    ptx::tma_load_2d<1>(sb + i * tile_n * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * C::kAtomElems,
+                                        nt * tile_n);
                 }
               }
               ptx::tma_load_2d<1>(sa, &map_a, full, kb * C::kAtomElems, (blk0 + j) * kBlockM);
@@ -634,12 +641,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       int slot = 0, b_slot = 0;
       uint32_t phase = 0, acc_phase = 0;
       const int slots = tall_slots();
-      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), b_atom = p.b_rows * kAtomBytes;
+      const uint32_t ring = ptx::smem_u32(smem), b_ring_addr = ptx::smem_u32(b_ring), b_atom = tile_n * kAtomBytes;
       for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
         int mt, nt;
         tile_coords(t, p, mt, nt);
         const int live = tall_live(mt);
-        const uint32_t idesc = make_idesc<KIND>(SPARSE, false, p.a_fmt, kBlockM, min(BLOCK_N, (int)p.N - nt * BLOCK_N),
+        const uint32_t idesc = make_idesc<KIND>(SPARSE, false, p.a_fmt, kBlockM, min(tile_n, (int)p.N - nt * tile_n),
                                                 KIND == 0 && p.acc_f16);
         if (!bounded_wait(&sh->tmem_empty[0], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
         ptx::tc_fence_after();
@@ -652,7 +659,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (!(ok = bounded_wait(&sh->full[slot], phase, sh, p.status, 3u, p.wait_limit))) break;
             ptx::tc_fence_after();
             // (metadata columns per slot: a full slot also says that nothing reads its columns any more)
-            const uint32_t sa = ring + slot * kSlotBytes, e_tmem = tmem_base + C::kECol + slot * 8, d_tmem = tmem_base + j * BLOCK_N;
+            const uint32_t sa = ring + slot * slot_bytes, e_tmem = tmem_base + C::kECol + slot * 8, d_tmem = tmem_base + j * BLOCK_N;
 #pragma unroll
             for (int i = 0; i < C::kEBlocks; ++i)
               ptx::tmem_cp_128x128b<CTAS>(e_tmem + 4 * i, ptx::smem_desc(sa + C::kABlockBytes + i * 2048, ptx::kLayoutNone, 128));
@@ -687,16 +694,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       int stage = 0;
       uint32_t phase = 0;
       constexpr int box_elems = C::kAtomElems;  // elements per 128-byte atom row
+      const int b_atom = C::b_rows(tile_n) * kAtomBytes;
       const uint32_t ring = ptx::smem_u32(smem);
       const uint32_t full0 = CTAS == 2 ? ptx::map_to_cta(ptx::smem_u32(&sh->full[0]), 0) : ptx::smem_u32(&sh->full[0]);
       for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
         int mt, nt;
         tile_coords(t, p, mt, nt);
         // the last n-tile may be narrower: the pair then splits only the columns that exist
-        const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
-        const int col0 = nt * BLOCK_N + (int)cta_rank * (n_eff / CTAS);  // first B row (N index)
+        const int n_eff = min(tile_n, (int)(p.N - (int64_t)nt * tile_n));
+        const int col0 = nt * tile_n + (int)cta_rank * (n_eff / CTAS);  // first B row (N index)
         const int row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M);
-        constexpr uint32_t tx_bytes = (uint32_t)((C::kABytes + C::kEBytes + C::kBBytes) * CTAS);
+        const uint32_t tx_bytes = (uint32_t)((C::kABytes + C::kEBytes + b_bytes) * CTAS);
         // implicit convolution: (image, row, column) of this CTA's first output pixel
         int conv_n = 0, conv_p = 0, conv_q = 0, conv_c0 = 0, conv_r = 0, conv_s = 0;
         if (p.conv) {
@@ -717,7 +725,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             continue;
           }
-          const uint32_t sa = ring + stage * C::kStageBytes, sb = sa + C::kABytes, se = sb + C::kBBytes;
+          const uint32_t sa = ring + stage * slot_bytes, sb = sa + C::kABytes, se = sb + b_bytes;
           const uint32_t full = full0 + 8 * stage;
           if (cta_rank == 0) ptx::mbar_expect_tx(&sh->full[stage], tx_bytes);
           // both m-blocks' rows and metadata blocks are neighbours: one box each
@@ -727,14 +735,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             ptx::tma_load_2d<CTAS>(sa + i * MBLK * kBlockM * kAtomBytes, &map_a, full, (kb * C::kABoxes + i) * box_elems, row0);
           if (B_MN) {
             // B stored N-contiguous: boxes of 128 bytes along N x all k-rows of the stage
-#pragma unroll
-            for (int c = 0; c < C::kBChunks; ++c)
+            for (int c = 0; c < C::b_chunks(tile_n); ++c)
               ptx::tma_load_2d<CTAS>(sb + c * C::kBChunkBytes, &map_b, full, col0 + c * C::kBChunkElems, kb * C::kKPerStage);
           } else if (p.conv) {
             // k = (r * 3 + s) * C + c: a stage holds channels of one filter tap; rows = output pixels
 #pragma unroll
             for (int i = 0; i < C::kBBoxes; ++i)
-              ptx::tma_load_im2col_4d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, conv_c0 + i * box_elems, conv_q - 1,
+              ptx::tma_load_im2col_4d<CTAS>(sb + i * b_atom, &map_b, full, conv_c0 + i * box_elems, conv_q - 1,
                                             conv_p - 1, conv_n, (uint16_t)conv_s, (uint16_t)conv_r);
             conv_c0 += C::kKPerStage;
             if (conv_c0 == p.conv_c) {
@@ -746,7 +753,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           } else {
 #pragma unroll
             for (int i = 0; i < C::kBBoxes; ++i)
-              ptx::tma_load_2d<CTAS>(sb + i * C::kBRows * kAtomBytes, &map_b, full, (kb * C::kBBoxes + i) * box_elems, col0);
+              ptx::tma_load_2d<CTAS>(sb + i * b_atom, &map_b, full, (kb * C::kBBoxes + i) * box_elems, col0);
           }
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
@@ -755,13 +762,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (cta_rank == 0 && ptx::elect_one()) {
+      const int b_atom = C::b_rows(tile_n) * kAtomBytes;
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, e_buf = 0;
       for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
         int mt, nt;
         tile_coords(t, p, mt, nt);
         // instruction N = the columns this tile really has (a multiple of 16, of 32 for int8)
-        const int n_eff = min(BLOCK_N, (int)(p.N - (int64_t)nt * BLOCK_N));
+        const int n_eff = min(tile_n, (int)(p.N - (int64_t)nt * tile_n));
         const int live = live_blocks<CTAS, MBLK>(mt, (int)p.M);  // m-blocks with rows (others are not multiplied)
         const uint32_t idesc = make_idesc<KIND>(SPARSE, B_MN, p.a_fmt, kBlockM * CTAS, n_eff, KIND == 0 && p.acc_f16);
         if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
@@ -770,9 +778,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
           ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem + stage * C::kStageBytes);
+          const uint32_t sa = ptx::smem_u32(smem) + stage * slot_bytes;
           const uint32_t sb = sa + C::kABytes;
-          const uint32_t se = sb + C::kBBytes;
+          const uint32_t se = sb + b_bytes;
           // metadata columns alternate between two small tensor-memory buffers from k-block to k-block
           const uint32_t e_base = tmem_base + C::kECol + e_buf * (MBLK * 8);
           e_buf ^= 1u;
@@ -799,7 +807,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 // 32 bytes of compressed A and 64 bytes of B per instruction
                 uint64_t da = ptx::smem_desc(saj + k * 32, ptx::kLayoutSw128, 1024);
                 uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 1) * C::kBRows * kAtomBytes + (k & 1) * 64, ptx::kLayoutSw128, 1024);
+                                   : ptx::smem_desc(sb + (k >> 1) * b_atom + (k & 1) * 64, ptx::kLayoutSw128, 1024);
                 if (!one_byte_operands(KIND)) {
                   // one 32-bit metadata column per instruction: even-aligned address + selector
                   ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + (k & ~1), idesc | (uint32_t)(k & 1), accumulate);
@@ -809,7 +817,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
               } else {
                 uint64_t da = ptx::smem_desc(saj + (k >> 2) * kBlockM * kAtomBytes + (k & 3) * 32, ptx::kLayoutSw128, 1024);
                 uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 2) * C::kBRows * kAtomBytes + (k & 3) * 32, ptx::kLayoutSw128, 1024);
+                                   : ptx::smem_desc(sb + (k >> 2) * b_atom + (k & 3) * 32, ptx::kLayoutSw128, 1024);
                 ptx::mma_dense<KIND, CTAS>(d_tmem, da, db, idesc, accumulate);
               }
             }
@@ -845,14 +853,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // (the buffer of box seq + 1 is claimed, for its C or its result, at the end of box seq: with two buffers one
     // store may still be reading its own then)
     uint8_t* my_bufs = epi + ew * warp_bytes;
-    constexpr int kSub = BLOCK_N / 32;
-    constexpr int kIters = MBLK * kSub;
+    const int subs = tile_n / 32, iters = MBLK * subs;
 
     // box `it` of the tile (mt, nt): first row / column and whether any of it lies inside the matrix
     auto box_of = [&](int mt, int nt, int it, int& row0, int& col0) -> bool {
-      const int j = it / kSub, sc = it - j * kSub;
+      const int j = it >= subs, sc = it - j * subs;
       row0 = first_row<CTAS, MBLK>(mt, (int)cta_rank, (int)p.M) + j * kBlockM + q * 32;
-      col0 = nt * BLOCK_N + sc * 32;
+      col0 = nt * tile_n + sc * 32;
       return j < live_blocks<CTAS, MBLK>(mt, (int)p.M) && row0 < p.M && col0 < p.N;
     };
     // cursor of the C loads over the same stream of boxes, one live box in front of the consumer
@@ -865,7 +872,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         int row0, col0;
         const bool live_box = box_of(pf_mt, pf_nt, pf_it, row0, col0);
         pf_it += split;
-        if (pf_it >= kIters) {
+        if (pf_it >= iters) {
           pf_it = first_it;
           pf_t += num_clusters;
           if (pf_t < num_tiles) tile_coords(pf_t, p, pf_mt, pf_nt);
@@ -893,13 +900,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::tmem_ld_32x32b(t_acc + first_it * 32, r_next);
       bool ok = true;
 #pragma unroll 1
-      for (int it = first_it; it < kIters; it += split) {
+      for (int it = first_it; it < iters; it += split) {
         uint32_t r[32];
         ptx::tmem_ld_wait(r_next);
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = r_next[e];
-        if (it + split < kIters) {
-          const int jn = (it + split) / kSub, scn = (it + split) - jn * kSub;
+        if (it + split < iters) {
+          const int jn = it + split >= subs, scn = (it + split) - jn * subs;
           ptx::tmem_ld_32x32b(t_acc + jn * BLOCK_N + scn * 32, r_next);
         }
         int row0, col0;
@@ -964,31 +971,34 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 }
 
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
-sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* A, const void* meta, const void* B,
+sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, const void* A, const void* meta, const void* B,
                    cudaStream_t stream) {
   using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   GemmParams p = base;
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
-  int tile_m = kBlockM * CTAS * MBLK, ring_stages = C::kRingStages, ring_bytes = C::kStageBytes, b_ring_bytes = 0;
-  uint32_t b_box_rows = C::kBRows;
+  p.tile_n = tile_n;
+  const int cs = elem_bytes(d->cd_type);
+  // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
+  // stage less cost the int8 configuration 9 %); a staged epilogue gets what is left.
+  p.epi_bytes = kEpiWarps * (C::staged_epilogue(cs, p.cd_col_major) ? 4096 : 2048);
+  int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n);
+  p.stages = C::ring_stages(ring_bytes, p.epi_bytes);
   if constexpr (is_tall<CTAS, MBLK>) {
-    p.b_rows = (int32_t)(d->N < BLOCK_N ? d->N : BLOCK_N);
     tile_m = p.mblk * kBlockM;
-    b_box_rows = p.b_rows;
     // slots of A (each k-block needs mblk) and of B: the split with the most of A in flight
-    const int b_slot = C::kBBoxes * p.b_rows * kAtomBytes, budget = C::kSmemLimit - 16384;
+    const int b_slot = C::b_bytes(tile_n), budget = C::kSmemLimit - p.epi_bytes;
     ring_bytes = C::kABlockBytes + C::kEBlockBytes;
-    ring_stages = 0;
+    p.stages = 0;
     for (int bs = 2; bs <= 8 && bs * b_slot < budget; ++bs) {
       int slots = (budget - bs * b_slot) / ring_bytes;
       if (slots > (bs - 1) * p.mblk + 1) slots = (bs - 1) * p.mblk + 1;
       if (slots > C::kMaxStages) slots = C::kMaxStages;
-      if (slots > ring_stages) { ring_stages = slots; p.b_stages = bs; }
+      if (slots > p.stages) { p.stages = slots; p.b_stages = bs; }
     }
-    b_ring_bytes = p.b_stages * b_slot;
   }
+  const uint32_t b_box_rows = (uint32_t)C::b_rows(tile_n);
   p.m_tiles = (int)((d->M + tile_m - 1) / tile_m);
-  p.n_tiles = (int)((d->N + BLOCK_N - 1) / BLOCK_N);
+  p.n_tiles = (int)((d->N + tile_n - 1) / tile_n);
   p.k_blocks = (int)((d->K + C::kKPerStage - 1) / C::kKPerStage);
   if (p.band > p.m_tiles) p.band = p.m_tiles;
   p.by_band_tiles = FastDiv::by((uint32_t)(p.band * p.n_tiles));
@@ -1002,11 +1012,11 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, (is_tall<CTAS, MBLK> ? 1 : MBLK) * kBlockM, 128);
   if (st != SP24_OK) return st;
   if (p.conv) {
-    // B = im2col view of the NHWC activation: boxes of kBRows output pixels x one 128-byte run of channels
+    // B = im2col view of the NHWC activation: boxes of b_rows output pixels x one 128-byte run of channels
     if (B_MN) return SP24_ERR_UNSUPPORTED;
     if (KIND == 2) return SP24_ERR_UNSUPPORTED;
     const uint64_t nb = (uint64_t)d->N / ((uint64_t)p.conv_h * p.conv_w);
-    st = make_im2col_map(&map_b, B, es, nb, p.conv_h, p.conv_w, p.conv_c, atom_elems, C::kBRows);
+    st = make_im2col_map(&map_b, B, es, nb, p.conv_h, p.conv_w, p.conv_c, atom_elems, b_box_rows);
   } else if (B_MN) {
     st = make_map(&map_b, B, es, d->K, d->N, d->ldb * es, C::kBChunkElems, C::kKPerStage,
                   KIND == 2 ? kSwizzle128Atom32 : 128);
@@ -1028,18 +1038,11 @@ sp24_status launch(const sp24_gemm_desc* d, const GemmParams& base, const void* 
   } else {
     map_e = map_a;
   }
-  const int cs = elem_bytes(d->cd_type);
-  // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
-  // stage less cost the int8 configuration 9 %); staging gets what is left, in powers of two from 16 KB.
-  p.stages = ring_stages;
-  p.epi_bytes = kEpiWarps * 2048;
   CUtensorMap map_c, map_d;
   if (!C::staged_epilogue(cs, p.cd_col_major)) {
     map_c = map_d = map_a;  // not used
   } else {
-    const int room = C::kSmemLimit - p.stages * ring_bytes - b_ring_bytes;
-    p.epi_bytes = kEpiWarps * 4096;
-    if (2 * p.epi_bytes <= room) p.epi_bytes *= 2;
+    if (C::kSmemLimit - p.stages * ring_bytes >= 2 * p.epi_bytes) p.epi_bytes *= 2;
     // C and D move in 32 x 32 boxes whose rows are 128 bytes
     st = make_map(&map_d, p.D, cs, d->M, d->N, d->ldd * cs, 32, 32, 128);
     if (st != SP24_OK) return st;
@@ -1087,7 +1090,7 @@ sp24_status launch_gemm(TileShape t, bool sparse, bool b_mn, const sp24_gemm_des
   auto is = [&](int ctas, int block_n, int mblk) { return t.ctas == ctas && t.block_n == block_n && t.mblk == mblk; };
 #define SP24_SHAPE(CT, BN, MB, MN)                                     \
   if (is(CT, BN, MB) && b_mn == MN)                                    \
-    return sparse ? launch<KIND, true, BN, CT, MB, MN>(d, p, A, meta, B, s) : launch<KIND, false, BN, CT, MB, MN>(d, p, A, meta, B, s);
+    return sparse ? launch<KIND, true, BN, CT, MB, MN>(t.tile_n, d, p, A, meta, B, s) : launch<KIND, false, BN, CT, MB, MN>(t.tile_n, d, p, A, meta, B, s);
   SP24_SHAPE(1, 128, 1, false)
   SP24_SHAPE(2, 224, 1, false)
   SP24_SHAPE(2, 224, 2, false)
@@ -1102,9 +1105,9 @@ sp24_status launch_gemm(TileShape t, bool sparse, bool b_mn, const sp24_gemm_des
     SP24_SHAPE(2, 240, 1, false)  // 2-byte outputs only
   }
   if constexpr (!tf32)  // dense variant only
-    if (is(2, 256, 2) && !sparse && !b_mn) return launch<KIND, false, 256, 2, 2, false>(d, p, A, meta, B, s);
+    if (is(2, 256, 2) && !sparse && !b_mn) return launch<KIND, false, 256, 2, 2, false>(t.tile_n, d, p, A, meta, B, s);
   if (t.ctas == 1 && t.block_n == 128 && (t.mblk == 2 || t.mblk == kTallBlocks) && sparse && !b_mn)
-    return launch<KIND, true, 128, 1, kTallBlocks, false>(d, p, A, meta, B, s);
+    return launch<KIND, true, 128, 1, kTallBlocks, false>(t.tile_n, d, p, A, meta, B, s);
 #undef SP24_SHAPE
   return SP24_ERR_UNSUPPORTED;
 }
