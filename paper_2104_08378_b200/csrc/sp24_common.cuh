@@ -76,6 +76,29 @@ inline sp24_status launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
   return cuda_status(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
 }
 
+// ---- streaming kernels ----------------------------------------------------------------------------------
+constexpr int kThreads = 256;
+
+// Block shape and grid of the vectorised kernels for `units` work units per row and `rows` rows:
+// TX (a power of two, 32..256) threads along the row, chosen to waste the fewest lanes.
+struct RowLaunch {
+  dim3 grid, block;
+  RowLaunch(int64_t units, int64_t rows, int unroll) {
+    int best_tx = 256;
+    int64_t best_cover = -1;
+    for (int tx = 256; tx >= 32; tx /= 2) {
+      int64_t per = (int64_t)tx * unroll;
+      int64_t cover = (units + per - 1) / per * per;
+      if (best_cover < 0 || cover < best_cover) { best_cover = cover; best_tx = tx; }
+    }
+    int ty = kThreads / best_tx;
+    block = dim3((unsigned)best_tx, (unsigned)ty, 1);
+    int64_t gy = (rows + ty - 1) / ty;
+    if (gy > 32768) gy = 32768;
+    grid = dim3((unsigned)(best_cover / ((int64_t)best_tx * unroll)), (unsigned)gy, 1);
+  }
+};
+
 #define SP24_RETURN_IF(cond, code) \
   do {                             \
     if (cond) return (code);       \

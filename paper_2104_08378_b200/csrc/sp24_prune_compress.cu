@@ -7,8 +7,6 @@
 namespace sp24 {
 namespace {
 
-constexpr int kThreads = 256;
-
 // ---- selection -------------------------------------------------------------------------
 // Bit p of the result is set iff position p of the group is kept.  Position a beats position b
 // (a < b) when key[a] >= key[b] -- equal magnitudes go to the lower index -- so the six
@@ -613,26 +611,6 @@ __global__ void __launch_bounds__(kThreads) decompress_f32_kernel(const uint8_t*
 }
 
 inline unsigned blocks_for(int64_t total, int per_block) { return (unsigned)((total + per_block - 1) / per_block); }
-
-// Block shape and grid of the vectorised kernels for `units` work units per row and `rows` rows:
-// TX (a power of two, 32..256) threads along the row, chosen to waste the fewest lanes.
-struct RowLaunch {
-  dim3 grid, block;
-  RowLaunch(int64_t units, int64_t rows, int unroll) {
-    int best_tx = 256;
-    int64_t best_cover = -1;
-    for (int tx = 256; tx >= 32; tx /= 2) {
-      int64_t per = (int64_t)tx * unroll;
-      int64_t cover = (units + per - 1) / per * per;
-      if (best_cover < 0 || cover < best_cover) { best_cover = cover; best_tx = tx; }
-    }
-    int ty = kThreads / best_tx;
-    block = dim3((unsigned)best_tx, (unsigned)ty, 1);
-    int64_t gy = (rows + ty - 1) / ty;
-    if (gy > 32768) gy = 32768;
-    grid = dim3((unsigned)(best_cover / ((int64_t)best_tx * unroll)), (unsigned)gy, 1);
-  }
-};
 
 }  // namespace
 
