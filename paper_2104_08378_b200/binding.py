@@ -1,4 +1,4 @@
-"""ctypes binding of the sp24 C ABI (include/sp24.h): argument marshalling only.
+"""Binding of the sp24 C ABI (include/sp24.h): argument marshalling only, by ctypes and, for the short calls, natively.
 
 Every function takes torch CUDA tensors (PyTorch is used for device memory and streams only),
 passes their device pointers and the current stream to ``libsp24.so`` and raises
@@ -106,6 +106,18 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 
+if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+    from . import _native      # compiled beside libsp24.so (csrc/sp24_native.cpp); missing: the import fails
+else:                          # a CPU-only build of torch has no CUDA tensors: every call is for the functions below
+    class _native:
+        gemm = gemm_i8_dequant = conv3x3_nhwc = compress = apply_mask = staticmethod(lambda *args: None)
+
+# Addresses for the native form of the short calls, which does what the functions below do if all arguments are of the
+# ordinary kind, and returns None if not (then they do it themselves) or the status of a call that was refused.
+_GEMM, _DEQUANT, _CONV, _COMPRESS, _META_BYTES, _APPLY_MASK = (
+    ctypes.cast(getattr(lib, name), ctypes.c_void_p).value
+    for name in ("sp24_gemm", "sp24_gemm_i8_dequant", "sp24_conv3x3_nhwc", "sp24_compress", "sp24_meta_bytes", "sp24_apply_mask"))
+
 
 def status_string(status: int) -> str:
     return lib.sp24_status_string(int(status)).decode()
@@ -159,6 +171,10 @@ def prune(x: torch.Tensor, out: torch.Tensor | None = None, dtype: str | None = 
 def compress(x: torch.Tensor, layout: int = META_TCGEN05, dtype: str | None = None,
              count_dropped: bool = False):
     """sp24_compress: returns (vals [M, K/2], meta uint8 [meta_bytes], dropped tensor or None)."""
+    if dtype is None and count_dropped is False:
+        done = _native.compress(_COMPRESS, _META_BYTES, x, layout)
+        if done is not None:
+            return done if type(done) is not int else _check(done, "sp24_compress")
     dt = _dtype_of(x, dtype)
     M, K = x.shape
     vals = x.new_empty((M, K // 2))
@@ -252,6 +268,10 @@ def gemm(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor, *, alpha=
     """sp24_gemm (sp24_gemm_f16acc with acc_f16=True).  A: vals [M, K/2] (or dense [M, K]); Bt: [N, K]
     (K contiguous), or with b_row_major=True the K x N matrix itself, [K, N] (N contiguous); C/D: [M, N],
     or with cd_col_major=True their transposes [N, M] (M contiguous)."""
+    if ab is None and acc_f16 is False:
+        done = _native.gemm(_GEMM, _workspaces, A, meta, Bt, alpha, beta, C, out, cd, a_is_dense, ws, b_row_major, cd_col_major)
+        if done is not None:
+            return done if type(done) is not int else _check(done, "sp24_gemm")
     ab = _dtype_of(A, ab)
     a_shape, b_shape = A.shape, Bt.shape
     M = a_shape[0]
@@ -337,6 +357,10 @@ def gemm_i8_dequant(A: torch.Tensor, meta: torch.Tensor | None, Bt: torch.Tensor
                     out: torch.Tensor | None = None, a_is_dense: bool = False, ws: torch.Tensor | None = None,
                     b_row_major: bool = False, cd_col_major: bool = False) -> torch.Tensor:
     """sp24_gemm_i8_dequant: int8 sparse GEMM, D = act(row_scale[i] * acc + bias[i]) as cd (bf16/f16/f32/i8)."""
+    done = _native.gemm_i8_dequant(_DEQUANT, _workspaces, A, meta, Bt, row_scale, bias, relu, out_scale, cd, out, a_is_dense,
+                                   ws, b_row_major, cd_col_major)
+    if done is not None:
+        return done if type(done) is not int else _check(done, "sp24_gemm_i8_dequant")
     a_shape = A.shape
     M = a_shape[0]
     K = a_shape[1] if a_is_dense else 2 * a_shape[1]
@@ -358,6 +382,10 @@ def conv3x3_nhwc(A: torch.Tensor, meta: torch.Tensor | None, x: torch.Tensor, *,
                  ab: str | None = None, a_is_dense: bool = False, ws: torch.Tensor | None = None,
                  nhwc_out: bool = False) -> torch.Tensor:
     """sp24_conv3x3_nhwc: x [Nb, H, W, Cin] -> D [Kout, Nb*H*W] (or NHWC [Nb*H*W, Kout] with nhwc_out)."""
+    if ab is None:
+        done = _native.conv3x3_nhwc(_CONV, _workspaces, A, meta, x, alpha, beta, C, out, cd, a_is_dense, ws, nhwc_out)
+        if done is not None:
+            return done if type(done) is not int else _check(done, "sp24_conv3x3_nhwc")
     ab = _dtype_of(A, ab)
     Nb, H, W, Cin = x.shape
     M = A.shape[0]
@@ -389,6 +417,10 @@ def kept_magnitude(x: torch.Tensor, perm: torch.Tensor | None = None, dtype: str
 def apply_mask(w: torch.Tensor, meta: torch.Tensor, layout: int = META_TCGEN05, out: torch.Tensor | None = None,
                dtype: str | None = None) -> torch.Tensor:
     """sp24_apply_mask: zero every position of w the metadata does not name as kept."""
+    if out is not None and dtype is None:
+        done = _native.apply_mask(_APPLY_MASK, w, meta, layout, out)
+        if done is not None:
+            return done if type(done) is not int else _check(done, "sp24_apply_mask")
     dt = _dtype_of(w, dtype)
     M, K = w.shape
     if out is None:

@@ -1,9 +1,12 @@
-"""Compile the CUDA library in-tree: csrc/*.cu -> libsp24.so (sm_100a SASS only), the sources side by side."""
+"""Compile the CUDA library in-tree: csrc/*.cu -> libsp24.so (sm_100a SASS only), the sources side by side, and the
+binding's native part, csrc/sp24_native.cpp -> _native.so."""
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
+import sysconfig
 import tempfile
 from concurrent.futures import ThreadPoolExecutor
 
@@ -12,6 +15,9 @@ _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libsp24.so")
 SOURCES = sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cuh"))) + [os.path.join(_ROOT, "include", "sp24.h")]
+
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
+NATIVE_SOURCES = [os.path.join(_HERE, "csrc", "sp24_native.cpp"), os.path.join(_ROOT, "include", "sp24.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -27,16 +33,31 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def _older(path: str, sources) -> bool:
+    return not os.path.exists(path) or any(os.path.getmtime(f) > os.path.getmtime(path) for f in sources)
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB_PATH):
-        return True
-    built = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(f) > built for f in SOURCES + HEADERS)
+    return _older(LIB_PATH, SOURCES + HEADERS) or _older(NATIVE_PATH, NATIVE_SOURCES)
+
+
+def _build_native() -> None:
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda_dir = os.path.dirname(os.path.dirname(_nvcc()))
+    include = [os.path.join(_ROOT, "include"), os.path.join(torch_dir, "include"),
+               os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+               os.path.join(cuda_dir or "/usr/local/cuda", "include")]
+    tmp = f"{NATIVE_PATH}.{os.getpid()}.tmp"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared"] + [f"-I{d}" for d in include] +
+                          ["-o", tmp, NATIVE_SOURCES[0], f"-L{torch_dir}/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, NATIVE_PATH)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Run nvcc if the library is missing or older than its sources; returns the .so path."""
-    if force or needs_build():
+    """Compile what is missing or older than its sources (everything with force); returns the CUDA library's path."""
+    if force or _older(NATIVE_PATH, NATIVE_SOURCES):
+        _build_native()
+    if force or _older(LIB_PATH, SOURCES + HEADERS):
         tmp = f"{LIB_PATH}.{os.getpid()}.tmp"
         compile_ = [_nvcc()] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else [])
         with tempfile.TemporaryDirectory() as objects, ThreadPoolExecutor(os.cpu_count()) as pool:
