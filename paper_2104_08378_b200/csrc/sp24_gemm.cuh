@@ -49,6 +49,7 @@ struct GemmParams {
   int32_t band;       // m-tiles per band of the tile sweep
   FastDiv by_band_tiles, by_band, by_last_band;  // tiles of a band; m-tiles of a band and of the last one
   int32_t tile_n;     // columns of a tile: the kernel's BLOCK_N or fewer
+  int32_t kps;        // k-blocks of a stage (1 or 2)
   int32_t mblk, b_stages;  // tall tiles only: m-blocks of a tile, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout): selects the kernel

@@ -97,7 +97,9 @@ struct Cfg {
   }
   static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
   static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
-  static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block
+  static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block and k-block
+  // Stages of two k-blocks (p.kps; see the producer)
+  static constexpr bool kPairsOfKBlocks = SPARSE && !B_MN && MBLK == 1;
   static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
   static_assert(ring_stages(stage_bytes(BLOCK_N), kEpiWarps * 2048) >= 2, "need at least two stages");
   // the epilogue moves 32-column boxes; a last box of 16 columns (240-column tiles) is handled only by
@@ -534,7 +536,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   static_assert(!kTall || (SPARSE && !B_MN && C::kABoxes == 1 && C::kBBoxes == 2), "tall tiles: sparse A, K-major B");
   // tall tiles: [slots of A and metadata | slots of B | epilogue staging]
   const int tile_n = p.tile_n, b_bytes = C::b_bytes(tile_n), b_slot_bytes = kTall ? b_bytes : 0;
-  const int slot_bytes = kTall ? C::kABlockBytes + C::kEBlockBytes : C::kABytes + b_bytes + C::kEAlloc;
+  const int kps = C::kPairsOfKBlocks ? p.kps : 1;  // k-blocks of a stage
+  const int slot_bytes = kTall ? C::kABlockBytes + C::kEBlockBytes : kps * (C::kABytes + b_bytes + C::kEAlloc);
   uint8_t* b_ring = smem + p.stages * slot_bytes;
   uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : 0);
   Shared* sh = reinterpret_cast<Shared*>(epi + p.epi_bytes);
@@ -687,6 +690,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   } else if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (ptx::elect_one()) {
+      // The thread that issues the loads needs about 390 cycles for a stage whatever its bytes (170 to look at the ring,
+      // 215 to issue three loads), more than the MMAs of a narrow tile take: its stages hold two k-blocks each, which
+      // are loaded by as many loads as one.  One k-block a stage and two, us, device: bf16 512 x 512 x 8192 16.0, 13.1;
+      // 4096 x 32 x 4096 9.1, 7.8; int8 4096 x 32 x 4096 6.0, 5.4.  Loops of their own: with the number of k-blocks as a
+      // variable of one loop, products with one a stage were up to 15 % slower.
       // (Shared-memory and barrier addresses as plain integers, as few loads per stage as the boxes allow: the
       // thread that issues them is busy for about 100 cycles per load, which delays the refill of a stage.
       // Three loads instead of six (two m-blocks) or four: 49152 x 32 x 12288 bf16 123.1 -> 119.6 us, int8
@@ -717,6 +725,21 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         // panel the wave before it has just finished with, saves 12 % of the DRAM reads and 1.5 % of the
         // time, but makes the rounding of a result depend on which CTA computed its tile: the same rows
         // and columns would no longer give the same bits when M or N is split differently.  Not done.)
+        if (kps == 2) {  // (A in whole 128-byte atoms: its atoms are a third dimension as B's are)
+          for (int kb = 0; kb < p.k_blocks; kb += 2) {
+            if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
+            if (!(p.test_skip_stage && t == cluster_id && kb == 2)) {  // (test hook: as below)
+              const uint32_t sa = ring + stage * slot_bytes, sb = sa + 2 * C::kABytes, se = sb + 2 * b_bytes;
+              const uint32_t full = full0 + 8 * stage;
+              if (cta_rank == 0) ptx::mbar_expect_tx(&sh->full[stage], 2 * tx_bytes);
+              ptx::tma_load_3d<CTAS>(se, &map_e, full, 0, 16 * kb * C::kEBlocks, row0 / kBlockM);
+              ptx::tma_load_3d<CTAS>(sa, &map_a, full, 0, row0, kb);
+              ptx::tma_load_3d<CTAS>(sb, &map_b, full, 0, col0, kb * C::kBBoxes);
+            }
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+          }
+          continue;
+        }
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
           if (p.test_skip_stage && t == cluster_id && kb == 1) {
@@ -763,6 +786,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // ------------------------------ MMA issuer ------------------------------
     if (cta_rank == 0 && ptx::elect_one()) {
       const int b_atom = C::b_rows(tile_n) * kAtomBytes;
+      const uint32_t ring = ptx::smem_u32(smem);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0, e_buf = 0;
       for (int t = cluster_id; t < num_tiles && !sh->abort; t += num_clusters) {
@@ -772,15 +796,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         const int n_eff = min(tile_n, (int)(p.N - (int64_t)nt * tile_n));
         const int live = live_blocks<CTAS, MBLK>(mt, (int)p.M);  // m-blocks with rows (others are not multiplied)
         const uint32_t idesc = make_idesc<KIND>(SPARSE, B_MN, p.a_fmt, kBlockM * CTAS, n_eff, KIND == 0 && p.acc_f16);
-        if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
-        ptx::tc_fence_after();
-        bool ok = true;
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
-          ptx::tc_fence_after();
-          const uint32_t sa = ptx::smem_u32(smem) + stage * slot_bytes;
-          const uint32_t sb = sa + C::kABytes;
-          const uint32_t se = sb + b_bytes;
+        // the MMAs of a k-block: A, B and metadata at sa, sb, se
+        auto multiply = [&](int kb, uint32_t sa, uint32_t sb, uint32_t se) {
           // metadata columns alternate between two small tensor-memory buffers from k-block to k-block
           const uint32_t e_base = tmem_base + C::kECol + e_buf * (MBLK * 8);
           e_buf ^= 1u;
@@ -794,20 +811,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                                             ptx::smem_desc(se + j * C::kEBlockBytes + i * 2048, ptx::kLayoutNone, 128));
             }
           }
+          const uint64_t db0 = B_MN ? ptx::smem_desc(sb, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes) : ptx::smem_desc(sb, ptx::kLayoutSw128, 1024);
 #pragma unroll
           for (int j = 0; j < MBLK; ++j) {
             if (j >= live) break;
             const uint32_t d_tmem = tmem_base + (acc * MBLK + j) * BLOCK_N;
             const uint32_t e_tmem = e_base + j * 8;
-            const uint32_t saj = sa + j * C::kABlockBytes;
+            const uint64_t da0 = ptx::smem_desc(sa + j * C::kABlockBytes, ptx::kLayoutSw128, 1024);
 #pragma unroll
             for (int k = 0; k < C::kMmasPerStage; ++k) {
               const uint32_t accumulate = (kb > 0 || k > 0) ? 1u : 0u;
               if (SPARSE) {
                 // 32 bytes of compressed A and 64 bytes of B per instruction
-                uint64_t da = ptx::smem_desc(saj + k * 32, ptx::kLayoutSw128, 1024);
-                uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 1) * b_atom + (k & 1) * 64, ptx::kLayoutSw128, 1024);
+                const uint64_t da = ptx::desc_at(da0, k * 32);
+                const uint64_t db = ptx::desc_at(db0, B_MN ? k * C::kBKStepBytes : (k >> 1) * b_atom + (k & 1) * 64);
                 if (!one_byte_operands(KIND)) {
                   // one 32-bit metadata column per instruction: even-aligned address + selector
                   ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + (k & ~1), idesc | (uint32_t)(k & 1), accumulate);
@@ -815,17 +832,39 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                   ptx::mma_sparse<KIND, CTAS>(d_tmem, da, db, e_tmem + 2 * k, idesc, accumulate);
                 }
               } else {
-                uint64_t da = ptx::smem_desc(saj + (k >> 2) * kBlockM * kAtomBytes + (k & 3) * 32, ptx::kLayoutSw128, 1024);
-                uint64_t db = B_MN ? ptx::smem_desc(sb + k * C::kBKStepBytes, C::kBMnLayout, C::kBMnSbo, C::kBChunkBytes)
-                                   : ptx::smem_desc(sb + (k >> 2) * b_atom + (k & 3) * 32, ptx::kLayoutSw128, 1024);
+                const uint64_t da = ptx::desc_at(da0, (k >> 2) * kBlockM * kAtomBytes + (k & 3) * 32);
+                const uint64_t db = ptx::desc_at(db0, B_MN ? k * C::kBKStepBytes : (k >> 2) * b_atom + (k & 3) * 32);
                 ptx::mma_dense<KIND, CTAS>(d_tmem, da, db, idesc, accumulate);
               }
             }
           }
-          // the stage may be refilled once these MMAs have read it
+        };
+        if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
+        ptx::tc_fence_after();
+        bool ok = true;
+        // the stage may be refilled once its MMAs have read it
+        auto release = [&] {
           if (CTAS == 1) ptx::tc_commit(&sh->empty[stage]);
           else ptx::tc_commit_pair(&sh->empty[stage], 3);
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+        };
+        if (kps == 2) {
+          for (int kb = 0; kb < p.k_blocks; kb += 2) {
+            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
+            ptx::tc_fence_after();
+            const uint32_t sa = ring + stage * slot_bytes, sb = sa + 2 * C::kABytes, se = sb + 2 * b_bytes;
+            multiply(kb, sa, sb, se);
+            if (kb + 1 < p.k_blocks) multiply(kb + 1, sa + C::kABytes, sb + b_bytes, se + C::kEAlloc);
+            release();
+          }
+        } else {
+          for (int kb = 0; kb < p.k_blocks; ++kb) {
+            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
+            ptx::tc_fence_after();
+            const uint32_t sa = ring + stage * slot_bytes;
+            multiply(kb, sa, sa + C::kABytes, sa + C::kABytes + b_bytes);
+            release();
+          }
         }
         if (!ok) break;
         if (CTAS == 1) ptx::tc_commit(&sh->tmem_full[acc]);
@@ -975,13 +1014,19 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
                    cudaStream_t stream) {
   using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   GemmParams p = base;
-  const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
   p.tile_n = tile_n;
   const int cs = elem_bytes(d->cd_type);
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); a staged epilogue gets what is left.
   p.epi_bytes = kEpiWarps * (C::staged_epilogue(cs, p.cd_col_major) ? 4096 : 2048);
-  int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n);
+  const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
+  const uint32_t atom_elems = kAtomBytes / es;
+  const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
+  // Two k-blocks a stage: A in whole 128-byte atoms, four k-blocks at least, and four such stages in the ring (with three
+  // the ring is too coarse, us: bf16 64 x 6592 x 1408 7.0 -> 7.4, 2048 x 1024 x 2048 7.07 -> 7.22).
+  p.kps = C::kPairsOfKBlocks && !p.conv && a_cols % atom_elems == 0 && a_cols / atom_elems >= 4 &&
+                  C::ring_stages(2 * C::stage_bytes(tile_n), p.epi_bytes) >= 4 ? 2 : 1;
+  int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n) * p.kps;
   p.stages = C::ring_stages(ring_bytes, p.epi_bytes);
   if constexpr (is_tall<CTAS, MBLK>) {
     tile_m = p.mblk * kBlockM;
@@ -1007,9 +1052,12 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
   // metadata blocks per 128-row block: 128 columns each (64 for the 1:2 pattern), an even number of them
   p.meta_kb = KIND == 2 ? (int)(2 * ((d->K + 127) / 128)) : (int)(2 * ((d->K + 255) / 256));
   CUtensorMap map_a, map_b, map_e;
-  const uint32_t atom_elems = kAtomBytes / es;
-  const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  sp24_status st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, (is_tall<CTAS, MBLK> ? 1 : MBLK) * kBlockM, 128);
+  sp24_status st;
+  if (p.kps == 2)
+    st = make_map(&map_a, MapShape{A, {atom_elems, (uint64_t)d->M, a_cols / atom_elems}, {(uint64_t)d->lda * es, kAtomBytes},
+                                   {atom_elems, kBlockM, 2}, es, 128});
+  else
+    st = make_map(&map_a, A, es, d->M, a_cols, d->lda * es, atom_elems, (is_tall<CTAS, MBLK> ? 1 : MBLK) * kBlockM, 128);
   if (st != SP24_OK) return st;
   if (p.conv) {
     // B = im2col view of the NHWC activation: boxes of b_rows output pixels x one 128-byte run of channels
@@ -1025,7 +1073,7 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
     // needs the zeros that only the two-dimensional map gives it)
     p.b_3d = 1;
     st = make_map(&map_b, MapShape{B, {atom_elems, (uint64_t)d->N, (uint64_t)d->K / atom_elems},
-                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, b_box_rows, (uint32_t)C::kBBoxes}, es, 128});
+                                   {(uint64_t)d->ldb * es, kAtomBytes}, {atom_elems, b_box_rows, (uint32_t)(C::kBBoxes * p.kps)}, es, 128});
   } else {
     st = make_map(&map_b, B, es, d->N, d->K, d->ldb * es, atom_elems, b_box_rows, 128);
   }
@@ -1033,7 +1081,7 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
   if (SPARSE) {
     // metadata as rows of 128 bytes: 16 * meta_kb of them per 128 rows of A
     st = make_map(&map_e, MapShape{meta, {128, (uint64_t)p.meta_kb * 16, (uint64_t)((d->M + 127) / 128)},
-                                   {128, (uint64_t)p.meta_kb * 2048}, {128, 16 * C::kEBlocks, is_tall<CTAS, MBLK> ? 1 : MBLK}, 1, 0});
+                                   {128, (uint64_t)p.meta_kb * 2048}, {128, (uint32_t)(16 * C::kEBlocks * p.kps), is_tall<CTAS, MBLK> ? 1 : MBLK}, 1, 0});
     if (st != SP24_OK) return st;
   } else {
     map_e = map_a;

@@ -224,6 +224,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t smem_addr, uint32_t layou
   d |= (uint64_t)layout << 61;
   return d;
 }
+// The descriptor `bytes` further on: its address field counts 16-byte units, and no address of the ring carries out of it.
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) {
+  return (desc & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)desc + (bytes >> 4));
+}
 
 // ---- MMA -------------------------------------------------------------------------------------------
 // KIND 0: kind::f16 (fp16 / bf16 operands, fp32 accumulate); KIND 1: kind::i8 (int32 accumulate);

@@ -11,7 +11,7 @@ TORCH = {"bf16": torch.bfloat16, "f16": torch.float16, "f32": torch.float32, "tf
 # less than one block of rows, one column of tiles of every width, widths that leave 16 or 32 columns over, enough
 # tiles for two rounds, pairs of CTAs (M >= 256 with more columns), a K of one and of two k-blocks
 SHAPES = [(16, 16, 64), (160, 48, 288), (256, 256, 512), (320, 1104, 128), (512, 208, 1344), (1184, 736, 1008), (1024, 2080, 256),
-          (2784, 1312, 272)]
+          (2784, 1312, 272), (64, 96, 1408), (304, 64, 2304)]   # (the last two: an odd number of k-blocks, two to a stage)
 
 
 @pytest.fixture(scope="module")
