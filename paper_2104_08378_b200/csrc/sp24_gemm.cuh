@@ -31,6 +31,18 @@ struct FastDiv {
   __host__ __device__ __forceinline__ int operator()(int n) const { return (int)(((uint64_t)(uint32_t)n * mul) >> shift); }
 };
 
+// The owner of a ring of barriers waits, after its last use of them, once for every slot, in the order in which it would use
+// them next and for what it would wait for then: `slot` and `phase` are those of its next use, wait(slot, parity) is its
+// wait for a free slot (at once for one that was never used).  After that nothing is on its way to these barriers.
+template <class Wait>
+__host__ __device__ __forceinline__ bool drain_ring(int slots, int slot, uint32_t phase, Wait wait) {
+  for (int i = 0; i < slots; ++i) {
+    if (!wait(slot, phase ^ 1u)) return false;
+    if (++slot == slots) { slot = 0; phase ^= 1u; }
+  }
+  return true;
+}
+
 struct GemmParams {
   int64_t M, N, K;
   int64_t ldc, ldd;   // elements

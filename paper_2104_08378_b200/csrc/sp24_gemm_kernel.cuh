@@ -781,6 +781,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      // (teardown of a pair: the last commits, which come from CTA 0, have arrived)
+      if (CTAS == 2 && !sh->abort)
+        drain_ring(p.stages, stage, phase, [&](int s, uint32_t parity) {
+          return bounded_wait(&sh->empty[s], parity, sh, p.status, 1u, p.wait_limit);
+        });
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
@@ -871,6 +876,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         else ptx::tc_commit_pair(&sh->tmem_full[acc], 3);
         if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
       }
+      // (teardown of a pair: the last accumulators have been handed back, CTA 1's warps' arrivals among them)
+      if (CTAS == 2 && !sh->abort)
+        drain_ring(C::kAccStages, acc, acc_phase, [&](int a, uint32_t parity) {
+          return bounded_wait(&sh->tmem_empty[a], parity, sh, p.status, 2u, p.wait_limit);
+        });
     }
   } else if (warp >= kFirstEpiWarp) {
     // ------------------------------ epilogue ------------------------------
@@ -992,13 +1002,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   // ------------------------------ teardown ------------------------------
   ptx::tc_fence_before();
   __syncthreads();
-  if (sh->abort) {
-    // copies issued before the abort may still be landing in this CTA's shared memory
-    for (int i = 0; i < 64; ++i) __nanosleep(1000);
-  }
+  // after waits that were given up: copies issued before them, and the other CTA's arrivals, may still be landing in this
+  // CTA's shared memory
+  auto settle = [&] {
+    if (sh->abort)
+      for (int i = 0; i < 64; ++i) __nanosleep(1000);
+  };
+  settle();
   if (CTAS == 2) {
-    // the pair leaves together: nothing arrives at the barriers, or reads the tensor memory, of a CTA that has gone
-    // (every such access has been waited for by then, so the arrival has no memory accesses to order)
+    // The pair leaves together.  The arrival orders no memory accesses, and need not: whatever a CTA sends to the other's
+    // barriers has a waiter there (loads: the issuer; commits and hand-backs: later tiles and, for the last ones,
+    // drain_ring above), and tensor memory has been read once tcgen05.wait::ld returns.
     ptx::cluster_arrive_relaxed();
     ptx::cluster_wait();
   }
@@ -1007,6 +1021,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     ptx::tc_fence_after();
     ptx::tmem_dealloc<CTAS>(tmem_base, kTmemCols);
   }
+  if (CTAS == 2) settle();
 }
 
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
