@@ -946,7 +946,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::tc_fence_after();
       uint32_t r_next[32];
       const uint32_t t_acc = tmem_base + (acc * MBLK) * BLOCK_N + ((uint32_t)(q * 32) << 16);
-      ptx::tmem_ld_32x32b(t_acc + first_it * 32, r_next);
+      // accumulator columns of box `it`
+      auto acc_of = [&](int it) -> uint32_t { return t_acc + (it >= subs ? BLOCK_N + (it - subs) * 32 : it * 32); };
+      if (first_it < iters) ptx::tmem_ld_32x32b(acc_of(first_it), r_next);  // (32 columns, one m-block: one box for two warps)
       bool ok = true;
 #pragma unroll 1
       for (int it = first_it; it < iters; it += split) {
@@ -954,10 +956,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         ptx::tmem_ld_wait(r_next);
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = r_next[e];
-        if (it + split < iters) {
-          const int jn = it + split >= subs, scn = (it + split) - jn * subs;
-          ptx::tmem_ld_32x32b(t_acc + jn * BLOCK_N + scn * 32, r_next);
-        }
+        if (it + split < iters) ptx::tmem_ld_32x32b(acc_of(it + split), r_next);
         int row0, col0;
         if (!box_of(mt, nt, it, row0, col0)) continue;  // same answer for the whole warp
         const int b = seq % nbuf;
