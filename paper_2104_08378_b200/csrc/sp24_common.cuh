@@ -99,6 +99,12 @@ struct RowLaunch {
   }
 };
 
+// The vectorised kernels hold offsets inside a row in 32 bits: of the matrix, and of the metadata in the operand order, where a
+// row's bytes are spread over those of its 128-row block.  Longer rows are for the kernels of any alignment.
+inline bool row_offsets_fit(int64_t K, int es, sp24_meta_layout l) {
+  return (l == SP24_META_TCGEN05 ? (K + 255) / 256 * 4096 : K * es) <= int64_t(1) << 32;
+}
+
 #define SP24_RETURN_IF(cond, code) \
   do {                             \
     if (cond) return (code);       \

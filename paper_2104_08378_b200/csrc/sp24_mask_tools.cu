@@ -410,7 +410,8 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t total = M * (K / 8), KB = 2 * ((K + 255) / 256);
   const int es = elem_bytes(t);
-  if (K % 16 == 0 && aligned16(w) && aligned16(y) && aligned16(meta) && (ldw * es) % 16 == 0 && (ldy * es) % 16 == 0) {
+  if (K % 16 == 0 && aligned16(w) && aligned16(y) && aligned16(meta) && (ldw * es) % 16 == 0 && (ldy * es) % 16 == 0 &&
+      row_offsets_fit(K, es, l)) {
     constexpr int UNROLL = 4;
     const RowLaunch L(K * es / 16, M, UNROLL);
     auto launch = [&](auto kernel) {
