@@ -553,14 +553,14 @@ __global__ void __launch_bounds__(kThreads) compress_f32_kernel(const uint8_t* _
                                                                 int64_t rows_pad, int64_t chunks_pad,
                                                                 unsigned long long* dropped) {
   const uint32_t chunk = blockIdx.x * blockDim.x + threadIdx.x, chunks = (uint32_t)(K >> 3), KB = (uint32_t)(chunks_pad >> 3);
-  const uint32_t moff = HW ? (chunk >> 3) * 2048u + 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * chunk;
+  const int64_t moff = HW ? (int64_t)(chunk >> 3) * 2048 + 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : (int64_t)chunk * 2;
   uint32_t lost = 0;
   for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows_pad;
        row += (int64_t)gridDim.y * blockDim.y) {
     if (chunk >= (uint32_t)chunks_pad) continue;
     uint32_t mbits = 0x4444u;
     if (row < M && chunk < chunks) {
-      const uint8_t* src = x + row * row_bytes_x + chunk * 32u;
+      const uint8_t* src = x + row * row_bytes_x + (int64_t)chunk * 32;
       const uint4 a = ld_stream(src), b = ld_stream(src + 16);
       const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
       uint32_t out[4];
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kThreads) compress_f32_kernel(const uint8_t* _
         mbits |= (sec ? 0xEu : 0x4u) << (4 * g);
         lost += ((sec ? w[2 * g] : w[2 * g + 1]) & 0x7FFFFFFFu) != 0;
       }
-      st_stream(vals + row * row_bytes_v + chunk * 16u, make_uint4(out[0], out[1], out[2], out[3]));
+      st_stream(vals + row * row_bytes_v + (int64_t)chunk * 16, make_uint4(out[0], out[1], out[2], out[3]));
     }
     const uint32_t r = (uint32_t)row & 127u;
     uint8_t* mr = HW ? meta + (row >> 7) * ((int64_t)KB * 2048) + (16u * (r & 7u) + 2u * ((r >> 3) & 1u) + 256u * (r >> 4))
@@ -589,13 +589,13 @@ __global__ void __launch_bounds__(kThreads) decompress_f32_kernel(const uint8_t*
                                                                   int64_t chunks_pad) {
   const uint32_t chunk = blockIdx.x * blockDim.x + threadIdx.x, chunks = (uint32_t)(K >> 3), KB = (uint32_t)(chunks_pad >> 3);
   if (chunk >= chunks) return;
-  const uint32_t moff = HW ? (chunk >> 3) * 2048u + 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * chunk;
+  const int64_t moff = HW ? (int64_t)(chunk >> 3) * 2048 + 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : (int64_t)chunk * 2;
   for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < M; row += (int64_t)gridDim.y * blockDim.y) {
     const uint32_t r = (uint32_t)row & 127u;
     const uint8_t* mr = HW ? meta + (row >> 7) * ((int64_t)KB * 2048) + (16u * (r & 7u) + 2u * ((r >> 3) & 1u) + 256u * (r >> 4))
                            : meta + row * (K >> 2);
     const uint32_t mbits = *reinterpret_cast<const uint16_t*>(mr + moff);
-    const uint4 v = ld_stream(vals + row * row_bytes_v + chunk * 16u);
+    const uint4 v = ld_stream(vals + row * row_bytes_v + (int64_t)chunk * 16);
     const uint32_t in[4] = {v.x, v.y, v.z, v.w};
     uint32_t w[8];
 #pragma unroll
@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(kThreads) decompress_f32_kernel(const uint8_t*
       w[2 * g] = sec ? 0u : in[g];
       w[2 * g + 1] = sec ? in[g] : 0u;
     }
-    uint8_t* dst = y + row * row_bytes_y + chunk * 32u;
+    uint8_t* dst = y + row * row_bytes_y + (int64_t)chunk * 32;
     st_stream(dst, make_uint4(w[0], w[1], w[2], w[3]));
     st_stream(dst + 16, make_uint4(w[4], w[5], w[6], w[7]));
   }
@@ -662,7 +662,8 @@ extern "C" sp24_status sp24_prune(sp24_dtype t, int64_t M, int64_t K, const void
   if ((st = check_arch()) != SP24_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int es = elem_bytes(t), f8 = is_fp8(t) ? 1 : 0;
-  const bool vec = aligned16(x) && aligned16(y) && (ldx * es) % 16 == 0 && (ldy * es) % 16 == 0 && (K * es) % 16 == 0;
+  const bool vec = aligned16(x) && aligned16(y) && (ldx * es) % 16 == 0 && (ldy * es) % 16 == 0 && (K * es) % 16 == 0 &&
+                   row_offsets_fit(K, es, SP24_META_CANONICAL);
   if (vec) {
     constexpr int UNROLL = 4;
     int64_t vpr = K * es / 16, rows = M;
@@ -724,7 +725,7 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
   const int64_t rows_pad = hw ? (M + 127) / 128 * 128 : M;
   const int64_t k_pad = hw ? (K + 255) / 256 * 256 : K;
   const bool vec = K % 16 == 0 && aligned16(x) && aligned16(vals) && aligned16(meta) && (ldx * es) % 16 == 0 &&
-                   (ldv * es) % (8 * es) == 0;
+                   (ldv * es) % (8 * es) == 0 && row_offsets_fit(K, es, l);
   if (vec) {
     constexpr int UNROLL = 4;
     const int64_t chunks_pad = k_pad / 16;

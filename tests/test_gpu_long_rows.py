@@ -55,3 +55,35 @@ def test_apply_mask(dtype, K, layout):
     for c in range(0, K, BLOCK):
         kept = keep[row[c // 8:(c + BLOCK) // 8].long()].view(-1)
         assert torch.equal(_bits(got)[0, c:c + BLOCK], torch.where(kept, _bits(w)[0, c:c + BLOCK], 0)), c
+
+
+@pytest.mark.parametrize("dtype,K,layout", [("bf16", 2**28 + 4096, 1), ("e5m2", 2**28 + 4096, 1), ("i8", 2**32 + 4096, 0)])
+def test_prune_and_compress(dtype, K, layout):
+    """One long row is, group by group, the matrix of its pieces: values, canonical metadata and pruned matrix of both are the
+    same bytes in the same order, and the operand order holds the same bits."""
+    from paper_2104_08378_b200 import binding as sp
+    x = _matrix(dtype, K, torch.Generator(device="cuda").manual_seed(42))
+    pieces = x.view(-1, 4096)
+    want_pruned, want_vals, want_meta, want_dropped = sp.prune_compress(pieces, layout=sp.META_CANONICAL, count_dropped=True)
+    vals, meta, dropped = sp.compress(x, layout=layout, count_dropped=True)
+    for v, m, d in ((vals, meta, dropped), sp.prune_compress(x, layout=layout, count_dropped=True)[1:]):
+        assert torch.equal(_bits(v).view(-1), _bits(want_vals).view(-1)) and torch.equal(d, want_dropped)
+        if layout == sp.META_CANONICAL:
+            assert torch.equal(m.view(-1), want_meta.view(-1))
+        else:
+            blocks, at = _first_row(m, x.element_size())
+            assert torch.equal(blocks[:, at], want_meta.view(torch.int16).view(-1, 8))
+            assert (blocks[:, [i + 8 for i in at]] == 0x4444).all()              # row 1: padding
+    assert torch.equal(_bits(sp.prune(x)).view(-1), _bits(want_pruned).view(-1))
+    assert torch.equal(_bits(sp.decompress(vals, meta, layout=layout)).view(-1), _bits(want_pruned).view(-1))
+
+
+def test_pairs_of_float32():
+    from paper_2104_08378_b200 import binding as sp
+    K = 2**27 + 4096                     # the operand order of the 1:2 pattern: 64 columns to a 2048-byte block
+    x = torch.randn((1, K), device="cuda", generator=torch.Generator(device="cuda").manual_seed(43))
+    want_vals, want_meta, _ = sp.compress(x.view(-1, 4096), layout=sp.META_CANONICAL)
+    vals, meta, _ = sp.compress(x)
+    blocks, at = _first_row(meta, 2)
+    assert torch.equal(vals.view(-1), want_vals.view(-1)) and torch.equal(blocks[:, at], want_meta.view(torch.int16).view(-1, 8))
+    assert torch.equal(sp.decompress(vals, meta).view(-1), sp.prune(x.view(-1, 4096)).view(-1))
