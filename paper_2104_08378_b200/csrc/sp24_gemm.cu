@@ -258,7 +258,8 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& cta
 // 170 random problems (256..16384 rows, 160..16384 columns, K 256..12288, every kind, with and without C), 11 to 17
 // shapes of each; mean error 5 to 10 % per shape.
 static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n) {
-  const int es = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
+  const int bytes = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
+  const int es = bytes > 0 ? bytes : 1;  // (a type that no product takes may still ask for its plan)
   const double k_blocks = (double)((d->K * es + 255) / 256);
   const int64_t rows = 128 * ctas * mblk, slots = sm_count() / ctas > 0 ? sm_count() / ctas : 1;
   const int64_t tiles = ((d->M + rows - 1) / rows) * ((d->N + tile_n - 1) / tile_n);

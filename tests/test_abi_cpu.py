@@ -109,3 +109,16 @@ def test_the_binding_imports_without_the_cuda_parts_of_torch():
         "assert sp.gemm_plan(sp.make_desc('bf16', 'bf16', 0, 32, 64, 32, 64, 32, 32)) is None\n")
     done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert "Sp24Error" in done.stderr and "status 3" in done.stderr, done.stderr
+
+
+def test_a_plan_for_types_that_no_product_takes():
+    """sp24_gemm_plan does not look at the types: one it does not know gets a plan too, whatever the orders."""
+    code = (
+        "from paper_2104_08378_b200 import binding as sp\n"
+        "for order_b in (sp.ROW_MAJOR, sp.COL_MAJOR):\n"
+        "    for ab in (99, sp.I32):\n"
+        "        for N in (96, 512):\n"
+        "            print(sp.gemm_plan(sp.GemmDesc(ab, 99, 256, N, 512, 256, 512, N, N, order_b, 0, 0, 0)))\n")
+    done = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    plans = done.stdout.split()    # (single CTAs; how many blocks each takes depends on the SMs)
+    assert done.returncode == 0 and len(plans) == 8 and all(p.startswith("1x128x") for p in plans), (done, plans)
