@@ -30,6 +30,9 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // The current device must be a compute-capability 10.x part; the answer is cached per device.
 sp24_status check_arch();
 
+// SMs of the current device, cached per device (1 if there is none).
+int sm_count();
+
 // The status of a runtime call.  A call that fails also leaves its code behind as the thread's last error, which the
 // plain launches read back with cudaGetLastError(): cleared here, so that only the call that failed reports it.
 inline sp24_status cuda_status(cudaError_t e) {

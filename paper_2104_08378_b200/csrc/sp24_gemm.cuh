@@ -18,7 +18,7 @@ constexpr int kNumThreads = 32 * (kFirstEpiWarp + kEpiWarps);
 constexpr long long kWaitTimeoutCycles = 2000ll * 1000ll * 1000ll;  // per wait: 1-2 s of SM clock
 constexpr uint32_t kTmemCols = 512;
 
-// n / d for n < 2^31 by a multiplication: mul / 2^(31 + log) is 1 / d rounded up, by less than 2^-31 / d, with 2^log the
+// n / d for n < 2^31 by a multiplication (Granlund and Montgomery, Division by Invariant Integers using Multiplication): mul / 2^(31 + log) is 1 / d rounded up, by less than 2^-31 / d, with 2^log the
 // first power of two >= d.  (A division by a divisor known only at run time takes the device about 150 cycles, and the
 // first load of a call waits for two.)
 struct FastDiv {
@@ -102,7 +102,6 @@ inline sp24_status make_map(CUtensorMap* map, const void* base, int es, uint64_t
 }
 sp24_status make_im2col_map(CUtensorMap* map, const void* x, int es, uint64_t nb, uint64_t h, uint64_t w, uint64_t c,
                             uint32_t channels_per_box, uint32_t pixels_per_box);
-int sm_count();
 
 // ---- in sp24_gemm_{f16,i8,tf32,f8}.cu --------------------------------------------------------------
 // One launch of the kernel for MMA kind KIND (0 = f16 / bf16, 1 = int8, 2 = tf32, 3 = 8-bit floating point (e4m3 /

@@ -731,13 +731,14 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
     const int64_t chunks_pad = k_pad / 16;
     const int64_t units = es == 2 ? chunks_pad * 2 : chunks_pad;  // 16-byte vectors per padded row
     RowLaunch L(units, rows_pad, UNROLL);
-    // What fits the L2 with its result is bound by instructions, a tenth of them a block's tables: 8 blocks an SM take all
-    // rows.  What does not is bound by HBM and wants the loads of all its blocks in flight.  Us, device, a block for every
-    // row step against 8 an SM: compress bf16 12288 x 3072 (118 MB in all) 19.9, 17.3; 49152 x 1024 (157 MB) 25.5, 22.5;
-    // 49152 x 12288 (1.9 GB) 323, 369; fused with prune bf16 16102 x 1088 (92 MB) 17.1, 14.9; 12288 x 3072 (193 MB) 30.3, 32.8;
-    // int8 49152 x 1024 (132 MB) 28.4, 25.7.
+    // A matrix of moderate size is bound by instructions, a tenth of them a block's tables: 8 blocks an SM take all rows.  A
+    // large one is bound by HBM and wants the loads of all its blocks in flight.  The line, 160 MB of traffic, lies between
+    // what was measured on either side of it (it is not the L2's 126 MB).  Us, device, a block for every row step against 8
+    // an SM: compress bf16 12288 x 3072 (118 MB in all) 19.9, 17.3; 49152 x 1024 (157 MB) 25.5, 22.5; 49152 x 12288 (1.9 GB)
+    // 323, 369; fused with prune bf16 16102 x 1088 (92 MB) 17.1, 14.9; 12288 x 3072 (193 MB) 30.3, 32.8; int8 49152 x 1024
+    // (132 MB) 28.4, 25.7.
     const int64_t moved = M * K * es * (y ? 5 : 3) / 2 + M * K / 8;
-    const unsigned few = (148 * 8 + L.grid.x - 1) / L.grid.x;
+    const unsigned few = (8 * (unsigned)sm_count() + L.grid.x - 1) / L.grid.x;
     if (moved <= (int64_t)160 << 20 && L.grid.y > few) L.grid.y = few;
     const bool full = rows_pad == M && k_pad == K && units % ((int64_t)L.block.x * UNROLL) == 0;
     const int variant = (y ? 8 : 0) | (dropped ? 4 : 0) | (hw ? 2 : 0) | (full ? 1 : 0);
