@@ -98,8 +98,15 @@ struct Cfg {
   static constexpr int kAccStages = MBLK >= 2 ? 1 : ((2 * BLOCK_N + (SPARSE ? 32 : 0) <= (int)kTmemCols) ? 2 : 1);
   static constexpr int kECol = kAccStages * MBLK * BLOCK_N;        // first metadata column in tensor memory
   static constexpr int kMmasPerStage = SPARSE ? 4 : 4 * kBBoxes;   // per m-block and k-block
-  // Stages of two k-blocks (p.kps; see the producer)
+  // Stages of two k-blocks (p.kps; see the producer): A in whole 128-byte atoms, four k-blocks at least, and four such stages
+  // in the ring (with three the ring is too coarse, us: bf16 64 x 6592 x 1408 7.0 -> 7.4, 2048 x 1024 x 2048 7.07 -> 7.22).
+  // That is 16-bit and TF32 tiles of 32 columns, of 64 in a pair without a staged epilogue; 8-bit kinds, whose metadata is
+  // twice as long, only in pairs of 32 columns.
   static constexpr bool kPairsOfKBlocks = SPARSE && !B_MN && MBLK == 1;
+  static constexpr int k_blocks_of_a_stage(int tile_n, int staging, int64_t a_cols, bool conv) {
+    return kPairsOfKBlocks && !conv && a_cols % kAtomElems == 0 && a_cols / kAtomElems >= 4 &&
+                   ring_stages(2 * stage_bytes(tile_n), staging) >= 4 ? 2 : 1;
+  }
   static constexpr int kSmemBytes = 232448;  // always the whole opt-in maximum
   static_assert(ring_stages(stage_bytes(BLOCK_N), kEpiWarps * 2048) >= 2, "need at least two stages");
   // the epilogue moves 32-column boxes; a last box of 16 columns (240-column tiles) is handled only by
@@ -691,10 +698,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // ------------------------------ TMA producer ------------------------------
     if (ptx::elect_one()) {
       // The thread that issues the loads needs about 390 cycles for a stage whatever its bytes (170 to look at the ring,
-      // 215 to issue three loads), more than the MMAs of a narrow tile take: its stages hold two k-blocks each, which
-      // are loaded by as many loads as one.  One k-block a stage and two, us, device: bf16 512 x 512 x 8192 16.0, 13.1;
-      // 4096 x 32 x 4096 9.1, 7.8; int8 4096 x 32 x 4096 6.0, 5.4.  Loops of their own: with the number of k-blocks as a
-      // variable of one loop, products with one a stage were up to 15 % slower.
+      // 215 to issue three loads), more than the MMAs of a narrow tile take: its stages hold two k-blocks each where the
+      // ring has room (k_blocks_of_a_stage), which are loaded by as many loads as one.  One k-block a stage and two, us,
+      // device: bf16 512 x 512 x 8192 16.0, 13.1; 4096 x 32 x 4096 9.1, 7.8.  Loops of their own: with the number of k-blocks
+      // as a variable of one loop, products with one a stage were up to 15 % slower.
       // (Shared-memory and barrier addresses as plain integers, as few loads per stage as the boxes allow: the
       // thread that issues them is busy for about 100 cycles per load, which delays the refill of a stage.
       // Three loads instead of six (two m-blocks) or four: 49152 x 32 x 12288 bf16 123.1 -> 119.6 us, int8
@@ -1036,10 +1043,7 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
   const uint32_t atom_elems = kAtomBytes / es;
   const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  // Two k-blocks a stage: A in whole 128-byte atoms, four k-blocks at least, and four such stages in the ring (with three
-  // the ring is too coarse, us: bf16 64 x 6592 x 1408 7.0 -> 7.4, 2048 x 1024 x 2048 7.07 -> 7.22).
-  p.kps = C::kPairsOfKBlocks && !p.conv && a_cols % atom_elems == 0 && a_cols / atom_elems >= 4 &&
-                  C::ring_stages(2 * C::stage_bytes(tile_n), p.epi_bytes) >= 4 ? 2 : 1;
+  p.kps = C::k_blocks_of_a_stage(tile_n, p.epi_bytes, (int64_t)a_cols, p.conv != 0);
   int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n) * p.kps;
   p.stages = C::ring_stages(ring_bytes, p.epi_bytes);
   if constexpr (is_tall<CTAS, MBLK>) {

@@ -8,10 +8,21 @@ pytestmark = pytest.mark.gpu
 
 TORCH = {"bf16": torch.bfloat16, "f16": torch.float16, "f32": torch.float32, "tf32": torch.float32, "i32": torch.int32,
          "e4m3": torch.float8_e4m3fn, "e5m2": torch.float8_e5m2}
-# less than one block of rows, one column of tiles of every width, widths that leave 16 or 32 columns over, enough
-# tiles for two rounds, pairs of CTAs (M >= 256 with more columns), a K of one and of two k-blocks
+# less than one block of rows, widths that leave 16 or 32 columns over, enough tiles for two rounds, a K of one and of two
+# k-blocks ...
 SHAPES = [(16, 16, 64), (160, 48, 288), (256, 256, 512), (320, 1104, 128), (512, 208, 1344), (1184, 736, 1008), (1024, 2080, 256),
-          (2784, 1312, 272), (64, 96, 1408), (304, 64, 2304)]   # (the last two: an odd number of k-blocks, two to a stage)
+          (2784, 1312, 272), (64, 96, 1408), (304, 64, 2304)]
+# ... and those that, with them, take every width of single CTAs and of pairs in every kind and order of B, and, two k-blocks
+# to a stage, an odd and an even number of them (test_tile_choice_cpu.py)
+SHAPES += [(800, 704, 320), (320, 3744, 288), (448, 3616, 288), (2464, 960, 288), (1376, 2048, 288), (3744, 832, 288),
+           (288, 3520, 1120), (3392, 1280, 288), (320, 1632, 1376), (2784, 1568, 288), (128, 32, 1152), (576, 3168, 320),
+           (832, 768, 768), (3168, 192, 896), (2336, 2816, 288), (448, 1216, 832)]
+KINDS = [("bf16", "bf16"), ("f16", "f32"), ("tf32", "f32"), ("e4m3", "bf16"), ("e5m2", "f32"), ("i8", "i32")]
+
+
+def shapes(kind):
+    unit = 32 if kind in ("e4m3", "e5m2", "i8") else 16
+    return [tuple((v + unit - 1) // unit * unit for v in shape) for shape in SHAPES]
 
 
 @pytest.fixture(scope="module")
@@ -27,13 +38,11 @@ def _matrix(kind, rows, cols, g, pad):
 
 
 @pytest.mark.parametrize("b_rows", [False, True])
-@pytest.mark.parametrize("kind,cd", [("bf16", "bf16"), ("f16", "f32"), ("tf32", "f32"), ("e4m3", "bf16"), ("e5m2", "f32"), ("i8", "i32")])
+@pytest.mark.parametrize("kind,cd", KINDS)
 def test_same_bits_as_128_columns(sp, force_tile, kind, cd, b_rows):
-    unit = 32 if kind in ("e4m3", "e5m2", "i8") else 16
     g = torch.Generator(device="cuda")
     g.manual_seed(11)
-    for M, N, K in SHAPES:
-        M, N, K = ((v + unit - 1) // unit * unit for v in (M, N, K))
+    for M, N, K in shapes(kind):
         for dense in (False, True):
             A, x = _matrix(kind, M, K, g, 0), _matrix(kind, *((K, N) if b_rows else (N, K)), g, 32)
             vals, meta = (A, None) if dense else sp.compress(A)[:2]

@@ -24,10 +24,12 @@ def fault_hooks(sp):
     sp.set_fault_hooks(0, False)
 
 
-@pytest.mark.parametrize("tile", ["1x128x1", "2x224x1", "2x224x2"])
-def test_expired_wait_is_reported_and_the_context_stays_usable(sp, force_tile, fault_hooks, tile):
+# (None: the library's own choice, 32 columns and 64 columns of a pair, with stages of two k-blocks)
+@pytest.mark.parametrize("tile,M,N", [("1x128x1", 512, 448), ("2x224x1", 512, 448), ("2x224x2", 512, 448), (None, 512, 448),
+                                      (None, 448, 1216)])
+def test_expired_wait_is_reported_and_the_context_stays_usable(sp, force_tile, fault_hooks, tile, M, N):
     torch.manual_seed(3)
-    M, N, K = 512, 448, 1024
+    K = 1024
     A = (torch.randn(M, K, device="cuda") * 0.1).bfloat16()
     Bt = torch.randn(N, K, device="cuda").bfloat16()
     vals, meta, _ = sp.compress(A)
