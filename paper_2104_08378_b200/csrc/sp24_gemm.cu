@@ -256,7 +256,8 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& cta
 // k-blocks (a fixed part and one per column, the same for all kinds: a k-block is 256 bytes of K), then the epilogue of a
 // tile by its columns (4-byte results and C cost more; 256-column tiles and two m-blocks cannot overlap it).  Fitted to
 // 170 random problems (256..16384 rows, 160..16384 columns, K 256..12288, every kind, with and without C), 11 to 17
-// shapes of each; mean error 5 to 10 % per shape.
+// shapes of each, before stages held two k-blocks: it puts bf16 512 x 512 x 8192 at 16.5 us, which now takes 13.1.  On 100
+// other problems of the same ranges the mean error of today's kernels is 9 to 13 % per shape, 16 % for two m-blocks.
 static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n) {
   const int bytes = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
   const int es = bytes > 0 ? bytes : 1;  // (a type that no product takes may still ask for its plan)
@@ -278,8 +279,8 @@ static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block
 // tiles is faster with narrower ones on more of them (us, device: f16 256 x 256 x 512 4.10 -> 3.23, f16 1184 x 736 x 1008
 // with C 7.6 -> 5.8, int8 992 x 480 x 6176 14.9 -> 9.5, bf16 512 x 192 x 10464 31.2 -> 19.8).  Over 150 other random
 // problems the choice below is 17 % faster in the mean than the widest tiles, one is slower by more than 2 % (int8 128 x
-// 3808 x 352 4.5 -> 4.7 us); over the 170 above it is 1.5 % behind the best of the shapes.  A pair keeps its shape, or its
-// two m-blocks, unless the estimate says 3 %, or 15 %: what it is wrong by.
+// 3808 x 352 4.5 -> 4.7 us); it is 1.5 % behind the best of the shapes over the 170 above, 2.3 % (at worst 22 %) over the 100.
+// A pair keeps its shape unless the estimate says 3 %, its two m-blocks unless it says 15 %: it puts those 12 % too high.
 static void choose_width(const sp24_gemm_desc* d, bool has_c, int& ctas, int& block_n, int& mblk, int& tile_n) {
   const int64_t n32 = (d->N + 31) / 32 * 32;
   auto widest = [&](int bn) { return n32 < bn ? (int)n32 : bn; };

@@ -1018,7 +1018,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   if (CTAS == 2) {
     // The pair leaves together.  The arrival orders no memory accesses, and need not: whatever a CTA sends to the other's
     // barriers has a waiter there (loads: the issuer; commits and hand-backs: later tiles and, for the last ones,
-    // drain_ring above), and tensor memory has been read once tcgen05.wait::ld returns.
+    // drain_ring above), and tensor memory has been read once tcgen05.wait::ld returns.  (With release instead of the issuer's
+    // drain it also waits for D's stores: BERT FFN 12.4 against 12.1 us, device; large products the same.)
     ptx::cluster_arrive_relaxed();
     ptx::cluster_wait();
   }
