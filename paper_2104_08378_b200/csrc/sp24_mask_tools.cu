@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kThreads) kept_magnitude_perm_kernel(const uin
 
 // ---- apply mask -----------------------------------------------------------------------------------
 // Vector path.  Work unit: one 16-byte vector (two groups of a 16-bit type = one metadata byte, four of an 8-bit type =
-// two bytes); launch geometry, unrolling and metadata addresses as in compress16_kernel / compress8_kernel.  A metadata
+// two bytes); launch geometry and unrolling as in prune_vec_kernel, metadata addresses as in compress_kernel.  A metadata
 // nibble indexes a table of byte-permute selectors that copy the two positions it names and zero the others.
 // Bound by HBM.  The result is stored without an evict-first hint: it is compressed next, and as much of it as fits is then
 // read from the L2.  One chunk of 16 columns per thread, metadata decoded by arithmetic and evict-first stores before; us, device,

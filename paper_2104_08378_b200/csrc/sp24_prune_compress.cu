@@ -28,25 +28,8 @@ __device__ __forceinline__ uint32_t mask_to_nibble(uint32_t mask) {
   return p0 | (p1 << 2);
 }
 
-// Which of a group's four 16-bit values (two words: lo = elements 0,1; hi = elements 2,3) are non-zero.
-struct Group16 {
-  static __device__ __forceinline__ uint32_t nonzero(uint32_t lo, uint32_t hi) {
-    return ((lo & 0x7FFFu) != 0) | (((lo >> 16) & 0x7FFFu) != 0) << 1 | ((hi & 0x7FFFu) != 0) << 2 |
-           (((hi >> 16) & 0x7FFFu) != 0) << 3;
-  }
-};
-
-// Which of a group's four int8 values (one word) are non-zero.
-struct Group8 {
-  static __device__ __forceinline__ uint32_t nonzero(uint32_t w) {
-    return ((w & 0xFFu) != 0) | ((w & 0xFF00u) != 0) << 1 | ((w & 0xFF0000u) != 0) << 2 |
-           ((w & 0xFF000000u) != 0) << 3;
-  }
-};
-
-// Magnitude keys of 8-bit elements: |x| for int8 (-128 -> 0x80 = 128, no saturation), the seven
+// Magnitude key of an 8-bit element: |x| for int8 (-128 -> 0x80 = 128, no saturation), the seven
 // bits below the sign for the 8-bit floating-point types (`f8` != 0).
-__device__ __forceinline__ uint32_t keys8(uint32_t w, int f8) { return f8 ? (w & 0x7F7F7F7Fu) : __vabs4(w); }
 __device__ __forceinline__ uint32_t key8(uint32_t e, int f8) { return f8 ? (e & 0x7Fu) : (uint32_t)abs((int)(int8_t)e); }
 
 __device__ __forceinline__ uint4 ld_stream(const void* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
@@ -91,136 +74,129 @@ __device__ __forceinline__ int64_t meta_offset(int layout, int64_t row, int64_t 
   return blk * 2048 + in_blk;
 }
 
-// ---- compress (fused prune + compress) ----------------------------------------------------
-// The domain is padded (rows to rows_pad, 16-column chunks to chunks_pad) so that the operand-
-// order layout gets its 0x4 padding nibbles from the same launch.  Every thread issues all of
-// its loads before it consumes any of them.
-//
-// Selection by table: the six comparisons of a group are made two at a time on packed 15-bit
-// keys -- ((a | 0x8000) - b) has bit 15 set iff a >= b, and two such differences fit one 32-bit
-// subtraction without a borrow between the halves -- and their six result bits index a 64-entry
-// table in shared memory that holds, per outcome, the metadata nibble, the keep mask and the
-// byte-permute selectors that gather the two kept values.
-__device__ __forceinline__ uint32_t selection_entry(uint32_t idx) {
-  // idx bits: 0 = c01, 1 = c03, 2 = c02, 3 = c23, 4 = c12, 5 = c13   (cab: key[a] >= key[b])
-  uint32_t c01 = idx & 1, c03 = (idx >> 1) & 1, c02 = (idx >> 2) & 1;
-  uint32_t c23 = (idx >> 3) & 1, c12 = (idx >> 4) & 1, c13 = (idx >> 5) & 1;
-  uint32_t b0 = 3u - (c01 + c02 + c03), b1 = c01 + 2u - (c12 + c13);
-  uint32_t b2 = c02 + c12 + 1u - c23, b3 = c03 + c13 + c23;
-  uint32_t mask = (b0 < 2u) | ((b1 < 2u) << 1) | ((b2 < 2u) << 2) | ((b3 < 2u) << 3);
-  if (__popc(mask) != 2) mask = 3;  // comparison outcomes no real keys can produce
-  uint32_t p0 = __ffs(mask) - 1, p1 = 31 - __clz(mask);
-  uint32_t sel8 = p0 | (p1 << 4);                                                // bytes p0, p1 of a word
-  uint32_t sel16 = (2 * p0) | ((2 * p0 + 1) << 4) | ((2 * p1) << 8) | ((2 * p1 + 1) << 12);  // halves p0, p1 of a pair
-  return (p0 | (p1 << 2)) | (mask << 4) | (sel8 << 8) | (sel16 << 16);
+// ---- selection of the vector kernels ------------------------------------------------------
+// A 16-byte vector is transposed so that word i holds element i of all its groups (two in 16-bit lanes, four in 8-bit
+// ones): each of the six comparisons is then one subtraction for all groups, whose result is the lane's top bit, and what
+// follows is logic on those bits.  No table: with one in shared memory, indexed by the six bits, a vector took 88
+// instructions and the look-ups met in the banks; it takes 57 with the kept values gathered by lane masks and about 40 now
+// that the bits are turned into byte-permute selectors by dot products, which run beside the ALU pipe (16-bit types).
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {  // __byte_perm with the selectors that copy a sign
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
 }
 
-__device__ __forceinline__ void build_selection_table(uint32_t* table) {
-  int t = threadIdx.y * blockDim.x + threadIdx.x;
-  if (t < 64) table[t] = selection_entry((uint32_t)t);
-  __syncthreads();
-}
-
-// k_lo = [key0, key1], k_hi = [key2, key3] as 16-bit lanes, every key < 2^15.
-__device__ __forceinline__ uint32_t selection_index(uint32_t k_lo, uint32_t k_hi) {
-  const uint32_t g = 0x80008000u;
-  uint32_t r1 = (k_lo | g) - k_hi;                              // bit 15: c02, bit 31: c13
-  uint32_t r2 = (k_lo | g) - __byte_perm(k_hi, 0, 0x1032);      // bit 15: c03, bit 31: c12
-  uint32_t r3 = (__byte_perm(k_lo, k_hi, 0x5410) | g) - __byte_perm(k_lo, k_hi, 0x7632);  // bit 15: c01, 31: c23
-  uint32_t t = (r1 & g) | ((r2 & g) >> 1) | ((r3 & g) >> 2);    // bits 15..13: c02 c03 c01, 31..29: c13 c12 c23
-  return ((t >> 13) & 7u) | ((t >> 26) & 0x38u);
-}
-
-// 16-bit types: the table indices of the two groups of one 16-byte vector at once.  lo/hi are the masked
-// key words of group 0 (k0k1, k2k3) and group 1; word p of the transposed form holds key p of both groups,
-// so each of the six comparisons is one subtraction for the two groups.
-__device__ __forceinline__ void selection_index_x2(uint32_t lo0, uint32_t hi0, uint32_t lo1, uint32_t hi1,
-                                                   uint32_t& idx0, uint32_t& idx1) {
-  const uint32_t p0 = __byte_perm(lo0, lo1, 0x5410), p1 = __byte_perm(lo0, lo1, 0x7632);
-  const uint32_t p2 = __byte_perm(hi0, hi1, 0x5410), p3 = __byte_perm(hi0, hi1, 0x7632);
-  const uint32_t g = 0x80008000u;
-  const uint32_t c01 = ((p0 | g) - p1) & g, c02 = ((p0 | g) - p2) & g, c03 = ((p0 | g) - p3) & g;
-  const uint32_t c12 = ((p1 | g) - p2) & g, c13 = ((p1 | g) - p3) & g, c23 = ((p2 | g) - p3) & g;
-  const uint32_t x = (c01 >> 15) | (c03 >> 14) | (c02 >> 13) | (c23 >> 12) | (c12 >> 11) | (c13 >> 10);
-  idx0 = x & 0xFFFFu;
-  idx1 = x >> 16;
-}
-
-// 8-bit types: the table indices of the four groups of one 16-byte vector at once.  a[g] holds the four
-// keys of group g, one per byte.  With all keys below 128 the keys are transposed (word p = key p of
-// the four groups) and each of the six comparisons is one byte-wise subtraction with a guard bit,
-// ((x | 0x80) - y) bit 7 = (x >= y); the six flag words are merged into one index byte per group.  A
-// key of 128 (int8 -128) does not fit the guard trick: such a vector takes the group-by-group path.
-__device__ __forceinline__ void selection_index_x4(const uint32_t (&a)[4], uint32_t (&idx)[4]) {
-  if ((a[0] | a[1] | a[2] | a[3]) & 0x80808080u) {
-#pragma unroll
-    for (int g = 0; g < 4; ++g) idx[g] = selection_index(__byte_perm(a[g], 0, 0x4140), __byte_perm(a[g], 0, 0x4342));
-    return;
+template <int ES>
+__device__ __forceinline__ void transpose(uint4 w, uint32_t (&p)[4]) {
+  if constexpr (ES == 2) {
+    p[0] = prmt(w.x, w.z, 0x5410); p[1] = prmt(w.x, w.z, 0x7632); p[2] = prmt(w.y, w.w, 0x5410); p[3] = prmt(w.y, w.w, 0x7632);
+  } else {
+    const uint32_t t0 = prmt(w.x, w.y, 0x5140), t1 = prmt(w.z, w.w, 0x5140), t2 = prmt(w.x, w.y, 0x7362), t3 = prmt(w.z, w.w, 0x7362);
+    p[0] = prmt(t0, t1, 0x5410); p[1] = prmt(t0, t1, 0x7632); p[2] = prmt(t2, t3, 0x5410); p[3] = prmt(t2, t3, 0x7632);
   }
-  const uint32_t t0 = __byte_perm(a[0], a[1], 0x5140), t1 = __byte_perm(a[2], a[3], 0x5140);
-  const uint32_t t2 = __byte_perm(a[0], a[1], 0x7362), t3 = __byte_perm(a[2], a[3], 0x7362);
-  const uint32_t p0 = __byte_perm(t0, t1, 0x5410), p1 = __byte_perm(t0, t1, 0x7632);
-  const uint32_t p2 = __byte_perm(t2, t3, 0x5410), p3 = __byte_perm(t2, t3, 0x7632);
-  const uint32_t g = 0x80808080u;
-  const uint32_t c01 = ((p0 | g) - p1) & g, c02 = ((p0 | g) - p2) & g, c03 = ((p0 | g) - p3) & g;
-  const uint32_t c12 = ((p1 | g) - p2) & g, c13 = ((p1 | g) - p3) & g, c23 = ((p2 | g) - p3) & g;
-  // index bits: 0 = c01, 1 = c03, 2 = c02, 3 = c23, 4 = c12, 5 = c13 (see selection_entry); byte g of x = group g
-  const uint32_t x = (c01 >> 7) | (c03 >> 6) | (c02 >> 5) | (c23 >> 4) | (c12 >> 3) | (c13 >> 2);
-  idx[0] = x & 0xFFu;
-  idx[1] = (x >> 8) & 0xFFu;
-  idx[2] = (x >> 16) & 0xFFu;
-  idx[3] = x >> 24;
+}
+template <int ES>
+__device__ __forceinline__ uint4 transpose_back(const uint32_t (&p)[4]) {
+  if constexpr (ES == 2)
+    return make_uint4(prmt(p[0], p[1], 0x5410), prmt(p[2], p[3], 0x5410), prmt(p[0], p[1], 0x7632), prmt(p[2], p[3], 0x7632));
+  const uint32_t a = prmt(p[0], p[1], 0x5140), b = prmt(p[2], p[3], 0x5140), c = prmt(p[0], p[1], 0x7362), d = prmt(p[2], p[3], 0x7362);
+  return make_uint4(prmt(a, b, 0x5410), prmt(a, b, 0x7632), prmt(c, d, 0x5410), prmt(c, d, 0x7632));
+}
+
+// The selection of a transposed vector.  (Top bit of each lane; the others are not defined.)
+template <int ES>
+struct Selection {
+  static constexpr uint32_t kTop = ES == 2 ? 0x80008000u : 0x80808080u;
+  uint32_t key[4];   // magnitudes (16-bit types: below the top bit; 8-bit types: 0..128)
+  uint32_t kept[4];  // is position i kept
+  // Position 0 is kept if it beats two of the others, and so on (see keep_mask4).
+  static __device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (a & c) | (b & c); }
+  // a >= b: with a's top bit set no lane borrows from the next.  8-bit keys use the top bit themselves (int8 -128): it
+  // decides, and if equal the rest does.
+  static __device__ __forceinline__ uint32_t at_least(uint32_t a, uint32_t b) {
+    if constexpr (ES == 2) return (a | kTop) - b;
+    const uint32_t rest = (a | kTop) - (b & ~kTop);
+    return (a & ~b) | (~(a ^ b) & rest);
+  }
+  __device__ __forceinline__ Selection(const uint32_t (&p)[4], int f8) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (ES == 2) {
+        key[i] = p[i] & ~kTop;
+      } else {
+        const uint32_t sign = prmt(p[i], 0, 0xBA98);
+        key[i] = f8 ? p[i] & ~kTop : (p[i] ^ sign) + (sign & 0x01010101u);
+      }
+    }
+    const uint32_t c01 = at_least(key[0], key[1]), c02 = at_least(key[0], key[2]), c03 = at_least(key[0], key[3]);
+    const uint32_t c12 = at_least(key[1], key[2]), c13 = at_least(key[1], key[3]), c23 = at_least(key[2], key[3]);
+    kept[0] = majority(c01, c02, c03);
+    kept[1] = majority(~c01, c12, c13);
+    kept[2] = majority(~c02, ~c12, c23);
+    kept[3] = majority(~c03, ~c13, ~c23);
+  }
+  // Bit i of the metadata nibble: first kept position in bits 0 and 1, second in bits 2 and 3.
+  template <int I>
+  __device__ __forceinline__ uint32_t nibble_bit() const {
+    return I == 0 ? ~kept[0] & kept[1] : I == 1 ? ~(kept[0] | kept[1]) : I == 2 ? kept[3] | ~kept[2] : kept[3] | kept[2];
+  }
+  __device__ __forceinline__ uint32_t keep_mask(int i) const { return prmt(kept[i], 0, ES == 2 ? 0xBB99u : 0xBA98u); }
+  // The vector with the positions that are not kept set to zero.
+  __device__ __forceinline__ uint4 pruned(const uint32_t (&p)[4]) const {
+    const uint32_t y[4] = {p[0] & keep_mask(0), p[1] & keep_mask(1), p[2] & keep_mask(2), p[3] & keep_mask(3)};
+    return transpose_back<ES>(y);
+  }
+  // Non-zero magnitudes that are not kept.
+  __device__ __forceinline__ uint32_t lost() const {
+    uint32_t n = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t d = key[i] & ~keep_mask(i);
+      n += __popc((((d & ~kTop) + ~kTop) | d) & kTop);
+    }
+    return n;
+  }
+};
+
+// c + the sum of weights[i] over the bytes of `bits` that are 0xFF (the others are 0).  The weights are given as the bytes of
+// their negatives, because such a byte counts as -1.
+__device__ __forceinline__ uint32_t weigh(uint32_t bits, uint32_t minus_weights, uint32_t c) {
+  return (uint32_t)__dp4a((int)bits, (int)minus_weights, (int)c);
+}
+
+// The kept values of a vector (8 bytes) and its metadata: two groups of a 16-bit type (8 bits), four of an 8-bit type (16).
+template <int ES>
+__device__ __forceinline__ uint32_t gather_kept(const Selection<ES>& s, uint4 w, uint32_t (&kept)[2]) {
+  const uint32_t bit0 = s.template nibble_bit<0>(), bit1 = s.template nibble_bit<1>(), bit2 = s.template nibble_bit<2>(), bit3 = s.template nibble_bit<3>();
+  if constexpr (ES == 2) {
+    // bytes: bit 0 and bit 1 of group 0, of group 1; bits 2 and 3 likewise
+    const uint32_t b01 = prmt(bit0, bit1, 0xFBD9), b23 = prmt(bit2, bit3, 0xFBD9);
+    // a kept position i takes bytes 2i and 2i + 1 of the group's two words: selector nibbles 0x10 + 0x22 * i
+    kept[0] = prmt(w.x, w.y, 256 * weigh(b23, 0x0000BCDEu, 0) + weigh(b01, 0x0000BCDEu, 0x1010));
+    kept[1] = prmt(w.z, w.w, 256 * weigh(b23, 0xBCDE0000u, 0) + weigh(b01, 0xBCDE0000u, 0x1010));
+    return weigh(b01, 0xE0F0FEFFu, weigh(b23, 0x80C0F8FCu, 0));  // 1, 2, 16, 32 and 4, 8, 64, 128
+  } else {
+    uint32_t meta[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {  // groups 0 and 1, groups 2 and 3: two words of one permutation
+      const uint32_t b01 = prmt(bit0, bit1, h ? 0xFBEAu : 0xD9C8u), b23 = prmt(bit2, bit3, h ? 0xFBEAu : 0xD9C8u);
+      const uint32_t first = weigh(b01, 0x0000FEFFu, weigh(b23, 0x0000E0F0u, 0x4400)), second = weigh(b01, 0xFEFF0000u, weigh(b23, 0xE0F00000u, 0));
+      kept[h] = prmt(h ? w.z : w.x, h ? w.w : w.y, 256 * second + first);
+      meta[h] = weigh(b01, 0xE0F0FEFFu, weigh(b23, 0x80C0F8FCu, 0));
+    }
+    return 256 * meta[1] + meta[0];
+  }
 }
 
 // ---- prune (vectorised) -------------------------------------------------------------------------
-// Launch geometry of the vectorised kernels: blockDim = (TX, 256/TX), a warp always lies inside
-// one row; thread (tx, ty) of block (bx, by) handles units (bx*UNROLL + u)*TX + tx, u < UNROLL, of
-// rows by*TY + ty, + gridDim.y*TY, ...  No integer division on the device.
-//
-// Per comparison outcome the byte-permute selectors that copy the kept elements and zero the others
-// (selector nibble 4 = a zero byte of the second operand): 16-bit types need one selector for each
-// of the group's two words, int8 one for its single word.
-template <int ES>
-__device__ __forceinline__ uint32_t prune_selectors(uint32_t idx) {
-  const uint32_t mask = (selection_entry(idx) >> 4) & 0xFu;
-  if (ES == 2) {
-    uint32_t lo = ((mask & 1u) ? 0x10u : 0x44u) | (((mask & 2u) ? 0x32u : 0x44u) << 8);
-    uint32_t hi = ((mask & 4u) ? 0x10u : 0x44u) | (((mask & 8u) ? 0x32u : 0x44u) << 8);
-    return lo | (hi << 16);
-  }
-  return ((mask & 1u) ? 0x0u : 0x4u) | (((mask & 2u) ? 0x1u : 0x4u) << 4) | (((mask & 4u) ? 0x2u : 0x4u) << 8) |
-         (((mask & 8u) ? 0x3u : 0x4u) << 12);
-}
-
-template <int ES>
-__device__ __forceinline__ uint4 prune_vec(uint4 v, const uint32_t* table, int f8) {
-  if (ES == 2) {
-    uint32_t i0, i1;
-    selection_index_x2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu, v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu, i0, i1);
-    const uint32_t s0 = table[i0], s1 = table[i1];
-    return make_uint4(__byte_perm(v.x, 0, s0 & 0xFFFFu), __byte_perm(v.y, 0, s0 >> 16), __byte_perm(v.z, 0, s1 & 0xFFFFu),
-                      __byte_perm(v.w, 0, s1 >> 16));
-  }
-  uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  const uint32_t a[4] = {keys8(w[0], f8), keys8(w[1], f8), keys8(w[2], f8), keys8(w[3], f8)};
-  uint32_t idx[4];
-  selection_index_x4(a, idx);
-#pragma unroll
-  for (int g = 0; g < 4; ++g) w[g] = __byte_perm(w[g], 0, table[idx[g]]);
-  return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// One 16-byte vector per thread and unroll step; `vpr` vectors per row.
+// Launch geometry: blockDim = (TX, 256/TX), a warp always lies inside one row; thread (tx, ty) of block (bx, by) handles
+// vectors (bx*UNROLL + u)*TX + tx, u < UNROLL, of rows by*TY + ty, + gridDim.y*TY, ...  No integer division on the device.
+// One 16-byte vector per thread and unroll step; `vpr` vectors per row.  HBM-bound (6.5
+// TB/s); us, device, with a table of selectors and now: int8 12288 x 3072 20.3, 13.8, 49152 x 12288 269, 184; bf16 the same.
 template <int ES, int UNROLL>
 __global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* x, int64_t row_bytes_x,
                                                              uint8_t* y, int64_t row_bytes_y, int64_t vpr,
                                                              int64_t rows, int f8) {
-  __shared__ uint32_t table[64];
-  {
-    const int t = threadIdx.y * blockDim.x + threadIdx.x;
-    if (t < 64) table[t] = prune_selectors<ES>((uint32_t)t);
-    __syncthreads();
-  }
   wait_for_stream();
   const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows;
@@ -236,17 +212,22 @@ __global__ void __launch_bounds__(kThreads) prune_vec_kernel(const uint8_t* x, i
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
       const uint32_t c = c0 + u * blockDim.x;
-      if (c < vpr) st_stream(yr + c * 16u, prune_vec<ES>(v[u], table, f8));
+      if (c < vpr) {
+        uint32_t p[4];
+        transpose<ES>(v[u], p);
+        st_stream(yr + c * 16u, Selection<ES>(p, f8).pruned(p));
+      }
     }
   }
 }
 
+// ---- compress (fused prune + compress) ----------------------------------------------------
 template <bool COUNT>
 __device__ __forceinline__ void count_dropped(uint32_t lost, unsigned long long* dropped) {
   if (!COUNT) return;
   lost = __reduce_add_sync(0xFFFFFFFFu, lost);
   __shared__ uint32_t warp_sum[kThreads / 32];
-  int t = threadIdx.y * blockDim.x + threadIdx.x;
+  const int t = threadIdx.x;
   if ((t & 31) == 0) warp_sum[t >> 5] = lost;
   __syncthreads();
   if (t == 0) {
@@ -257,148 +238,135 @@ __device__ __forceinline__ void count_dropped(uint32_t lost, unsigned long long*
   }
 }
 
-// 16-bit types.  Work unit: 8 columns (two groups) = one 16-byte load, 8 bytes of values and one
-// metadata byte out, so a warp reads 512 and writes 256 contiguous bytes per step.  Lanes 2j and
-// 2j+1 hold the two halves of a 16-column chunk; the even lane stores the chunk's 16 metadata bits.
-// HW: metadata goes straight into the tensor-core operand order.  FULL: the launch covers exactly
-// the matrix (no padding rows / columns, no ragged block), so no bounds are checked.
-// PRUNE: the pruned matrix is written as well (y, same shape as x; may be x itself), so that one
-// pass over x yields everything the separate prune and compress passes would.
-template <int UNROLL, bool COUNT, bool HW, bool FULL, bool PRUNE>
-__global__ void __launch_bounds__(kThreads, 4) compress16_kernel(const uint8_t* x, int64_t row_bytes_x,
-                                                              uint8_t* __restrict__ vals, int64_t row_bytes_v,
-                                                              uint8_t* __restrict__ meta, int64_t M, int64_t K,
-                                                              int64_t rows_pad, int64_t chunks_pad,
-                                                              unsigned long long* dropped, uint8_t* y,
-                                                              int64_t row_bytes_y) {
-  __shared__ uint32_t table[64];
-  __shared__ uint32_t ptable[PRUNE ? 64 : 1];
-  if (PRUNE) {
-    const int t = threadIdx.y * blockDim.x + threadIdx.x;
-    if (t < 64) ptable[t] = prune_selectors<2>((uint32_t)t);
-  }
-  build_selection_table(table);
-  wait_for_stream();
-  const uint32_t halves = (uint32_t)(K >> 3), halves_pad = (uint32_t)chunks_pad * 2, KB = (uint32_t)(chunks_pad >> 3);
-  const uint32_t h0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
-  // metadata offset of this thread's chunks inside a row: fixed for the whole kernel
-  uint32_t moff[UNROLL];
-#pragma unroll
-  for (int u = 0; u < UNROLL; ++u) {
-    const uint32_t chunk = (h0 + u * blockDim.x) >> 1;
-    moff[u] = HW ? (chunk >> 3) * 2048u + 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * chunk;
-  }
-  uint32_t lost = 0;
-  for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows_pad;
-       row += (int64_t)gridDim.y * blockDim.y) {
-    const uint8_t* xr = x + row * row_bytes_x;
-    uint8_t* vr = vals + row * row_bytes_v;
-    const uint32_t r = (uint32_t)row & 127u;
-    uint8_t* mr = HW ? meta + (row >> 7) * ((int64_t)KB * 2048) + (16u * (r & 7u) + 2u * ((r >> 3) & 1u) + 256u * (r >> 4))
-                     : meta + row * (K >> 3);
-    const bool row_live = FULL || row < M;
-    uint4 in[UNROLL];
-#pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const uint32_t half = h0 + u * blockDim.x;
-      if (row_live && (FULL || half < halves)) in[u] = ld_stream(xr + half * 16u);
-    }
-#pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const uint32_t half = h0 + u * blockDim.x;
-      uint32_t mbyte = 0x44u;  // padding: positions (0, 1) in both groups
-      if (row_live && (FULL || half < halves)) {
-        const uint32_t w[4] = {in[u].x, in[u].y, in[u].z, in[u].w};
-        uint32_t i0, i1;
-        selection_index_x2(w[0] & 0x7FFF7FFFu, w[1] & 0x7FFF7FFFu, w[2] & 0x7FFF7FFFu, w[3] & 0x7FFF7FFFu, i0, i1);
-        const uint32_t e0 = table[i0], e1 = table[i1];
-        if (PRUNE) {
-          const uint32_t s0 = ptable[i0], s1 = ptable[i1];
-          st_stream(y + row * row_bytes_y + half * 16u,
-                    make_uint4(__byte_perm(w[0], 0, s0 & 0xFFFFu), __byte_perm(w[1], 0, s0 >> 16),
-                               __byte_perm(w[2], 0, s1 & 0xFFFFu), __byte_perm(w[3], 0, s1 >> 16)));
-        }
-        __stcs(reinterpret_cast<uint2*>(vr + half * 8u),
-               make_uint2(__byte_perm(w[0], w[1], e0 >> 16), __byte_perm(w[2], w[3], e1 >> 16)));
-        mbyte = (e0 & 0xFu) | ((e1 & 0xFu) << 4);
-        if (COUNT)
-          lost += __popc(Group16::nonzero(w[0], w[1]) & ~(e0 >> 4) & 0xFu) +
-                  __popc(Group16::nonzero(w[2], w[3]) & ~(e1 >> 4) & 0xFu);
-      }
-      const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, mbyte, 1);
-      if ((threadIdx.x & 1) == 0 && (FULL || half < halves_pad))
-        *reinterpret_cast<uint16_t*>(mr + moff[u]) = (uint16_t)(mbyte | (other << 8));
-    }
-  }
-  count_dropped<COUNT>(lost, dropped);
+// 32 bytes at a 32-byte boundary, read or written once.
+__device__ __forceinline__ void ld_stream32(const void* p, uint4 (&v)[2]) {
+  asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x), "=r"(v[1].y), "=r"(v[1].z), "=r"(v[1].w)
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st_stream32(void* p, const uint4 (&v)[2]) {
+  asm volatile("st.global.L1::no_allocate.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0].x),
+               "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w)
+               : "memory");
 }
 
-// int8.  Work unit: one chunk of 16 columns (four groups) = one 16-byte load, 8 bytes of values and
-// 16 bits of metadata out.
-template <int UNROLL, bool COUNT, bool HW, bool FULL, bool PRUNE>
-__global__ void __launch_bounds__(kThreads, 4) compress8_kernel(const uint8_t* x, int64_t row_bytes_x,
-                                                             uint8_t* __restrict__ vals, int64_t row_bytes_v,
-                                                             uint8_t* __restrict__ meta, int64_t M, int64_t K,
-                                                             int64_t rows_pad, int64_t chunks_pad,
-                                                             unsigned long long* dropped, int f8, uint8_t* y,
-                                                             int64_t row_bytes_y) {
-  __shared__ uint32_t table[64];
-  __shared__ uint32_t ptable[PRUNE ? 64 : 1];
-  if (PRUNE) {
-    const int t = threadIdx.y * blockDim.x + threadIdx.x;
-    if (t < 64) ptable[t] = prune_selectors<1>((uint32_t)t);
-  }
-  build_selection_table(table);
+// What a launch of compress_kernel may do with whole cells at once: x or y by 32 bytes, the values of an 8-bit cell by 16.
+enum { kWideX = 1, kWideY = 2, kWideVals = 4 };
+
+// Work unit ("cell"): 32 bytes of a row (16 columns of a 16-bit type, 32 of an 8-bit one) = 16 bytes of values and 2 or 4
+// bytes of metadata.  A thread has a cell of the rows r and r + 8 of a 16-row group: in the operand order of a 16-bit type the
+// two share each 32-bit word.  A warp has 16 cells of 2 neighbouring rows (8 of 4 rows where the row ends in half of that) and
+// their partners, so that it writes whole 32-byte sectors of metadata: with 16-byte units and a row to a warp
+// metadata went out in 2-byte pieces.  gridDim.y strides over the row groups.
+// The domain is padded (rows to a multiple of 128, columns of 256) so that the operand order gets its 0x4 padding nibbles from
+// the same launch.  HW: metadata straight into that order.  FULL: the launch covers exactly the matrix, so no bounds are
+// checked.  PRUNE: the pruned matrix is written as well (y, same shape as x; may be x itself), so that one pass over x yields
+// everything the separate prune and compress passes would.
+// Bound by HBM where the matrix is large and cold, by the ALU pipe where it comes out of the L2 (ncu, bf16 12288 x 3072 right
+// after apply_mask: 5 of 75 MB read from DRAM, ALU pipe 73 % busy with 57 instructions a vector).  Us, device, table
+// kernels of before / now: compress bf16 49152 x 12288 332, 281 (6.7 TB/s); 4096 x 4096 9.0, 7.4; 49152 x 256 13.4, 5.9; int8
+// 49152 x 12288 292, 160; 12288 x 3072 22.0, 11.1; fused with prune bf16 49152 x 12288 534, 474; int8 340, 247; after
+// apply_mask, both calls, bf16 12288 x 3072 40.4, 36.0.
+// (Registers: five blocks an SM where nothing spills; 8-bit types are faster with four.)
+template <int ES, bool COUNT, bool PRUNE>
+constexpr int kCompressBlocks = ES == 2 && !COUNT && !PRUNE ? 5 : 4;
+
+template <int ES, bool COUNT, bool HW, bool FULL, bool PRUNE>
+__global__ void __launch_bounds__(kThreads, kCompressBlocks<ES, COUNT, PRUNE>)
+compress_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t row_bytes_v, uint8_t* meta, int64_t M, int64_t K,
+                uint32_t row_groups, uint32_t cells_pad, int cell_shift, int wide, unsigned long long* dropped, int f8, uint8_t* y,
+                int64_t row_bytes_y) {
+  constexpr uint32_t kCols = ES == 2 ? 16 : 32;  // columns of a cell
   wait_for_stream();
-  const uint32_t chunks = (uint32_t)(K >> 4), cpad = (uint32_t)chunks_pad, KB = (uint32_t)(chunks_pad >> 3);
-  const uint32_t c0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
-  uint32_t moff[UNROLL];
-#pragma unroll
-  for (int u = 0; u < UNROLL; ++u) {
-    const uint32_t chunk = c0 + u * blockDim.x;
-    moff[u] = HW ? (chunk >> 3) * 2048u + 2u * (chunk & 7u) : 2u * chunk;
-  }
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t rows_of_warp = 32u >> cell_shift, cell = (blockIdx.x << cell_shift) + (lane & ((1u << cell_shift) - 1u));
+  const uint32_t thread_row = warp * rows_of_warp + (lane >> cell_shift);  // eight of these to a row group
+  const uint32_t in_group = thread_row & 7u, step = gridDim.y * rows_of_warp;
+  const bool live_cell = FULL || (int64_t)cell * kCols < K, meta_cell = FULL || cell < cells_pad;
+  const bool half_cell = ES == 1 && !FULL && K - (int64_t)cell * kCols == 16;
+  // metadata of the cell in the first row of its 128-row block that this thread may have (canonical: in row 0)
+  const uint32_t chunk = ES == 2 ? cell : 2 * cell, KB = ES == 2 ? cells_pad >> 3 : cells_pad >> 2;
+  uint8_t* const meta_cell0 = meta + (!HW ? 2 * chunk
+                                          : (chunk >> 3) * 2048u + 16u * in_group +
+                                                (ES == 2 ? 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * (chunk & 7u)));
+  uint32_t n = blockIdx.y * rows_of_warp + (thread_row >> 3);  // row group
+  const int64_t row0 = (int64_t)n * 16 + in_group;
+  const uint8_t* xp = x + row0 * row_bytes_x + (int64_t)cell * 32;
+  uint8_t* vp = vals + row0 * row_bytes_v + (int64_t)cell * 16;
+  uint8_t* yp = PRUNE ? y + row0 * row_bytes_y + (int64_t)cell * 32 : nullptr;
   uint32_t lost = 0;
-  for (int64_t row = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; row < rows_pad;
-       row += (int64_t)gridDim.y * blockDim.y) {
-    const uint8_t* xr = x + row * row_bytes_x;
-    uint8_t* vr = vals + row * row_bytes_v;
-    uint8_t* mr = HW ? meta + (row >> 7) * ((int64_t)KB * 2048) + 16u * ((uint32_t)row & 127u) : meta + row * (K >> 3);
-    const bool row_live = FULL || row < M;
-    uint4 in[UNROLL];
+#pragma unroll 1
+  for (; n < row_groups; n += step, xp += (int64_t)step * 16 * row_bytes_x, vp += (int64_t)step * 16 * row_bytes_v) {
+    uint4 in[2][2];
+    bool live[2];
 #pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const uint32_t chunk = c0 + u * blockDim.x;
-      if (row_live && (FULL || chunk < chunks)) in[u] = ld_stream(xr + chunk * 16u);
-    }
-#pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const uint32_t chunk = c0 + u * blockDim.x;
-      if (!FULL && chunk >= cpad) continue;
-      uint32_t mbits = 0x4444u;
-      if (row_live && (FULL || chunk < chunks)) {
-        const uint32_t w[4] = {in[u].x, in[u].y, in[u].z, in[u].w};
-        uint32_t out[2] = {0, 0};
-        uint32_t pw[4];
-        mbits = 0;
-        const uint32_t keys[4] = {keys8(w[0], f8), keys8(w[1], f8), keys8(w[2], f8), keys8(w[3], f8)};
-        uint32_t idx4[4];
-        selection_index_x4(keys, idx4);
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const uint32_t a = keys[g];
-          const uint32_t idx = idx4[g];
-          const uint32_t e = table[idx];
-          if (PRUNE) pw[g] = __byte_perm(w[g], 0, ptable[idx]);
-          const uint32_t pair = __byte_perm(w[g], 0, ((e >> 8) & 0xFFu) | 0x4400u);
-          out[g >> 1] |= pair << (16 * (g & 1));
-          mbits |= (e & 0xFu) << (4 * g);
-          if (COUNT) lost += __popc(Group8::nonzero(a) & ~(e >> 4) & 0xFu);
+    for (int h = 0; h < 2; ++h) {
+      live[h] = live_cell && (FULL || (int64_t)n * 16 + in_group + 8 * h < M);
+      if (live[h]) {
+        const uint8_t* src = xp + 8 * h * row_bytes_x;
+        if (wide & kWideX) {
+          ld_stream32(src, in[h]);
+        } else {
+          in[h][0] = ld_stream(src);
+          in[h][1] = half_cell ? make_uint4(0, 0, 0, 0) : ld_stream(src + 16);
         }
-        __stcs(reinterpret_cast<uint2*>(vr + chunk * 8u), make_uint2(out[0], out[1]));
-        if (PRUNE) st_stream(y + row * row_bytes_y + chunk * 16u, make_uint4(pw[0], pw[1], pw[2], pw[3]));
       }
-      *reinterpret_cast<uint16_t*>(mr + moff[u]) = (uint16_t)mbits;
+    }
+    uint32_t bits[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bits[h] = ES == 2 ? 0x4444u : 0x44444444u;  // padding: positions (0, 1) in all groups
+      if (live[h]) {
+        uint32_t kept[2][2], m[2];
+        uint4 out[2];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          uint32_t p[4];
+          transpose<ES>(in[h][v], p);
+          const Selection<ES> s(p, f8);
+          m[v] = gather_kept<ES>(s, in[h][v], kept[v]);
+          if (PRUNE) out[v] = s.pruned(p);
+          if (COUNT) lost += s.lost();
+        }
+        bits[h] = m[1] * (ES == 2 ? 256u : 65536u) + m[0];
+        uint8_t* v = vp + 8 * h * row_bytes_v;
+        if (ES == 2 || (wide & kWideVals)) {
+          st_stream(v, make_uint4(kept[0][0], kept[0][1], kept[1][0], kept[1][1]));
+        } else {
+          __stcs(reinterpret_cast<uint2*>(v), make_uint2(kept[0][0], kept[0][1]));
+          if (!half_cell) __stcs(reinterpret_cast<uint2*>(v + 8), make_uint2(kept[1][0], kept[1][1]));
+        }
+        if (PRUNE) {
+          uint8_t* dst = yp + 8 * h * row_bytes_y;
+          if (wide & kWideY) {
+            st_stream32(dst, out);
+          } else {
+            st_stream(dst, out[0]);
+            if (!half_cell) st_stream(dst + 16, out[1]);
+          }
+        }
+      }
+    }
+    if (PRUNE) yp += (int64_t)step * 16 * row_bytes_y;
+    if (!meta_cell) continue;
+    if constexpr (HW) {
+      uint8_t* mr = meta_cell0 + ((uint64_t)(n >> 3) * KB << 11) + 256u * (n & 7u);
+      if constexpr (ES == 2) {
+        *reinterpret_cast<uint32_t*>(mr) = bits[1] * 65536u + bits[0];
+      } else {
+        *reinterpret_cast<uint32_t*>(mr) = bits[0];
+        *reinterpret_cast<uint32_t*>(mr + 128) = bits[1];
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t row = (int64_t)n * 16 + in_group + 8 * h;
+        if (!FULL && row >= M) continue;
+        uint16_t* mr = reinterpret_cast<uint16_t*>(meta_cell0 + row * (K >> 3));
+        mr[0] = (uint16_t)bits[h];
+        if (ES == 1 && !half_cell) mr[1] = (uint16_t)(bits[h] >> 16);
+      }
     }
   }
   count_dropped<COUNT>(lost, dropped);
@@ -694,19 +662,6 @@ extern "C" sp24_status sp24_prune(sp24_dtype t, int64_t M, int64_t K, const void
 namespace sp24 {
 namespace {
 
-template <int ES, bool COUNT, bool HW, bool FULL, bool PRUNE>
-sp24_status launch_compress_vec(const RowLaunch& L, cudaStream_t s, const uint8_t* xs, int64_t rbx, uint8_t* vs, int64_t rbv,
-                                uint8_t* ms, int64_t M, int64_t K, int64_t rows_pad, int64_t chunks_pad,
-                                unsigned long long* dropped, int f8, uint8_t* ys, int64_t rby) {
-  constexpr int UNROLL = 4;
-  if constexpr (ES == 2)
-    return launch_overlapped(compress16_kernel<UNROLL, COUNT, HW, FULL, PRUNE>, L.grid, L.block, 0, s, 1, xs, rbx, vs, rbv, ms,
-                             M, K, rows_pad, chunks_pad, dropped, ys, rby);
-  else
-    return launch_overlapped(compress8_kernel<UNROLL, COUNT, HW, FULL, PRUNE>, L.grid, L.block, 0, s, 1, xs, rbx, vs, rbv, ms,
-                             M, K, rows_pad, chunks_pad, dropped, f8, ys, rby);
-}
-
 // compress (y == nullptr) or fused prune + compress (y = pruned matrix, vector kernels only: returns
 // SP24_ERR_UNSUPPORTED when they cannot take the operands) for the 2:4 types.
 sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int64_t ldx, void* y, int64_t ldy,
@@ -727,31 +682,33 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
   const bool vec = K % 16 == 0 && aligned16(x) && aligned16(vals) && aligned16(meta) && (ldx * es) % 16 == 0 &&
                    (ldv * es) % (8 * es) == 0 && row_offsets_fit(K, es, l);
   if (vec) {
-    constexpr int UNROLL = 4;
-    const int64_t chunks_pad = k_pad / 16;
-    const int64_t units = es == 2 ? chunks_pad * 2 : chunks_pad;  // 16-byte vectors per padded row
-    RowLaunch L(units, rows_pad, UNROLL);
-    // A matrix of moderate size is bound by instructions, a tenth of them a block's tables: 8 blocks an SM take all rows.  A
-    // large one is bound by HBM and wants the loads of all its blocks in flight.  The line, 160 MB of traffic, lies between
-    // what was measured on either side of it (it is not the L2's 126 MB).  Us, device, a block for every row step against 8
-    // an SM: compress bf16 12288 x 3072 (118 MB in all) 19.9, 17.3; 49152 x 1024 (157 MB) 25.5, 22.5; 49152 x 12288 (1.9 GB)
-    // 323, 369; fused with prune bf16 16102 x 1088 (92 MB) 17.1, 14.9; 12288 x 3072 (193 MB) 30.3, 32.8; int8 49152 x 1024
-    // (132 MB) 28.4, 25.7.
+    const int64_t cols = es == 2 ? 16 : 32, cells_pad = (k_pad + cols - 1) / cols;
+    const int shift = (cells_pad - 1) % 16 < 8 ? 3 : 4;  // cells of a row to a warp: 8 or 16, whichever leaves fewer lanes idle
+    const int64_t units = (cells_pad + (1 << shift) - 1) >> shift, groups = (rows_pad + 15) / 16, per_block = 32 >> shift;
+    int64_t steps = (groups + per_block - 1) / per_block;
+    if (steps > 32768) steps = 32768;
+    // A matrix of moderate size is bound by instructions: two rounds of the blocks that fit the SMs take all rows, so that no
+    // last round is nearly empty and the set-up of a block is paid for once.  A large one is bound by HBM and wants the loads
+    // of all its blocks in flight.  The line, 160 MB of traffic, lies between what was measured on either side of it (it is
+    // not the L2's 126 MB).  Us, device, a block for every row step against two rounds: compress bf16 16102 x 1088 (53 MB in
+    // all) 10.0, 8.8; apply_mask + compress of 4096 x 4096 18.4, 18.1, of 12288 x 3072 37.3, 36.8; compress of 49152 x 12288
+    // (1.9 GB) 281, 310 (16 blocks an SM).
     const int64_t moved = M * K * es * (y ? 5 : 3) / 2 + M * K / 8;
-    const unsigned few = (8 * (unsigned)sm_count() + L.grid.x - 1) / L.grid.x;
-    if (moved <= (int64_t)160 << 20 && L.grid.y > few) L.grid.y = few;
-    const bool full = rows_pad == M && k_pad == K && units % ((int64_t)L.block.x * UNROLL) == 0;
+    const int64_t two_rounds = (2 * (es == 2 && !dropped && !y ? kCompressBlocks<2, false, false> : kCompressBlocks<1, true, true>) * sm_count() + units - 1) / units;
+    if (moved <= (int64_t)160 << 20 && steps > two_rounds) steps = two_rounds;
+    const dim3 grid((unsigned)units, (unsigned)steps, 1);
+    const bool whole_cells = K % cols == 0;
+    const bool full = rows_pad == M && M % 16 == 0 && k_pad == K && whole_cells && cells_pad == units << shift;
+    auto by32 = [&](const void* p, int64_t ld) { return whole_cells && reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
+    const int wide = (by32(x, ldx) ? kWideX : 0) | (y && by32(y, ldy) ? kWideY : 0) | (whole_cells && ldv * es % 16 == 0 ? kWideVals : 0);
     const int variant = (y ? 8 : 0) | (dropped ? 4 : 0) | (hw ? 2 : 0) | (full ? 1 : 0);
     const uint8_t* xs = (const uint8_t*)x;
     uint8_t *vs = (uint8_t*)vals, *ms = (uint8_t*)meta, *ys = (uint8_t*)y;
-#define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                            \
-  case V:                                                                                                             \
-    if (es == 2)                                                                                                      \
-      st = launch_compress_vec<2, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
-                                                     dropped, f8, ys, ldy * es);                                      \
-    else                                                                                                              \
-      st = launch_compress_vec<1, COUNT, HW, FULL, PRUNE>(L, s, xs, ldx * es, vs, ldv * es, ms, M, K, rows_pad, chunks_pad, \
-                                                     dropped, f8, ys, ldy * es);                                      \
+#define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                                 \
+  case V:                                                                                                                  \
+    st = launch_overlapped(es == 2 ? compress_kernel<2, COUNT, HW, FULL, PRUNE> : compress_kernel<1, COUNT, HW, FULL, PRUNE>, grid, \
+                           dim3(kThreads), 0, s, 1, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)cells_pad, \
+                           shift, wide, dropped, f8, ys, ldy * es);                                                        \
     break;
     switch (variant) {
       SP24_CV(0, false, false, false, false)
