@@ -184,6 +184,13 @@ __device__ __forceinline__ float2 fma2(float2 a, float s, float2 c) {
   return d;
 }
 
+// c << 16 | a << 8 | b, a and b clamped to the range of int8
+__device__ __forceinline__ uint32_t pack_sat_s8(int a, int b, uint32_t c) {
+  uint32_t d;
+  asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
 // ---- tensor memory -----------------------------------------------------------------------------
 template <int CTAS>
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t cols) {
