@@ -252,16 +252,44 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& cta
   }
 }
 
+// Clusters of 2^log single CTAs that the device holds at one time (a GPC may end in SMs that make no whole cluster), asked
+// once per device; every GEMM CTA fills its SM.
+__global__ void cluster_probe() {}
+static int split_clusters(int log) {
+  static std::atomic<int> known[64][4];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const bool cacheable = dev >= 0 && dev < 64;
+  if (cacheable && (n = known[dev][log].load(std::memory_order_relaxed)) > 0) return n;
+  constexpr int smem = 227 * 1024;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 1u << log;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(1u << log);
+  cfg.blockDim = dim3(kNumThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cuda_status(cudaFuncSetAttribute(cluster_probe, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != SP24_OK ||
+      cuda_status(cudaOccupancyMaxActiveClusters(&n, cluster_probe, &cfg)) != SP24_OK || n <= 0)
+    n = (sm_count() >> log) * 3 / 4;
+  if (cacheable) known[dev][log].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 // Time of a product with tiles of (128 * ctas * mblk) x tile_n, us on an idle chip: start, and per round of tiles the
 // k-blocks (a fixed part and one per column, the same for all kinds: a k-block is 256 bytes of K), then the epilogue of a
 // tile by its columns (4-byte results and C cost more; 256-column tiles and two m-blocks cannot overlap it).  Fitted to
 // 170 random problems (256..16384 rows, 160..16384 columns, K 256..12288, every kind, with and without C), 11 to 17
 // shapes of each, before stages held two k-blocks: it puts bf16 512 x 512 x 8192 at 16.5 us, which now takes 13.1.  On 100
 // other problems of the same ranges the mean error of today's kernels is 9 to 13 % per shape, 16 % for two m-blocks.
-static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n) {
+// split_log: the CTAs of a cluster share the k-blocks.
+static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n, int split_log = 0) {
   const int bytes = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
   const int es = bytes > 0 ? bytes : 1;  // (a type that no product takes may still ask for its plan)
-  const double k_blocks = (double)((d->K * es + 255) / 256);
+  const double k_blocks = (double)((((d->K * es + 255) >> 8) + (1 << split_log) - 1) >> split_log);
   const int64_t rows = 128 * ctas * mblk, slots = sm_count() / ctas > 0 ? sm_count() / ctas : 1;
   const int64_t tiles = ((d->M + rows - 1) / rows) * ((d->N + tile_n - 1) / tile_n);
   const double rounds = (double)((tiles + slots - 1) / slots), w = tile_n / 100.0;
@@ -281,7 +309,14 @@ static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block
 // problems the choice below is 17 % faster in the mean than the widest tiles, one is slower by more than 2 % (int8 128 x
 // 3808 x 352 4.5 -> 4.7 us); it is 1.5 % behind the best of the shapes over the 170 above, 2.3 % (at worst 22 %) over the 100.
 // A pair keeps its shape unless the estimate says 3 %, its two m-blocks unless it says 15 %: it puts those 12 % too high.
-static void choose_width(const sp24_gemm_desc* d, bool has_c, int& ctas, int& block_n, int& mblk, int& tile_n) {
+//
+// INT32 accumulators of single CTAs: a cluster of 2, 4 or 8 of them may share the k-blocks of a tile (split_log), which the
+// estimate has as its k-blocks in so many parts and the exchange of the accumulators, by their columns.  Where few tiles
+// have many k-blocks this uses SMs that have none; the sums are integers, the same in any order, so the result does not
+// depend on it (those of floating-point kinds would).  Us, device, one CTA to a tile and the choice: 4096 x 32 x 4096 5.9, 4.7;
+// 512 x 512 x 8192 9.2, 6.6; 256 x 256 x 12288 12.3, 6.1; 1056 x 32 x 10816 with C 11.6, 5.2; 2048 x 64 x 2048 4.3, 4.1.
+static void choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ctas, int& block_n, int& mblk, int& tile_n, int& split_log) {
+  split_log = 0;
   const int64_t n32 = (d->N + 31) / 32 * 32;
   auto widest = [&](int bn) { return n32 < bn ? (int)n32 : bn; };
   tile_n = widest(block_n);
@@ -294,11 +329,23 @@ static void choose_width(const sp24_gemm_desc* d, bool has_c, int& ctas, int& bl
   double best = now * (ctas == 1 ? 1.0 : mblk == 2 ? 0.85 : 0.97);
   auto try_shape = [&](int c, int bn, int tn) {
     const double t = tile_time(d, has_c, c, bn, 1, tn);
-    if (t < best) { best = t; ctas = c; block_n = bn; mblk = 1; tile_n = tn; }
+    if (t < best) { best = t; ctas = c; block_n = bn; mblk = 1; tile_n = tn; split_log = 0; }
   };
   const bool pairs = !d->a_is_dense && d->N > 128 && d->M >= 256 && (d->M / 256) * ((d->N + 223) / 224) >= 4;
   const bool k_major_b = d->order_b == SP24_COL_MAJOR, one = ctas == 1;
   const bool has_240 = k_major_b && elem_bytes(d->ab_type) == 2 && elem_bytes(d->cd_type) == 2;
+  if (d->ab_type == SP24_I8 && !d->a_is_dense && d->order_b == SP24_COL_MAJOR && !conv) {
+    const int64_t blocks = (d->M + kBlockM - 1) / kBlockM, k_blocks = (d->K + 255) / 256;
+    for (int w = widest(128); w > 0; w -= 32) {
+      const int64_t tiles = blocks * ((d->N + w - 1) / w);
+      for (int log = 1; log <= 3 && k_blocks >= 2 << log; ++log) {
+        if (tiles > (sm_count() >> log) || tiles > split_clusters(log)) break;
+        const double columns = w / 100.0, exchange = log == 1 ? 0.4 + columns : (log == 2 ? 0.5 : 0.9) + 2.0 * columns;
+        const double t = 1.04 * (tile_time(d, has_c, 1, 128, 1, w, log) + exchange);
+        if (t < best) { best = t; ctas = 1; block_n = 128; mblk = 1; tile_n = w; split_log = log; }
+      }
+    }
+  }
   if (!one) try_shape(1, 128, widest(128));
   for (int w = 96; w >= 32; w -= 32)
     if (w < n32) try_shape(1, 128, w);
@@ -311,9 +358,9 @@ static void choose_width(const sp24_gemm_desc* d, bool has_c, int& ctas, int& bl
 extern "C" sp24_status sp24_gemm_plan(const sp24_gemm_desc* d, int* ctas, int* block_n, int* mblk) {
   SP24_RETURN_IF(d == nullptr || ctas == nullptr || block_n == nullptr || mblk == nullptr, SP24_ERR_NULL);
   SP24_RETURN_IF(d->M <= 0 || d->N <= 0 || d->K <= 0, SP24_ERR_SHAPE);
-  int tile_n;
+  int tile_n, split_log;
   choose_tile(d, false, false, *ctas, *block_n, *mblk);
-  choose_width(d, false, *ctas, *block_n, *mblk, tile_n);
+  choose_width(d, false, false, *ctas, *block_n, *mblk, tile_n, split_log);
   Settings& cfg = settings();
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     *ctas = c;
@@ -440,26 +487,27 @@ static sp24_status run_gemm(const sp24_gemm_desc* d, const void* alpha, const vo
   const bool sparse = !d->a_is_dense;
   const bool i8 = d->ab_type == SP24_I8, tf32 = d->ab_type == SP24_F32, f8 = is_fp8(d->ab_type);
   int ctas, block_n, mblk;
-  int tile_n;
+  int tile_n, split_log;
   choose_tile(d, has_c, cv != nullptr, ctas, block_n, mblk);
-  choose_width(d, has_c, ctas, block_n, mblk, tile_n);
+  choose_width(d, has_c, cv != nullptr, ctas, block_n, mblk, tile_n, split_log);
   p.band = 16 / mblk;
   if (const int c = cfg.ctas.load(std::memory_order_relaxed)) {
     ctas = c;
     block_n = cfg.block_n.load(std::memory_order_relaxed);
     mblk = cfg.mblk.load(std::memory_order_relaxed);
     tile_n = ctas == 1 && mblk > 1 && d->N < block_n ? (int)d->N : block_n;
+    split_log = 0;
   }
   SP24_RETURN_IF(cv && ctas == 1 && mblk != 1, SP24_ERR_UNSUPPORTED);  // a forced tall tile
   p.mblk = mblk;
   if (const int b = cfg.band.load(std::memory_order_relaxed)) p.band = b;
   const bool b_mn = d->order_b == SP24_ROW_MAJOR;  // B stored N-contiguous
   if (cfg.log.load(std::memory_order_relaxed))
-    fprintf(stderr, "sp24_gemm: M=%lld N=%lld K=%lld ab=%d cd=%d %s%s tile=%dx%dx%d columns=%d band=%d beta=%g%s%s\n", (long long)d->M,
+    fprintf(stderr, "sp24_gemm: M=%lld N=%lld K=%lld ab=%d cd=%d %s%s tile=%dx%dx%d columns=%d split=%d band=%d beta=%g%s%s\n", (long long)d->M,
             (long long)d->N, (long long)d->K, (int)d->ab_type, (int)d->cd_type, sparse ? "sparse" : "dense",
-            b_mn ? " B:N-contiguous" : "", ctas, block_n, mblk, tile_n, p.band, (double)fbeta, dq ? " dequant" : "",
+            b_mn ? " B:N-contiguous" : "", ctas, block_n, mblk, tile_n, 1 << split_log, p.band, (double)fbeta, dq ? " dequant" : "",
             cv ? " conv3x3" : (acc_f16 ? " fp16-accumulate" : ""));
-  const TileShape tile = {ctas, block_n, mblk, tile_n};
+  const TileShape tile = {ctas, block_n, mblk, tile_n, split_log};
   if (i8) return launch_gemm<1>(tile, sparse, b_mn, d, p, A, meta, B, s);
   if (tf32) return launch_gemm<2>(tile, sparse, b_mn, d, p, A, meta, B, s);
   if (f8) return launch_gemm<3>(tile, sparse, b_mn, d, p, A, meta, B, s);

@@ -62,6 +62,8 @@ struct GemmParams {
   FastDiv by_band_tiles, by_band, by_last_band;  // tiles of a band; m-tiles of a band and of the last one
   int32_t tile_n;     // columns of a tile: the kernel's BLOCK_N or fewer
   int32_t kps;        // k-blocks of a stage (1 or 2)
+  int32_t split_log;  // log2 of the CTAs (a cluster) that share a tile's k-blocks; INT32 accumulators of single CTAs only
+  int32_t part_bytes; // ... and the room for the other CTAs' parts of the boxes that a CTA finishes
   int32_t mblk, b_stages;  // tall tiles only: m-blocks of a tile, slots of the B ring
   int32_t b_3d;       // map_b is three-dimensional: a stage of B is one load
   int32_t cd_col_major;  // C and D stored M-contiguous (the [tokens, out_features] layout): selects the kernel
@@ -109,6 +111,7 @@ sp24_status make_im2col_map(CUtensorMap* map, const void* x, int es, uint64_t nb
 // built.  Each kind is instantiated in a source file of its own, so that they compile side by side.
 struct TileShape {
   int ctas, block_n, mblk, tile_n;
+  int split_log;  // see GemmParams
 };
 template <int KIND>
 sp24_status launch_gemm(TileShape tile, bool sparse, bool b_mn, const sp24_gemm_desc* d, const GemmParams& p, const void* A,

@@ -49,6 +49,12 @@ constexpr int kTallBlocks = 3;
 template <int CTAS, int MBLK>
 constexpr bool is_tall = CTAS == 1 && MBLK == kTallBlocks;
 
+// A cluster of CTAs may share the k-blocks of a tile (p.split_log): INT32 accumulators, which are the same in any order of the
+// sums.  Kernels of their own (SPLIT): with it as a choice inside the others, short calls that do not split took up to 0.2 us
+// (6 %) more.
+template <int KIND, bool SPARSE, int CTAS, int MBLK, bool B_MN>
+constexpr bool can_split = KIND == 1 && SPARSE && CTAS == 1 && MBLK == 1 && !B_MN;
+
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
 struct Cfg {
   // 128-byte atoms per stage: sparse A is half as wide as B; the dense variant with two
@@ -119,22 +125,25 @@ struct Cfg {
 
 struct Shared {
   uint64_t full[12], empty[12], tmem_full[2], tmem_empty[2];
+  uint64_t split_full;             // the other CTAs' parts of the boxes that this one finishes are there
   uint64_t c_full[kEpiWarps][2];   // per epilogue warp and staging buffer: C box has landed
   uint32_t tmem_base;
   volatile uint32_t abort;
 };
 static_assert(sizeof(Shared) <= 512, "barrier block");
 
+template <bool CLUSTER = false>  // (for what another CTA has written)
 __device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, Shared* sh, uint32_t* status,
                                              uint32_t code, long long limit) {
+  auto try_wait = [&] { return CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity); };
   // fast path: poll a while before any bookkeeping; try_wait itself suspends the thread briefly
 #pragma unroll 1
   for (int i = 0; i < 64; ++i)
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (try_wait()) return true;
   const long long t0 = clock64();
   uint32_t spins = 0;
   while (true) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (try_wait()) return true;
     if ((++spins & 255u) == 0) {
       if (sh->abort) return false;
       if (clock64() - t0 > limit) {
@@ -339,10 +348,10 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // half as wide, meet in pairs).
 // C is loaded in the order of the stores (whole 64-byte row segments as well) into registers, four boxes ahead, the
 // first four of a tile before its accumulators are complete, and goes to the rows' owners through the buffer.
-template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES>
+template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES, bool SPLIT>
 __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
-                                              int lane) {
+                                              int lane, uint32_t parts, int split_rank) {
   constexpr int kCols = CS == 4 ? 16 : 32;  // columns of a box
   constexpr int W = kCols * CS / 4;         // 32-bit words of one box row
   constexpr int P = 4;                      // boxes whose C values are held in registers
@@ -355,7 +364,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   uint8_t* Db = static_cast<uint8_t*>(p.D);
   const size_t ldc_b = (size_t)p.ldc * CS, ldd_b = (size_t)p.ldd * CS;
   const int M = (int)p.M, N = (int)p.N;
-  const bool has_c = CS != 1 && p.has_c != 0;
+  const bool has_c = CS != 1 && !(KIND == 1 && CS == 2) && p.has_c != 0;  // (int8: only INT32 results are added to)
   // this lane's row of the buffer, its unit 0 under the swizzle (xor the unit into bits 4..5) ...
   const uint32_t own_row = ptx::smem_u32(stage) + (uint32_t)(lane * 64 + ((((lane >> 1) ^ (lane >> 3)) & 3) << 4));
   // ... for ldmatrix / stmatrix ...
@@ -365,6 +374,17 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   // rows on)
   const int st_r = lane / kUnits, st_u = lane % kUnits;
   const uint32_t st_row = ptx::smem_u32(stage) + (uint32_t)(st_r * 64 + ((st_u ^ (((st_r >> 1) ^ (st_r >> 3)) & 3)) << 4));
+  // K-blocks shared by a cluster of CTAs: the boxes of warp w are finished by CTA w mod the cluster's size.  The other CTAs'
+  // warps w send it their accumulators of these boxes (16-byte units of 32 lanes) into shared memory kept for them; it adds
+  // them up as it takes a box from its own tensor memory.
+  const int split_log = SPLIT ? p.split_log : 0, split = 1 << split_log;
+  const int owner = (warp - kFirstEpiWarp) & (split - 1);
+  const bool mine = owner == split_rank;
+  const int warp_boxes = (p.tile_n / kCols + 1) / 2, owner_boxes = (kEpiWarps >> split_log) * warp_boxes;  // (room for)
+  auto part_of = [&](int from_rank, int sc) {
+    const int i = ((from_rank - owner - 1) & (split - 1)) * owner_boxes + ((warp - kFirstEpiWarp) >> split_log) * warp_boxes + (sc >> 1);
+    return parts + (uint32_t)(i * (kCols * 128) + lane * 16);
+  };
   auto st_addr = [&](int k) { return (st_row ^ (uint32_t)(((k * kRowsPerStore) >> 3) << 4)) + k * kRowsPerStore * 64; };
   int acc = 0;
   uint32_t acc_phase = 0;
@@ -501,13 +521,25 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
       step(cj, csc, kEpiWarps / 4);
     };
     auto box = [&](uint32_t (&c)[W]) -> bool {
-      const int row0 = row_q + j * kBlockM, col0 = tile_col + sc * kCols, j0 = j;
+      const int row0 = row_q + j * kBlockM, col0 = tile_col + sc * kCols, j0 = j, sc0 = sc;
       step(j, sc, kEpiWarps / 4);
       const bool more = j < blocks;
       uint32_t o[W];
       if (has_c) share_c(c);
       ptx::tmem_ld_wait(r);
       if (!more) hand_back();
+      if constexpr (SPLIT) {
+#pragma unroll 1
+        for (int i = 1; i < split; ++i) {
+          const uint32_t from = part_of(split_rank + i, sc0);
+#pragma unroll
+          for (int u = 0; u < kCols / 4; ++u) {
+            uint32_t x[4];
+            ptx::ld_shared_v4(from + u * 512, x[0], x[1], x[2], x[3]);
+            r[4 * u] += x[0]; r[4 * u + 1] += x[1]; r[4 * u + 2] += x[2]; r[4 * u + 3] += x[3];
+          }
+        }
+      }
       if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
       compute_row<KIND, CS, kCols>(r, c, has_c, p, scale, bias, o);
       if (more) {
@@ -518,14 +550,33 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
       store(o, row0, col0);
       return more;
     };
-    const bool any = j < blocks;
+    const bool any = mine && j < blocks;
     if (any) load_scale(row_q + j * kBlockM);
-    if (has_c) {
+    if (has_c && mine) {
 #pragma unroll
       for (int n = 0; n < P; ++n) fetch_c(creg[n]);
     }
     if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
     ptx::tc_fence_after();
+    if constexpr (SPLIT) {
+      if (!mine) {
+        const uint32_t bar = ptx::map_to_cta(ptx::smem_u32(&sh->split_full), (uint32_t)owner);
+#pragma unroll 1
+        for (; j < blocks; step(j, sc, kEpiWarps / 4)) {
+          const uint32_t to = ptx::map_to_cta(part_of(split_rank, sc), (uint32_t)owner);
+          ptx::tmem_ld_32x32b(t_acc + sc * kCols, r);
+          ptx::tmem_ld_wait(r);
+#pragma unroll
+          for (int u = 0; u < kCols / 4; ++u) ptx::st_async_v4(to + u * 512, r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3], bar);
+        }
+      } else {
+        if (lane == 0) {
+          const int boxes = blocks > 0 && nsub > half ? (nsub - half + 1) / 2 : 0;
+          ptx::mbar_expect_tx(&sh->split_full, (uint32_t)(boxes * (split - 1) * kCols * 128));
+        }
+        if (!bounded_wait<true>(&sh->split_full, 0, sh, p.status, 6u, p.wait_limit)) break;
+      }
+    }
     if (!any) {
       hand_back();
     } else {
@@ -551,7 +602,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
 // CS, COLS: bytes of an output element, column-major output.  A kernel for each form of the output, so that it holds
 // one epilogue: with all of them behind branches of one kernel, a tile's epilogue took up to twice as long whatever
 // the form (us, branches -> own kernels: bf16 24576 x 224 x 4096 with 512 x 224 tiles 39.8 -> 34.3, with C 43.6 -> 37.8).
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS>
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS, bool SPLIT = false>
 __global__ void __launch_bounds__(kNumThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_c,
@@ -567,12 +618,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   const int kps = C::kPairsOfKBlocks ? p.kps : 1;  // k-blocks of a stage
   const int slot_bytes = kTall ? C::kABlockBytes + C::kEBlockBytes : kps * (C::kABytes + b_bytes + C::kEAlloc);
   uint8_t* b_ring = smem + p.stages * slot_bytes;
-  uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : 0);
+  uint8_t* epi = b_ring + (kTall ? p.b_stages * b_slot_bytes : SPLIT ? p.part_bytes : 0);
   Shared* sh = reinterpret_cast<Shared*>(epi + p.epi_bytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t cta_rank = CTAS == 2 ? ptx::cluster_ctarank() : 0;
-  const int cluster_id = blockIdx.x / CTAS, num_clusters = gridDim.x / CTAS;
+  static_assert(!SPLIT || can_split<KIND, SPARSE, CTAS, MBLK, B_MN>, "only INT32 sums may be split");
+  const int split_log = SPLIT ? p.split_log : 0, split_rank = SPLIT ? (int)ptx::cluster_ctarank() : 0;
+  const int cluster_id = SPLIT ? blockIdx.x >> split_log : blockIdx.x / CTAS;
+  const int num_clusters = SPLIT ? gridDim.x >> split_log : gridDim.x / CTAS;
+  // this CTA's k-blocks
+  const int kb_begin = SPLIT ? (p.k_blocks * split_rank) >> split_log : 0;
+  const int kb_end = SPLIT ? (p.k_blocks * (split_rank + 1)) >> split_log : p.k_blocks;
   const int num_tiles = p.m_tiles * p.n_tiles;
 
   // Set-up: lanes of a warp initialise the barriers, and the pair meets without a release.  All that a CTA of a pair has
@@ -590,11 +647,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       ptx::mbar_init(&sh->tmem_empty[lane], kEpiWarps * CTAS);  // one arrival per epilogue warp of the pair
     }
     if (C::staged_epilogue(CS, COLS) && lane < 2 * kEpiWarps) ptx::mbar_init(&sh->c_full[lane >> 1][lane & 1], 1);
+    if (SPLIT && lane == 0) ptx::mbar_init(&sh->split_full, kEpiWarps >> split_log);
     if (lane == 0) sh->abort = 0;
     ptx::fence_barrier_init();
     __syncwarp();
   }
-  if (CTAS == 2) ptx::cluster_arrive_relaxed();
+  if (CTAS == 2 || SPLIT) ptx::cluster_arrive_relaxed();
   if (warp == 1) {
     ptx::tmem_alloc<CTAS>(&sh->tmem_base, kTmemCols);
     ptx::tmem_relinquish<CTAS>();
@@ -768,9 +826,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           }
           continue;
         }
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
+        for (int kb = kb_begin; kb < kb_end; ++kb) {
           if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
-          if (p.test_skip_stage && t == cluster_id && kb == 1) {
+          if (p.test_skip_stage && t == cluster_id && kb == kb_begin + 1) {
             // test hook: this k-block of the first tile is neither armed nor loaded by either CTA, so
             // the MMA issuer's wait for it expires and every role leaves through the abort path
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -891,11 +949,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             release();
           }
         } else {
-          for (int kb = 0; kb < p.k_blocks; ++kb) {
+          for (int kb = kb_begin; kb < kb_end; ++kb) {
             if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t sa = ring + stage * slot_bytes;
-            multiply(kb, sa, sa + C::kABytes, sa + C::kABytes + b_bytes);
+            multiply(kb - kb_begin, sa, sa + C::kABytes, sa + C::kABytes + b_bytes);
             release();
           }
         }
@@ -914,8 +972,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // ------------------------------ epilogue ------------------------------
     if constexpr (!C::staged_epilogue(CS, COLS)) {
       // loads and stores by the epilogue warps themselves
-      epilogue_direct<KIND, CS, COLS, BLOCK_N, CTAS, MBLK, C::kAccStages>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
-                                                                          num_clusters, num_tiles, warp, lane);
+      if (SPLIT) ptx::cluster_wait();  // (the set-up's: the other CTAs' barriers are there)
+      epilogue_direct<KIND, CS, COLS, BLOCK_N, CTAS, MBLK, C::kAccStages, SPLIT>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
+                                                                          num_clusters, num_tiles, warp, lane, ptx::smem_u32(b_ring), split_rank);
+      // (all that this warp sends is on its way: the cluster may leave when every warp has come so far)
+      if (SPLIT) {
+        __syncwarp();
+        ptx::cluster_arrive_relaxed();
+      }
     } else {
     // 4-byte row-major outputs when every epilogue warp can have a box buffer of its own.  The two warps
     // of a lane quarter own its 32 accumulator rows and take its 32 x 32 boxes in turn: TMA load of the C
@@ -1027,6 +1091,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   }
 
   // ------------------------------ teardown ------------------------------
+  if (SPLIT && warp < kFirstEpiWarp) {
+    __syncwarp();
+    ptx::cluster_wait();
+    ptx::cluster_arrive_relaxed();
+  }
   ptx::tc_fence_before();
   __syncthreads();
   // after waits that were given up: copies issued before them, and the other CTA's arrivals, may still be landing in this
@@ -1043,21 +1112,24 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     // drain it also waits for D's stores: BERT FFN 12.4 against 12.1 us, device; large products the same.)
     ptx::cluster_arrive_relaxed();
     ptx::cluster_wait();
+  } else if (SPLIT) {
+    ptx::cluster_wait();  // (what was sent to this CTA has a waiter, split_full; after waits that were given up, settle() is it)
   }
   if (warp == 1) {
     __syncwarp();
     ptx::tc_fence_after();
     ptx::tmem_dealloc<CTAS>(tmem_base, kTmemCols);
   }
-  if (CTAS == 2) settle();
+  if (CTAS == 2 || SPLIT) settle();
 }
 
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
-sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, const void* A, const void* meta, const void* B,
+sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmParams& base, const void* A, const void* meta, const void* B,
                    cudaStream_t stream) {
   using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   GemmParams p = base;
-  p.tile_n = tile_n;
+  const int tile_n = p.tile_n = tile.tile_n;
+  p.split_log = can_split<KIND, SPARSE, CTAS, MBLK, B_MN> ? tile.split_log : 0;
   const int cs = elem_bytes(d->cd_type);
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); a staged epilogue gets what is left.
@@ -1065,9 +1137,13 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
   const uint32_t atom_elems = kAtomBytes / es;
   const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
-  p.kps = C::k_blocks_of_a_stage(tile_n, p.epi_bytes, (int64_t)a_cols, p.conv != 0);
+  p.kps = p.split_log ? 1 : C::k_blocks_of_a_stage(tile_n, p.epi_bytes, (int64_t)a_cols, p.conv != 0);
+  if (p.split_log) {  // (as epilogue_direct lays them out)
+    const int cols = cs == 4 ? 16 : 32;
+    p.part_bytes = ((1 << p.split_log) - 1) * (kEpiWarps >> p.split_log) * ((tile_n / cols + 1) / 2) * cols * 128;
+  }
   int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n) * p.kps;
-  p.stages = C::ring_stages(ring_bytes, p.epi_bytes);
+  p.stages = C::ring_stages(ring_bytes, p.epi_bytes + p.part_bytes);
   if constexpr (is_tall<CTAS, MBLK>) {
     tile_m = p.mblk * kBlockM;
     // slots of A (each k-block needs mblk) and of B: the split with the most of A in flight
@@ -1140,13 +1216,16 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
   }
   // the kernels of the output forms
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams);
-  Kernel forms[6] = {};
-#define SP24_FORM(CS_, COLS_) forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;
+  constexpr bool kCanSplit = can_split<KIND, SPARSE, CTAS, MBLK, B_MN>;
+  Kernel forms[6] = {}, split_forms[6] = {};
+#define SP24_FORM(CS_, COLS_)                                                                                   \
+  forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;              \
+  if constexpr (kCanSplit) split_forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, true>;
   if constexpr (KIND == 1) { SP24_FORM(1, false) SP24_FORM(1, true) }
   if constexpr (KIND != 2) { SP24_FORM(2, false) SP24_FORM(2, true) }
   if constexpr (BLOCK_N % 32 == 0) { SP24_FORM(4, false) SP24_FORM(4, true) }  // 240-column tiles: 2-byte outputs only
 #undef SP24_FORM
-  const Kernel kernel = forms[2 * (cs >> 1) + p.cd_col_major];
+  const Kernel kernel = (p.split_log ? split_forms : forms)[2 * (cs >> 1) + p.cd_col_major];
   if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
     // the shared-memory opt-in is per kernel and device: once is enough.  All forms at once, so that a call with one
@@ -1157,15 +1236,16 @@ sp24_status launch(int tile_n, const sp24_gemm_desc* d, const GemmParams& base, 
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 0 || dev >= 64 || !done[dev]) {
-      for (const Kernel k : forms)
-        if (k != nullptr) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+      for (int i = 0; i < 12; ++i)
+        if (const Kernel k = i < 6 ? forms[i] : split_forms[i - 6]) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
       if (dev >= 0 && dev < 64) done[dev] = true;
     }
   }
   const int tiles = p.m_tiles * p.n_tiles;
   int clusters = sm_count() / CTAS;
-  if (clusters > tiles) clusters = tiles;
-  return launch_overlapped(kernel, dim3((unsigned)(clusters * CTAS)), dim3(kNumThreads), C::kSmemBytes, stream, CTAS, map_a,
+  if (clusters > tiles || p.split_log) clusters = tiles;  // (k-blocks shared: one tile to a cluster)
+  const int cluster_ctas = CTAS << p.split_log;
+  return launch_overlapped(kernel, dim3((unsigned)(clusters * cluster_ctas)), dim3(kNumThreads), C::kSmemBytes, stream, cluster_ctas, map_a,
                            map_b, map_e, map_c, map_d, p);
 }
 
@@ -1178,7 +1258,7 @@ sp24_status launch_gemm(TileShape t, bool sparse, bool b_mn, const sp24_gemm_des
   auto is = [&](int ctas, int block_n, int mblk) { return t.ctas == ctas && t.block_n == block_n && t.mblk == mblk; };
 #define SP24_SHAPE(CT, BN, MB, MN)                                     \
   if (is(CT, BN, MB) && b_mn == MN)                                    \
-    return sparse ? launch<KIND, true, BN, CT, MB, MN>(t.tile_n, d, p, A, meta, B, s) : launch<KIND, false, BN, CT, MB, MN>(t.tile_n, d, p, A, meta, B, s);
+    return sparse ? launch<KIND, true, BN, CT, MB, MN>(t, d, p, A, meta, B, s) : launch<KIND, false, BN, CT, MB, MN>(t, d, p, A, meta, B, s);
   SP24_SHAPE(1, 128, 1, false)
   SP24_SHAPE(2, 224, 1, false)
   SP24_SHAPE(2, 224, 2, false)
@@ -1193,9 +1273,9 @@ sp24_status launch_gemm(TileShape t, bool sparse, bool b_mn, const sp24_gemm_des
     SP24_SHAPE(2, 240, 1, false)  // 2-byte outputs only
   }
   if constexpr (!tf32)  // dense variant only
-    if (is(2, 256, 2) && !sparse && !b_mn) return launch<KIND, false, 256, 2, 2, false>(t.tile_n, d, p, A, meta, B, s);
+    if (is(2, 256, 2) && !sparse && !b_mn) return launch<KIND, false, 256, 2, 2, false>(t, d, p, A, meta, B, s);
   if (t.ctas == 1 && t.block_n == 128 && (t.mblk == 2 || t.mblk == kTallBlocks) && sparse && !b_mn)
-    return launch<KIND, true, 128, 1, kTallBlocks, false>(t.tile_n, d, p, A, meta, B, s);
+    return launch<KIND, true, 128, 1, kTallBlocks, false>(t, d, p, A, meta, B, s);
 #undef SP24_SHAPE
   return SP24_ERR_UNSUPPORTED;
 }
