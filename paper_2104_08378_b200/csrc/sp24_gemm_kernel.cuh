@@ -306,19 +306,19 @@ __device__ __forceinline__ void widen_f16_accumulators(uint32_t (&r)[COLUMNS]) {
 // TMA-staged form of a 4-byte row-major box (rows of 128 bytes in the TMA's 128-byte swizzle: 16-byte
 // unit v of row r sits at unit v ^ (r & 7), which also keeps the row-per-thread accesses free of bank
 // conflicts): C, if any, is in the staging buffer; the result replaces it there.
-template <int KIND>
+template <int KIND, bool HAS_C>
 __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint8_t* buf, int lane, const GemmParams& p,
                                                    float scale, float bias) {
   uint32_t c[32], o[32];
   uint8_t* row = buf + lane * 128;
-  if (p.has_c) {
+  if (HAS_C) {
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
       const uint4 x = *reinterpret_cast<const uint4*>(row + ((v ^ (lane & 7)) << 4));
       c[4 * v] = x.x; c[4 * v + 1] = x.y; c[4 * v + 2] = x.z; c[4 * v + 3] = x.w;
     }
   }
-  compute_row<KIND, 4, 32>(r, c, p.has_c != 0, p, scale, bias, o);
+  compute_row<KIND, 4, 32>(r, c, HAS_C, p, scale, bias, o);
 #pragma unroll
   for (int v = 0; v < 8; ++v)
     *reinterpret_cast<uint4*>(row + ((v ^ (lane & 7)) << 4)) = make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
@@ -348,7 +348,7 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // half as wide, meet in pairs).
 // C is loaded in the order of the stores (whole 64-byte row segments as well) into registers, four boxes ahead, the
 // first four of a tile before its accumulators are complete, and goes to the rows' owners through the buffer.
-template <int KIND, int CS, bool COLS, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES, bool SPLIT>
+template <int KIND, int CS, bool COLS, bool HAS_C, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES, bool SPLIT>
 __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
                                               int lane, uint32_t parts, int split_rank) {
@@ -364,7 +364,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   uint8_t* Db = static_cast<uint8_t*>(p.D);
   const size_t ldc_b = (size_t)p.ldc * CS, ldd_b = (size_t)p.ldd * CS;
   const int M = (int)p.M, N = (int)p.N;
-  const bool has_c = CS != 1 && !(KIND == 1 && CS == 2) && p.has_c != 0;  // (int8: only INT32 results are added to)
+  constexpr bool has_c = HAS_C;
   // this lane's row of the buffer, its unit 0 under the swizzle (xor the unit into bits 4..5) ...
   const uint32_t own_row = ptx::smem_u32(stage) + (uint32_t)(lane * 64 + ((((lane >> 1) ^ (lane >> 3)) & 3) << 4));
   // ... for ldmatrix / stmatrix ...
@@ -599,10 +599,12 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   }
 }
 
-// CS, COLS: bytes of an output element, column-major output.  A kernel for each form of the output, so that it holds
-// one epilogue: with all of them behind branches of one kernel, a tile's epilogue took up to twice as long whatever
-// the form (us, branches -> own kernels: bf16 24576 x 224 x 4096 with 512 x 224 tiles 39.8 -> 34.3, with C 43.6 -> 37.8).
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS, bool SPLIT = false>
+// CS, COLS, HAS_C: bytes of an output element, column-major output, C is added.  A kernel for each form of the output, so that
+// it holds one epilogue: with all of them behind branches of one kernel, a tile's epilogue took up to twice as long whatever
+// the form (us, branches -> own kernels: bf16 24576 x 224 x 4096 with 512 x 224 tiles 39.8 -> 34.3, with C 43.6 -> 37.8).  With
+// and without C apart (the registers of four boxes of it): f16 256 x 256 x 512 3.29 -> 3.19, BERT FFN 12.48 -> 12.26, bf16
+// 8480 x 896 x 384 7.83 -> 7.46, with C 9920 x 544 x 1216 16.1 -> 15.6, f16 1184 x 736 x 1008 5.92 -> 5.82; none slower.
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS, bool HAS_C, bool SPLIT = false>
 __global__ void __launch_bounds__(kNumThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_c,
@@ -661,7 +663,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     ptx::prefetch_tensormap(&map_b);
     if (SPARSE) ptx::prefetch_tensormap(&map_e);
     if (C::staged_epilogue(CS, COLS)) {
-      if (p.has_c) ptx::prefetch_tensormap(&map_c);
+      if (HAS_C) ptx::prefetch_tensormap(&map_c);
       ptx::prefetch_tensormap(&map_d);
     }
   }
@@ -973,7 +975,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if constexpr (!C::staged_epilogue(CS, COLS)) {
       // loads and stores by the epilogue warps themselves
       if (SPLIT) ptx::cluster_wait();  // (the set-up's: the other CTAs' barriers are there)
-      epilogue_direct<KIND, CS, COLS, BLOCK_N, CTAS, MBLK, C::kAccStages, SPLIT>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
+      epilogue_direct<KIND, CS, COLS, HAS_C, BLOCK_N, CTAS, MBLK, C::kAccStages, SPLIT>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
                                                                           num_clusters, num_tiles, warp, lane, ptx::smem_u32(b_ring), split_rank);
       // (all that this warp sends is on its way: the cluster may leave when every warp has come so far)
       if (SPLIT) {
@@ -1027,7 +1029,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
       }
     };
-    if (p.has_c && lane == 0) issue_c_load();
+    if (HAS_C && lane == 0) issue_c_load();
 
     int acc = 0;
     uint32_t acc_phase = 0, seq = 0;
@@ -1053,7 +1055,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (!box_of(mt, nt, it, row0, col0)) continue;  // same answer for the whole warp
         const int b = seq % nbuf;
         uint8_t* buf = my_bufs + b * buf_bytes;
-        if (p.has_c && !bounded_wait(&sh->c_full[ew][b], (seq / nbuf) & 1u, sh, p.status, 5u, p.wait_limit)) { ok = false; break; }
+        if (HAS_C && !bounded_wait(&sh->c_full[ew][b], (seq / nbuf) & 1u, sh, p.status, 5u, p.wait_limit)) { ok = false; break; }
         if (KIND == 0 && p.acc_f16) widen_f16_accumulators(r);
         float scale = 1.f, bias = 0.f;
         if (KIND == 1 && p.dequant) {
@@ -1062,7 +1064,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           scale = p.row_scale[row];
           bias = p.bias ? p.bias[row] : 0.f;
         }
-        convert_row_staged<KIND>(r, buf, lane, p, scale, bias);
+        convert_row_staged<KIND, HAS_C>(r, buf, lane, p, scale, bias);
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
@@ -1071,7 +1073,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           // the buffer claimed next is free once the store that used it last has read it
           if (nbuf == 2) ptx::bulk_wait_group_read<1>();
           else ptx::bulk_wait_group_read<0>();
-          if (p.has_c) issue_c_load();
+          if (HAS_C) issue_c_load();
         }
         __syncwarp();
         ++seq;
@@ -1217,15 +1219,18 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   // the kernels of the output forms
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams);
   constexpr bool kCanSplit = can_split<KIND, SPARSE, CTAS, MBLK, B_MN>;
-  Kernel forms[6] = {}, split_forms[6] = {};
-#define SP24_FORM(CS_, COLS_)                                                                                   \
-  forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_>;              \
-  if constexpr (kCanSplit) split_forms[2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, true>;
-  if constexpr (KIND == 1) { SP24_FORM(1, false) SP24_FORM(1, true) }
-  if constexpr (KIND != 2) { SP24_FORM(2, false) SP24_FORM(2, true) }
-  if constexpr (BLOCK_N % 32 == 0) { SP24_FORM(4, false) SP24_FORM(4, true) }  // 240-column tiles: 2-byte outputs only
+  Kernel forms[24] = {};  // [split][with C][bytes][order]
+#define SP24_FORM(CS_, COLS_, C_)                                                                                                   \
+  forms[6 * C_ + 2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, C_>;                     \
+  if constexpr (kCanSplit) forms[12 + 6 * C_ + 2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, C_, true>;
+  if constexpr (KIND == 1) { SP24_FORM(1, false, false) SP24_FORM(1, true, false) }
+  if constexpr (KIND != 2) { SP24_FORM(2, false, false) SP24_FORM(2, true, false) }
+  if constexpr (KIND != 2 && KIND != 1) { SP24_FORM(2, false, true) SP24_FORM(2, true, true) }  // (int8: only INT32 results are added to)
+  if constexpr (BLOCK_N % 32 == 0) {  // 240-column tiles: 2-byte outputs only
+    SP24_FORM(4, false, false) SP24_FORM(4, true, false) SP24_FORM(4, false, true) SP24_FORM(4, true, true)
+  }
 #undef SP24_FORM
-  const Kernel kernel = (p.split_log ? split_forms : forms)[2 * (cs >> 1) + p.cd_col_major];
+  const Kernel kernel = forms[12 * (p.split_log != 0) + 6 * p.has_c + 2 * (cs >> 1) + p.cd_col_major];
   if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
     // the shared-memory opt-in is per kernel and device: once is enough.  All forms at once, so that a call with one
@@ -1236,8 +1241,8 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 0 || dev >= 64 || !done[dev]) {
-      for (int i = 0; i < 12; ++i)
-        if (const Kernel k = i < 6 ? forms[i] : split_forms[i - 6]) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+      for (const Kernel k : forms)
+        if (k != nullptr) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
       if (dev >= 0 && dev < 64) done[dev] = true;
     }
   }
