@@ -31,7 +31,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <mutex>
+#include <atomic>
 
 #include "sp24_gemm.cuh"
 #include "sp24_ptx.cuh"
@@ -1233,17 +1233,17 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   const Kernel kernel = forms[12 * (p.split_log != 0) + 6 * p.has_c + 2 * (cs >> 1) + p.cd_col_major];
   if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
-    // the shared-memory opt-in is per kernel and device: once is enough.  All forms at once, so that a call with one
-    // form also loads the others' code: none is loaded for the first time inside a stream capture after that.
-    static std::mutex mu;
-    static bool done[64] = {};
+    // the shared-memory opt-in is per kernel and device: once is enough (by several threads at a time does no harm).  All
+    // forms at once, so that a call with one form also loads the others' code: none is loaded for the first time inside a
+    // stream capture after that.
+    static std::atomic<bool> done[64];
     int dev = 0;
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !done[dev]) {
+    const bool kept = dev >= 0 && dev < 64;
+    if (!kept || !done[dev].load(std::memory_order_acquire)) {
       for (const Kernel k : forms)
         if (k != nullptr) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-      if (dev >= 0 && dev < 64) done[dev] = true;
+      if (kept) done[dev].store(true, std::memory_order_release);
     }
   }
   const int tiles = p.m_tiles * p.n_tiles;
