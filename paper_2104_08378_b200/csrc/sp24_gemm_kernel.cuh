@@ -123,6 +123,15 @@ struct Cfg {
                 "tensor memory overflow");
 };
 
+// Kernels with twelve epilogue warps beside the ones with eight (WARPS): int8 results of pairs, whose arithmetic is the longest,
+// on a short K in several rounds of tiles, where it and not the main loop bounds a round.  Up to six k-blocks, us, device, eight
+// warps and twelve: 3072 x 4096 x 256 10.3, 9.7; x 768 11.2, 10.6; x 1536 13.0, 12.4; 10944 x 5824 x 512 40.2, 37.1.  Not on a
+// longer K (x 2048 14.3, 14.6) or in one round (288 x 4736 x 1344 5.4, 5.6); not for 16-bit results (4096 x 4096 x 768 12.5, 12.1
+// but 9632 x 13344 x 416 70, 72, the stores bound it), other kinds (BERT FFN the same with twelve or sixteen) or wider tiles,
+// whose ring would lose a stage.
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
+constexpr bool twelve_warps = KIND == 1 && SPARSE && CTAS == 2 && MBLK == 1 && !B_MN && BLOCK_N == 224;
+
 struct Shared {
   uint64_t full[12], empty[12], tmem_full[2], tmem_empty[2];
   uint64_t split_full;             // the other CTAs' parts of the boxes that this one finishes are there
@@ -348,7 +357,7 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // half as wide, meet in pairs).
 // C is loaded in the order of the stores (whole 64-byte row segments as well) into registers, four boxes ahead, the
 // first four of a tile before its accumulators are complete, and goes to the rows' owners through the buffer.
-template <int KIND, int CS, bool COLS, bool HAS_C, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES, bool SPLIT>
+template <int KIND, int CS, bool COLS, bool HAS_C, int BLOCK_N, int CTAS, int MBLK, int ACC_STAGES, int WARPS, bool SPLIT>
 __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh, uint8_t* epi, uint32_t tmem_base,
                                               int cta_rank, int cluster_id, int num_clusters, int num_tiles, int warp,
                                               int lane, uint32_t parts, int split_rank) {
@@ -358,7 +367,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
   constexpr int kUnits = W / 4;             // 16-byte units of a buffer row that hold data
   constexpr int kUnitElems = 16 / CS;       // elements per 16-byte unit
   constexpr int kRowsPerStore = 32 / kUnits;
-  const int q = warp & 3, half = (warp - kFirstEpiWarp) >> 2;
+  const int q = warp & 3, turn = (warp - kFirstEpiWarp) >> 2;  // lane quarter, and first box of this warp there
   uint8_t* stage = epi + (warp - kFirstEpiWarp) * 2048;
   const uint8_t* Cb = static_cast<const uint8_t*>(p.C);
   uint8_t* Db = static_cast<uint8_t*>(p.D);
@@ -392,7 +401,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
     int mt, nt;
     tile_coords(t, p, mt, nt);
     const int tile_col = nt * p.tile_n, col_end = min(N, tile_col + p.tile_n);  // columns of this tile stop here
-    // the boxes of this lane quarter: `nsub` in a row, `blocks` rows of them (m-blocks); this warp takes every other one
+    // the boxes of this lane quarter: `nsub` in a row, `blocks` rows of them (m-blocks); the warps take them in turn
     const int row_q = (is_tall<CTAS, MBLK> ? mt * p.mblk * kBlockM : first_row<CTAS, MBLK>(mt, cta_rank, M)) + q * 32;
     const int nsub = (col_end - tile_col + kCols - 1) / kCols;
     const int blocks = min(is_tall<CTAS, MBLK> ? p.mblk : live_blocks<CTAS, MBLK>(mt, M), (M - row_q + kBlockM - 1) / kBlockM);
@@ -401,7 +410,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
       while (sc >= nsub) { sc -= nsub; ++j; }
     };
     int j = 0, sc = 0;  // the box at hand
-    step(j, sc, half);
+    step(j, sc, turn);
     // C values of a box, in the order of the stores
     auto load_c = [&](int row0, int col0, uint32_t (&c)[W]) {
       if constexpr (CS == 1) {
@@ -518,11 +527,11 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
     int cj = j, csc = sc;  // has_c: the next box whose C values are fetched
     auto fetch_c = [&](uint32_t (&c)[W]) {
       if (cj < blocks) load_c(row_q + cj * kBlockM, tile_col + csc * kCols, c);
-      step(cj, csc, kEpiWarps / 4);
+      step(cj, csc, WARPS / 4);
     };
     auto box = [&](uint32_t (&c)[W]) -> bool {
       const int row0 = row_q + j * kBlockM, col0 = tile_col + sc * kCols, j0 = j, sc0 = sc;
-      step(j, sc, kEpiWarps / 4);
+      step(j, sc, WARPS / 4);
       const bool more = j < blocks;
       uint32_t o[W];
       if (has_c) share_c(c);
@@ -562,7 +571,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
       if (!mine) {
         const uint32_t bar = ptx::map_to_cta(ptx::smem_u32(&sh->split_full), (uint32_t)owner);
 #pragma unroll 1
-        for (; j < blocks; step(j, sc, kEpiWarps / 4)) {
+        for (; j < blocks; step(j, sc, WARPS / 4)) {
           const uint32_t to = ptx::map_to_cta(part_of(split_rank, sc), (uint32_t)owner);
           ptx::tmem_ld_32x32b(t_acc + sc * kCols, r);
           ptx::tmem_ld_wait(r);
@@ -571,7 +580,7 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
         }
       } else {
         if (lane == 0) {
-          const int boxes = blocks > 0 && nsub > half ? (nsub - half + 1) / 2 : 0;
+          const int boxes = blocks > 0 && nsub > turn ? (nsub - turn + 1) / 2 : 0;
           ptx::mbar_expect_tx(&sh->split_full, (uint32_t)(boxes * (split - 1) * kCols * 128));
         }
         if (!bounded_wait<true>(&sh->split_full, 0, sh, p.status, 6u, p.wait_limit)) break;
@@ -604,8 +613,8 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
 // the form (us, branches -> own kernels: bf16 24576 x 224 x 4096 with 512 x 224 tiles 39.8 -> 34.3, with C 43.6 -> 37.8).  With
 // and without C apart (the registers of four boxes of it): f16 256 x 256 x 512 3.29 -> 3.19, BERT FFN 12.48 -> 12.26, bf16
 // 8480 x 896 x 384 7.83 -> 7.46, with C 9920 x 544 x 1216 16.1 -> 15.6, f16 1184 x 736 x 1008 5.92 -> 5.82; none slower.
-template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS, bool HAS_C, bool SPLIT = false>
-__global__ void __launch_bounds__(kNumThreads, 1)
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN, int CS, bool COLS, bool HAS_C, bool SPLIT = false, int WARPS = kEpiWarps>
+__global__ void __launch_bounds__(32 * (kFirstEpiWarp + WARPS), 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_c,
             const __grid_constant__ CUtensorMap map_d, const GemmParams p) {
@@ -625,6 +634,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t cta_rank = CTAS == 2 ? ptx::cluster_ctarank() : 0;
+  static_assert(WARPS == kEpiWarps || !(SPLIT || C::staged_epilogue(CS, COLS)), "these count on eight epilogue warps");
   static_assert(!SPLIT || can_split<KIND, SPARSE, CTAS, MBLK, B_MN>, "only INT32 sums may be split");
   const int split_log = SPLIT ? p.split_log : 0, split_rank = SPLIT ? (int)ptx::cluster_ctarank() : 0;
   const int cluster_id = SPLIT ? blockIdx.x >> split_log : blockIdx.x / CTAS;
@@ -646,7 +656,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
     if (lane < 2) {
       ptx::mbar_init(&sh->tmem_full[lane], 1);
-      ptx::mbar_init(&sh->tmem_empty[lane], kEpiWarps * CTAS);  // one arrival per epilogue warp of the pair
+      ptx::mbar_init(&sh->tmem_empty[lane], WARPS * CTAS);  // one arrival per epilogue warp of the pair
     }
     if (C::staged_epilogue(CS, COLS) && lane < 2 * kEpiWarps) ptx::mbar_init(&sh->c_full[lane >> 1][lane & 1], 1);
     if (SPLIT && lane == 0) ptx::mbar_init(&sh->split_full, kEpiWarps >> split_log);
@@ -975,7 +985,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if constexpr (!C::staged_epilogue(CS, COLS)) {
       // loads and stores by the epilogue warps themselves
       if (SPLIT) ptx::cluster_wait();  // (the set-up's: the other CTAs' barriers are there)
-      epilogue_direct<KIND, CS, COLS, HAS_C, BLOCK_N, CTAS, MBLK, C::kAccStages, SPLIT>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
+      epilogue_direct<KIND, CS, COLS, HAS_C, BLOCK_N, CTAS, MBLK, C::kAccStages, WARPS, SPLIT>(p, sh, epi, tmem_base, (int)cta_rank, cluster_id,
                                                                           num_clusters, num_tiles, warp, lane, ptx::smem_u32(b_ring), split_rank);
       // (all that this warp sends is on its way: the cluster may leave when every warp has come so far)
       if (SPLIT) {
@@ -1135,7 +1145,11 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   const int cs = elem_bytes(d->cd_type);
   // Shared-memory split.  The ring comes first (these kernels are bound by the operand feed: one
   // stage less cost the int8 configuration 9 %); a staged epilogue gets what is left.
-  p.epi_bytes = kEpiWarps * (C::staged_epilogue(cs, p.cd_col_major) ? 4096 : 2048);
+  constexpr bool kTwelve = twelve_warps<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
+  int tile_m = kBlockM * CTAS * MBLK;
+  const int warps = kTwelve && cs == 1 && d->K <= 6 * C::kKPerStage &&
+                            (d->M + tile_m - 1) / tile_m * ((d->N + tile_n - 1) / tile_n) > sm_count() / CTAS ? 12 : kEpiWarps;
+  p.epi_bytes = warps * (C::staged_epilogue(cs, p.cd_col_major) ? 4096 : 2048);
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
   const uint32_t atom_elems = kAtomBytes / es;
   const uint64_t a_cols = SPARSE ? d->K / 2 : d->K;
@@ -1144,7 +1158,7 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
     const int cols = cs == 4 ? 16 : 32;
     p.part_bytes = ((1 << p.split_log) - 1) * (kEpiWarps >> p.split_log) * ((tile_n / cols + 1) / 2) * cols * 128;
   }
-  int tile_m = kBlockM * CTAS * MBLK, ring_bytes = C::stage_bytes(tile_n) * p.kps;
+  int ring_bytes = C::stage_bytes(tile_n) * p.kps;
   p.stages = C::ring_stages(ring_bytes, p.epi_bytes + p.part_bytes);
   if constexpr (is_tall<CTAS, MBLK>) {
     tile_m = p.mblk * kBlockM;
@@ -1219,9 +1233,10 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   // the kernels of the output forms
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmParams);
   constexpr bool kCanSplit = can_split<KIND, SPARSE, CTAS, MBLK, B_MN>;
-  Kernel forms[24] = {};  // [split][with C][bytes][order]
+  Kernel forms[24] = {}, twelve[2] = {};  // [split][with C][bytes][order]
 #define SP24_FORM(CS_, COLS_, C_)                                                                                                   \
   forms[6 * C_ + 2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, C_>;                     \
+  if constexpr (kTwelve && CS_ == 1) twelve[COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, false, false, 12>; \
   if constexpr (kCanSplit) forms[12 + 6 * C_ + 2 * (CS_ >> 1) + COLS_] = gemm_kernel<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN, CS_, COLS_, C_, true>;
   if constexpr (KIND == 1) { SP24_FORM(1, false, false) SP24_FORM(1, true, false) }
   if constexpr (KIND != 2) { SP24_FORM(2, false, false) SP24_FORM(2, true, false) }
@@ -1230,7 +1245,7 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
     SP24_FORM(4, false, false) SP24_FORM(4, true, false) SP24_FORM(4, false, true) SP24_FORM(4, true, true)
   }
 #undef SP24_FORM
-  const Kernel kernel = forms[12 * (p.split_log != 0) + 6 * p.has_c + 2 * (cs >> 1) + p.cd_col_major];
+  const Kernel kernel = warps == 12 ? twelve[p.cd_col_major] : forms[12 * (p.split_log != 0) + 6 * p.has_c + 2 * (cs >> 1) + p.cd_col_major];
   if (kernel == nullptr) return SP24_ERR_UNSUPPORTED;
   {
     // the shared-memory opt-in is per kernel and device: once is enough (by several threads at a time does no harm).  All
@@ -1241,8 +1256,8 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
     SP24_CUDA_CHECK(cudaGetDevice(&dev));
     const bool kept = dev >= 0 && dev < 64;
     if (!kept || !done[dev].load(std::memory_order_acquire)) {
-      for (const Kernel k : forms)
-        if (k != nullptr) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+      for (int i = 0; i < 26; ++i)
+        if (const Kernel k = i < 24 ? forms[i] : twelve[i - 24]) SP24_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
       if (kept) done[dev].store(true, std::memory_order_release);
     }
   }
@@ -1250,7 +1265,7 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   int clusters = sm_count() / CTAS;
   if (clusters > tiles || p.split_log) clusters = tiles;  // (k-blocks shared: one tile to a cluster)
   const int cluster_ctas = CTAS << p.split_log;
-  return launch_overlapped(kernel, dim3((unsigned)(clusters * cluster_ctas)), dim3(kNumThreads), C::kSmemBytes, stream, cluster_ctas, map_a,
+  return launch_overlapped(kernel, dim3((unsigned)(clusters * cluster_ctas)), dim3(32 * (kFirstEpiWarp + warps)), C::kSmemBytes, stream, cluster_ctas, map_a,
                            map_b, map_e, map_c, map_d, p);
 }
 
