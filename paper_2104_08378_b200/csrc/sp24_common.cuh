@@ -82,6 +82,25 @@ inline sp24_status launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
 // ---- streaming kernels ----------------------------------------------------------------------------------
 constexpr int kThreads = 256;
 
+__device__ __forceinline__ uint4 ld_stream(const void* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ void st_stream(void* p, uint4 v) { __stcs(reinterpret_cast<uint4*>(p), v); }
+// 32 bytes at a 32-byte boundary, read or written once.
+__device__ __forceinline__ void ld_stream32(const void* p, uint4 (&v)[2]) {
+  asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x), "=r"(v[1].y), "=r"(v[1].z), "=r"(v[1].w)
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st_stream32(void* p, const uint4 (&v)[2]) {
+  asm volatile("st.global.L1::no_allocate.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0].x),
+               "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w)
+               : "memory");
+}
+
+// What a kernel that works on cells (32 bytes of a row, see compress_kernel) may do with a whole one at once: read or write 32
+// bytes, write 16 bytes of values of an 8-bit type.
+enum { kWideX = 1, kWideY = 2, kWideVals = 4 };
+
 // Block shape and grid of the vectorised kernels for `units` work units per row and `rows` rows:
 // TX (a power of two, 32..256) threads along the row, chosen to waste the fewest lanes.
 struct RowLaunch {

@@ -143,31 +143,107 @@ __global__ void __launch_bounds__(kThreads) kept_magnitude_perm_kernel(const uin
 }
 
 // ---- apply mask -----------------------------------------------------------------------------------
-// Vector path.  Work unit: one 16-byte vector (two groups of a 16-bit type = one metadata byte, four of an 8-bit type =
-// two bytes); launch geometry and unrolling as in prune_vec_kernel, metadata addresses as in compress_kernel.  A metadata
-// nibble indexes a table of byte-permute selectors that copy the two positions it names and zero the others.
+// A metadata nibble indexes a table of byte-permute selectors that copy the two positions it names and zero the others (16 words:
+// no two of them share a bank).
+template <int ES>
+__device__ __forceinline__ void mask_selectors(uint32_t (&table)[16], uint32_t t) {
+  if (t < 16) {
+    const uint32_t keep = (1u << (t & 3u)) | (1u << (t >> 2));
+    // selector nibble 4 = a zero byte of the second operand; 16-bit types: a selector for each of a group's two words
+    uint32_t sel = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i)
+      sel |= ES == 2 ? ((keep >> i) & 1u ? (i & 1u ? 0x32u : 0x10u) : 0x44u) << (8 * i) : ((keep >> i) & 1u ? i : 4u) << (4 * i);
+    table[t] = sel;
+  }
+  __syncthreads();
+}
+
+// Rows of whole cells (32 bytes) at 32-byte boundaries: cells of two rows to a thread and metadata addresses as in compress_kernel,
+// so that a thread's metadata is one or two words.
+// Bound by HBM, by the instructions where the rows are short.  The result is stored without an evict-first hint: it is
+// compressed next, and as much of it as fits is then read from the L2.  With 16-byte units of one row, a metadata byte or two read
+// for each, a vector took 59 instructions (int8 76).  Us, device, with the compression, units and cells: bf16 49152 x 256 18.4,
+// 13.4; 16102 x 1088 21.8, 20.4; 4096 x 4096 18.3, 17.8; 12288 x 3072 36.1, 35.8; 49152 x 12288 639, 640; int8 49152 x 256 17.4,
+// 9.1; 12288 x 3072 24.7, 24.1.  (Cells by two 16-byte accesses at other boundaries: 5 to 20 % slower than the units.)
+template <int ES, bool HW, bool FULL>
+__global__ void __launch_bounds__(kThreads, 5) apply_mask_vec_kernel(const uint8_t* w, int64_t row_bytes_w, const uint8_t* meta,
+                                                                     uint8_t* y, int64_t row_bytes_y, int64_t M, int64_t K,
+                                                                     uint32_t row_groups, uint32_t KB, int cell_shift) {
+  constexpr uint32_t kCols = ES == 2 ? 16 : 32;  // columns of a cell
+  __shared__ uint32_t table[16];
+  mask_selectors<ES>(table, threadIdx.x);
+  wait_for_stream();
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t rows_of_warp = 32u >> cell_shift, cell = (blockIdx.x << cell_shift) + (lane & ((1u << cell_shift) - 1u));
+  const uint32_t thread_row = warp * rows_of_warp + (lane >> cell_shift);  // eight of these to a row group
+  const uint32_t in_group = thread_row & 7u, step = gridDim.y * rows_of_warp;
+  if (!FULL && (int64_t)cell * kCols >= K) return;
+  const uint32_t chunk = ES == 2 ? cell : 2 * cell;
+  const uint8_t* const meta_cell0 = meta + (!HW ? 2 * chunk
+                                                : (chunk >> 3) * 2048u + 16u * in_group +
+                                                      (ES == 2 ? 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * (chunk & 7u)));
+  uint32_t n = blockIdx.y * rows_of_warp + (thread_row >> 3);  // row group
+  const int64_t row0 = (int64_t)n * 16 + in_group;
+  const uint8_t* wp = w + row0 * row_bytes_w + (int64_t)cell * 32;
+  uint8_t* yp = y + row0 * row_bytes_y + (int64_t)cell * 32;
+#pragma unroll 1
+  for (; n < row_groups; n += step, wp += (int64_t)step * 16 * row_bytes_w, yp += (int64_t)step * 16 * row_bytes_y) {
+    uint4 in[2][2];
+    bool live[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      live[h] = FULL || (int64_t)n * 16 + in_group + 8 * h < M;
+      if (live[h]) ld_stream32(wp + 8 * h * row_bytes_w, in[h]);
+    }
+    uint32_t bits[2] = {0, 0};  // 16-bit types: in the lower half
+    if constexpr (HW) {
+      const uint8_t* mr = meta_cell0 + ((uint64_t)(n >> 3) * KB << 11) + 256u * (n & 7u);
+      bits[0] = *reinterpret_cast<const uint32_t*>(mr);
+      bits[1] = ES == 2 ? bits[0] >> 16 : *reinterpret_cast<const uint32_t*>(mr + 128);
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!live[h]) continue;
+        const uint16_t* mr = reinterpret_cast<const uint16_t*>(meta_cell0 + ((int64_t)n * 16 + in_group + 8 * h) * (K >> 3));
+        bits[h] = mr[0];
+        if (ES == 1) bits[h] |= (uint32_t)mr[1] << 16;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!live[h]) continue;
+      uint32_t v[8] = {in[h][0].x, in[h][0].y, in[h][0].z, in[h][0].w, in[h][1].x, in[h][1].y, in[h][1].z, in[h][1].w};
+#pragma unroll
+      for (int g = 0; g < 8 / ES; ++g) {
+        const uint32_t sel = table[(bits[h] >> (4 * g)) & 15u];
+        if constexpr (ES == 2) {
+          v[2 * g] = __byte_perm(v[2 * g], 0, sel & 0xFFFFu);
+          v[2 * g + 1] = __byte_perm(v[2 * g + 1], 0, sel >> 16);
+        } else {
+          v[g] = __byte_perm(v[g], 0, sel);
+        }
+      }
+      uint8_t* dst = yp + 8 * h * row_bytes_y;
+      asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                   "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                   : "memory");
+    }
+  }
+}
+
+// Operands at 16-byte boundaries.  Work unit: one 16-byte vector (two groups of a 16-bit type = one metadata byte, four of an 8-bit type =
+// two bytes); launch geometry and unrolling as in prune_vec_kernel, metadata addresses as in compress_kernel.
 // Bound by HBM.  The result is stored without an evict-first hint: it is compressed next, and as much of it as fits is then
 // read from the L2.  One chunk of 16 columns per thread, metadata decoded by arithmetic and evict-first stores before; us, device,
 // before and now: bf16 12288 x 3072 23.5 -> 22.7, followed by its compression 43.4 -> 40.9 (42.7 with evict-first stores);
 // bf16 49152 x 12288 458 -> 361; int8 12288 x 3072 15.2 -> 9.4.
 template <int ES, int UNROLL, bool HW>
-__global__ void __launch_bounds__(kThreads) apply_mask_vec_kernel(const uint8_t* w, int64_t row_bytes_w, const uint8_t* meta,
+__global__ void __launch_bounds__(kThreads) apply_mask_units_kernel(const uint8_t* w, int64_t row_bytes_w, const uint8_t* meta,
                                                                   uint8_t* y, int64_t row_bytes_y, int64_t M, int64_t K,
                                                                   int64_t KB) {
   __shared__ uint32_t table[16];
-  {
-    const uint32_t t = threadIdx.y * blockDim.x + threadIdx.x;
-    if (t < 16) {
-      const uint32_t keep = (1u << (t & 3u)) | (1u << (t >> 2));
-      // selector nibble 4 = a zero byte of the second operand; 16-bit types: a selector for each of a group's two words
-      uint32_t sel = 0;
-#pragma unroll
-      for (uint32_t i = 0; i < 4; ++i)
-        sel |= ES == 2 ? ((keep >> i) & 1u ? (i & 1u ? 0x32u : 0x10u) : 0x44u) << (8 * i) : ((keep >> i) & 1u ? i : 4u) << (4 * i);
-      table[t] = sel;
-    }
-    __syncthreads();
-  }
+  mask_selectors<ES>(table, threadIdx.y * blockDim.x + threadIdx.x);
   wait_for_stream();
   const uint32_t units = (uint32_t)(K * ES >> 4), u0 = blockIdx.x * UNROLL * blockDim.x + threadIdx.x;
   uint32_t moff[UNROLL];  // metadata offset of this thread's units inside a row: fixed for the whole kernel
@@ -412,15 +488,36 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
   const int es = elem_bytes(t);
   if (K % 16 == 0 && aligned16(w) && aligned16(y) && aligned16(meta) && (ldw * es) % 16 == 0 && (ldy * es) % 16 == 0 &&
       row_offsets_fit(K, es, l)) {
+    const bool hw = l == SP24_META_TCGEN05;
+    const int64_t cols = es == 2 ? 16 : 32, cells = K / cols;
+    auto by32 = [&](const void* p, int64_t ld) { return reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
+    if (K % cols == 0 && by32(w, ldw) && by32(y, ldy)) {
+      // Cells of a row to a warp: 32, 16 or 8, the most of which few lanes are idle (32 and fewer, us, with the compression: bf16
+      // 49152 x 256 15.3, 13.5; 49152 x 12288 640, 645; 6088 x 11632, whose 727 cells are whole only by 8, 77.4, 78.3).
+      auto padded = [&](int log) { return (cells + (1 << log) - 1) >> log << log; };
+      const int64_t most = padded(3) + cells / 16;
+      const int shift = padded(5) <= most ? 5 : padded(4) <= most ? 4 : 3;
+      const int64_t units = padded(shift) >> shift, groups = (M + 15) / 16, per_block = 32 >> shift;
+      int64_t steps = (groups + per_block - 1) / per_block;
+      if (steps > 32768) steps = 32768;
+      const bool full = M % 16 == 0 && cells == units << shift;
+      auto launch = [&](auto kernel) {
+        return launch_overlapped(kernel, dim3((unsigned)units, (unsigned)steps, 1), dim3(kThreads), 0, s, 1, (const uint8_t*)w, ldw * es,
+                                 (const uint8_t*)meta, (uint8_t*)y, ldy * es, M, K, (uint32_t)groups, (uint32_t)KB, shift);
+      };
+      if (es == 2 && full) return hw ? launch(apply_mask_vec_kernel<2, true, true>) : launch(apply_mask_vec_kernel<2, false, true>);
+      if (es == 2) return hw ? launch(apply_mask_vec_kernel<2, true, false>) : launch(apply_mask_vec_kernel<2, false, false>);
+      if (full) return hw ? launch(apply_mask_vec_kernel<1, true, true>) : launch(apply_mask_vec_kernel<1, false, true>);
+      return hw ? launch(apply_mask_vec_kernel<1, true, false>) : launch(apply_mask_vec_kernel<1, false, false>);
+    }
     constexpr int UNROLL = 4;
     const RowLaunch L(K * es / 16, M, UNROLL);
     auto launch = [&](auto kernel) {
       return launch_overlapped(kernel, L.grid, L.block, 0, s, 1, (const uint8_t*)w, ldw * es, (const uint8_t*)meta, (uint8_t*)y,
                                ldy * es, M, K, KB);
     };
-    const bool hw = l == SP24_META_TCGEN05;
-    if (es == 2) return hw ? launch(apply_mask_vec_kernel<2, UNROLL, true>) : launch(apply_mask_vec_kernel<2, UNROLL, false>);
-    return hw ? launch(apply_mask_vec_kernel<1, UNROLL, true>) : launch(apply_mask_vec_kernel<1, UNROLL, false>);
+    if (es == 2) return hw ? launch(apply_mask_units_kernel<2, UNROLL, true>) : launch(apply_mask_units_kernel<2, UNROLL, false>);
+    return hw ? launch(apply_mask_units_kernel<1, UNROLL, true>) : launch(apply_mask_units_kernel<1, UNROLL, false>);
   }
   const unsigned blocks = (unsigned)((total + kThreads - 1) / kThreads);
   if (elem_bytes(t) == 2)

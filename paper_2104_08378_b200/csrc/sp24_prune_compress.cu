@@ -32,9 +32,6 @@ __device__ __forceinline__ uint32_t mask_to_nibble(uint32_t mask) {
 // bits below the sign for the 8-bit floating-point types (`f8` != 0).
 __device__ __forceinline__ uint32_t key8(uint32_t e, int f8) { return f8 ? (e & 0x7Fu) : (uint32_t)abs((int)(int8_t)e); }
 
-__device__ __forceinline__ uint4 ld_stream(const void* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
-__device__ __forceinline__ void st_stream(void* p, uint4 v) { __stcs(reinterpret_cast<uint4*>(p), v); }
-
 // ---- prune -----------------------------------------------------------------------------
 // Any alignment / leading dimension: one thread per group, element-wise accesses.
 template <typename T>
@@ -78,8 +75,8 @@ __device__ __forceinline__ int64_t meta_offset(int layout, int64_t row, int64_t 
 // A 16-byte vector is transposed so that word i holds element i of all its groups (two in 16-bit lanes, four in 8-bit
 // ones): each of the six comparisons is then one subtraction for all groups, whose result is the lane's top bit, and what
 // follows is logic on those bits.  No table: with one in shared memory, indexed by the six bits, a vector took 88
-// instructions and the look-ups met in the banks; it takes 57 with the kept values gathered by lane masks and about 40 now
-// that the bits are turned into byte-permute selectors by dot products, which run beside the ALU pipe (16-bit types).
+// instructions and the look-ups met in the banks; it took 57 (ALU pipe 73 % busy) with the kept values gathered by lane masks and
+// takes 53 (50 %) now that the bits are turned into byte-permute selectors by dot products, which run beside the ALU pipe.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {  // __byte_perm with the selectors that copy a sign
   uint32_t d;
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
@@ -237,22 +234,6 @@ __device__ __forceinline__ void count_dropped(uint32_t lost, unsigned long long*
     if (s) atomicAdd(dropped, (unsigned long long)s);
   }
 }
-
-// 32 bytes at a 32-byte boundary, read or written once.
-__device__ __forceinline__ void ld_stream32(const void* p, uint4 (&v)[2]) {
-  asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x), "=r"(v[1].y), "=r"(v[1].z), "=r"(v[1].w)
-               : "l"(p)
-               : "memory");
-}
-__device__ __forceinline__ void st_stream32(void* p, const uint4 (&v)[2]) {
-  asm volatile("st.global.L1::no_allocate.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0].x),
-               "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z), "r"(v[1].w)
-               : "memory");
-}
-
-// What a launch of compress_kernel may do with whole cells at once: x or y by 32 bytes, the values of an 8-bit cell by 16.
-enum { kWideX = 1, kWideY = 2, kWideVals = 4 };
 
 // Work unit ("cell"): 32 bytes of a row (16 columns of a 16-bit type, 32 of an 8-bit one) = 16 bytes of values and 2 or 4
 // bytes of metadata.  A thread has a cell of the rows r and r + 8 of a 16-row group: in the operand order of a 16-bit type the
