@@ -1,7 +1,7 @@
 // Native form of the binding's short calls (a Python extension module over torch's C++ API): argument marshalling, the
 // allocation of the result, and the call of the C ABI.  For a small product the marshalling in Python costs more than the
 // kernel takes (f16 256 x 256 x 512: 9.9 us of host time a call for 3.2 us on the device; 2.9 of it the allocation through
-// torch's Python layer, 3 the marshalling, 1 ctypes, 3.1 the launch); here the call takes 4.6 us, 3.1 with the result given.
+// torch's Python layer, 3 the marshalling, 1 ctypes, 3.1 the launch); here the call takes 4.5 us, 2.8 with the result given.
 //
 // Every function takes what the Python one has been given and returns None if anything about it is out of the ordinary
 // (another type than a plain CUDA tensor, an active torch-function mode, a type or shape that the Python form rejects, no
