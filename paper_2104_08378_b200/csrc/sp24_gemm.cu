@@ -252,15 +252,16 @@ static void choose_tile(const sp24_gemm_desc* d, bool has_c, bool conv, int& cta
   }
 }
 
-// Clusters of 2^log single CTAs that the device holds at one time (a GPC may end in SMs that make no whole cluster), asked
-// once per device; every GEMM CTA fills its SM.
+// Clusters of 2^log single CTAs that the device holds at one time (a GPC may end in SMs that make no whole cluster), 0 if it
+// holds none; every GEMM CTA fills its SM.  Asked once per device.  A query that fails is not an answer: -1, and the next call
+// asks again.
 __global__ void cluster_probe() {}
 static int split_clusters(int log) {
-  static std::atomic<int> known[64][4];
+  static std::atomic<int> known[64][4];  // the answer + 1
   int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   const bool cacheable = dev >= 0 && dev < 64;
-  if (cacheable && (n = known[dev][log].load(std::memory_order_relaxed)) > 0) return n;
+  if (cacheable && (n = known[dev][log].load(std::memory_order_relaxed)) > 0) return n - 1;
   constexpr int smem = 227 * 1024;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr = {};
@@ -273,9 +274,9 @@ static int split_clusters(int log) {
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   if (cuda_status(cudaFuncSetAttribute(cluster_probe, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != SP24_OK ||
-      cuda_status(cudaOccupancyMaxActiveClusters(&n, cluster_probe, &cfg)) != SP24_OK || n <= 0)
-    n = (sm_count() >> log) * 3 / 4;
-  if (cacheable) known[dev][log].store(n, std::memory_order_relaxed);
+      cuda_status(cudaOccupancyMaxActiveClusters(&n, cluster_probe, &cfg)) != SP24_OK || n < 0)
+    return -1;
+  if (cacheable) known[dev][log].store(n + 1, std::memory_order_relaxed);
   return n;
 }
 
@@ -315,16 +316,18 @@ static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block
 // have many k-blocks this uses SMs that have none; the sums are integers, the same in any order, so the result does not
 // depend on it (those of floating-point kinds would).  Us, device, one CTA to a tile and the choice: 4096 x 32 x 4096 5.9, 4.7;
 // 512 x 512 x 8192 9.2, 6.6; 256 x 256 x 12288 12.3, 6.1; 1056 x 32 x 10816 with C 11.6, 5.2; 2048 x 64 x 2048 4.3, 4.1.
-static void choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ctas, int& block_n, int& mblk, int& tile_n, int& split_log) {
+// False if the device did not say how many clusters it holds: nothing is split then, and the choice is not to be kept.
+static bool choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ctas, int& block_n, int& mblk, int& tile_n, int& split_log) {
   split_log = 0;
+  bool answered = true;
   const int64_t n32 = (d->N + 31) / 32 * 32;
   auto widest = [&](int bn) { return n32 < bn ? (int)n32 : bn; };
   tile_n = widest(block_n);
   if (ctas == 1 && mblk > 1) {  // tall tiles: all the columns there are
     if (d->N < tile_n) tile_n = (int)d->N;
-    return;
+    return true;
   }
-  if (ctas == 2 && (d->a_is_dense || d->N <= 128)) return;
+  if (ctas == 2 && (d->a_is_dense || d->N <= 128)) return true;
   const double now = tile_time(d, has_c, ctas, block_n, mblk, ctas == 2 ? block_n : tile_n);
   double best = now * (ctas == 1 ? 1.0 : mblk == 2 ? 0.85 : 0.97);
   auto try_shape = [&](int c, int bn, int tn) {
@@ -339,7 +342,10 @@ static void choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ct
     for (int w = widest(128); w > 0; w -= 32) {
       const int64_t tiles = blocks * ((d->N + w - 1) / w);
       for (int log = 1; log <= 3 && k_blocks >= 2 << log; ++log) {
-        if (tiles > (sm_count() >> log) || tiles > split_clusters(log)) break;
+        if (tiles > (sm_count() >> log)) break;
+        const int room = split_clusters(log);
+        if (room < 0) answered = false;
+        if (tiles > room) break;
         const double columns = w / 100.0, exchange = log == 1 ? 0.4 + columns : (log == 2 ? 0.5 : 0.9) + 2.0 * columns;
         const double t = 1.04 * (tile_time(d, has_c, 1, 128, 1, w, log) + exchange);
         if (t < best) { best = t; ctas = 1; block_n = 128; mblk = 1; tile_n = w; split_log = log; }
@@ -349,10 +355,11 @@ static void choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ct
   if (!one) try_shape(1, 128, widest(128));
   for (int w = 96; w >= 32; w -= 32)
     if (w < n32) try_shape(1, 128, w);
-  if (!pairs) return;
+  if (!pairs) return answered;
   for (int w = 224; w >= 64; w -= 32) try_shape(2, 224, widest(w));
   if (has_240) try_shape(2, 240, 240);
   if (k_major_b) try_shape(2, 256, widest(256));
+  return answered;
 }
 
 // The shape, width and split of a product, a pure function of what is compared here and of the device.  The last ones of a
@@ -379,8 +386,8 @@ static TileShape choose(const sp24_gemm_desc* d, bool has_c, bool conv) {
     if (kept.key[i] == key) return kept.shape[i];
   TileShape t;
   choose_tile(d, has_c, conv, t.ctas, t.block_n, t.mblk);
-  choose_width(d, has_c, conv, t.ctas, t.block_n, t.mblk, t.tile_n, t.split_log);
-  if (known) {
+  const bool answered = choose_width(d, has_c, conv, t.ctas, t.block_n, t.mblk, t.tile_n, t.split_log);
+  if (known && answered) {
     const int slot = kept.used < kKept ? kept.used++ : (kept.next++ % kKept);
     kept.key[slot] = key;
     kept.shape[slot] = t;
