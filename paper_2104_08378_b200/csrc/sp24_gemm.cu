@@ -323,11 +323,17 @@ static bool choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ct
   const int64_t n32 = (d->N + 31) / 32 * 32;
   auto widest = [&](int bn) { return n32 < bn ? (int)n32 : bn; };
   tile_n = widest(block_n);
+  // Room for clusters.  Every INT8 product that has the kernels with the split beside its own asks, also where nothing will be
+  // split: a program's first call, before it captures a stream, is then the one that loads the probe.
+  int room[4] = {};
+  if (d->ab_type == SP24_I8 && !d->a_is_dense && d->order_b == SP24_COL_MAJOR)
+    for (int log = 1; log <= 3; ++log)
+      if ((room[log] = split_clusters(log)) < 0) answered = false;
   if (ctas == 1 && mblk > 1) {  // tall tiles: all the columns there are
     if (d->N < tile_n) tile_n = (int)d->N;
-    return true;
+    return answered;
   }
-  if (ctas == 2 && (d->a_is_dense || d->N <= 128)) return true;
+  if (ctas == 2 && (d->a_is_dense || d->N <= 128)) return answered;
   const double now = tile_time(d, has_c, ctas, block_n, mblk, ctas == 2 ? block_n : tile_n);
   double best = now * (ctas == 1 ? 1.0 : mblk == 2 ? 0.85 : 0.97);
   auto try_shape = [&](int c, int bn, int tn) {
@@ -342,10 +348,7 @@ static bool choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ct
     for (int w = widest(128); w > 0; w -= 32) {
       const int64_t tiles = blocks * ((d->N + w - 1) / w);
       for (int log = 1; log <= 3 && k_blocks >= 2 << log; ++log) {
-        if (tiles > (sm_count() >> log)) break;
-        const int room = split_clusters(log);
-        if (room < 0) answered = false;
-        if (tiles > room) break;
+        if (tiles > (sm_count() >> log) || tiles > room[log]) break;
         const double columns = w / 100.0, exchange = log == 1 ? 0.4 + columns : (log == 2 ? 0.5 : 0.9) + 2.0 * columns;
         const double t = 1.04 * (tile_time(d, has_c, 1, 128, 1, w, log) + exchange);
         if (t < best) { best = t; ctas = 1; block_n = 128; mblk = 1; tile_n = w; split_log = log; }

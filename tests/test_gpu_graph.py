@@ -67,3 +67,28 @@ def test_captured_step_replays_bit_exact(sp, ab):
             assert np.array_equal(got_D.cpu().numpy(), ref)
         else:
             check_fp(got_D.to(torch.float64).cpu().numpy(), ref, oracle.gemm_abs(v_ref, m_ref, Bt_h, ab))
+
+
+def test_a_split_product_in_a_capture_after_one_that_is_not_split(sp):
+    """The kernels that share a tile's k-blocks, and what their choice asks the device, are ready after any INT8 product."""
+    from test_gpu_split_k_blocks import SHAPES
+    rng = np.random.default_rng(7)
+    sets = []
+    for M, N, K in ((64, 64, 512), SHAPES[0][:3]):
+        a, bt = (rng.integers(-128, 128, s, dtype=np.int8) for s in ((M, K), (N, K)))
+        vals, meta, _ = sp.compress(to_device(a, "i8"))
+        acc = (oracle.prune(a, "i8").astype(np.float64) @ bt.astype(np.float64).T).astype(np.int32)   # (exact)
+        sets.append((vals, meta, to_device(bt, "i8"), acc))
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    vals, meta, x, acc = sets[0]
+    assert np.array_equal(sp.gemm(vals, meta, x, cd="i32", ws=ws).cpu().numpy(), acc)
+    vals, meta, x, acc = sets[1]
+    out = torch.zeros(acc.shape, dtype=torch.int32, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sp.gemm(vals, meta, x, cd="i32", ws=ws, out=out)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert sp.gemm_status(ws) == 0 and np.array_equal(out.cpu().numpy(), acc)

@@ -37,3 +37,12 @@ def test_a_question_that_fails_is_asked_again(exe):
     got = tile_choice.details(exe, [(I8, I32, M, N, K, 0, 0, 0, 0)] * 12, FAILING_QUERIES=9)
     assert got[0].parts == 1 and got[-1].parts == parts, got
     assert got[-1].queries == 0, got        # and an answer is kept
+
+
+def test_the_first_int8_product_asks_whatever_it_splits(exe):
+    """So that none of it is left to a stream capture that follows."""
+    M, N, K, parts = SHAPES[0]
+    first = [(64, 64, 512), (3072, 4096, 768), (8192, 8192, 8192)]
+    for shape in first:
+        got = tile_choice.details(exe, [(I8, I32, *shape, 0, 0, 0, 0), (I8, I32, M, N, K, 0, 0, 0, 0)])
+        assert [(c.parts, c.queries) for c in got] == [(1, 3), (parts, 0)], (shape, got)
