@@ -253,6 +253,9 @@ __device__ __forceinline__ void count_dropped(uint32_t lost, unsigned long long*
 template <int ES, bool COUNT, bool PRUNE>
 constexpr int kCompressBlocks = ES == 2 && !COUNT && !PRUNE ? 5 : 4;
 
+template <bool COUNT, bool PRUNE>
+constexpr int kUnitBlocks = COUNT && PRUNE ? 4 : 5;
+
 template <int ES, bool COUNT, bool HW, bool FULL, bool PRUNE>
 __global__ void __launch_bounds__(kThreads, kCompressBlocks<ES, COUNT, PRUNE>)
 compress_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t row_bytes_v, uint8_t* meta, int64_t M, int64_t K,
@@ -347,6 +350,82 @@ compress_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t ro
         uint16_t* mr = reinterpret_cast<uint16_t*>(meta_cell0 + row * (K >> 3));
         mr[0] = (uint16_t)bits[h];
         if (ES == 1 && !half_cell) mr[1] = (uint16_t)(bits[h] >> 16);
+      }
+    }
+  }
+  count_dropped<COUNT>(lost, dropped);
+}
+
+// Units of 16 bytes: a thread has one of the rows r and r + 8, a warp 32 (16, 8) neighbouring ones of 1 (2, 4) rows; neighbouring
+// lanes put their metadata together, so that words of the operand order are still written whole.  Half a cell to a thread:
+// for matrices of few cells, where compress_kernel's threads go through four vectors one after another on a part of the SMs.
+// Bound by the latency of that chain.  Us, device, cells and units: compress bf16 360 x 512 1.47, 1.26; int8 406 x 128 1.73, 1.37,
+// with the count 2.05, 1.63, fused with prune 1.89, 1.47; 1184 x 1024 1.83, 1.56, 2.10, 1.78, 2.05, 1.62.
+template <int ES, bool COUNT, bool HW, bool PRUNE>
+__global__ void __launch_bounds__(kThreads, kUnitBlocks<COUNT, PRUNE>)
+compress_units_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t row_bytes_v, uint8_t* meta, int64_t M, int64_t K,
+                      uint32_t row_groups, uint32_t units_pad, int unit_shift, unsigned long long* dropped, int f8, uint8_t* y,
+                      int64_t row_bytes_y) {
+  wait_for_stream();
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, odd = lane & 1u;
+  const uint32_t rows_of_warp = 32u >> unit_shift, unit = (blockIdx.x << unit_shift) + (lane & ((1u << unit_shift) - 1u));
+  const uint32_t thread_row = warp * rows_of_warp + (lane >> unit_shift);  // eight of these to a row group
+  const uint32_t in_group = thread_row & 7u, step = gridDim.y * rows_of_warp;
+  const bool live_unit = (int64_t)unit * (16 / ES) < K, meta_unit = unit < units_pad;
+  // metadata of the unit and its neighbour in the first row of a 128-row block that this thread may write (canonical: in row 0)
+  const uint32_t chunk = ES == 2 ? unit >> 1 : unit, KB = ES == 2 ? units_pad >> 4 : units_pad >> 3;
+  uint8_t* const meta_unit0 =
+      meta + (!HW ? 2 * chunk
+                  : (chunk >> 3) * 2048u + 16u * in_group +
+                        (ES == 2 ? 128u * (chunk & 1u) + 4u * ((chunk >> 1) & 3u) : 2u * (chunk & 6u) + 128u * odd));
+  uint32_t n = blockIdx.y * rows_of_warp + (thread_row >> 3);  // row group, the same for all lanes of a warp
+  const int64_t row0 = (int64_t)n * 16 + in_group;
+  const uint8_t* xp = x + row0 * row_bytes_x + (int64_t)unit * 16;
+  uint8_t* vp = vals + row0 * row_bytes_v + (int64_t)unit * 8;
+  uint8_t* yp = PRUNE ? y + row0 * row_bytes_y + (int64_t)unit * 16 : nullptr;
+  uint32_t lost = 0;
+#pragma unroll 1
+  for (; n < row_groups; n += step, xp += (int64_t)step * 16 * row_bytes_x, vp += (int64_t)step * 16 * row_bytes_v) {
+    uint4 in[2];
+    bool live[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      live[h] = live_unit && (int64_t)n * 16 + in_group + 8 * h < M;
+      if (live[h]) in[h] = ld_stream(xp + 8 * h * row_bytes_x);
+    }
+    uint32_t bits[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bits[h] = ES == 2 ? 0x44u : 0x4444u;  // padding: positions (0, 1) in all groups
+      if (live[h]) {
+        uint32_t kept[2], p[4];
+        transpose<ES>(in[h], p);
+        const Selection<ES> s(p, f8);
+        bits[h] = gather_kept<ES>(s, in[h], kept);
+        __stcs(reinterpret_cast<uint2*>(vp + 8 * h * row_bytes_v), make_uint2(kept[0], kept[1]));
+        if (PRUNE) st_stream(yp + 8 * h * row_bytes_y, s.pruned(p));
+        if (COUNT) lost += s.lost();
+      }
+    }
+    if (PRUNE) yp += (int64_t)step * 16 * row_bytes_y;
+    uint8_t* const mr = meta_unit0 + ((uint64_t)(n >> 3) * KB << 11) + 256u * (n & 7u);  // (operand order)
+    if constexpr (ES == 2) {  // a byte of either row: 16 bits with the neighbour's
+      const uint32_t own = bits[1] * 65536u + bits[0], other = __shfl_xor_sync(0xFFFFFFFFu, own, 1);
+      const uint32_t word = odd ? own * 256u + other : other * 256u + own;
+      if constexpr (HW) {
+        if (meta_unit && !odd) *reinterpret_cast<uint32_t*>(mr) = word;
+      } else {  // (a row has an even number of units)
+        const int64_t row = (int64_t)n * 16 + in_group + 8 * odd;
+        if (meta_unit && row < M) *reinterpret_cast<uint16_t*>(meta_unit0 + row * (K >> 3)) = (uint16_t)(odd ? word >> 16 : word);
+      }
+    } else if constexpr (HW) {  // 16 bits of either row: the even lane writes a word of row r, the odd one of r + 8
+      const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, odd ? bits[0] : bits[1], 1);
+      if (meta_unit) *reinterpret_cast<uint32_t*>(mr) = odd ? bits[1] * 65536u + other : other * 65536u + bits[0];
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t row = (int64_t)n * 16 + in_group + 8 * h;
+        if (meta_unit && row < M) *reinterpret_cast<uint16_t*>(meta_unit0 + row * (K >> 3)) = (uint16_t)bits[h];
       }
     }
   }
@@ -663,28 +742,61 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
   const bool vec = K % 16 == 0 && aligned16(x) && aligned16(vals) && aligned16(meta) && (ldx * es) % 16 == 0 &&
                    (ldv * es) % (8 * es) == 0 && row_offsets_fit(K, es, l);
   if (vec) {
+    const uint8_t* xs = (const uint8_t*)x;
+    uint8_t *vs = (uint8_t*)vals, *ms = (uint8_t*)meta, *ys = (uint8_t*)y;
+    // Blocks along the rows, for warps with 2^shift units of a row.  A matrix of moderate size is bound by instructions: about two
+    // rounds of the blocks that fit the SMs take all rows (whole rows of blocks, so a few blocks may make a third), and the set-up
+    // of a block is paid for once.  A large one is bound by HBM and wants the loads of all its blocks in flight.  The line, 160 MB
+    // of traffic, is that of apply_mask + compress and of the fused pass.  Us, device, a block for every row step and two rounds,
+    // at MB of traffic: apply_mask + compress bf16 4096 x 4096 (50) 13.4, 13.2; 12288 x 3072 (112) 35.8, 35.0; 12288 x 4096 (150)
+    // 49.8, 49.6; 8192 x 8192 (200) 68.4, 69.2; 16384 x 8192 (400) 141, 149; int8 8192 x 8192 (104) 38.7, 37.5; fused bf16 4096 x
+    // 4096 (82) 10.0, 9.4; 12288 x 3072 (184) 29.8, 31.5; int8 12288 x 4096 (126) 21.7, 19.9; 8192 x 8192 (168) 28.9, 29.9; alone
+    // on operands that stay in the L2 bf16 12288 x 3072 (112) 14.8, 15.8, int8 9000 x 16384 (229) 49.2, 42.6.
+    const int64_t groups = (rows_pad + 15) / 16, moved = M * K * es * (y ? 5 : 3) / 2 + M * K / 8;
+    auto row_steps = [&](int shift, int64_t columns, int blocks_of_sm) {
+      int64_t steps = (groups + (32 >> shift) - 1) / (32 >> shift);
+      if (steps > 32768) steps = 32768;
+      const int64_t two_rounds = (2 * blocks_of_sm * sm_count() + columns - 1) / columns;
+      return moved <= (int64_t)160 << 20 && steps > two_rounds ? two_rounds : steps;
+    };
     const int64_t cols = es == 2 ? 16 : 32, cells_pad = (k_pad + cols - 1) / cols;
     const int shift = (cells_pad - 1) % 16 < 8 ? 3 : 4;  // cells of a row to a warp: 8 or 16, whichever leaves fewer lanes idle
-    const int64_t units = (cells_pad + (1 << shift) - 1) >> shift, groups = (rows_pad + 15) / 16, per_block = 32 >> shift;
-    int64_t steps = (groups + per_block - 1) / per_block;
-    if (steps > 32768) steps = 32768;
-    // A matrix of moderate size is bound by instructions: two rounds of the blocks that fit the SMs take all rows, so that no
-    // last round is nearly empty and the set-up of a block is paid for once.  A large one is bound by HBM and wants the loads
-    // of all its blocks in flight.  The line, 160 MB of traffic, lies between what was measured on either side of it (it is
-    // not the L2's 126 MB).  Us, device, a block for every row step against two rounds: compress bf16 16102 x 1088 (53 MB in
-    // all) 10.0, 8.8; apply_mask + compress of 4096 x 4096 18.4, 18.1, of 12288 x 3072 37.3, 36.8; compress of 49152 x 12288
-    // (1.9 GB) 281, 310 (16 blocks an SM).
-    const int64_t moved = M * K * es * (y ? 5 : 3) / 2 + M * K / 8;
-    const int64_t two_rounds = (2 * (es == 2 && !dropped && !y ? kCompressBlocks<2, false, false> : kCompressBlocks<1, true, true>) * sm_count() + units - 1) / units;
-    if (moved <= (int64_t)160 << 20 && steps > two_rounds) steps = two_rounds;
+    const int64_t units = (cells_pad + (1 << shift) - 1) >> shift;
+    const int64_t steps = row_steps(shift, units, es == 2 && !dropped && !y ? kCompressBlocks<2, false, false> : kCompressBlocks<1, true, true>);
+    // Fewer blocks of cells than SMs: units of half a cell.  The line is where the two meet (int8, cells over units, alone and
+    // fused: 1.0 MB 1.21, 1.38; 1.4 MB 1.00, 1.06; 1.6 MB 1.00, 1.10; 3.2 MB 0.90, 0.93; bf16 0.7 MB 1.15, 1.14; 1.3 MB 0.96, 1.00;
+    // 5.3 MB 0.98, 0.98).
+    if (units * steps < sm_count()) {
+      const int64_t units_pad = k_pad / (16 / es);
+      auto padded = [&](int log) { return (units_pad + (1 << log) - 1) >> log << log; };
+      const int64_t most = padded(3) + units_pad / 16;  // 32, 16 or 8 units of a row to a warp: the most of which few lanes are idle
+      const int log = padded(5) <= most ? 5 : padded(4) <= most ? 4 : 3;
+      const int64_t columns = padded(log) >> log;
+      const dim3 grid((unsigned)columns, (unsigned)row_steps(log, columns, dropped && y ? kUnitBlocks<true, true> : kUnitBlocks<false, false>), 1);
+#define SP24_CU(V, COUNT, HW, PRUNE)                                                                                              \
+  case V:                                                                                                                        \
+    return launch_overlapped(es == 2 ? compress_units_kernel<2, COUNT, HW, PRUNE> : compress_units_kernel<1, COUNT, HW, PRUNE>, grid, \
+                             dim3(kThreads), 0, s, 1, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)units_pad, log, \
+                             dropped, f8, ys, ldy * es);
+      switch ((y ? 4 : 0) | (dropped ? 2 : 0) | (hw ? 1 : 0)) {
+        SP24_CU(0, false, false, false)
+        SP24_CU(1, false, true, false)
+        SP24_CU(2, true, false, false)
+        SP24_CU(3, true, true, false)
+        SP24_CU(4, false, false, true)
+        SP24_CU(5, false, true, true)
+        SP24_CU(6, true, false, true)
+        default:
+          SP24_CU(7, true, true, true)
+      }
+#undef SP24_CU
+    }
     const dim3 grid((unsigned)units, (unsigned)steps, 1);
     const bool whole_cells = K % cols == 0;
     const bool full = rows_pad == M && M % 16 == 0 && k_pad == K && whole_cells && cells_pad == units << shift;
     auto by32 = [&](const void* p, int64_t ld) { return whole_cells && reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
     const int wide = (by32(x, ldx) ? kWideX : 0) | (y && by32(y, ldy) ? kWideY : 0) | (whole_cells && ldv * es % 16 == 0 ? kWideVals : 0);
     const int variant = (y ? 8 : 0) | (dropped ? 4 : 0) | (hw ? 2 : 0) | (full ? 1 : 0);
-    const uint8_t* xs = (const uint8_t*)x;
-    uint8_t *vs = (uint8_t*)vals, *ms = (uint8_t*)meta, *ys = (uint8_t*)y;
 #define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                                 \
   case V:                                                                                                                  \
     st = launch_overlapped(es == 2 ? compress_kernel<2, COUNT, HW, FULL, PRUNE> : compress_kernel<1, COUNT, HW, FULL, PRUNE>, grid, \
