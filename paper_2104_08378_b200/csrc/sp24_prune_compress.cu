@@ -357,10 +357,12 @@ compress_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t ro
 }
 
 // Units of 16 bytes: a thread has one of the rows r and r + 8, a warp 32 (16, 8) neighbouring ones of 1 (2, 4) rows; neighbouring
-// lanes put their metadata together, so that words of the operand order are still written whole.  Half a cell to a thread:
-// for matrices of few cells, where compress_kernel's threads go through four vectors one after another on a part of the SMs.
-// Bound by the latency of that chain.  Us, device, cells and units: compress bf16 360 x 512 1.47, 1.26; int8 406 x 128 1.73, 1.37,
-// with the count 2.05, 1.63, fused with prune 1.89, 1.47; 1184 x 1024 1.83, 1.56, 2.10, 1.78, 2.05, 1.62.
+// lanes put their metadata together, so that words of the operand order are still written whole.  Half a cell to a thread: for
+// matrices of few cells, where compress_kernel's threads go through four vectors one after another on a part of the SMs, and for
+// the fused pass at 16-byte boundaries, where the two accesses of a cell meet in its sectors (see compress_any). Bound by the
+// latency of that chain, in the fused pass by HBM or the L2.  Us, device, cells and units: compress bf16 360 x 512 1.47, 1.26;
+// int8 406 x 128 1.73, 1.37, with the count 2.05, 1.63, fused with prune 1.89, 1.47; 1184 x 1024 1.83, 1.56, 2.10, 1.78, 2.05,
+// 1.62.
 template <int ES, bool COUNT, bool HW, bool PRUNE>
 __global__ void __launch_bounds__(kThreads, kUnitBlocks<COUNT, PRUNE>)
 compress_units_kernel(const uint8_t* x, int64_t row_bytes_x, uint8_t* vals, int64_t row_bytes_v, uint8_t* meta, int64_t M, int64_t K,
@@ -760,13 +762,23 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
       return moved <= (int64_t)160 << 20 && steps > two_rounds ? two_rounds : steps;
     };
     const int64_t cols = es == 2 ? 16 : 32, cells_pad = (k_pad + cols - 1) / cols;
+    const bool whole_cells = K % cols == 0;
+    auto by32 = [&](const void* p, int64_t ld) { return whole_cells && reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
     const int shift = (cells_pad - 1) % 16 < 8 ? 3 : 4;  // cells of a row to a warp: 8 or 16, whichever leaves fewer lanes idle
     const int64_t units = (cells_pad + (1 << shift) - 1) >> shift;
+    const bool full = rows_pad == M && M % 16 == 0 && k_pad == K && whole_cells && cells_pad == units << shift;
     const int64_t steps = row_steps(shift, units, es == 2 && !dropped && !y ? kCompressBlocks<2, false, false> : kCompressBlocks<1, true, true>);
     // Fewer blocks of cells than SMs: units of half a cell.  The line is where the two meet (int8, cells over units, alone and
     // fused: 1.0 MB 1.21, 1.38; 1.4 MB 1.00, 1.06; 1.6 MB 1.00, 1.10; 3.2 MB 0.90, 0.93; bf16 0.7 MB 1.15, 1.14; 1.3 MB 0.96, 1.00;
     // 5.3 MB 0.98, 0.98).
-    if (units * steps < sm_count()) {
+    // The fused pass on rows that are not at 32-byte boundaries too, up to 40 M elements, 64 M where they end in half a cell:
+    // each of a cell's two stores would leave halves of sectors to the other.  (Whole 8-bit matrices are faster in cells all the
+    // same.)  Us, 16-byte vectors of one row, cells and units: bf16 3072 x 1024 3.28, 3.51, 2.98; 4096 x 4096 11.6, 13.0, 10.1;
+    // 12928 x 1488 14.5, 15.9, 12.9; 12288 x 3072 30.7, 31.3, 31.1; 49152 x 12288 538, 493, 495; int8 4100 x 4112 9.9, 8.3, 7.9;
+    // 4096 x 4096 7.3, 6.6, 7.1; 7468 x 9312 in place 34.6, 33.4, 35.9; with half a cell 32243 x 1040 21.8, 18.0, 16.5; 9098 x
+    // 4752 22.1, 25.9, 20.3; 17858 x 8336 75.4, 73.7, 74.6.
+    const bool split_stores = y && !(by32(x, ldx) && by32(y, ldy)) && (es == 2 || !full);
+    if (units * steps < sm_count() || (split_stores && M * K <= (int64_t)(whole_cells ? 40 : 64) << 20)) {
       const int64_t units_pad = k_pad / (16 / es);
       auto padded = [&](int log) { return (units_pad + (1 << log) - 1) >> log << log; };
       const int64_t most = padded(3) + units_pad / 16;  // 32, 16 or 8 units of a row to a warp: the most of which few lanes are idle
@@ -792,9 +804,6 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
 #undef SP24_CU
     }
     const dim3 grid((unsigned)units, (unsigned)steps, 1);
-    const bool whole_cells = K % cols == 0;
-    const bool full = rows_pad == M && M % 16 == 0 && k_pad == K && whole_cells && cells_pad == units << shift;
-    auto by32 = [&](const void* p, int64_t ld) { return whole_cells && reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
     const int wide = (by32(x, ldx) ? kWideX : 0) | (y && by32(y, ldy) ? kWideY : 0) | (whole_cells && ldv * es % 16 == 0 ? kWideVals : 0);
     const int variant = (y ? 8 : 0) | (dropped ? 4 : 0) | (hw ? 2 : 0) | (full ? 1 : 0);
 #define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                                 \
