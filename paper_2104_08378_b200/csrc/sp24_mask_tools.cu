@@ -164,7 +164,7 @@ __device__ __forceinline__ void mask_selectors(uint32_t (&table)[16], uint32_t t
 // Bound by HBM, by the instructions where the rows are short.  The result is stored without an evict-first hint: it is
 // compressed next, and as much of it as fits is then read from the L2.  With 16-byte units of one row, a metadata byte or two read
 // for each, a vector took 59 instructions (int8 76).  Us, device, with the compression, units and cells: bf16 49152 x 256 18.4,
-// 13.4; 16102 x 1088 21.8, 20.4; 4096 x 4096 18.3, 17.8; 12288 x 3072 36.1, 35.8; 49152 x 12288 639, 640; int8 49152 x 256 17.4,
+// 13.4; 16102 x 1088 21.8, 20.4; 4096 x 4096 18.3, 17.8; 12288 x 3072 36.1, 35.8; int8 49152 x 256 17.4,
 // 9.1; 12288 x 3072 24.7, 24.1.  (Cells by two 16-byte accesses at other boundaries: 5 to 20 % slower than the units.)
 template <int ES, bool HW, bool FULL>
 __global__ void __launch_bounds__(kThreads, 5) apply_mask_vec_kernel(const uint8_t* w, int64_t row_bytes_w, const uint8_t* meta,
@@ -232,12 +232,11 @@ __global__ void __launch_bounds__(kThreads, 5) apply_mask_vec_kernel(const uint8
   }
 }
 
-// Operands at 16-byte boundaries.  Work unit: one 16-byte vector (two groups of a 16-bit type = one metadata byte, four of an 8-bit type =
-// two bytes); launch geometry and unrolling as in prune_vec_kernel, metadata addresses as in compress_kernel.
+// Operands at 16-byte boundaries, and large ones.  Work unit: one 16-byte vector (two groups of a 16-bit type = one metadata byte,
+// four of an 8-bit type = two bytes); launch geometry and unrolling as in prune_vec_kernel, metadata addresses as in
+// compress_kernel.
 // Bound by HBM.  The result is stored without an evict-first hint: it is compressed next, and as much of it as fits is then
-// read from the L2.  One chunk of 16 columns per thread, metadata decoded by arithmetic and evict-first stores before; us, device,
-// before and now: bf16 12288 x 3072 23.5 -> 22.7, followed by its compression 43.4 -> 40.9 (42.7 with evict-first stores);
-// bf16 49152 x 12288 458 -> 361; int8 12288 x 3072 15.2 -> 9.4.
+// read from the L2 (bf16 12288 x 3072 with its compression of then 40.9 us against 42.7, device).
 template <int ES, int UNROLL, bool HW>
 __global__ void __launch_bounds__(kThreads) apply_mask_units_kernel(const uint8_t* w, int64_t row_bytes_w, const uint8_t* meta,
                                                                   uint8_t* y, int64_t row_bytes_y, int64_t M, int64_t K,
@@ -491,9 +490,17 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
     const bool hw = l == SP24_META_TCGEN05;
     const int64_t cols = es == 2 ? 16 : 32, cells = K / cols;
     auto by32 = [&](const void* p, int64_t ld) { return reinterpret_cast<uintptr_t>(p) % 32 == 0 && ld * es % 32 == 0; };
-    if (K % cols == 0 && by32(w, ldw) && by32(y, ldy)) {
+    constexpr int UNROLL = 4;
+    const RowLaunch L(K * es / 16, M, UNROLL);
+    // Whole cells of a matrix beyond 80 MiB go by units as well, unless these leave three of ten lanes idle: HBM bounds both, and a
+    // warp's units are 512 bytes of one row.  Us, device, units and cells, alone and with the compression: bf16 53517 x 3248 107.3,
+    // 111.4, 193.3, 197.0; 16801 x 14736 152.2, 155.0, 275.1, 277.9; 49152 x 12288 362.5, 362.5, 641, 641; int8 306380 x 1568 153.6,
+    // 162.8, 327, 336; below the line bf16 6172 x 5424 (67 MB) 18.2, 17.5, 33.6, 33.6, int8
+    // 9740 x 7424 (72 MB) 22.9, 21.5, 44.9, 43.8.
+    const bool large = M * K * es > (int64_t)80 << 20 && 10 * (K * es / 16) >= 7 * (int64_t)L.grid.x * L.block.x * UNROLL;
+    if (K % cols == 0 && by32(w, ldw) && by32(y, ldy) && !large) {
       // Cells of a row to a warp: 32, 16 or 8, the most of which few lanes are idle (32 and fewer, us, with the compression: bf16
-      // 49152 x 256 15.3, 13.5; 49152 x 12288 640, 645; 6088 x 11632, whose 727 cells are whole only by 8, 77.4, 78.3).
+      // 49152 x 256 15.3, 13.5; 6088 x 11632, whose 727 cells are whole only by 8, 77.4, 78.3).
       auto padded = [&](int log) { return (cells + (1 << log) - 1) >> log << log; };
       const int64_t most = padded(3) + cells / 16;
       const int shift = padded(5) <= most ? 5 : padded(4) <= most ? 4 : 3;
@@ -510,8 +517,6 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
       if (full) return hw ? launch(apply_mask_vec_kernel<1, true, true>) : launch(apply_mask_vec_kernel<1, false, true>);
       return hw ? launch(apply_mask_vec_kernel<1, true, false>) : launch(apply_mask_vec_kernel<1, false, false>);
     }
-    constexpr int UNROLL = 4;
-    const RowLaunch L(K * es / 16, M, UNROLL);
     auto launch = [&](auto kernel) {
       return launch_overlapped(kernel, L.grid, L.block, 0, s, 1, (const uint8_t*)w, ldw * es, (const uint8_t*)meta, (uint8_t*)y,
                                ldy * es, M, K, KB);
