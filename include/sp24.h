@@ -299,7 +299,9 @@ sp24_status sp24_set_tile_override(int ctas, int block_n, int mblk, int band);
 /* Test support for the failure path, not for production use: shortens the limit of every
  * device-side wait to `wait_cycles` SM cycles (values below 1 000 000 restore the default of
  * about a second) and, with skip_stage != 0, makes the TMA producers leave out one k-block of
- * their first tile so that a wait expires.  Nothing faults or hangs: the kernel returns early
+ * their first tile so that a wait expires; 2 + r: where several CTAs share the k-blocks of a tile,
+ * only that of rank r does, whose own waits then have four times the limit: the others' waits for
+ * its sums are the first to expire.  Nothing faults or hangs: the kernel returns early
  * and sp24_gemm_status reports SP24_ERR_TIMEOUT.  Never read from the environment. */
 sp24_status sp24_test_set_fault_hooks(long long wait_cycles, int skip_stage);
 

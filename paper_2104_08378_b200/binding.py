@@ -319,9 +319,9 @@ def set_tile_override(tile: str | None = None, band: int = 0):
     _check(lib.sp24_set_tile_override(c, n, m, band), "sp24_set_tile_override")
 
 
-def set_fault_hooks(wait_cycles: int = 0, skip_stage: bool = False):
+def set_fault_hooks(wait_cycles: int = 0, skip_stage: bool | int = False):
     """sp24_test_set_fault_hooks (failure-path tests only)."""
-    _check(lib.sp24_test_set_fault_hooks(int(wait_cycles), 1 if skip_stage else 0), "sp24_test_set_fault_hooks")
+    _check(lib.sp24_test_set_fault_hooks(int(wait_cycles), int(skip_stage)), "sp24_test_set_fault_hooks")
 
 
 def im2col_nhwc_3x3(x: torch.Tensor, dtype: str | None = None, out: torch.Tensor | None = None) -> torch.Tensor:

@@ -624,7 +624,7 @@ extern "C" sp24_status sp24_set_tile_override(int ctas, int block_n, int mblk, i
 extern "C" sp24_status sp24_test_set_fault_hooks(long long wait_cycles, int skip_stage) {
   Settings& cfg = settings();
   cfg.test_wait_cycles.store(wait_cycles, std::memory_order_relaxed);
-  cfg.test_skip_stage.store(skip_stage ? 1 : 0, std::memory_order_relaxed);
+  cfg.test_skip_stage.store(skip_stage < 0 ? 1 : skip_stage, std::memory_order_relaxed);
   return SP24_OK;
 }
 

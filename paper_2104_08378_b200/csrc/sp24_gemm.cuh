@@ -57,7 +57,7 @@ struct GemmParams {
   int32_t has_c;
   int32_t stages, epi_bytes;  // shared memory: ring stages and bytes of epilogue staging
   long long wait_limit;       // SM cycles after which a device-side wait gives up
-  int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires
+  int32_t test_skip_stage;    // test hook: the producers leave out one k-block, so that a wait expires (2 + r: only CTA r of those that share a tile's)
   int32_t band;       // m-tiles per band of the tile sweep
   FastDiv by_band_tiles, by_band, by_last_band;  // tiles of a band; m-tiles of a band and of the last one
   int32_t tile_n;     // columns of a tile: the kernel's BLOCK_N or fewer

@@ -132,6 +132,14 @@ struct Cfg {
 template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
 constexpr bool twelve_warps = KIND == 1 && SPARSE && CTAS == 2 && MBLK == 1 && !B_MN && BLOCK_N == 224;
 
+template <int KIND, bool SPARSE, int BLOCK_N, int CTAS, int MBLK, bool B_MN>
+int epilogue_warps(const sp24_gemm_desc* d, int tile_n) {
+  using C = Cfg<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
+  const int tile_m = kBlockM * CTAS * MBLK;
+  return twelve_warps<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN> && elem_bytes(d->cd_type) == 1 && d->K <= 6 * C::kKPerStage &&
+                 (d->M + tile_m - 1) / tile_m * ((d->N + tile_n - 1) / tile_n) > sm_count() / CTAS ? 12 : kEpiWarps;
+}
+
 struct Shared {
   uint64_t full[12], empty[12], tmem_full[2], tmem_empty[2];
   uint64_t split_full;             // the other CTAs' parts of the boxes that this one finishes are there
@@ -565,7 +573,8 @@ __device__ __forceinline__ void epilogue_direct(const GemmParams& p, Shared* sh,
 #pragma unroll
       for (int n = 0; n < P; ++n) fetch_c(creg[n]);
     }
-    if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, p.wait_limit)) break;
+    const long long limit = SPLIT && p.test_skip_stage == 2 + split_rank ? 4 * p.wait_limit : p.wait_limit;  // (as in gemm_kernel)
+    if (!bounded_wait(&sh->tmem_full[acc], acc_phase, sh, p.status, 4u, limit)) break;
     ptx::tc_fence_after();
     if constexpr (SPLIT) {
       if (!mine) {
@@ -643,6 +652,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   const int kb_begin = SPLIT ? (p.k_blocks * split_rank) >> split_log : 0;
   const int kb_end = SPLIT ? (p.k_blocks * (split_rank + 1)) >> split_log : p.k_blocks;
   const int num_tiles = p.m_tiles * p.n_tiles;
+  // (test hook: the CTA whose k-block is left out waits longer, so that the others' waits for its sums are the first to expire)
+  auto wait_limit = [&] { return SPLIT && p.test_skip_stage == 2 + split_rank ? 4 * p.wait_limit : p.wait_limit; };
 
   // Set-up: lanes of a warp initialise the barriers, and the pair meets without a release.  All that a CTA of a pair has
   // to know before it goes on is that the peer's barriers are there, and fence.mbarrier_init publishes those; that the
@@ -825,7 +836,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         // and columns would no longer give the same bits when M or N is split differently.  Not done.)
         if (kps == 2) {  // (A in whole 128-byte atoms: its atoms are a third dimension as B's are)
           for (int kb = 0; kb < p.k_blocks; kb += 2) {
-            if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
+            if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, wait_limit())) break;
             if (!(p.test_skip_stage && t == cluster_id && kb == 2)) {  // (test hook: as below)
               const uint32_t sa = ring + stage * slot_bytes, sb = sa + 2 * C::kABytes, se = sb + 2 * b_bytes;
               const uint32_t full = full0 + 8 * stage;
@@ -839,10 +850,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           continue;
         }
         for (int kb = kb_begin; kb < kb_end; ++kb) {
-          if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, p.wait_limit)) break;
-          if (p.test_skip_stage && t == cluster_id && kb == kb_begin + 1) {
-            // test hook: this k-block of the first tile is neither armed nor loaded by either CTA, so
-            // the MMA issuer's wait for it expires and every role leaves through the abort path
+          if (!bounded_wait(&sh->empty[stage], phase ^ 1u, sh, p.status, 1u, wait_limit())) break;
+          if (p.test_skip_stage && (!SPLIT || p.test_skip_stage == 1 || p.test_skip_stage == 2 + split_rank) && t == cluster_id &&
+              kb == kb_begin + 1) {
+            // test hook: this k-block of the first tile is neither armed nor loaded by either CTA (by one of those that share
+            // the tile's k-blocks), so the MMA issuer's wait for it expires and every role leaves through the abort path
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             continue;
           }
@@ -882,7 +894,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       // (teardown of a pair: the last commits, which come from CTA 0, have arrived)
       if (CTAS == 2 && !sh->abort)
         drain_ring(p.stages, stage, phase, [&](int s, uint32_t parity) {
-          return bounded_wait(&sh->empty[s], parity, sh, p.status, 1u, p.wait_limit);
+          return bounded_wait(&sh->empty[s], parity, sh, p.status, 1u, wait_limit());
         });
     }
   } else if (warp == 1) {
@@ -942,7 +954,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             }
           }
         };
-        if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, p.wait_limit)) break;
+        if (!bounded_wait(&sh->tmem_empty[acc], acc_phase ^ 1u, sh, p.status, 2u, wait_limit())) break;
         ptx::tc_fence_after();
         bool ok = true;
         // the stage may be refilled once its MMAs have read it
@@ -953,7 +965,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         };
         if (kps == 2) {
           for (int kb = 0; kb < p.k_blocks; kb += 2) {
-            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
+            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, wait_limit())) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t sa = ring + stage * slot_bytes, sb = sa + 2 * C::kABytes, se = sb + 2 * b_bytes;
             multiply(kb, sa, sb, se);
@@ -962,7 +974,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
           }
         } else {
           for (int kb = kb_begin; kb < kb_end; ++kb) {
-            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, p.wait_limit)) { ok = false; break; }
+            if (!bounded_wait(&sh->full[stage], phase, sh, p.status, 3u, wait_limit())) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t sa = ring + stage * slot_bytes;
             multiply(kb - kb_begin, sa, sa + C::kABytes, sa + C::kABytes + b_bytes);
@@ -977,7 +989,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       // (teardown of a pair: the last accumulators have been handed back, CTA 1's warps' arrivals among them)
       if (CTAS == 2 && !sh->abort)
         drain_ring(C::kAccStages, acc, acc_phase, [&](int a, uint32_t parity) {
-          return bounded_wait(&sh->tmem_empty[a], parity, sh, p.status, 2u, p.wait_limit);
+          return bounded_wait(&sh->tmem_empty[a], parity, sh, p.status, 2u, wait_limit());
         });
     }
   } else if (warp >= kFirstEpiWarp) {
@@ -1147,8 +1159,7 @@ sp24_status launch(const TileShape& tile, const sp24_gemm_desc* d, const GemmPar
   // stage less cost the int8 configuration 9 %); a staged epilogue gets what is left.
   constexpr bool kTwelve = twelve_warps<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>;
   int tile_m = kBlockM * CTAS * MBLK;
-  const int warps = kTwelve && cs == 1 && d->K <= 6 * C::kKPerStage &&
-                            (d->M + tile_m - 1) / tile_m * ((d->N + tile_n - 1) / tile_n) > sm_count() / CTAS ? 12 : kEpiWarps;
+  const int warps = epilogue_warps<KIND, SPARSE, BLOCK_N, CTAS, MBLK, B_MN>(d, tile_n);
   p.epi_bytes = warps * (C::staged_epilogue(cs, p.cd_col_major) ? 4096 : 2048);
   const int es = KIND == 0 ? 2 : (one_byte_operands(KIND) ? 1 : 4);
   const uint32_t atom_elems = kAtomBytes / es;

@@ -10,7 +10,11 @@ from gpu_util import to_device
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,N,K", [(5920, 960, 256), (3104, 4128, 768), (2080, 9248, 1504), (4640, 3424, 1568), (19232, 224, 32)])
+# (test_split_choice_cpu.py holds them to twelve warps and the one of seven k-blocks to eight)
+SHAPES = [(5920, 960, 256), (3104, 4128, 768), (2080, 9248, 1504), (4640, 3424, 1568), (19232, 224, 32)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
 def test_against_the_exact_product(M, N, K):
     from paper_2104_08378_b200 import binding as sp
     rng = np.random.default_rng(M + N + K)

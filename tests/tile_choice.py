@@ -25,7 +25,8 @@ sp24_status report(TileShape t, bool sparse, bool b_mn, const sp24_gemm_desc* d,
   if (sparse && !b_mn && t.mblk == 1)
     k = t.ctas == 1 ? kps(Cfg<KIND, true, 128, 1, 1, false>{}) : t.block_n == 256 ? kps(Cfg<KIND, true, 256, 2, 1, false>{})
         : kps(Cfg<KIND, true, 224, 2, 1, false>{});
-  printf("%dx%dx%d %d %d %d %d\n", t.ctas, t.block_n, t.mblk, t.tile_n, k, 1 << t.split_log, queries);
+  const int warps = sparse && !b_mn && t.ctas == 2 && t.block_n == 224 && t.mblk == 1 ? epilogue_warps<KIND, true, 224, 2, 1, false>(d, t.tile_n) : kEpiWarps;
+  printf("%dx%dx%d %d %d %d %d %d\n", t.ctas, t.block_n, t.mblk, t.tile_n, k, 1 << t.split_log, queries, warps);
   queries = 0;
   return SP24_OK;
 }
@@ -79,7 +80,7 @@ def compile_harness(folder):
     return str(exe)
 
 
-Choice = collections.namedtuple("Choice", "tile columns k_blocks parts queries")
+Choice = collections.namedtuple("Choice", "tile columns k_blocks parts queries warps")
 
 
 def details(exe, problems, **env):
