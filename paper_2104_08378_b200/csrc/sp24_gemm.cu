@@ -285,7 +285,8 @@ static int split_clusters(int log) {
 // tile by its columns (4-byte results and C cost more; 256-column tiles and two m-blocks cannot overlap it).  Fitted to
 // 170 random problems (256..16384 rows, 160..16384 columns, K 256..12288, every kind, with and without C), 11 to 17
 // shapes of each, before stages held two k-blocks: it puts bf16 512 x 512 x 8192 at 16.5 us, which now takes 13.1.  On 100
-// other problems of the same ranges the mean error of today's kernels is 9 to 13 % per shape, 16 % for two m-blocks.
+// other problems of the same ranges the mean error of later kernels is 9 to 13 % per shape, 16 % for two m-blocks.  (An int8
+// result counts as a 16-bit one: the fit is older than its arithmetic by pairs and its twelve warps.)
 // split_log: the CTAs of a cluster share the k-blocks.
 static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block_n, int mblk, int tile_n, int split_log = 0) {
   const int bytes = elem_bytes(d->ab_type), cs = elem_bytes(d->cd_type);
@@ -314,8 +315,12 @@ static double tile_time(const sp24_gemm_desc* d, bool has_c, int ctas, int block
 // INT32 accumulators of single CTAs: a cluster of 2, 4 or 8 of them may share the k-blocks of a tile (split_log), which the
 // estimate has as its k-blocks in so many parts and the exchange of the accumulators, by their columns.  Where few tiles
 // have many k-blocks this uses SMs that have none; the sums are integers, the same in any order, so the result does not
-// depend on it (those of floating-point kinds would).  Us, device, one CTA to a tile and the choice: 4096 x 32 x 4096 5.9, 4.7;
-// 512 x 512 x 8192 9.2, 6.6; 256 x 256 x 12288 12.3, 6.1; 1056 x 32 x 10816 with C 11.6, 5.2; 2048 x 64 x 2048 4.3, 4.1.
+// depend on it (those of floating-point kinds would).  Us, device, one CTA to a tile and the choice: 4096 x 32 x 4096 5.7, 4.5;
+// 512 x 512 x 8192 9.0, 6.3; 256 x 256 x 12288 12.2, 5.9; 1056 x 32 x 10816 with C 11.4, 5.0; 2048 x 64 x 2048 4.2, 4.2.
+// The exchange was set from a few shapes (0.7 us for 2 CTAs, 1.2 for 4, 1.5 for 8 at 32 columns), the 4 % so that nearly equal
+// ones are not split.  Over 100 random int8 products (64..9000 rows, 32..2000 columns, K 512..12288, up to 74 tiles of 128 x 128,
+// every result type), at every width and number of parts, the mean error of the estimate is 9 % for 2 parts and 11 % for 4 and
+// 8 (one: 10 %); the choice is 0.9 % behind the best (at worst 14 %), and 1.20 times as fast as the best unsplit one in the mean.
 // False if the device did not say how many clusters it holds: nothing is split then, and the choice is not to be kept.
 static bool choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ctas, int& block_n, int& mblk, int& tile_n, int& split_log) {
   split_log = 0;
@@ -367,7 +372,8 @@ static bool choose_width(const sp24_gemm_desc* d, bool has_c, bool conv, int& ct
 
 // The shape, width and split of a product, a pure function of what is compared here and of the device.  The last ones of a
 // host thread are kept: the estimates take 0.3 to 0.8 us of host time, and a short call is bound by that (f16 256 x 256 x 512
-// in a loop 5.36 -> 5.10; int8 4096 x 32 x 4096 5.57 -> 5.18).
+// in a loop 5.36 -> 5.10; int8 4096 x 32 x 4096 5.57 -> 5.18).  These are loops over one product: a first call of a shape has
+// the estimate as before, and a thread with more than sixteen in rotation the search as well (up to 0.1 us).
 struct Choice {
   int device, ab, cd, order_b, order_d, dense, has_c, conv;
   int64_t M, N, K;

@@ -9,7 +9,8 @@
 //            memory (tcgen05.cp), issues the tcgen05.mma[.sp] of the stage, commits the stage
 //            back to the producer and, after the last k-block, the accumulators to the epilogue;
 //            owns the tensor-memory allocation;
-//   warps 2-9 epilogue, two per tensor-memory lane quarter taking alternate 32-column boxes:
+//   warps 2-9 epilogue (2-13 in the kernels of twelve_warps), two (three) per tensor-memory lane quarter taking 32-column boxes
+//            in turn:
 //            tcgen05.ld accumulator -> registers, alpha / beta / conversion in registers, then one of two
 //            forms.  4-byte row-major outputs: a
 //            staging box per warp, C boxes TMA-loaded one box ahead, TMA store of the D box, if
@@ -18,6 +19,8 @@
 //            as soon as their last box is in registers.
 // CTAS == 2 runs a pair of CTAs (cluster of two): each CTA loads its 128 rows of A / metadata per
 // m-block and its half of B, CTA 0 issues cta_group::2 MMAs (M = 256) for both.
+// SPLIT runs a cluster of 2, 4 or 8 CTAs on one tile of INT32 sums, each with a part of the k-blocks
+// and MMAs of its own; the epilogue warps exchange the accumulators.
 // MBLK == 2 gives every CTA two m-blocks (two accumulators, one B tile): what an SM can pull in
 // from the L2 per clock, not the tensor pipe, bounds this kernel, and sharing the B tile between
 // two m-blocks cuts the bytes per flop by about a third.  The two accumulators then fill tensor
@@ -348,8 +351,7 @@ __device__ __forceinline__ void convert_row_staged(const uint32_t (&r)[32], uint
 // cannot hide that.  So: one short loop over the boxes that exist, with C a loop of four, shared-memory accesses in
 // groups so that they overlap, packed FP32 arithmetic.  Cycles from the accumulators of a 512 x 224 tile being complete
 // to their hand-back, unrolled and now (timestamps included): 16-bit results 12,700 and 5,800, with C 18,400 and 9,600,
-// column-major 14,800 and 6,300, with C 20,800 and 9,500.  More warps make it slower (12 or 16 instead of 8, BERT FFN
-// 12.9 -> 14.7, 17.7 us, 256 x 256 x 512 4.2 -> 4.7, 5.3): registers for fewer boxes of C, and set-up.
+// column-major 14,800 and 6,300, with C 20,800 and 9,500.  (Where more than eight warps pay: twelve_warps.)
 // A box is 32 rows x 64 bytes of output (32 columns, 16 of a 4-byte type; 32 bytes of a 1-byte type).  Per box: the
 // accumulators of this thread's row come out of tensor memory (loaded while the box before is stored), are converted
 // in registers and stored by way of a 2 KB buffer of the warp.

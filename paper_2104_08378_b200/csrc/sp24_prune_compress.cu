@@ -244,8 +244,8 @@ __device__ __forceinline__ void count_dropped(uint32_t lost, unsigned long long*
 // the same launch.  HW: metadata straight into that order.  FULL: the launch covers exactly the matrix, so no bounds are
 // checked.  PRUNE: the pruned matrix is written as well (y, same shape as x; may be x itself), so that one pass over x yields
 // everything the separate prune and compress passes would.
-// Bound by HBM where the matrix is large and cold, by the ALU pipe where it comes out of the L2 (ncu, bf16 12288 x 3072 right
-// after apply_mask: 5 of 75 MB read from DRAM, ALU pipe 73 % busy with 57 instructions a vector).  Us, device, table
+// Bound by HBM where the matrix is large and cold.  Where it comes out of the L2 (bf16 12288 x 3072 right after apply_mask: 5 of
+// 75 MB read from DRAM) the longest stall is memory and the ALU pipe half busy (52 %, 53 instructions a vector).  Us, device, table
 // kernels of before / now: compress bf16 49152 x 12288 332, 281 (6.7 TB/s); 4096 x 4096 9.0, 7.4; 49152 x 256 13.4, 5.9; int8
 // 49152 x 12288 292, 160; 12288 x 3072 22.0, 11.1; fused with prune bf16 49152 x 12288 534, 474; int8 340, 247; after
 // apply_mask, both calls, bf16 12288 x 3072 40.4, 36.0.
@@ -774,7 +774,7 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
     // The fused pass on rows that are not at 32-byte boundaries too, up to 40 M elements, 64 M where they end in half a cell:
     // each of a cell's two stores would leave halves of sectors to the other.  (Whole 8-bit matrices are faster in cells all the
     // same.)  Us, 16-byte vectors of one row, cells and units: bf16 3072 x 1024 3.28, 3.51, 2.98; 4096 x 4096 11.6, 13.0, 10.1;
-    // 12928 x 1488 14.5, 15.9, 12.9; 12288 x 3072 30.7, 31.3, 31.1; 49152 x 12288 538, 493, 495; int8 4100 x 4112 9.9, 8.3, 7.9;
+    // 12928 x 1488 14.5, 15.9, 12.9; 12288 x 3072 30.7, 31.3, 31.1; 67606 x 7296 449, 408, 420; int8 4100 x 4112 9.9, 8.3, 7.9;
     // 4096 x 4096 7.3, 6.6, 7.1; 7468 x 9312 in place 34.6, 33.4, 35.9; with half a cell 32243 x 1040 21.8, 18.0, 16.5; 9098 x
     // 4752 22.1, 25.9, 20.3; 17858 x 8336 75.4, 73.7, 74.6.
     const bool split_stores = y && !(by32(x, ldx) && by32(y, ldy)) && (es == 2 || !full);
