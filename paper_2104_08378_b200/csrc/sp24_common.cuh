@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "sp24.h"
 
 namespace sp24 {
@@ -81,6 +83,32 @@ inline sp24_status launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
 
 // ---- streaming kernels ----------------------------------------------------------------------------------
 constexpr int kThreads = 256;
+
+// A streaming kernel of few blocks behind a product: blocks that come in early find room only on the SMs that the product leaves
+// idle, and all of them together there, where they then do the whole work.  So a launch of up to four blocks to an SM asks for as
+// much (unused) shared memory as leaves room for an even spread only; the other blocks wait for the product's SMs.  Us a call in a
+// CUDA graph, as they come and spread, each behind the product of its rows with 256 columns: prune_compress int8 3264 x 448 7.4,
+// 6.1; bf16 3456 x 224 6.7, 5.5; 4448 x 448 8.2, 7.4; compress 7.0, 5.9; 6.3, 5.3; 7.9, 7.1; apply_mask and compress 8.2, 7.4; 7.5,
+// 6.8; 10.2, 8.9.  By themselves, or behind other kernels, they take as long as before; without the early start 6.8, 6.2, 8.1.
+template <auto KERNEL>
+struct Kernel {};  // a kernel as an argument's type
+
+template <auto KERNEL, typename... Args>
+inline sp24_status launch_streaming(Kernel<KERNEL>, dim3 grid, dim3 block, cudaStream_t stream, Args... args) {
+  static std::atomic<bool> allowed[64];  // the shared-memory opt-in, per kernel and device
+  const int64_t sms = sm_count(), blocks_of_sm = sms > 0 ? ((int64_t)grid.x * grid.y + sms - 1) / sms : 0;
+  constexpr int most = 227 * 1024 - 2048;  // (static shared memory and the KB that each block takes)
+  int dev = 0;
+  size_t smem = 0;
+  if (blocks_of_sm >= 1 && blocks_of_sm <= 4 && cudaGetDevice(&dev) == cudaSuccess) {
+    const bool kept = dev >= 0 && dev < 64;
+    bool ok = kept && allowed[dev].load(std::memory_order_relaxed);
+    if (!ok && (ok = cuda_status(cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) == SP24_OK) && kept)
+      allowed[dev].store(true, std::memory_order_relaxed);
+    if (ok) smem = (size_t)(227 * 1024 / blocks_of_sm - 2048);
+  }
+  return launch_overlapped(KERNEL, grid, block, smem, stream, 1, args...);
+}
 
 __device__ __forceinline__ uint4 ld_stream(const void* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
 __device__ __forceinline__ void st_stream(void* p, uint4 v) { __stcs(reinterpret_cast<uint4*>(p), v); }

@@ -509,20 +509,19 @@ extern "C" sp24_status sp24_apply_mask(sp24_dtype t, int64_t M, int64_t K, const
       if (steps > 32768) steps = 32768;
       const bool full = M % 16 == 0 && cells == units << shift;
       auto launch = [&](auto kernel) {
-        return launch_overlapped(kernel, dim3((unsigned)units, (unsigned)steps, 1), dim3(kThreads), 0, s, 1, (const uint8_t*)w, ldw * es,
-                                 (const uint8_t*)meta, (uint8_t*)y, ldy * es, M, K, (uint32_t)groups, (uint32_t)KB, shift);
+        return launch_streaming(kernel, dim3((unsigned)units, (unsigned)steps, 1), dim3(kThreads), s, (const uint8_t*)w, ldw * es,
+                                (const uint8_t*)meta, (uint8_t*)y, ldy * es, M, K, (uint32_t)groups, (uint32_t)KB, shift);
       };
-      if (es == 2 && full) return hw ? launch(apply_mask_vec_kernel<2, true, true>) : launch(apply_mask_vec_kernel<2, false, true>);
-      if (es == 2) return hw ? launch(apply_mask_vec_kernel<2, true, false>) : launch(apply_mask_vec_kernel<2, false, false>);
-      if (full) return hw ? launch(apply_mask_vec_kernel<1, true, true>) : launch(apply_mask_vec_kernel<1, false, true>);
-      return hw ? launch(apply_mask_vec_kernel<1, true, false>) : launch(apply_mask_vec_kernel<1, false, false>);
+      if (es == 2 && full) return hw ? launch(Kernel<apply_mask_vec_kernel<2, true, true>>{}) : launch(Kernel<apply_mask_vec_kernel<2, false, true>>{});
+      if (es == 2) return hw ? launch(Kernel<apply_mask_vec_kernel<2, true, false>>{}) : launch(Kernel<apply_mask_vec_kernel<2, false, false>>{});
+      if (full) return hw ? launch(Kernel<apply_mask_vec_kernel<1, true, true>>{}) : launch(Kernel<apply_mask_vec_kernel<1, false, true>>{});
+      return hw ? launch(Kernel<apply_mask_vec_kernel<1, true, false>>{}) : launch(Kernel<apply_mask_vec_kernel<1, false, false>>{});
     }
     auto launch = [&](auto kernel) {
-      return launch_overlapped(kernel, L.grid, L.block, 0, s, 1, (const uint8_t*)w, ldw * es, (const uint8_t*)meta, (uint8_t*)y,
-                               ldy * es, M, K, KB);
+      return launch_streaming(kernel, L.grid, L.block, s, (const uint8_t*)w, ldw * es, (const uint8_t*)meta, (uint8_t*)y, ldy * es, M, K, KB);
     };
-    if (es == 2) return hw ? launch(apply_mask_units_kernel<2, UNROLL, true>) : launch(apply_mask_units_kernel<2, UNROLL, false>);
-    return hw ? launch(apply_mask_units_kernel<1, UNROLL, true>) : launch(apply_mask_units_kernel<1, UNROLL, false>);
+    if (es == 2) return hw ? launch(Kernel<apply_mask_units_kernel<2, UNROLL, true>>{}) : launch(Kernel<apply_mask_units_kernel<2, UNROLL, false>>{});
+    return hw ? launch(Kernel<apply_mask_units_kernel<1, UNROLL, true>>{}) : launch(Kernel<apply_mask_units_kernel<1, UNROLL, false>>{});
   }
   const unsigned blocks = (unsigned)((total + kThreads - 1) / kThreads);
   if (elem_bytes(t) == 2)

@@ -705,10 +705,10 @@ extern "C" sp24_status sp24_prune(sp24_dtype t, int64_t M, int64_t K, const void
     RowLaunch L(vpr, rows, UNROLL);
     int64_t rbx = ldx == K && ldy == K ? vpr * 16 : ldx * es, rby = ldx == K && ldy == K ? vpr * 16 : ldy * es;
     if (es == 2)
-      return launch_overlapped(prune_vec_kernel<2, UNROLL>, L.grid, L.block, 0, s, 1, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
+      return launch_streaming(Kernel<prune_vec_kernel<2, UNROLL>>{}, L.grid, L.block, s, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
                                vpr, rows, f8);
     else
-      return launch_overlapped(prune_vec_kernel<1, UNROLL>, L.grid, L.block, 0, s, 1, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
+      return launch_streaming(Kernel<prune_vec_kernel<1, UNROLL>>{}, L.grid, L.block, s, (const uint8_t*)x, rbx, (uint8_t*)y, rby,
                                vpr, rows, f8);
   } else {
     int64_t gpr = K / 4, total = M * gpr;
@@ -768,9 +768,10 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
     const int64_t units = (cells_pad + (1 << shift) - 1) >> shift;
     const bool full = rows_pad == M && M % 16 == 0 && k_pad == K && whole_cells && cells_pad == units << shift;
     const int64_t steps = row_steps(shift, units, es == 2 && !dropped && !y ? kCompressBlocks<2, false, false> : kCompressBlocks<1, true, true>);
-    // Fewer blocks of cells than SMs: units of half a cell.  The line is where the two meet (int8, cells over units, alone and
-    // fused: 1.0 MB 1.21, 1.38; 1.4 MB 1.00, 1.06; 1.6 MB 1.00, 1.10; 3.2 MB 0.90, 0.93; bf16 0.7 MB 1.15, 1.14; 1.3 MB 0.96, 1.00;
-    // 5.3 MB 0.98, 0.98).
+    // Fewer blocks of cells than three for two SMs (3.6 MB where no lanes are idle): units of half a cell.  Cells over units, means of
+    // 3 to 12 matrices, bf16 and int8: compression alone 0.3 to 0.8 MB 1.16, 1.22; 1.2 to 1.8 MB 0.97, 0.99; 2.4 to 3.6 MB 1.02,
+    // 1.06; 3.6 to 4.9 MB 0.98, 1.01; 6.5 to 10 MB 0.90, 0.91; fused and a product behind it 1.2 to 1.8 MB 1.01, 1.01; 2.4 to 3.6 MB
+    // 1.05, 1.02; 3.6 to 4.9 MB 0.98, 1.01; 6.5 to 10 MB 0.98, 0.98.
     // The fused pass on rows that are not at 32-byte boundaries too, up to 40 M elements, 64 M where they end in half a cell:
     // each of a cell's two stores would leave halves of sectors to the other.  (Whole 8-bit matrices are faster in cells all the
     // same.)  Us, 16-byte vectors of one row, cells and units: bf16 3072 x 1024 3.28, 3.51, 2.98; 4096 x 4096 11.6, 13.0, 10.1;
@@ -778,18 +779,20 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
     // 4096 x 4096 7.3, 6.6, 7.1; 7468 x 9312 in place 34.6, 33.4, 35.9; with half a cell 32243 x 1040 21.8, 18.0, 16.5; 9098 x
     // 4752 22.1, 25.9, 20.3; 17858 x 8336 75.4, 73.7, 74.6.
     const bool split_stores = y && !(by32(x, ldx) && by32(y, ldy)) && (es == 2 || !full);
-    if (units * steps < sm_count() || (split_stores && M * K <= (int64_t)(whole_cells ? 40 : 64) << 20)) {
+    if (2 * units * steps < 3 * sm_count() || (split_stores && M * K <= (int64_t)(whole_cells ? 40 : 64) << 20)) {
       const int64_t units_pad = k_pad / (16 / es);
       auto padded = [&](int log) { return (units_pad + (1 << log) - 1) >> log << log; };
       const int64_t most = padded(3) + units_pad / 16;  // 32, 16 or 8 units of a row to a warp: the most of which few lanes are idle
       const int log = padded(5) <= most ? 5 : padded(4) <= most ? 4 : 3;
       const int64_t columns = padded(log) >> log;
       const dim3 grid((unsigned)columns, (unsigned)row_steps(log, columns, dropped && y ? kUnitBlocks<true, true> : kUnitBlocks<false, false>), 1);
-#define SP24_CU(V, COUNT, HW, PRUNE)                                                                                              \
-  case V:                                                                                                                        \
-    return launch_overlapped(es == 2 ? compress_units_kernel<2, COUNT, HW, PRUNE> : compress_units_kernel<1, COUNT, HW, PRUNE>, grid, \
-                             dim3(kThreads), 0, s, 1, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)units_pad, log, \
-                             dropped, f8, ys, ldy * es);
+      auto launch = [&](auto kernel) {
+        return launch_streaming(kernel, grid, dim3(kThreads), s, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)units_pad, log,
+                                dropped, f8, ys, ldy * es);
+      };
+#define SP24_CU(V, COUNT, HW, PRUNE) \
+  case V:                            \
+    return es == 2 ? launch(Kernel<compress_units_kernel<2, COUNT, HW, PRUNE>>{}) : launch(Kernel<compress_units_kernel<1, COUNT, HW, PRUNE>>{});
       switch ((y ? 4 : 0) | (dropped ? 2 : 0) | (hw ? 1 : 0)) {
         SP24_CU(0, false, false, false)
         SP24_CU(1, false, true, false)
@@ -806,12 +809,13 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
     const dim3 grid((unsigned)units, (unsigned)steps, 1);
     const int wide = (by32(x, ldx) ? kWideX : 0) | (y && by32(y, ldy) ? kWideY : 0) | (whole_cells && ldv * es % 16 == 0 ? kWideVals : 0);
     const int variant = (y ? 8 : 0) | (dropped ? 4 : 0) | (hw ? 2 : 0) | (full ? 1 : 0);
-#define SP24_CV(V, COUNT, HW, FULL, PRUNE)                                                                                 \
-  case V:                                                                                                                  \
-    st = launch_overlapped(es == 2 ? compress_kernel<2, COUNT, HW, FULL, PRUNE> : compress_kernel<1, COUNT, HW, FULL, PRUNE>, grid, \
-                           dim3(kThreads), 0, s, 1, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)cells_pad, \
-                           shift, wide, dropped, f8, ys, ldy * es);                                                        \
-    break;
+    auto launch = [&](auto kernel) {
+      return launch_streaming(kernel, grid, dim3(kThreads), s, xs, ldx * es, vs, ldv * es, ms, M, K, (uint32_t)groups, (uint32_t)cells_pad, shift,
+                              wide, dropped, f8, ys, ldy * es);
+    };
+#define SP24_CV(V, COUNT, HW, FULL, PRUNE) \
+  case V:                                  \
+    return es == 2 ? launch(Kernel<compress_kernel<2, COUNT, HW, FULL, PRUNE>>{}) : launch(Kernel<compress_kernel<1, COUNT, HW, FULL, PRUNE>>{});
     switch (variant) {
       SP24_CV(0, false, false, false, false)
       SP24_CV(1, false, false, true, false)
@@ -832,7 +836,6 @@ sp24_status compress_any(sp24_dtype t, int64_t M, int64_t K, const void* x, int6
         SP24_CV(15, true, true, true, true)
     }
 #undef SP24_CV
-    return st;
   } else {
     if (y != nullptr) return SP24_ERR_UNSUPPORTED;
     int64_t bytes_pad = k_pad / 8, total = rows_pad * bytes_pad;

@@ -10,9 +10,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("layout", [0, 1])
 @pytest.mark.parametrize("pad,shift", [(0, 0), (16, 0), (0, 16), (8, 8)])
-@pytest.mark.parametrize("dtype,M,K", [("bf16", 9500, 16), ("bf16", 4745, 144), ("bf16", 4704, 256), ("bf16", 4705, 256),
-                                       ("bf16", 3200, 272), ("bf16", 2432, 512), ("i8", 9500, 48), ("i8", 4704, 512),
-                                       ("i8", 4705, 512), ("i8", 3200, 528), ("i8", 3201, 768)])
+@pytest.mark.parametrize("dtype,M,K", [("bf16", 14220, 16), ("bf16", 7113, 144), ("bf16", 7072, 256), ("bf16", 7073, 256),
+                                       ("bf16", 4750, 272), ("bf16", 3560, 512), ("i8", 14220, 48), ("i8", 7072, 512),
+                                       ("i8", 7073, 512), ("i8", 4750, 528), ("i8", 4751, 768)])
 def test_both_sides_of_the_line(dtype, M, K, pad, shift, layout):
     cells.test_units_against_the_oracle(dtype, M, K, pad, shift, layout)
 
